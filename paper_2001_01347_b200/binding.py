@@ -115,6 +115,19 @@ def _dev_ptr(t: torch.Tensor | None, dtype, numel: int, name: str) -> int | None
     return t.data_ptr()
 
 
+# The raw handle of a device's current stream without building a Stream object around it (0.2 against 2.2 us: a call on a
+# small instance is bound by what the host does before the launch).
+_raw_current_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None) or \
+    (lambda index: torch.cuda.current_stream(index).cuda_stream)
+
+
+def _stream(stream: torch.cuda.Stream | None, device: torch.device) -> int:
+    if stream is not None:
+        return stream.cuda_stream
+    index = device.index
+    return _raw_current_stream(torch.cuda.current_device() if index is None else index) if device.type == "cuda" else 0
+
+
 @dataclass
 class Selection:
     idx: torch.Tensor       # [B, n] int32
@@ -137,21 +150,22 @@ class ZipLine:
     # -- zl_select_batched ---------------------------------------------------------------
     def select_batched(self, ts: torch.Tensor, out: Selection | None = None, stream: torch.cuda.Stream | None = None) -> Selection:
         """ts: CUDA int64 [B, n, R].  Enqueues on ``stream`` (default: the current stream)."""
-        if ts.dim() != 3 or ts.shape[1] != self.n or ts.shape[2] != self.R:
+        shape = ts.shape
+        if len(shape) != 3 or shape[1] != self.n or shape[2] != self.R:
             raise ValueError(f"ts must be [B, {self.n}, {self.R}]")
-        B = ts.shape[0]
+        B = shape[0]
         if out is None:
             dev = ts.device
             out = Selection(torch.empty((B, self.n), dtype=torch.int32, device=dev),
                             torch.empty(B, dtype=torch.int64, device=dev),
                             torch.empty(B, dtype=torch.int64, device=dev),
                             torch.empty(B, dtype=torch.int32, device=dev))
-        s = stream if stream is not None else torch.cuda.current_stream(ts.device)
+        s = _stream(stream, ts.device)
         rc = lib.zl_select_batched(self._h, _dev_ptr(ts, torch.int64, B * self.n * self.R, "ts"), B,
                                    _dev_ptr(out.idx, torch.int32, B * self.n, "idx"),
                                    _dev_ptr(out.barrier, torch.int64, B, "barrier"),
                                    _dev_ptr(out.wait, torch.int64, B, "wait"),
-                                   _dev_ptr(out.status, torch.int32, B, "status"), s.cuda_stream)
+                                   _dev_ptr(out.status, torch.int32, B, "status"), s)
         _check(rc, "zl_select_batched")
         return out
 
@@ -168,13 +182,13 @@ class ZipLine:
                             torch.empty(B, dtype=torch.int64, device=dev),
                             torch.empty(B, dtype=torch.int64, device=dev),
                             torch.empty(B, dtype=torch.int32, device=dev))
-        s = stream if stream is not None else torch.cuda.current_stream(last.device)
+        s = _stream(stream, last.device)
         rc = lib.zl_predict_select_batched(self._h, _dev_ptr(last, torch.int64, B * self.n, "last"),
                                            _dev_ptr(interval, torch.int64, B * self.n, "interval"), B,
                                            _dev_ptr(out.idx, torch.int32, B * self.n, "idx"),
                                            _dev_ptr(out.barrier, torch.int64, B, "barrier"),
                                            _dev_ptr(out.wait, torch.int64, B, "wait"),
-                                           _dev_ptr(out.status, torch.int32, B, "status"), s.cuda_stream)
+                                           _dev_ptr(out.status, torch.int32, B, "status"), s)
         _check(rc, "zl_predict_select_batched")
         return out
 
@@ -272,9 +286,9 @@ def zl_predict_batched(last: torch.Tensor, interval: torch.Tensor, R: int,
     """Phase 1 of ZipLine: CUDA int64 [B, n] last end timestamps and intervals -> [B, n, R] predictions."""
     B, n = last.shape
     out = torch.empty((B, n, R), dtype=torch.int64, device=last.device)
-    s = stream if stream is not None else torch.cuda.current_stream(last.device)
+    s = _stream(stream, last.device)
     rc = lib.zl_predict_batched(_dev_ptr(last, torch.int64, B * n, "last"), _dev_ptr(interval, torch.int64, B * n, "interval"),
-                                B, n, R, out.data_ptr(), s.cuda_stream)
+                                B, n, R, out.data_ptr(), s)
     _check(rc, "zl_predict_batched")
     return out
 
@@ -288,9 +302,9 @@ def zl_gridscan_batched(ts: torch.Tensor, full: bool = False, stream: torch.cuda
     idx = torch.empty((B, n), dtype=torch.int32, device=dev)
     barrier = torch.empty(B, dtype=torch.int64, device=dev)
     wait = torch.empty(B, dtype=torch.int64, device=dev)
-    s = stream if stream is not None else torch.cuda.current_stream(dev)
+    s = _stream(stream, dev)
     rc = lib.zl_gridscan_batched(_dev_ptr(ts, torch.int64, B * n * R, "ts"), B, n, R, int(bool(full)),
-                                 scratch.data_ptr(), idx.data_ptr(), barrier.data_ptr(), wait.data_ptr(), s.cuda_stream)
+                                 scratch.data_ptr(), idx.data_ptr(), barrier.data_ptr(), wait.data_ptr(), s)
     _check(rc, "zl_gridscan_batched")
     return idx, barrier, wait
 
@@ -301,9 +315,9 @@ def zl_probe_read_batched(ts: torch.Tensor, count: torch.Tensor, sink: torch.Ten
     ts: CUDA int64 [..., R]; count: CUDA int32, one per row; sink: CUDA int64/uint64 scalar."""
     R = ts.shape[-1]
     rows = ts.numel() // R
-    s = stream if stream is not None else torch.cuda.current_stream(ts.device)
+    s = _stream(stream, ts.device)
     rc = lib.zl_probe_read_batched(_dev_ptr(ts, torch.int64, rows * R, "ts"), _dev_ptr(count, torch.int32, rows, "count"),
-                                   rows, R, sink.data_ptr(), s.cuda_stream)
+                                   rows, R, sink.data_ptr(), s)
     _check(rc, "zl_probe_read_batched")
 
 
@@ -322,12 +336,12 @@ def zl_select_batched_noalloc(ts: torch.Tensor, out: Selection, objective: int =
     caller's result tensors (this wrapper allocates nothing either).  Calls that overlap on the GPU
     race on the shared array; keep them on one stream."""
     B, n, R = ts.shape
-    s = stream if stream is not None else torch.cuda.current_stream(ts.device)
+    s = _stream(stream, ts.device)
     rc = lib.zl_select_batched_noalloc(n, R, objective, flags, _dev_ptr(ts, torch.int64, B * n * R, "ts"), B,
                                        _dev_ptr(out.idx, torch.int32, B * n, "idx"),
                                        _dev_ptr(out.barrier, torch.int64, B, "barrier"),
                                        _dev_ptr(out.wait, torch.int64, B, "wait"),
-                                       _dev_ptr(out.status, torch.int32, B, "status"), s.cuda_stream)
+                                       _dev_ptr(out.status, torch.int32, B, "status"), s)
     _check(rc, "zl_select_batched_noalloc")
     return out
 
@@ -341,8 +355,8 @@ def zl_trace_batched(ts: torch.Tensor, stream: torch.cuda.Stream | None = None) 
     """Per-position intermediates of the sweep for small instances; ts: CUDA int64 [B, n, R]."""
     B, n, R = ts.shape
     out = {k: torch.empty((B, n * R), dtype=dt, device=ts.device) for k, dt in TRACE_FIELDS}
-    s = stream if stream is not None else torch.cuda.current_stream(ts.device)
+    s = _stream(stream, ts.device)
     rc = lib.zl_trace_batched(_dev_ptr(ts, torch.int64, B * n * R, "ts"), B, n, R,
-                              *[out[k].data_ptr() for k, _ in TRACE_FIELDS], s.cuda_stream)
+                              *[out[k].data_ptr() for k, _ in TRACE_FIELDS], s)
     _check(rc, "zl_trace_batched")
     return out
