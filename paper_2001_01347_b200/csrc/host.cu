@@ -13,6 +13,8 @@
 //   sum_route.cu  the bucket route (SUM, and RANGE instances that are one shared-memory batch): the whole instance
 //                 is put into time order bucket by bucket.
 //   sweep.cu      the segment sweep (fallback of both fast routes) and k_finalize (K5).
+//   cells.cu      the cell route: branch and bound over time cells (both objectives, all but the smallest instances), and what it
+//                 leaves over; the routes above serve a handle's first calls and those the cells do not work out for.
 //   baselines.cu  GridScan / FullGridScan, the predictor, the per-position trace.
 #include <cuda_runtime.h>
 #include <stddef.h>
@@ -43,7 +45,7 @@ struct zl_handle {
     cudaStream_t s_stream;
     size_t staging_bytes;
     // options (0 = automatic)
-    int opt_threads, opt_lanes, opt_segments, opt_round_factor, opt_no_filter, opt_filter_threads, opt_filter_rows, opt_pdl_off, opt_prologue_threads, opt_tail_threads, opt_filter_round, opt_cluster, opt_filter_stages, opt_checks_off, opt_filter_bulk, opt_tail_cap, opt_max_rounds, opt_no_small, opt_rest_split;
+    int opt_threads, opt_lanes, opt_segments, opt_round_factor, opt_no_filter, opt_filter_threads, opt_filter_rows, opt_pdl_off, opt_prologue_threads, opt_tail_threads, opt_filter_round, opt_cluster, opt_filter_stages, opt_checks_off, opt_filter_bulk, opt_tail_cap, opt_max_rounds, opt_no_small, opt_rest_split, opt_no_cells, opt_cells;
     int epoch;               // calls so far: the two sets of per-call flags alternate
     int last_cuda_error;
     int launches;
@@ -56,6 +58,11 @@ struct zl_handle {
     // RANGE filter route: one word of pinned host memory that the last kernel of a call writes (did some instance have
     // more survivors than one CTA finishes?); the next call reads it, without waiting, to choose the form of its last stage
     uint32_t *h_hint, *d_hint;
+    // cell route
+    uint32_t *d_cflags;      // eight words, then the word last written to the hint
+    uint32_t cells_epoch;    // calls on the cell route
+    int cells_last;          // the previous call took the cell route
+    int cells_fails, cells_wait;   // calls it did not work out for so far; calls left until it is tried (again)
 };
 
 namespace {
@@ -65,6 +72,8 @@ using zl::Pipeline;
 using zl::pow2_ceil;
 using zl::pow2_floor;
 constexpr int PROF_EVENTS = 5;
+constexpr int CELLS_AFTER = 8;                 // calls of a handle before it tries the cell route
+constexpr int CELLS_MIN_WORKERS = 8;           // fewer workers: their few elements are sorted as cheaply, and the bounds of a cell are loose
 constexpr size_t CANARY_BYTES = 64;
 constexpr int CANARY_BYTE = 0xC5;
 
@@ -83,6 +92,10 @@ void enqueue(const Pipeline &q, const LaunchPlan &p, cudaStream_t st, cudaEvent_
     zl::FilterBufs fb = q.fb;
     if (!filter && !sumfast) memset(&fb, 0, sizeof(fb));
     if (ev) cudaEventRecord(ev[0], st);
+    if (q.cells) {
+        zl::enqueue_cells(q, q.fb, p, st, ev, src);
+        return;
+    }
     if constexpr (!arith) {
         if (q.small) {
             // a few thousand timestamps an instance: everything in one kernel
@@ -129,6 +142,7 @@ cudaError_t raise_shared_memory_limits() {
     cudaError_t e = zl::prologue_limits();
     if (e == cudaSuccess) e = zl::range_limits();
     if (e == cudaSuccess) e = zl::small_limits();
+    if (e == cudaSuccess) e = zl::cell_limits();
     if (e == cudaSuccess) e = zl::filter_limits();
     if (e == cudaSuccess) e = zl::heavy_limits();
     if (e == cudaSuccess) e = zl::range_rest_limits();
@@ -237,6 +251,7 @@ zl_status zl_create(const zl_config *cfg, zl_handle **out) {
     if (!h) return ZL_ERR_NOMEM;
     memset(h, 0, sizeof(*h));
     h->cfg = *cfg;
+    h->cells_wait = CELLS_AFTER;
     DeviceScope scope(cfg->device);                               // the caller's device is current again on return
     cudaError_t e = scope.err;
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, cfg->device);
@@ -285,10 +300,6 @@ zl_status zl_create(const zl_config *cfg, zl_handle **out) {
             filter_b += sizes[i];
         }
         if (e == cudaSuccess) e = cudaMemset(f.flags, 0, 128);      // two sets of eight per-call words, then words that outlive a call
-        if (e == cudaSuccess) e = cudaHostAlloc((void **)&h->h_hint, 64, cudaHostAllocMapped);
-        if (e == cudaSuccess) { memset(h->h_hint, 0, 64); e = cudaHostGetDevicePointer((void **)&h->d_hint, h->h_hint, 0); }
-        f.hint = h->d_hint;
-        f.hint_last = e == cudaSuccess ? f.flags + 16 : nullptr;
         if (cfg->flags & ZL_FLAG_DEBUG_CHECKS) {
             // the violation record, then 16 clock stamps per CTA of the head kernel and of the filter kernel
             const size_t dbg_b = 64 + (ctas + mb * ((size_t)cfg->n_workers + 1) / 2 + 1) * 16 * 8;
@@ -326,6 +337,15 @@ zl_status zl_create(const zl_config *cfg, zl_handle **out) {
             memset(&f, 0, sizeof(f));
         }
     }
+    if ((cfg->objective == ZL_OBJ_RANGE && !range_small) || (long long)cfg->n_workers * cfg->lookahead_R > zl::SMALL_MAX) {
+        // cell route, and the words by which a call tells the next one how it went
+        if (e == cudaSuccess) e = alloc((void **)&h->d_cflags, 128);
+        filter_b += 128;
+        if (e == cudaSuccess) e = cudaMemset(h->d_cflags, 0, 128);
+        if (e == cudaSuccess) e = cudaHostAlloc((void **)&h->h_hint, 64, cudaHostAllocMapped);
+        if (e == cudaSuccess) { memset(h->h_hint, 0, 64); e = cudaHostGetDevicePointer((void **)&h->d_hint, h->h_hint, 0); }
+        if (e == cudaSuccess) { h->fb.hint = h->d_hint; h->fb.hint_last = h->d_cflags + 16; }
+    }
     const size_t seg_b = (size_t)cfg->max_batch * h->nres * sizeof(zl::SegResult);
     if (e == cudaSuccess) e = alloc((void **)&h->d_meta, meta_b);
     if (e == cudaSuccess) e = alloc((void **)&h->d_seg, seg_b);
@@ -334,7 +354,7 @@ zl_status zl_create(const zl_config *cfg, zl_handle **out) {
     if (e == cudaSuccess) e = raise_shared_memory_limits();   // more than the default 48 KB of dynamic shared memory
     if (e != cudaSuccess) {
         zl_status st = cuda_fail(nullptr, e);
-        cudaFree(h->d_meta); cudaFree(h->d_seg); cudaFree(h->d_pred);
+        cudaFree(h->d_meta); cudaFree(h->d_seg); cudaFree(h->d_pred); cudaFree(h->d_cflags);
         if (h->h_hint) cudaFreeHost(h->h_hint);
         cudaFree(h->fb.table); cudaFree(h->fb.rowhint); cudaFree(h->fb.cellmax); cudaFree(h->fb.rcnt);
         cudaFree(h->fb.list1); cudaFree(h->fb.bcnt); cudaFree(h->fb.list2); cudaFree(h->fb.tilemax); cudaFree(h->fb.flags);
@@ -401,7 +421,7 @@ zl_status zl_profile_read(zl_handle *h, int32_t *calls, float *ms_stage) {
 zl_status zl_destroy(zl_handle *h) {
     if (!h) return ZL_OK;
     DeviceScope scope(h->cfg.device);
-    cudaFree(h->d_meta); cudaFree(h->d_seg); cudaFree(h->d_pred);
+    cudaFree(h->d_meta); cudaFree(h->d_seg); cudaFree(h->d_pred); cudaFree(h->d_cflags);
     cudaFree(h->fb.table); cudaFree(h->fb.rowhint); cudaFree(h->fb.cellmax); cudaFree(h->fb.rcnt);
     cudaFree(h->fb.list1); cudaFree(h->fb.bcnt); cudaFree(h->fb.list2); cudaFree(h->fb.tilemax); cudaFree(h->fb.flags);
     cudaFree(h->fb.bnd); cudaFree(h->fb.cellacc); cudaFree(h->fb.itab); cudaFree(h->fb.part); cudaFree(h->fb.ptab); cudaFree(h->fb.dbg); cudaFree(h->fb.done);
@@ -441,6 +461,10 @@ zl_status zl_set_option(zl_handle *h, const char *key, int32_t value) {
         h->opt_rest_split = value;                  // RANGE filter route, what the tail kernel leaves: 1 a kernel per phase, 2 the single last kernel
     } else if (!strcmp(key, "no_small")) {
         h->opt_no_small = value != 0;               // small instances take the route larger ones would (bucket route)
+    } else if (!strcmp(key, "cells")) {
+        h->opt_cells = value != 0;                  // the cell route from the first call on, whatever it leaves over
+    } else if (!strcmp(key, "no_cells")) {
+        h->opt_no_cells = value != 0;               // larger instances take the filter route (RANGE) or the bucket route (SUM)
     } else if (!strcmp(key, "max_rounds")) {
         h->opt_max_rounds = value;                  // the segment sweep gives up (ZL_ERR_TIMEOUT) after this many rounds of a segment
     } else if (!strcmp(key, "tail_cap")) {
@@ -488,9 +512,47 @@ static int rest_split_now(const zl_handle *h) {
     return h->h_hint && *(volatile const uint32_t *)h->h_hint != 0;
 }
 
+// The cell route: every shape above the one-launch sizes, unless the handle asks for another route (every timestamp
+// examined, self-checks, a tuning knob of the other routes).
+static bool cells_allowed(const zl_handle *h) {
+    return h->d_cflags && !h->opt_no_filter && !(h->cfg.flags & (ZL_FLAG_FULL_SWEEP | ZL_FLAG_DEBUG_CHECKS | ZL_FLAG_FORCE_FILTER)) &&
+           (long long)h->cfg.n_workers * h->cfg.lookahead_R > zl::SMALL_MAX && h->cfg.n_workers >= CELLS_MIN_WORKERS &&
+           !h->opt_filter_bulk && !h->opt_rest_split && !h->opt_filter_round && !h->opt_filter_threads &&
+           !h->opt_filter_rows && !h->opt_cluster && !h->opt_tail_cap && !h->opt_tail_threads && !h->opt_prologue_threads && !h->opt_no_cells;
+}
+// Whether the next call takes it.  A handle's first calls go down the other routes, whose time depends little on how the
+// timestamps fall; then the cells are tried, and stay for as long as they leave nothing over.  A call that did leave some
+// instance to the segment sweep (the word in pinned memory says so) sends the next ones down the other routes again, twice
+// as many after every such call.
+static bool cells_now(const zl_handle *h) {
+    if (!cells_allowed(h)) return false;
+    if (h->opt_cells) return true;
+    if (h->cells_last && ((volatile const uint32_t *)h->h_hint)[1] != 0) return false;
+    return h->cells_wait == 0;
+}
+// The decision at a call, and its bookkeeping.
+static bool cells_take(zl_handle *h) {
+    const bool now = cells_now(h);
+    if (h->cells_last && !now && cells_allowed(h)) {
+        ((volatile uint32_t *)h->h_hint)[1] = 0;
+        ++h->cells_fails;
+        h->cells_wait = CELLS_AFTER << std::min(h->cells_fails, 8);
+    } else if (!now && h->cells_wait > 0) {
+        --h->cells_wait;
+    }
+    h->cells_last = now;
+    return now;
+}
+static void set_cells(Pipeline &q, zl_handle *h) {
+    q.cells = !q.small && cells_take(h) ? 1 : 0;
+    q.cflags = h->d_cflags;
+    q.epoch = ++h->cells_epoch;
+}
+
 int32_t zl_launches_per_call(const zl_handle *h) {
     if (!h) return 0;
     if (small_route(h)) return 1;
+    if (cells_now(h)) return 2;
     const bool filter = h->cfg.objective == ZL_OBJ_RANGE && !h->opt_no_filter && h->fb.table != nullptr;
     const bool sumfast = !filter && !h->opt_no_filter && h->fb.scap != 0;
     return (filter ? (rest_split_now(h) ? 9 : 4) : 3) + (sumfast ? (h->fb.scells ? 3 : 2) : 0) + ((h->cfg.flags & ZL_FLAG_CHECK_SORTED) ? 1 : 0);
@@ -534,10 +596,11 @@ zl_status zl_select_batched(zl_handle *h, const int64_t *d_ts, int32_t B, int32_
         ++h->epoch;
     }
     q.idx = d_idx; q.barrier = d_barrier; q.wait = d_wait; q.status = d_status;
+    h->launches += zl_launches_per_call(h);
+    set_cells(q, h);
     enqueue(q, p, st, ev, zl::MatBatch{d_ts});
     if (ev) ++h->prof_calls;
     ZL_CUDA(h, cudaGetLastError());
-    h->launches += zl_launches_per_call(h);
     return ZL_OK;
 }
 
@@ -601,8 +664,8 @@ zl_status zl_predict_select_batched(zl_handle *h, const int64_t *d_last, const i
     if (!h || !h->d_pred) return ZL_ERR_INVALID_ARG;
     if (B < 1 || B > h->cfg.max_batch) return ZL_ERR_INVALID_ARG;
     if (!on_device(h->cfg.device)) return ZL_ERR_INVALID_ARG;
-    if (h->cfg.objective == ZL_OBJ_RANGE && h->fb.table != nullptr) {
-        // the filter route (and its fallback) on generated rows: the predicted matrix is never written
+    if ((h->cfg.objective == ZL_OBJ_RANGE && h->fb.table != nullptr) || cells_now(h)) {
+        // the cell route, or (RANGE) the filter route and its fallback, on generated rows: the predicted matrix is never written
         if (!d_last || !d_interval || !d_idx || !d_barrier || !d_wait) return ZL_ERR_INVALID_ARG;
         if (((uintptr_t)d_last & 7) || ((uintptr_t)d_interval & 7) || ((uintptr_t)d_barrier & 7) || ((uintptr_t)d_wait & 7) ||
             ((uintptr_t)d_idx & 3) || ((uintptr_t)d_status & 3))
@@ -611,7 +674,7 @@ zl_status zl_predict_select_batched(zl_handle *h, const int64_t *d_last, const i
         if (p.smem > 200 * 1024) return ZL_ERR_UNSUPPORTED;
         cudaEvent_t *ev = (h->prof_ev && h->prof_calls < h->prof_cap) ? h->prof_ev + PROF_EVENTS * (size_t)h->prof_calls : nullptr;
         Pipeline q;
-        q.ts = nullptr; q.B = B; q.n = h->cfg.n_workers; q.R = h->cfg.lookahead_R; q.objective = ZL_OBJ_RANGE;
+        q.ts = nullptr; q.B = B; q.n = h->cfg.n_workers; q.R = h->cfg.lookahead_R; q.objective = h->cfg.objective;
         q.flags = h->cfg.flags & ~ZL_FLAG_CHECK_SORTED; q.num_sms = h->num_sms;
         q.meta = h->d_meta; q.seg = h->d_seg; q.nres = h->nres;
         q.fb = h->fb;
@@ -627,10 +690,11 @@ zl_status zl_predict_select_batched(zl_handle *h, const int64_t *d_last, const i
             ++h->epoch;
         }
         q.idx = d_idx; q.barrier = d_barrier; q.wait = d_wait; q.status = d_status;
+        h->launches += zl_launches_per_call(h);
+        set_cells(q, h);
         enqueue(q, p, (cudaStream_t)cuda_stream, ev, zl::AriBatch{d_last, d_interval});
         if (ev) ++h->prof_calls;
         ZL_CUDA(h, cudaGetLastError());
-        h->launches += zl_launches_per_call(h);
         return ZL_OK;
     }
     zl_status rc = zl_predict_batched(d_last, d_interval, B, h->cfg.n_workers, h->cfg.lookahead_R, h->d_pred, cuda_stream);
@@ -675,7 +739,8 @@ namespace {
 constexpr int NOALLOC_MAX_BATCH = 256;
 constexpr int NOALLOC_MAX_SEGS = 16384;                       // B * (time segments per instance) of one call
 constexpr size_t NOALLOC_META_BYTES = (size_t)NOALLOC_MAX_BATCH * sizeof(zl::InstMeta);
-constexpr size_t NOALLOC_BYTES = NOALLOC_META_BYTES + (size_t)NOALLOC_MAX_SEGS * sizeof(zl::SegResult);
+constexpr size_t NOALLOC_WORD_BYTES = 256;                     // the cell route's words
+constexpr size_t NOALLOC_BYTES = NOALLOC_META_BYTES + NOALLOC_WORD_BYTES + (size_t)NOALLOC_MAX_SEGS * sizeof(zl::SegResult);
 static_assert(NOALLOC_META_BYTES % 256 == 0, "segment records must start on a 256-byte boundary");
 constexpr int NOALLOC_MAX_DEVICES = 64;
 }  // namespace
@@ -686,6 +751,7 @@ namespace {
 std::mutex g_noalloc_mutex;
 void *g_noalloc_ptr[NOALLOC_MAX_DEVICES];                     // device address of the array, per device
 int g_noalloc_sms[NOALLOC_MAX_DEVICES];
+uint32_t g_noalloc_calls[NOALLOC_MAX_DEVICES];
 }  // namespace
 
 int32_t zl_noalloc_max_batch(void) { return NOALLOC_MAX_BATCH; }
@@ -728,6 +794,7 @@ zl_status zl_select_batched_noalloc(int32_t n_workers, int32_t lookahead_R, int3
             g_noalloc_ptr[dev] = ptr;
         }
         tmp.num_sms = g_noalloc_sms[dev];
+        tmp.cells_epoch = ++g_noalloc_calls[dev];
     }
     const LaunchPlan p = make_plan(&tmp, B);
     if (p.smem > 200 * 1024) return ZL_ERR_UNSUPPORTED;
@@ -737,7 +804,7 @@ zl_status zl_select_batched_noalloc(int32_t n_workers, int32_t lookahead_R, int3
         return ZL_ERR_UNSUPPORTED;
     }
     zl::InstMeta *meta = (zl::InstMeta *)g_noalloc_ptr[dev];
-    zl::SegResult *seg = (zl::SegResult *)((unsigned char *)g_noalloc_ptr[dev] + NOALLOC_META_BYTES);
+    zl::SegResult *seg = (zl::SegResult *)((unsigned char *)g_noalloc_ptr[dev] + NOALLOC_META_BYTES + NOALLOC_WORD_BYTES);
     // Nothing in the scratch has to start at zero: the prologue rewrites every InstMeta of this call and
     // every sweep CTA rewrites its SegResult before finalize reads them, so the last call's contents are
     // never read.  (The filter path of the handle-based entry point needs two more buffers and is not used here.)
@@ -747,6 +814,8 @@ zl_status zl_select_batched_noalloc(int32_t n_workers, int32_t lookahead_R, int3
     memset(&q.fb, 0, sizeof(q.fb));
     q.filter_threads = q.filter_rows = q.filter_round = 0; q.pdl_off = 0; q.prologue_threads = q.tail_threads = 0; q.cluster = q.filter_stages = 0; q.checks_off = 0; q.filter_bulk = 0; q.tail_cap = 0; q.rest_per_sm = 0; q.max_rounds = 0; q.rest_split = 0; q.small = (long long)n_workers * lookahead_R <= zl::SMALL_MAX && B <= 4 * std::max(1, tmp.num_sms) ? 1 : 0;
     q.idx = d_idx; q.barrier = d_barrier; q.wait = d_wait; q.status = d_status;
+    q.cells = (long long)n_workers * lookahead_R > zl::SMALL_MAX && !(flags & ZL_FLAG_FULL_SWEEP) && n_workers >= CELLS_MIN_WORKERS ? 1 : 0;
+    q.cflags = (uint32_t *)((unsigned char *)g_noalloc_ptr[dev] + NOALLOC_META_BYTES); q.epoch = tmp.cells_epoch;
     enqueue(q, p, (cudaStream_t)cuda_stream, nullptr, zl::MatBatch{d_ts});
     return cudaGetLastError() == cudaSuccess ? ZL_OK : ZL_ERR_CUDA;
 }

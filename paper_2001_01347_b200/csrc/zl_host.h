@@ -36,6 +36,8 @@ struct Pipeline {
     int max_rounds;                                               // 0: automatic; else the segment sweep's round limit
     int rest_per_sm;                                              // CTAs of k_range_rest resident per SM (0: ask the runtime)
     int checks_off;                                               // debug handle: unchecked kernels, clock stamps still taken
+    int cells;                                                    // 1: the cell route
+    uint32_t *cflags, epoch;                                      // its eight words; the number of the call
     int32_t *idx; int64_t *barrier; int64_t *wait; int32_t *status;
 };
 
@@ -94,6 +96,11 @@ cudaError_t range_rest_limits();
 // sum_route.cu: the bucket route (plan, index pass, bucket kernel); `mid` is recorded before the bucket kernel
 void enqueue_bucket_route(const Pipeline &q, FilterBufs &fb, cudaStream_t st, cudaEvent_t mid);
 cudaError_t bucket_route_limits();
+
+// cells.cu: the cell route (both objectives): branch and bound over time cells, a cluster per instance in one launch
+void enqueue_cells(const Pipeline &q, const FilterBufs &fb, const LaunchPlan &p, cudaStream_t st, cudaEvent_t *ev, const MatBatch &src);
+void enqueue_cells(const Pipeline &q, const FilterBufs &fb, const LaunchPlan &p, cudaStream_t st, cudaEvent_t *ev, const AriBatch &src);
+cudaError_t cell_limits();
 
 // small.cu: the whole search for small instances in one launch
 void enqueue_small(const Pipeline &q, const LaunchPlan &p, cudaStream_t st, const MatBatch &src);

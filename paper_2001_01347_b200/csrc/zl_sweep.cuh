@@ -373,4 +373,29 @@ __device__ __forceinline__ RowEnds finalize_first_ends(const SRC &src, int B, in
     return row_ends(src, (int)(item / rc), (int)(item % rc), n, R);
 }
 
+// ------------------------------------------------------------------------------ grid-wide barrier
+constexpr unsigned GRID_POLL_LIMIT = 1u << 22;                     // polls of a grid-wide barrier before it gives up
+
+// Every CTA of the grid arrives at the counter; the k-th barrier of the kernel is passed when gridDim.x * k arrivals
+// have been counted.  What the CTAs wrote before the barrier is visible, past the L1 cache, to loads after it.  A CTA
+// that polls GRID_POLL_LIMIT times without seeing the count reports it through `gaveup` and goes on: the call then ends
+// with ZL_ERR_TIMEOUT for every instance instead of never ending.
+__device__ __forceinline__ bool grid_barrier(unsigned int *arrivals, unsigned int *gaveup, unsigned int k) {
+    __shared__ unsigned int ok;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        atomicAdd(arrivals, 1u);
+        const unsigned int want = gridDim.x * k;
+        unsigned int polls = 0;
+        bool seen = false;
+        while (!(seen = ldcg32(arrivals) >= want) && ++polls < GRID_POLL_LIMIT) __nanosleep(64);
+        if (!seen) atomicExch(gaveup, 1u);
+        __threadfence();
+        ok = seen;
+    }
+    __syncthreads();
+    return ok != 0;
+}
+
 }  // namespace zl
