@@ -40,8 +40,8 @@ constexpr int CELL_ALIVE = 128;           // most cells of an instance that the 
 constexpr int CELL_BATCH = 16;            // most cells that the rows are asked for at once
 constexpr int CELL_NODES = 1024;          // most elements in those
 constexpr int CELL_CLUSTER = 16;          // most CTAs of a cluster
-constexpr int CELL_FIRST = 4;             // most cells that are evaluated before any is discarded
-constexpr long long CELL_ASK = 8;         // asking a row for a cell costs about as much as looking through this many of its elements
+constexpr long long CELL_ASK = 16;        // asking a row for a cell costs about as much as looking through this many of its elements
+constexpr int CELL_FEW = 8;               // so many cells are asked for in any case
 constexpr int CELL_SLACK = 4;             // elements by which a row may be off its estimate before a further piece is read
 constexpr int GUARD_BINS = 64;            // rows by their span, eight bins to a factor of two below the longest
 constexpr float RANGE_CELLS = 100.f;      // RANGE: cells to the longest mean iteration
@@ -76,6 +76,13 @@ template <> struct RowReader<MatBatch> {
         for (int k = 0; k < 9; ++k) T[k] = (uint32_t)v[k] - tminlo;
     }
     __device__ __forceinline__ int align(int row, int i) const { return i - (int)(((uintptr_t)(inst + (size_t)row * R + i) >> 3) & 3u); }
+    __device__ __forceinline__ void prefetch(int row, int i) const {
+        const int64_t *p = inst + (size_t)row * R + i;
+        if (i >= 0 && i + 8 <= R) {
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(p + 4));
+        }
+    }
 };
 template <> struct RowReader<AriBatch> {
     const int64_t *last, *iv; int R; uint32_t tminlo;
@@ -91,6 +98,7 @@ template <> struct RowReader<AriBatch> {
         for (int k = 0; k < 9; ++k, t += v) T[k] = i + k - 1 < 0 ? 0u : i + k - 1 < R ? t : INF32;
     }
     __device__ __forceinline__ int align(int, int i) const { return i; }
+    __device__ __forceinline__ void prefetch(int, int) const {}
 };
 template <class RD>
 __device__ __forceinline__ uint32_t element(const RD &rd, int row, int i) { return i < 0 ? 0u : i < rd.R ? rd.in(row, i) : INF32; }
@@ -119,20 +127,35 @@ __device__ __forceinline__ void stream_rows(const RD &rd, int R, int row, bool h
     for (int d = 1; d < 32; d <<= 1) { const int y = __shfl_up_sync(FULL, incl, d); if (lane >= d) incl += y; }
     const int total = __shfl_sync(FULL, incl, 31);
     const int sb = s0 - 8 * (incl - np);                          // piece q of the warp starts at element sb + 8 q of its row
-#pragma unroll 1
-    for (int q0 = 0; q0 < total; q0 += 32) {
+    // the lane's piece of the 32 from q0 on: its row, its first element, whether it is its row's first or last one
+    int r = 0, ns = 0;
+    unsigned edge = 0;
+    auto assign = [&](int q0) {
         const int q = min(q0 + lane, total - 1);
         int j = 0;                                                // the lane whose row piece q belongs to
 #pragma unroll
         for (int d = 16; d > 0; d >>= 1) if (__shfl_sync(FULL, incl, j + d - 1) <= q) j += d;
-        const int r = __shfl_sync(FULL, row, j), end = __shfl_sync(FULL, incl, j), first = end - __shfl_sync(FULL, np, j);
-        int s = __shfl_sync(FULL, sb, j) + 8 * q;
-        if (q0 + lane < total) {
-            int back = q == first ? s : 0, fwd = q == end - 1 ? s + 8 : R + 1;     // where the row may have to be read on
+        const int end = __shfl_sync(FULL, incl, j), first = end - __shfl_sync(FULL, np, j);
+        r = __shfl_sync(FULL, row, j);
+        ns = __shfl_sync(FULL, sb, j) + 8 * q;
+        edge = (q == first ? 1u : 0u) | (q == end - 1 ? 2u : 0u);
+    };
+    if (total > 0) assign(0);
+#pragma unroll 1
+    for (int q0 = 0; q0 < total; q0 += 32) {
+        const bool mine = q0 + lane < total;
+        const int row_q = r;
+        int s = ns;
+        int back = (edge & 1u) ? s : 0, fwd = (edge & 2u) ? s + 8 : R + 1;     // where the row may have to be read on
+        if (q0 + 32 < total) {                                    // the next piece on its way to the L2 while this one is worked on
+            assign(q0 + 32);
+            if (q0 + 32 + lane < total) rd.prefetch(r, ns);
+        }
+        if (mine) {
 #pragma unroll 1
             for (;;) {
                 uint32_t T[9];
-                rd.eight(r, s, T);
+                rd.eight(row_q, s, T);
                 act(T);
                 if (s <= back && (s <= 0 || T[0] < a)) back = 0;  // the row's start of the range is covered
                 if (s + 8 >= fwd && T[8] >= b) fwd = R + 1;       // ... and its end
@@ -222,10 +245,10 @@ struct CellParams {
 struct CellShared {
     // from every CTA of the cluster (each array is written by the others before one cluster barrier and read after it, so no
     // two exchanges share one): minima and maxima of its rows' ends; whether one of its rows decreases; SUM its rows' wait at
-    // the sample time; the key of its best cell, and S there
+    // the sample time; the key of its best cell, and G or S at its start
     unsigned long long ex[4][CELL_CLUSTER], exc[CELL_CLUSTER], exs[CELL_CLUSTER], exv[CELL_CLUSTER], exb[CELL_CLUSTER];
-    unsigned long long red[4][16];
-    unsigned long long acc, total, key;
+    unsigned long long red[4][32];
+    unsigned long long acc, total, key, kbase;
     uint32_t hist[GUARD_BINS];
     float span;                                   // RANGE: rows of at least this span are guards
     unsigned long long later;                     // RANGE: about how many timestamps of the other rows lie in the range
@@ -234,8 +257,7 @@ struct CellShared {
     uint64_t base[CELL_ALIVE];                    // RANGE: a lower bound of G at the cell's start, SUM: S there
     uint64_t lb[CELL_ALIVE];                      // lower bound of the objective in the cell
     unsigned short order[CELL_ALIVE];
-    unsigned int ncells, nfirst;
-    uint32_t done[CELL_FIRST];                    // cells evaluated before the list was made
+    unsigned int ncells;
     uint32_t gmaxl[CELL_BATCH], gminl[CELL_BATCH];   // RANGE: latest and earliest of the own rows' first elements at or after the cell's start
     // in the first CTA: what the rows answered
     uint32_t gmax[CELL_BATCH], gmin[CELL_BATCH];  // RANGE: ... of all rows'
@@ -340,7 +362,7 @@ __device__ __noinline__ bool evaluate_cells(CellShared &sh, int from, int ns, co
 // Dynamic shared memory: the slice's cells [cap + 4] u32 | rows' first and last element, relative [n] uint2 | SUM: per 128
 // cells the scan before them and the smallest lower bound among them [cap / 128] two u64.
 template <int OBJ, class SRC>
-__global__ void __launch_bounds__(512, 2) k_cells(const SRC src, const CellParams P) {
+__global__ void __launch_bounds__(1024, 1) k_cells(const SRC src, const CellParams P) {
     grid_dep_wait();
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ CellShared sh;
@@ -373,7 +395,7 @@ __global__ void __launch_bounds__(512, 2) k_cells(const SRC src, const CellParam
             if (lane == 0) sh.red[k][warp] = q[k];
         }
         if (tid == 0) {
-            sh.acc = 0; sh.total = 0; sh.key = ~0ull; sh.ncells = 0; sh.nfirst = 0; sh.nnodes = 0; sh.sstatus = 0; sh.later = 0;
+            sh.acc = 0; sh.total = 0; sh.key = ~0ull; sh.ncells = 0; sh.nnodes = 0; sh.sstatus = 0; sh.later = 0;
             sh.best.d = sh.best.t = ~0ull; sh.best.valid = 0; sh.best.status = 0;
         }
         if (tid < CELL_BATCH) { sh.gmax[tid] = sh.gmaxl[tid] = 0; sh.gmin[tid] = sh.gminl[tid] = INF32; }
@@ -532,10 +554,10 @@ __global__ void __launch_bounds__(512, 2) k_cells(const SRC src, const CellParam
     const int m = (int)(c1 - c0), nblk = (m + 127) >> 7;
     const uint32_t a = lo + (c0 << shift), bnd = c1 == ncells ? hi : lo + (c1 << shift);
     bool fits = true;
+    uint32_t gap = 0;                                             // RANGE: no cell's bound is below this
 #pragma unroll 1
     for (int stage = 0;; ++stage) {                               // RANGE: the guards, then (seldom) the other rows too
         // ---- the rows' elements in the slice
-        const uint32_t gap = stage ? (uint32_t)min(sh.best.d, (uint64_t)(INF32 - 1u)) : 0u;
         if (m > 0) {
             uint64_t carry = 0, total = 0;                        // SUM: the rows' last elements before a, and all deltas in the slice
             const uint32_t w = bnd - a;
@@ -557,7 +579,7 @@ __global__ void __launch_bounds__(512, 2) k_cells(const SRC src, const CellParam
                         // cell[k] becomes a lower bound of G at the start of cell k (before the prefix maximum): an element
                         // says that G is at least its successor for the cells after its own.  Elements before the slice
                         // count for its first cell; those in its last cell or behind it go to cell[m], which is not looked
-                        // at.  A gap of at most `gap` cannot push a cell's bound, G less the cell's end, beyond that.
+                        // at.  A gap of at most `gap` cannot push a cell's bound, G less the cell's end, beyond that: it discards no cell.
                         uint32_t longer = 0;
 #pragma unroll
                         for (int j = 0; j < 8; ++j) longer = max(longer, T[j + 1] - T[j]);
@@ -611,7 +633,6 @@ __global__ void __launch_bounds__(512, 2) k_cells(const SRC src, const CellParam
             uint32_t run = t0;
 #pragma unroll 1
             for (int w = 0; w < warp; ++w) run = max(run, (uint32_t)sh.red[0][w]);
-            uint32_t lbm = INF32, at = 0;
 #pragma unroll 1
             for (int k = k0; k < k1; ++k) {
                 uint4 v = *reinterpret_cast<const uint4 *>(cell + 128 * k + 4 * lane);
@@ -624,15 +645,16 @@ __global__ void __launch_bounds__(512, 2) k_cells(const SRC src, const CellParam
                 v.x = max(v.x, before); v.y = max(v.y, before); v.z = max(v.z, before); v.w = max(v.w, before);
                 *reinterpret_cast<uint4 *>(cell + 128 * k + 4 * lane) = v;
                 run = max(run, __shfl_sync(FULL, inc, 31));
+                // the most promising cell: the smallest G(start) - end.  (The optimum lies where G is about to rise.)
                 const uint32_t g[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     const int c = 128 * k + 4 * lane + j;
-                    const uint32_t end = min(a + ((uint32_t)(c + 1) << shift) - 1u, bnd - 1u), l = g[j] > end ? g[j] - end : 0u;
-                    if (c < m && l < lbm) { lbm = l; at = (uint32_t)c; }
+                    const uint32_t end = min(a + ((uint32_t)(c + 1) << shift) - 1u, bnd - 1u);
+                    const uint64_t q = (uint64_t)(g[j] > end ? g[j] - end : 0u) << 24 | (c0 + (uint32_t)c + 1u);      // never 0
+                    if (c < m && g[j] != INF32 && q < key) { key = q; kbase = g[j]; }
                 }
             }
-            if (lbm != INF32) key = (uint64_t)lbm << 24 | (c0 + at + 1u);        // never 0
         } else {
             uint64_t run = sh.acc, all = 0;
 #pragma unroll 1
@@ -667,57 +689,43 @@ __global__ void __launch_bounds__(512, 2) k_cells(const SRC src, const CellParam
             // a cell's 32-bit sum wrapped around: nothing in the slice can be trusted
             if (all != sh.total) fits = false;
         }
-        if (stage == 0) {
+        {
             const uint64_t mine = warp_reduce(key, OpMin());
             if (lane == 0) atomicMin(&sh.key, (unsigned long long)mine);
             __syncthreads();
-            if (OBJ == ZL_OBJ_SUM && key != ~0ull && key == sh.key) sh.acc = kbase;      // (keys are different)
+            if (key != ~0ull && key == sh.key) sh.kbase = kbase;  // (keys are different)
             __syncthreads();
             if (tid < G) {
                 CellShared &to = *cl.map_shared_rank(&sh, tid);
                 to.exv[rank] = fits ? sh.key : 0ull;
-                if (OBJ == ZL_OBJ_SUM) to.exb[rank] = sh.acc;
-            }
-            cl.sync();
-            if (OBJ == ZL_OBJ_SUM) {
-#pragma unroll 1
-                for (int r = 0; r < G; ++r) fits &= sh.exv[r] != 0ull;
-                if (!fits) break;
-            }
-            // ---- the most promising cells, one of a slice and CELL_FIRST of them at most, exactly
-            if (tid == 0) {
-                unsigned k = 0;
-                uint64_t low = 0;
-#pragma unroll 1
-                while (k < (unsigned)CELL_FIRST) {
-                    uint64_t q = ~0ull;
-                    int from = 0;
-#pragma unroll 1
-                    for (int r = 0; r < G; ++r) if (sh.exv[r] > low && sh.exv[r] < q) { q = sh.exv[r]; from = r; }
-                    if (q == ~0ull) break;
-                    low = q;
-                    const uint32_t c = (uint32_t)(q & 0xffffffu) - 1u, l = (uint32_t)(q >> 24);
-                    sh.done[k] = sh.cell[k] = c; sh.order[k] = (unsigned short)k;
-                    sh.base[k] = OBJ == ZL_OBJ_SUM ? (uint64_t)sh.exb[from] : l ? (uint64_t)l + min(lo + ((c + 1) << shift) - 1u, hi - 1u) : 0ull;
-                    ++k;
-                }
-                sh.nfirst = k;
-            }
-            __syncthreads();
-            const int first = (int)sh.nfirst;
-            if (first) {
-                fits = evaluate_cells<OBJ>(sh, 0, first, rd, ends, n, R, r0, nrows, lo, hi, shift);
-                if (!fits) break;
+                to.exb[rank] = sh.kbase;
             }
         }
-        if (rank == 0 && tid == 0) sh.ncells = 0;
-        cl.sync();                                                // the list is empty (and, after a first stage, its length has been read)
+        cl.sync();
+        uint64_t best_key = sh.exv[0];
+        int owner = 0;
+#pragma unroll 1
+        for (int r = 0; r < G; ++r) {
+            fits &= sh.exv[r] != 0ull;
+            if (sh.exv[r] < best_key) { best_key = sh.exv[r]; owner = r; }
+        }
+        if (!fits || best_key == ~0ull) { fits = false; break; }
+        // ---- the most promising cell exactly
+        const uint32_t primary = (uint32_t)(best_key & 0xffffffu) - 1u;
+        if (OBJ == ZL_OBJ_RANGE) gap = (uint32_t)(best_key >> 24);
+        if (tid == 0) {
+            sh.cell[0] = primary; sh.order[0] = 0;
+            sh.base[0] = sh.exb[owner];
+            if (rank == 0) sh.ncells = 0;
+        }
+        __syncthreads();
+        fits = evaluate_cells<OBJ>(sh, 0, 1, rd, ends, n, R, r0, nrows, lo, hi, shift);
+        if (!fits) break;
         // ---- the cells that may still hold a smaller one, or the same one earlier
         const uint64_t d = sh.best.d;
         CellShared &ld = *cl.map_shared_rank(&sh, 0);
         auto keep = [&](uint32_t c, uint64_t base, uint64_t l) {
-#pragma unroll 1
-            for (unsigned i = 0; i < sh.nfirst; ++i) if (sh.done[i] == c) return;
+            if (c == primary) return;
             const unsigned pos = atomicAdd(&ld.ncells, 1u);
             if (pos < CELL_ALIVE) {
                 // every CTA gets the list
@@ -763,9 +771,8 @@ __global__ void __launch_bounds__(512, 2) k_cells(const SRC src, const CellParam
         const int ns = (int)ld.ncells;
         if (ns == 0) break;
         // asking every row for each of them, or looking through the other rows first?
-        if (OBJ == ZL_OBJ_RANGE && stage == 0 && sh.span > 0.f && (ns > CELL_ALIVE || (long long)ns * n * CELL_ASK > (long long)sh.later)) {
-            cl.sync();                                            // everybody has read the length
-            continue;
+        if (OBJ == ZL_OBJ_RANGE && stage == 0 && sh.span > 0.f && (ns > CELL_ALIVE || (ns > CELL_FEW && (long long)ns * n * CELL_ASK > (long long)sh.later))) {
+            continue;                                             // (a cluster barrier follows before the length is touched again)
         }
         if (ns > CELL_ALIVE) { fits = false; break; }
 #pragma unroll 1
@@ -777,7 +784,7 @@ __global__ void __launch_bounds__(512, 2) k_cells(const SRC src, const CellParam
             sh.order[at] = (unsigned short)k;
         }
         __syncthreads();
-        const int batch = max(4, min(CELL_BATCH, 4 * nt / P.rpc));
+        const int batch = max(4, min(CELL_BATCH, 2 * nt / P.rpc));
 #pragma unroll 1
         for (int from = 0; from < ns && fits; from += batch) {
             if (sh.lb[sh.order[from]] > sh.best.d) break;
@@ -838,22 +845,24 @@ struct CellShape { int cluster, threads, cap; size_t smem; };
 
 static CellShape cell_shape(int n, int R, int B, int objective, int num_sms) {
     CellShape s;
-    // CTAs: about two for every SM, each with 16 rows at least to ask; clusters of 16 only for the largest instances, of which
-    // few fill the GPU
+    // CTAs: as many as there are SMs, each with 16 rows at least to ask; clusters of 16 only for the largest instances, of
+    // which few fill the GPU.  Threads: as many as an SM holds (clusters of 16: for two CTAs an SM, or not all of eight
+    // clusters find room at once), one to so many timestamps (RANGE looks through an eighth of them).
     const int most = (long long)n * R >= (1 << 22) ? CELL_CLUSTER : 8;
     s.cluster = 1;
-    while (s.cluster < most && (long long)B * s.cluster * 2 <= 2LL * num_sms && n / (s.cluster * 2) >= 16) s.cluster *= 2;
+    while (s.cluster < most && (long long)B * s.cluster * 2 <= num_sms && n / (s.cluster * 2) >= 16) s.cluster *= 2;
     const long long ctas = (long long)B * s.cluster;
-    s.threads = ctas > 4LL * num_sms ? 128 : ctas > 2LL * num_sms ? 256 : 512;
-    s.threads = (int)std::min<long long>(s.threads, std::max<long long>(128, 32 * (((long long)n * R / s.cluster + 1023) / 1024)));
+    s.threads = ctas > 4LL * num_sms ? 128 : ctas > 2LL * num_sms ? 256 : ctas > num_sms || s.cluster > 8 ? 512 : 1024;
+    const int per_thread = 32 * (objective == ZL_OBJ_RANGE ? 48 : 16);
+    s.threads = (int)std::min<long long>(s.threads, std::max<long long>(128, 32 * (((long long)n * R / s.cluster + per_thread - 1) / per_thread)));
     // Cells an instance can use.  RANGE: RANGE_CELLS to an iteration of the slowest row, of which there are rarely more than
-    // half R before the first row runs out.  SUM: see SUM_WIDTH, about 3 sqrt(n) cells an iteration.  No more than lets the
+    // half R before the first row runs out.  SUM: see SUM_WIDTH, 3 to 6 sqrt(n) cells an iteration.  No more than lets the
     // CTAs of the call (up to eight an SM) be resident together: they are bound by latency, not by what they move.
-    double want = objective == ZL_OBJ_RANGE ? RANGE_CELLS * 0.5 * R : 3.0 * R * std::sqrt((double)n);
+    double want = objective == ZL_OBJ_RANGE ? RANGE_CELLS * 0.5 * R : 6.0 * R * std::sqrt((double)n);
     want = std::max(256.0, std::min(want, (double)(1 << 18)));
-    const long long per_sm = std::max<long long>(2, std::min<long long>(8, (ctas + num_sms - 1) / num_sms));
+    const long long per_sm = s.cluster > 8 ? 2 : std::max<long long>(1, std::min<long long>(8, (ctas + num_sms - 1) / num_sms));
     const double cell_bytes = objective == ZL_OBJ_RANGE ? 4.0 : 4.125;
-    const double room = ((224.0 * 1024 / (double)per_sm) - sizeof(CellShared) - 1024 - 8.0 * n - 64) / cell_bytes;
+    const double room = (std::min(200.0, 224.0 / (double)per_sm) * 1024 - sizeof(CellShared) - 1024 - 8.0 * n - 64) / cell_bytes;
     const int most_cells = std::max(2048, (int)room & ~127);
     s.cap = std::min(most_cells, ((int)(want / s.cluster) + 127) & ~127);
     s.cap = std::max(256, s.cap);
