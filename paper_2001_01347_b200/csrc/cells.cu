@@ -5,7 +5,7 @@
 // search is branch and bound over the cells:
 //   RANGE  The best Z whose minimum is at time t has max(Z) = G(t) = max over the rows of their first element at or after t,
 //          so d = G(T) - T, and every candidate of a cell has d >= G(start) - end.  G is set by the rows with long
-//          iterations: the slowest fifth of the rows or so ("guards": an eighth of the timestamps) give a lower bound of G
+//          iterations: the slowest fifth to half of the rows ("guards": an eighth of the timestamps or so) give a lower bound of G
 //          at every cell's start - a maximum per cell, then a prefix maximum.  The cells with the smallest bounds are
 //          evaluated exactly (every row is asked for its elements in them: a search from the row's ends, a few loads); the
 //          smallest d discards nearly all other cells, and the ones it does not are evaluated the same way, most promising
@@ -41,9 +41,11 @@ constexpr int CELL_BATCH = 16;            // most cells that the rows are asked 
 constexpr int CELL_NODES = 1024;          // most elements in those
 constexpr int CELL_CLUSTER = 16;          // most CTAs of a cluster
 constexpr long long CELL_ASK = 16;        // asking a row for a cell costs about as much as looking through this many of its elements
+constexpr int CELL_ROUNDS = 48;           // most cells evaluated one by one before an instance is given up
 constexpr int CELL_FEW = 8;               // so many cells are asked for in any case
 constexpr int CELL_SLACK = 4;             // elements by which a row may be off its estimate before a further piece is read
 constexpr int GUARD_BINS = 64;            // rows by their span, eight bins to a factor of two below the longest
+constexpr float GUARD_IRREGULAR = 32.f;   // bins by which more rows are looked through, to a unit of their gaps' relative deviation above 0.1
 constexpr float RANGE_CELLS = 100.f;      // RANGE: cells to the longest mean iteration
 constexpr float SUM_WIDTH = 0.23f;        // SUM: n cell widths against the spread of the wait over time (see k_cells)
 
@@ -246,7 +248,9 @@ struct CellShared {
     // from every CTA of the cluster (each array is written by the others before one cluster barrier and read after it, so no
     // two exchanges share one): minima and maxima of its rows' ends; whether one of its rows decreases; SUM its rows' wait at
     // the sample time; the key of its best cell, and G or S at its start
-    unsigned long long ex[4][CELL_CLUSTER], exc[CELL_CLUSTER], exs[CELL_CLUSTER], exv[CELL_CLUSTER], exb[CELL_CLUSTER];
+    unsigned long long ex[4][CELL_CLUSTER];
+    float exi[CELL_CLUSTER];                      // RANGE: how irregular its rows are (sum over a few of them, see k_cells)
+    unsigned long long exc[CELL_CLUSTER], exs[CELL_CLUSTER], exv[CELL_CLUSTER], exb[CELL_CLUSTER];
     unsigned long long red[4][32];
     unsigned long long acc, total, key, kbase;
     uint32_t hist[GUARD_BINS];
@@ -379,10 +383,19 @@ __global__ void __launch_bounds__(1024, 1) k_cells(const SRC src, const CellPara
     {
         const typename SRC::Rows rows = src.inst(b, n, R);
         uint64_t q[4] = {~0ull, 0, ~0ull, 0};                     // order-preserving unsigned images of int64
+        float irr = 0.f;
+        const int step = (n + 31) / 32;
 #pragma unroll 1
         for (int p = tid; p < nrows; p += nt) {
             const auto row = rows.row(r0 + p);
             const int64_t x = row.at(0), y = row.at(R - 1);
+            if (OBJ == ZL_OBJ_RANGE && R > 2 && (r0 + p) % step == 0) {
+                // RANGE, a few dozen rows: how far the row's middle element is from where a row of equal gaps has it, in gaps: after h of R - 1
+                // gaps with a standard deviation of s (in gaps) that is s * sqrt(h * (R - 1 - h) / (R - 1)) on average
+                const int h = (R - 1) / 2;
+                const float span = (float)(y - x), off = (float)(row.at(h) - x) * (float)(R - 1) - span * (float)h;
+                if (span > 0.f) irr += off * off / (span * span) * ((float)(R - 1) / ((float)h * (float)(R - 1 - h)));
+            }
             const uint64_t ux = (uint64_t)x ^ (1ull << 63), uy = (uint64_t)y ^ (1ull << 63);
             q[0] = min(q[0], ux); q[1] = max(q[1], ux); q[2] = min(q[2], uy); q[3] = max(q[3], uy);
             const uint2 e = make_uint2((uint32_t)(uint64_t)x, (uint32_t)(uint64_t)y);
@@ -393,6 +406,10 @@ __global__ void __launch_bounds__(1024, 1) k_cells(const SRC src, const CellPara
         for (int k = 0; k < 4; ++k) {
             q[k] = (k & 1) ? warp_reduce(q[k], OpMax()) : warp_reduce(q[k], OpMin());
             if (lane == 0) sh.red[k][warp] = q[k];
+        }
+        if (OBJ == ZL_OBJ_RANGE) {
+            irr = warp_sum(irr);
+            if (lane == 0) sh.tmp[warp] = (uint64_t)__float_as_uint(irr);
         }
         if (tid == 0) {
             sh.acc = 0; sh.total = 0; sh.key = ~0ull; sh.ncells = 0; sh.nnodes = 0; sh.sstatus = 0; sh.later = 0;
@@ -408,6 +425,12 @@ __global__ void __launch_bounds__(1024, 1) k_cells(const SRC src, const CellPara
 #pragma unroll 1
             for (int w = 1; w < nw; ++w) v = (k & 1) ? max(v, sh.red[k][w]) : min(v, sh.red[k][w]);
             cl.map_shared_rank(&sh, r)->ex[k][rank] = v;
+            if (OBJ == ZL_OBJ_RANGE && k == 0) {
+                float v = 0.f;
+#pragma unroll 1
+                for (int w = 0; w < nw; ++w) v += __uint_as_float((uint32_t)sh.tmp[w]);
+                cl.map_shared_rank(&sh, r)->exi[rank] = v;
+            }
         }
     }
 #pragma unroll 1
@@ -476,7 +499,13 @@ __global__ void __launch_bounds__(1024, 1) k_cells(const SRC src, const CellPara
 #pragma unroll 1
         for (int w = 1; w < nw; ++w) longest = max(longest, (uint32_t)sh.red[0][w]);
         if (OBJ == ZL_OBJ_RANGE) {
-            // guards: the rows of the longest spans, a fifth of them at least, and those within a few per cent of these
+            // Guards: the rows that can set G near the optimum.  At a random time row i's next element is uniform in its mean
+            // gap m_i away, so all are within x with probability prod(x / m_i) over the rows with m_i > x; the smallest d of
+            // about N = n * R tries is the x where sum(log(m_i / x)) reaches log(N), and rows with gaps shorter than that
+            // hardly matter.  With the rows counted by the logarithm of their span that is a prefix sum of a prefix sum.  Rows
+            // a bin shorter are taken along, and more of them where single gaps are much longer than the row's mean.  (A fifth
+            // to a half of the rows on the workloads at hand.  A fixed fifth leaves dozens of cells where single gaps are
+            // long: n=1024, R=1024, B=64 87 us; a fixed half costs n=128, R=256, B=1024 68 us instead of 53.)
             const int top = __float_as_int((float)longest) >> 20;
 #pragma unroll 1
             for (int p = tid; p < n; p += nt) {
@@ -485,14 +514,24 @@ __global__ void __launch_bounds__(1024, 1) k_cells(const SRC src, const CellPara
             }
             __syncthreads();
             if (warp == 0) {
-                const uint32_t want = (uint32_t)max(n / 5, min(n, 8));
                 const uint32_t x0 = sh.hist[2 * lane], x1 = sh.hist[2 * lane + 1];
-                uint32_t inc = x0 + x1;
+                uint32_t inc = x0 + x1;                           // rows in the bins up to the lane's second one
 #pragma unroll
                 for (int d = 1; d < 32; d <<= 1) { const uint32_t y = __shfl_up_sync(FULL, inc, d); if (lane >= d) inc += y; }
-                const uint32_t exc = inc - x0 - x1;
-                const int k = __reduce_min_sync(FULL, exc + x0 >= want ? 2 * lane : inc >= want ? 2 * lane + 1 : GUARD_BINS);
-                if (lane == 0) sh.span = k >= GUARD_BINS - 1 ? 0.f : 0.95f * __int_as_float((top - k) << 20);
+                const uint32_t n0 = inc - x1, n1 = inc;           // rows up to bin 2 lane, 2 lane + 1
+                uint32_t dep = n0 + n1;                           // sum of these over the bins: (bin - own bin) over the rows, from the next bin on
+#pragma unroll
+                for (int d = 1; d < 32; d <<= 1) { const uint32_t y = __shfl_up_sync(FULL, dep, d); if (lane >= d) dep += y; }
+                const uint32_t d0 = dep - n0 - n1, d1 = dep - n1; // that sum at bin 2 lane, 2 lane + 1
+                const uint32_t tries = (uint32_t)(8.f * log2f((float)n * (float)R)), least = (uint32_t)min(n, 8);
+                int k = __reduce_min_sync(FULL, d0 >= tries ? 2 * lane : d1 >= tries ? 2 * lane + 1 : GUARD_BINS);
+                float irr = 0.f;
+#pragma unroll 1
+                for (int r = 0; r < G; ++r) irr += sh.exi[r];
+                const float dev = sqrtf(irr / (float)((n + (n + 31) / 32 - 1) / ((n + 31) / 32)));
+                k += 1 + (int)(GUARD_IRREGULAR * max(0.f, min(1.f, dev) - 0.1f));
+                k = max(k, __reduce_min_sync(FULL, n0 >= least ? 2 * lane : n1 >= least ? 2 * lane + 1 : GUARD_BINS));
+                if (lane == 0) sh.span = k >= min(GUARD_BINS - 1, top) ? 0.f : __int_as_float((top - k) << 20);
             }
             __syncthreads();
             const float span = sh.span;
@@ -555,10 +594,12 @@ __global__ void __launch_bounds__(1024, 1) k_cells(const SRC src, const CellPara
     const uint32_t a = lo + (c0 << shift), bnd = c1 == ncells ? hi : lo + (c1 << shift);
     bool fits = true;
     uint32_t gap = 0;                                             // RANGE: no cell's bound is below this
+    uint64_t low = 0;                                             // cells with keys up to this have been evaluated
+    int stage = 0, streamed = -1;                                 // RANGE: 0 the guards, 1 (seldom) the other rows too
 #pragma unroll 1
-    for (int stage = 0;; ++stage) {                               // RANGE: the guards, then (seldom) the other rows too
+    for (int round = 0;; ++round) {                               // a round: the most promising cell is evaluated, the rest counted
         // ---- the rows' elements in the slice
-        if (m > 0) {
+        if (m > 0 && streamed != stage) {
             uint64_t carry = 0, total = 0;                        // SUM: the rows' last elements before a, and all deltas in the slice
             const uint32_t w = bnd - a;
 #pragma unroll 1
@@ -611,6 +652,7 @@ __global__ void __launch_bounds__(1024, 1) k_cells(const SRC src, const CellPara
                 if (lane == 0) { atomicAdd(&sh.acc, (unsigned long long)carry); atomicAdd(&sh.total, (unsigned long long)total); }
             }
         }
+        streamed = stage;
         __syncthreads();
         // ---- what the sweep knows at every cell's start; a warp takes a run of 128-cell blocks, four cells a lane
         const int bpw = (nblk + nw - 1) / nw, k0 = min(warp * bpw, nblk), k1 = min(k0 + bpw, nblk);
@@ -652,7 +694,7 @@ __global__ void __launch_bounds__(1024, 1) k_cells(const SRC src, const CellPara
                     const int c = 128 * k + 4 * lane + j;
                     const uint32_t end = min(a + ((uint32_t)(c + 1) << shift) - 1u, bnd - 1u);
                     const uint64_t q = (uint64_t)(g[j] > end ? g[j] - end : 0u) << 24 | (c0 + (uint32_t)c + 1u);      // never 0
-                    if (c < m && g[j] != INF32 && q < key) { key = q; kbase = g[j]; }
+                    if (c < m && g[j] != INF32 && q > low && q < key) { key = q; kbase = g[j]; }
                 }
             }
         } else {
@@ -679,7 +721,7 @@ __global__ void __launch_bounds__(1024, 1) k_cells(const SRC src, const CellPara
                         const uint64_t u = nn * end - S[j], l = nn * start > S[j] ? nn * start - S[j] : 0ull;
                         lbm = min(lbm, l);
                         const uint64_t q = min(u, (uint64_t)0xffffffffffull) << 24 | (c0 + (uint32_t)c + 1u);
-                        if (q < key) { key = q; kbase = S[j] - dv[j]; }
+                        if (q > low && q < key) { key = q; kbase = S[j] - dv[j]; }
                     }
                 }
                 lbm = warp_reduce(lbm, OpMin());
@@ -711,10 +753,10 @@ __global__ void __launch_bounds__(1024, 1) k_cells(const SRC src, const CellPara
         }
         if (!fits || best_key == ~0ull) { fits = false; break; }
         // ---- the most promising cell exactly
-        const uint32_t primary = (uint32_t)(best_key & 0xffffffu) - 1u;
-        if (OBJ == ZL_OBJ_RANGE) gap = (uint32_t)(best_key >> 24);
+        if (OBJ == ZL_OBJ_RANGE && round == 0) gap = (uint32_t)(best_key >> 24);
+        low = best_key;
         if (tid == 0) {
-            sh.cell[0] = primary; sh.order[0] = 0;
+            sh.cell[0] = (uint32_t)(best_key & 0xffffffu) - 1u; sh.order[0] = 0;
             sh.base[0] = sh.exb[owner];
             if (rank == 0) sh.ncells = 0;
         }
@@ -725,7 +767,6 @@ __global__ void __launch_bounds__(1024, 1) k_cells(const SRC src, const CellPara
         const uint64_t d = sh.best.d;
         CellShared &ld = *cl.map_shared_rank(&sh, 0);
         auto keep = [&](uint32_t c, uint64_t base, uint64_t l) {
-            if (c == primary) return;
             const unsigned pos = atomicAdd(&ld.ncells, 1u);
             if (pos < CELL_ALIVE) {
                 // every CTA gets the list
@@ -742,7 +783,7 @@ __global__ void __launch_bounds__(1024, 1) k_cells(const SRC src, const CellPara
                 for (int j = 0; j < 4; ++j) {
                     const uint32_t end = min(a + ((uint32_t)(c + j + 1) << shift) - 1u, bnd - 1u);
                     const uint64_t l = g[j] > end ? (uint64_t)(g[j] - end) : 0ull;
-                    if (c + j < m && l <= d) keep(c0 + (uint32_t)(c + j), g[j], l);
+                    if (c + j < m && l <= d && (l << 24 | (c0 + (uint32_t)(c + j) + 1u)) > low) keep(c0 + (uint32_t)(c + j), g[j], l);
                 }
             }
         } else {
@@ -761,8 +802,10 @@ __global__ void __launch_bounds__(1024, 1) k_cells(const SRC src, const CellPara
                 for (int j = 0; j < 4; ++j) {
                     const uint32_t c = (uint32_t)(128 * k + 4 * lane + j);
                     if (dv[j] != 0u) {
-                        const uint64_t st = (uint64_t)n * (a + (c << shift)), l = st > S[j] ? st - S[j] : 0ull;
-                        if (l <= d) keep(c0 + c, S[j] - dv[j], l);
+                        const uint32_t start = a + (c << shift), end = min(start + ((1u << shift) - 1u), bnd - 1u);
+                        const uint64_t st = (uint64_t)n * start, l = st > S[j] ? st - S[j] : 0ull;
+                        const uint64_t q = min((uint64_t)n * end - S[j], (uint64_t)0xffffffffffull) << 24 | (c0 + c + 1u);
+                        if (l <= d && q > low) keep(c0 + c, S[j] - dv[j], l);
                     }
                 }
             }
@@ -772,9 +815,14 @@ __global__ void __launch_bounds__(1024, 1) k_cells(const SRC src, const CellPara
         if (ns == 0) break;
         // asking every row for each of them, or looking through the other rows first?
         if (OBJ == ZL_OBJ_RANGE && stage == 0 && sh.span > 0.f && (ns > CELL_ALIVE || (ns > CELL_FEW && (long long)ns * n * CELL_ASK > (long long)sh.later))) {
+            stage = 1; low = 0;
             continue;                                             // (a cluster barrier follows before the length is touched again)
         }
-        if (ns > CELL_ALIVE) { fits = false; break; }
+        if (ns > CELL_ALIVE) {                                    // more than there is room for: the next best cell may discard them
+            fits = round < CELL_ROUNDS;
+            if (fits) continue;
+            break;
+        }
 #pragma unroll 1
         for (int k = tid; k < ns; k += nt) {                      // most promising first
             const uint64_t l = sh.lb[k];

@@ -1,0 +1,110 @@
+"""The cell route (branch and bound over time cells) against the CPU oracle at the sizes where it can go wrong.  Whole numbers:
+every comparison is exact."""
+import numpy as np
+import pytest
+import torch
+
+import oracle as o
+import zl_inputs as zi
+
+pytestmark = pytest.mark.gpu
+
+if torch.cuda.is_available():
+    import paper_2001_01347_b200 as zl
+
+
+def select(ts, objective, flags=0):
+    B, n, R = ts.shape
+    h = zl.ZipLine(n, R, B, objective, 0, flags)
+    h.set_option("cells", 1)
+    assert h.launches_per_call == 2
+    sel = h.select_batched(torch.from_numpy(np.ascontiguousarray(ts)).cuda())
+    torch.cuda.synchronize()
+    left = h.filter_counts(B)[2]
+    h.destroy()
+    return sel, left
+
+
+def assert_oracle(ts, objective, sel):
+    for b in range(ts.shape[0]):
+        w, t, idx = o.sweep_window(ts[b], objective)
+        assert int(sel.status[b]) == 0
+        assert (int(sel.wait[b]), int(sel.barrier[b])) == (w, t), b
+        assert (sel.idx[b].cpu().numpy() == idx).all(), b
+
+
+@pytest.mark.parametrize("objective", [0, 1])
+@pytest.mark.parametrize("n,R,B", [(8, 513, 3), (8, 5000, 2), (15, 300, 5), (17, 257, 160), (31, 133, 9), (33, 129, 2), (63, 67, 700),
+                                   (97, 211, 40), (128, 33, 20), (255, 65, 1), (257, 64, 7), (1000, 15, 1), (1025, 9, 3), (4096, 2, 2),
+                                   (4095, 130, 1)])
+def test_shapes_around_the_pieces_slices_and_clusters(n, R, B, objective):
+    # rows of odd length and start (pieces of eight elements on 32-byte boundaries), row counts around the CTAs of a
+    # cluster, batches that change its size; spread workers with rare long iterations, so that estimates are off
+    w = zi.CONFIGS["c4"].with_(B=B, n=n, R=R)
+    ts = zi.generate(w, first_instance=n)
+    sel, left = select(ts, objective)
+    assert max(left) == 0 or n < 16
+    assert_oracle(ts, objective, sel)
+
+
+@pytest.mark.parametrize("objective", [0, 1])
+def test_ties_flat_rows_and_far_from_arithmetic(objective):
+    rng = np.random.default_rng(5 + objective)
+    for n, R, B, hi in ((40, 120, 6, 3), (100, 60, 4, 2), (300, 30, 3, 40)):
+        ts = (rng.integers(0, 5, size=(B, n, 1)) + np.cumsum(rng.integers(0, hi, size=(B, n, R)), axis=2)).astype(np.int64)
+        assert_oracle(ts, objective, select(ts, objective)[0])
+    inc = np.where(rng.random((9, 64, 100)) < 0.02, 5000, rng.integers(1, 30, size=(9, 64, 100)))
+    assert_oracle(np.cumsum(inc, axis=2), objective, select(np.cumsum(inc, axis=2).astype(np.int64), objective)[0])
+    ts = np.full((2, 70, 60), 77, dtype=np.int64)                  # one timestamp everywhere
+    assert_oracle(ts, objective, select(ts, objective)[0])
+
+
+@pytest.mark.parametrize("objective", [0, 1])
+def test_what_the_cells_leave_over_and_errors(objective):
+    # one batch: a regular instance, one whose span needs 64 bits (segment sweep), identical rows, an unsorted one, a
+    # negative timestamp
+    n, R = 64, 128
+    regular = zi.generate(zi.CONFIGS["c3"].with_(B=1, n=n, R=R))[0]
+    same = np.broadcast_to(np.cumsum(np.arange(1, R + 1)) * 1000, (n, R))
+    unsorted = regular.copy()
+    unsorted[5, 60] = unsorted[5, 58] - 1
+    negative = regular.copy()
+    negative[3, 0] = -4
+    ts = np.stack([regular, regular * 50_000, same, unsorted, negative, regular + 9]).astype(np.int64)
+    sel, left = select(ts, objective, zl.ZL_FLAG_CHECK_SORTED)
+    bad = [0, 0, 0, zl.binding.ZL_ERR_UNSORTED, zl.binding.ZL_ERR_INVALID_ARG, 0]
+    assert sel.status.tolist() == bad
+    assert (sel.idx[3:5] == -1).all() and (sel.wait[3:5] == np.iinfo(np.int64).min).all()
+    keep = [0, 1, 2, 5]
+    assert_oracle(ts[keep], objective, zl.Selection(sel.idx[keep], sel.barrier[keep], sel.wait[keep], sel.status[keep]))
+
+
+@pytest.mark.parametrize("objective", [0, 1])
+def test_predicted_rows(objective):
+    rng = np.random.default_rng(11)
+    for n, R, B in ((16, 300, 5), (100, 150, 3), (513, 200, 2)):
+        iv = np.maximum(1, (100_000 * np.exp(0.5 * rng.standard_normal((B, n)))).astype(np.int64))
+        last = rng.integers(0, 100_000, size=(B, n))
+        h = zl.ZipLine(n, R, B, objective, 0, zl.ZL_FLAG_PREDICTOR)
+        h.set_option("cells", 1)
+        sel = h.predict_select_batched(torch.from_numpy(last).cuda(), torch.from_numpy(iv).cuda())
+        torch.cuda.synchronize()
+        assert_oracle(np.stack([o.predict(last[b], iv[b], R) for b in range(B)]), objective, sel)
+        h.destroy()
+
+
+def test_a_handle_takes_the_route_after_its_first_calls_and_leaves_it_when_it_fails():
+    n, R = 64, 128
+    good = torch.from_numpy(zi.generate(zi.CONFIGS["c3"].with_(B=4, n=n, R=R))).cuda()
+    wide = good * 50_000                                           # every instance is left to the segment sweep
+    h = zl.ZipLine(n, R, 4, 0)
+    ref = h.select_batched(good)
+    for _ in range(9):
+        h.select_batched(good)
+    assert h.launches_per_call == 2
+    a = h.select_batched(good)
+    b = h.select_batched(wide)
+    torch.cuda.synchronize()
+    assert torch.equal(a.idx, ref.idx) and torch.equal(a.wait, ref.wait) and torch.equal(a.barrier, ref.barrier)
+    assert torch.equal(b.idx, ref.idx) and torch.equal(b.wait, ref.wait * 50_000)
+    h.destroy()
