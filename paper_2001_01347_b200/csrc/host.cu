@@ -13,6 +13,8 @@
 //   sum_route.cu  the bucket route (SUM, and RANGE instances that are one shared-memory batch): the whole instance
 //                 is put into time order bucket by bucket.
 //   sweep.cu      the segment sweep (fallback of both fast routes) and k_finalize (K5).
+//   small.cu      instances of a few thousand timestamps in one launch, a CTA each; walk.cu: the same for RANGE and few workers,
+//                 a warp each.
 //   cells.cu      the cell route: branch and bound over time cells (both objectives, all but the smallest instances), and what it
 //                 leaves over; the routes above serve a handle's first calls and those the cells do not work out for.
 //   baselines.cu  GridScan / FullGridScan, the predictor, the per-position trace.
@@ -45,7 +47,7 @@ struct zl_handle {
     cudaStream_t s_stream;
     size_t staging_bytes;
     // options (0 = automatic)
-    int opt_threads, opt_lanes, opt_segments, opt_round_factor, opt_no_filter, opt_filter_threads, opt_filter_rows, opt_pdl_off, opt_prologue_threads, opt_tail_threads, opt_filter_round, opt_cluster, opt_filter_stages, opt_checks_off, opt_filter_bulk, opt_tail_cap, opt_max_rounds, opt_no_small, opt_rest_split, opt_no_cells, opt_cells;
+    int opt_threads, opt_lanes, opt_segments, opt_round_factor, opt_no_filter, opt_filter_threads, opt_filter_rows, opt_pdl_off, opt_prologue_threads, opt_tail_threads, opt_filter_round, opt_cluster, opt_filter_stages, opt_checks_off, opt_filter_bulk, opt_tail_cap, opt_max_rounds, opt_no_small, opt_rest_split, opt_no_cells, opt_cells, opt_no_walk;
     int epoch;               // calls so far: the two sets of per-call flags alternate
     int last_cuda_error;
     int launches;
@@ -97,6 +99,11 @@ void enqueue(const Pipeline &q, const LaunchPlan &p, cudaStream_t st, cudaEvent_
         return;
     }
     if constexpr (!arith) {
+        if (q.walk) {
+            zl::enqueue_walk(q, st);
+            if (ev) for (int k = 1; k < PROF_EVENTS; ++k) cudaEventRecord(ev[k], st);
+            return;
+        }
         if (q.small) {
             // a few thousand timestamps an instance: everything in one kernel
             zl::enqueue_small(q, p, st, src);
@@ -143,6 +150,7 @@ cudaError_t raise_shared_memory_limits() {
     if (e == cudaSuccess) e = zl::range_limits();
     if (e == cudaSuccess) e = zl::small_limits();
     if (e == cudaSuccess) e = zl::cell_limits();
+    if (e == cudaSuccess) e = zl::walk_limits();
     if (e == cudaSuccess) e = zl::filter_limits();
     if (e == cudaSuccess) e = zl::heavy_limits();
     if (e == cudaSuccess) e = zl::range_rest_limits();
@@ -461,6 +469,8 @@ zl_status zl_set_option(zl_handle *h, const char *key, int32_t value) {
         h->opt_rest_split = value;                  // RANGE filter route, what the tail kernel leaves: 1 a kernel per phase, 2 the single last kernel
     } else if (!strcmp(key, "no_small")) {
         h->opt_no_small = value != 0;               // small instances take the route larger ones would (bucket route)
+    } else if (!strcmp(key, "no_walk")) {
+        h->opt_no_walk = value != 0;                // small RANGE instances take a CTA each (one launch, or the bucket route)
     } else if (!strcmp(key, "cells")) {
         h->opt_cells = value != 0;                  // the cell route from the first call on, whatever it leaves over
     } else if (!strcmp(key, "no_cells")) {
@@ -502,6 +512,12 @@ size_t zl_workspace_bytes(const zl_handle *h) { return h ? h->ws_bytes + h->stag
 static bool small_route(const zl_handle *h) {
     return (long long)h->cfg.n_workers * h->cfg.lookahead_R <= zl::SMALL_MAX && h->cfg.max_batch <= 4 * std::max(1, h->num_sms) &&
            !h->opt_no_filter && !h->opt_no_small && !(h->cfg.flags & ZL_FLAG_FORCE_FILTER);
+}
+
+// RANGE, small instances of few workers, whatever the batch: a warp each (walk.cu).
+static bool walk_route(const zl_handle *h) {
+    return h->cfg.objective == ZL_OBJ_RANGE && zl::walk_shape(h->cfg.n_workers, h->cfg.lookahead_R) && !h->opt_no_filter && !h->opt_no_small &&
+           !h->opt_no_walk && !(h->cfg.flags & (ZL_FLAG_FORCE_FILTER | ZL_FLAG_FULL_SWEEP | ZL_FLAG_DEBUG_CHECKS));
 }
 
 // The form of the RANGE filter route's last stage for the handle's next call: a kernel per phase when the shape is large,
@@ -551,7 +567,7 @@ static void set_cells(Pipeline &q, zl_handle *h) {
 
 int32_t zl_launches_per_call(const zl_handle *h) {
     if (!h) return 0;
-    if (small_route(h)) return 1;
+    if (small_route(h) || walk_route(h)) return 1;
     if (cells_now(h)) return 2;
     const bool filter = h->cfg.objective == ZL_OBJ_RANGE && !h->opt_no_filter && h->fb.table != nullptr;
     const bool sumfast = !filter && !h->opt_no_filter && h->fb.scap != 0;
@@ -588,7 +604,7 @@ zl_status zl_select_batched(zl_handle *h, const int64_t *d_ts, int32_t B, int32_
     q.prologue_threads = h->opt_prologue_threads; q.tail_threads = h->opt_tail_threads;
     if (h->opt_no_filter) { q.fb.table = nullptr; q.fb.scap = 0; }
     q.cluster = h->opt_cluster; q.filter_stages = h->opt_filter_stages;
-    q.checks_off = h->opt_checks_off; q.filter_bulk = h->opt_filter_bulk; q.tail_cap = h->opt_tail_cap; q.rest_per_sm = 0; q.max_rounds = h->opt_max_rounds; q.small = small_route(h) ? 1 : 0; q.rest_split = rest_split_now(h) ? 1 : 2;
+    q.checks_off = h->opt_checks_off; q.filter_bulk = h->opt_filter_bulk; q.tail_cap = h->opt_tail_cap; q.rest_per_sm = 0; q.max_rounds = h->opt_max_rounds; q.small = small_route(h) ? 1 : 0; q.walk = walk_route(h) ? 1 : 0; q.rest_split = rest_split_now(h) ? 1 : 2;
     if (q.fb.flags) {                           // the two sets of per-call flags alternate; a call zeroes the next call's set
         uint32_t *base = h->fb.flags;
         q.fb.flags = base + 8 * (h->epoch & 1);
@@ -682,7 +698,7 @@ zl_status zl_predict_select_batched(zl_handle *h, const int64_t *d_last, const i
         q.prologue_threads = h->opt_prologue_threads; q.tail_threads = h->opt_tail_threads;
         if (h->opt_no_filter) { q.fb.table = nullptr; q.fb.scap = 0; }
         q.cluster = h->opt_cluster; q.filter_stages = h->opt_filter_stages;
-        q.checks_off = h->opt_checks_off; q.filter_bulk = h->opt_filter_bulk; q.tail_cap = h->opt_tail_cap; q.rest_per_sm = 0; q.max_rounds = h->opt_max_rounds; q.small = small_route(h) ? 1 : 0; q.rest_split = rest_split_now(h) ? 1 : 2;
+        q.checks_off = h->opt_checks_off; q.filter_bulk = h->opt_filter_bulk; q.tail_cap = h->opt_tail_cap; q.rest_per_sm = 0; q.max_rounds = h->opt_max_rounds; q.small = small_route(h) ? 1 : 0; q.walk = walk_route(h) ? 1 : 0; q.rest_split = rest_split_now(h) ? 1 : 2;
         if (q.fb.flags) {                           // the two sets of per-call flags alternate; a call zeroes the next call's set
             uint32_t *base = h->fb.flags;
             q.fb.flags = base + 8 * (h->epoch & 1);
@@ -814,6 +830,7 @@ zl_status zl_select_batched_noalloc(int32_t n_workers, int32_t lookahead_R, int3
     memset(&q.fb, 0, sizeof(q.fb));
     q.filter_threads = q.filter_rows = q.filter_round = 0; q.pdl_off = 0; q.prologue_threads = q.tail_threads = 0; q.cluster = q.filter_stages = 0; q.checks_off = 0; q.filter_bulk = 0; q.tail_cap = 0; q.rest_per_sm = 0; q.max_rounds = 0; q.rest_split = 0; q.small = (long long)n_workers * lookahead_R <= zl::SMALL_MAX && B <= 4 * std::max(1, tmp.num_sms) ? 1 : 0;
     q.idx = d_idx; q.barrier = d_barrier; q.wait = d_wait; q.status = d_status;
+    q.walk = objective == ZL_OBJ_RANGE && !(flags & ZL_FLAG_FULL_SWEEP) && zl::walk_shape(n_workers, lookahead_R) ? 1 : 0;
     q.cells = (long long)n_workers * lookahead_R > zl::SMALL_MAX && !(flags & ZL_FLAG_FULL_SWEEP) && n_workers >= CELLS_MIN_WORKERS ? 1 : 0;
     q.cflags = (uint32_t *)((unsigned char *)g_noalloc_ptr[dev] + NOALLOC_META_BYTES); q.epoch = tmp.cells_epoch;
     enqueue(q, p, (cudaStream_t)cuda_stream, nullptr, zl::MatBatch{d_ts});

@@ -33,6 +33,7 @@ struct Pipeline {
     int tail_cap;                                                 // 0: default; else survivors the finishing CTA of the filter kernel has room for
     int rest_split;                                               // RANGE filter route's last stage: 0 by shape, 1 a kernel per phase, 2 the single kernel
     int small;                                                    // 1: the one-launch route (instances of a few thousand timestamps)
+    int walk;                                                     // 1: RANGE, small instances, a warp each
     int max_rounds;                                               // 0: automatic; else the segment sweep's round limit
     int rest_per_sm;                                              // CTAs of k_range_rest resident per SM (0: ask the runtime)
     int checks_off;                                               // debug handle: unchecked kernels, clock stamps still taken
@@ -101,6 +102,11 @@ cudaError_t bucket_route_limits();
 void enqueue_cells(const Pipeline &q, const FilterBufs &fb, const LaunchPlan &p, cudaStream_t st, cudaEvent_t *ev, const MatBatch &src);
 void enqueue_cells(const Pipeline &q, const FilterBufs &fb, const LaunchPlan &p, cudaStream_t st, cudaEvent_t *ev, const AriBatch &src);
 cudaError_t cell_limits();
+
+// walk.cu: RANGE, small instances of up to 128 workers, a warp per instance in one launch
+bool walk_shape(int n, int R);
+void enqueue_walk(const Pipeline &q, cudaStream_t st);
+cudaError_t walk_limits();
 
 // small.cu: the whole search for small instances in one launch
 void enqueue_small(const Pipeline &q, const LaunchPlan &p, cudaStream_t st, const MatBatch &src);
