@@ -181,7 +181,7 @@ STAGES = {  # names of what runs between the library's stage events, by route
     1: ("k_range_head", "k_filter", "k_tail", "k_range_rest"),     # large shapes: the last stage is one kernel per phase
     2: ("k_prologue", "k_sum_plan+k_sum_index", "k_sum_buckets+k_sweep", "k_finalize"),
     0: ("k_prologue", "-", "k_sweep", "k_finalize"),
-    3: ("k_small", "-", "-", "-"),
+    3: ("k_small or k_walk", "-", "-", "-"),
 }
 
 
@@ -304,7 +304,8 @@ def main():
     t_main = timed(h, args.steps, args.warmup)                           # the headline: no per-stage events in the stream
     t_prof = timed(h, max(3, min(args.steps, 20)), 3, profile=True, inner=max(1, t_main["inner"] // 4))   # stage events serialise the stages
     status_ok = bool((t_main["sel"].status == 0).all().item())
-    launches = h.launches_per_call * t_main["calls"]
+    h_launches = h.launches_per_call
+    launches = h_launches * t_main["calls"]
     ms_step = t_main["total_ms"] / t_main["calls"]
     value = world * nts / (ms_step * 1e-3)
 
@@ -359,7 +360,7 @@ def main():
 
     # ---- roofline of the dominant kernel: algorithmic bytes = 8 per timestamp it must examine
     peak, peak_kind = measured_peak_gbs()
-    names = STAGES[route]
+    names = STAGES[3] if h_launches == 1 else ("k_cells", "-", "-", "k_cell_rest") if h_launches == 2 else STAGES[route]
 
     def dominant(pr):
         stages = {}

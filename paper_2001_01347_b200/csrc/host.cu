@@ -516,7 +516,7 @@ static bool small_route(const zl_handle *h) {
 
 // RANGE, small instances of few workers, whatever the batch: a warp each (walk.cu).
 static bool walk_route(const zl_handle *h) {
-    return h->cfg.objective == ZL_OBJ_RANGE && zl::walk_shape(h->cfg.n_workers, h->cfg.lookahead_R) && !h->opt_no_filter && !h->opt_no_small &&
+    return h->cfg.objective == ZL_OBJ_RANGE && zl::walk_shape(h->cfg.n_workers, h->cfg.lookahead_R, h->cfg.max_batch, std::max(1, h->num_sms)) && !h->opt_no_filter && !h->opt_no_small &&
            !h->opt_no_walk && !(h->cfg.flags & (ZL_FLAG_FORCE_FILTER | ZL_FLAG_FULL_SWEEP | ZL_FLAG_DEBUG_CHECKS));
 }
 
@@ -830,7 +830,7 @@ zl_status zl_select_batched_noalloc(int32_t n_workers, int32_t lookahead_R, int3
     memset(&q.fb, 0, sizeof(q.fb));
     q.filter_threads = q.filter_rows = q.filter_round = 0; q.pdl_off = 0; q.prologue_threads = q.tail_threads = 0; q.cluster = q.filter_stages = 0; q.checks_off = 0; q.filter_bulk = 0; q.tail_cap = 0; q.rest_per_sm = 0; q.max_rounds = 0; q.rest_split = 0; q.small = (long long)n_workers * lookahead_R <= zl::SMALL_MAX && B <= 4 * std::max(1, tmp.num_sms) ? 1 : 0;
     q.idx = d_idx; q.barrier = d_barrier; q.wait = d_wait; q.status = d_status;
-    q.walk = objective == ZL_OBJ_RANGE && !(flags & ZL_FLAG_FULL_SWEEP) && zl::walk_shape(n_workers, lookahead_R) ? 1 : 0;
+    q.walk = objective == ZL_OBJ_RANGE && !(flags & ZL_FLAG_FULL_SWEEP) && zl::walk_shape(n_workers, lookahead_R, B, std::max(1, tmp.num_sms)) ? 1 : 0;
     q.cells = (long long)n_workers * lookahead_R > zl::SMALL_MAX && !(flags & ZL_FLAG_FULL_SWEEP) && n_workers >= CELLS_MIN_WORKERS ? 1 : 0;
     q.cflags = (uint32_t *)((unsigned char *)g_noalloc_ptr[dev] + NOALLOC_META_BYTES); q.epoch = tmp.cells_epoch;
     enqueue(q, p, (cudaStream_t)cuda_stream, nullptr, zl::MatBatch{d_ts});

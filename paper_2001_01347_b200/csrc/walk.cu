@@ -1,23 +1,25 @@
 // k_walk: the RANGE search for instances of a few thousand timestamps of up to 128 workers, a warp per instance, in one launch.
 // Nothing is sorted and no barrier but the warp's own is passed.
 //
-// The best selection whose minimum is at time t has max(Z) = G(t) = max over the rows of their first element at or after t.
-// The timeline up to the first exhausted row is cut into a few hundred cells.  One pass over the elements (a maximum of `next`
-// per cell, then a prefix maximum) gives G at every cell's start: every candidate of a cell has d >= G(start) - end, and a
-// cell that raises G holds one with d <= G(next start) - start.  A second pass collects the elements that raise G in the
-// cells that the smallest of these upper bounds does not discard - a few dozen - and each of them gets its exact d from the
-// others of its cell.  More of them than there is room for (many equal times): the rows are walked from barrier to barrier.
+// The best selection whose minimum is the element at time T has max(Z) = G(T) = max over the rows of their first element at or
+// after T, and only elements whose passing raises G matter.  The timeline up to the first exhausted row is cut into a few
+// hundred cells; one pass over the elements (a maximum of `next` per cell, then a prefix maximum) gives G at every cell's
+// start and so a lower bound of every element's d.  The element with the smallest bound is evaluated exactly - a row a lane,
+// a search in shared memory -, a second pass collects the ones that its d does not discard (a few, rarely dozens), and these
+// are evaluated in the order of their bounds until none is left below the smallest d.  More of them than there is room for
+// (many equal times): the rows are walked from barrier to barrier.
 #include "zl_batch.cuh"
 #include "zl_host.h"
 
 namespace zl {
 
-constexpr int WALK_MAX_R = 256;
+constexpr int WALK_ALONE = 256;
 constexpr int WALK_MAX_CELLS = 512;
+constexpr int WALK_PASSES = 24;            // most passes that take a single candidate
 constexpr unsigned WALK_NODES = 128;       // room for candidates
 
 struct WalkParams {
-    int n, R, B, stride, cells, words, check_sorted;      // stride: words between rows in shared memory (odd: no bank conflicts by row)
+    int n, R, B, stride, cells, words, check_sorted;      // stride: words between rows in shared memory: R and one that reads as infinite
     const int64_t *ts;
     int32_t *idx; int64_t *barrier; int64_t *wait; int32_t *status;
 };
@@ -89,97 +91,113 @@ __device__ __forceinline__ int first_from(const ROWS &rows, int p, int R, typena
 
 // The cells of an instance and what they leave.  cell: `most` (a power of two, at least 64) words plus 32, node: WALK_NODES, both
 // the warp's.  False: more candidates than there is room for.
+template <int K>
 __device__ __forceinline__ bool search_cells(const NarrowRows &rows, int n, int R, uint32_t t0, uint32_t lmin, uint32_t *cell, int most, uint64_t *node,
                                              uint32_t &bd, uint32_t &bt) {
-    const int lane = threadIdx.x & 31, N = n * R;
+    const int lane = threadIdx.x & 31, N = n * rows.stride;       // all words of the rows, one after the other
     const int per = most / 32, ps = __ffs(per) - 1;               // a run of cells a lane; cell c sits at c + c / per (no bank conflicts)
-    int sh = 0;
-    while (((lmin - 1u) >> sh) >= (uint32_t)most) ++sh;
-    const int m = (int)((lmin - 1u) >> sh) + 1;                   // cells: cell c holds the times (c << sh) + 1 .. (c + 1) << sh
+    // (T - 1) < lmin for every T <= lmin, so its cell ((T - 1) * scale) >> 32 is below `most`
+    const uint32_t scale = (uint32_t)min((uint64_t)0xffffffffu, ((uint64_t)most << 32) / lmin);
+    auto cell_at = [&](uint32_t T) { const uint32_t k = __umulhi(T - 1u, scale); return cell + k + (k >> ps); };
 #pragma unroll 1
     for (int c = lane; c < most + 32; c += 32) cell[c] = t0;
     __syncwarp();
     // cell c becomes the maximum of `next` over its elements
     {
-        int r = 0, c = lane;
 #pragma unroll 4
         for (int f = lane; f < N; f += 32) {
-            while (c >= R) { c -= R; ++r; }
-            const uint32_t T = rows.at(r, c);
-            const uint32_t nx = c + 1 < R ? rows.at(r, c + 1) : NarrowRows::INF;
-            const uint32_t k = (T - 1u) >> sh;
-            if (k < (uint32_t)m) {
-                uint32_t *w = cell + k + (k >> ps);
+            const uint32_t T = rows.at(0, f), nx = rows.at(0, f + 1);
+            if (T <= lmin) {
+                uint32_t *w = cell_at(T);
                 if (*w < nx) atomicMax(w, nx);
             }
-            c += 32;
         }
     }
     __syncwarp();
-    // ... and then G at its start: the prefix maximum, exclusive; the smallest upper bound on the way
-    uint32_t run = 0;
-    uint32_t *mine = cell + lane * (per + 1);
-#pragma unroll 1
-    for (int j = 0; j < per; ++j) run = max(run, mine[j]);
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) { const uint32_t y = __shfl_up_sync(FULL, run, d); if (lane >= d) run = max(run, y); }
-    run = __shfl_up_sync(FULL, run, 1);
-    run = lane == 0 ? t0 : max(run, t0);
-    uint32_t ub = 0xffffffffu;
-#pragma unroll 1
-    for (int j = 0; j < per; ++j) {
-        const int c = lane * per + j;
-        const uint32_t v = mine[j], start = ((uint32_t)c << sh) + 1u;
-        mine[j] = run;
-        // the element that raises G first has d = G(start) - T at most where G(start) is later than it, else 0; all that
-        // raise it end at v at the latest
-        if (c < m && v > run && v != NarrowRows::INF) ub = min(ub, v - start);
-        run = max(run, v);
-    }
-    ub = __reduce_min_sync(FULL, ub);
-    __syncwarp();
-    // the elements that raise G in the cells that are left
-    unsigned fill = 0;
+    // ... and then a lower bound of G inside it: the exclusive prefix maximum
     {
-        int r = 0, c = lane;
-#pragma unroll 2
+        uint32_t run = 0;
+        uint32_t *mine = cell + lane * (per + 1);
+#pragma unroll 4
+        for (int j = 0; j < per; ++j) run = max(run, mine[j]);
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) { const uint32_t y = __shfl_up_sync(FULL, run, d); if (lane >= d) run = max(run, y); }
+        run = __shfl_up_sync(FULL, run, 1);
+        run = lane == 0 ? t0 : max(run, t0);
+#pragma unroll 4
+        for (int j = 0; j < per; ++j) { const uint32_t v = mine[j]; mine[j] = run; run = max(run, v); }
+    }
+    __syncwarp();
+    // d of the element at time T: all rows' first elements at or after it
+    auto exact = [&](uint32_t T) {
+        uint32_t g = T;
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            const int p = 32 * k + lane;
+            if (p < n) { const int i = first_from(rows, p, R, T); g = max(g, i < R ? rows.at(p, i) : NarrowRows::INF); }
+        }
+        return __reduce_max_sync(FULL, g);
+    };
+    // Best first: (bound, time) of the elements, in that order.  A pass over the elements collects those behind the last one
+    // evaluated whose bound does not exceed d; while there are more than there is room for, only the first of them is taken.
+    uint32_t d = NarrowRows::INF, t = NarrowRows::INF;
+    uint64_t after = 0;
+    unsigned fill = 0;
+#pragma unroll 1
+    for (int pass = 0;; ++pass) {
+        uint64_t first = ~0ull;
+        fill = 0;
+#pragma unroll 4
         for (int f0 = 0; f0 < N; f0 += 32) {
-            while (c >= R) { c -= R; ++r; }
             bool keep = false;
-            uint32_t T = 0, nx = 0;
+            uint64_t q = ~0ull;
             if (f0 + lane < N) {
-                T = rows.at(r, c);
-                nx = c + 1 < R ? rows.at(r, c + 1) : NarrowRows::INF;
-                const uint32_t k = (T - 1u) >> sh;
-                if (k < (uint32_t)m) {
-                    const uint32_t g = cell[k + (k >> ps)], end = min((uint32_t)((uint64_t)(k + 1u) << sh), lmin);
-                    keep = nx > g && nx > T && (g <= end || g - end <= ub);
+                const uint32_t T = rows.at(0, f0 + lane), nx = rows.at(0, f0 + lane + 1);
+                if (T <= lmin) {
+                    const uint32_t g = max(*cell_at(T), T), l = g - T;
+                    q = ((uint64_t)l << 32) | T;
+                    keep = nx > g && l <= d && q >= after;
                 }
             }
+            if (keep) first = min(first, q);
             const unsigned km = __ballot_sync(FULL, keep);
-            const unsigned pos = fill + __popc(km & ((1u << lane) - 1u));
-            if (keep && pos < WALK_NODES) node[pos] = ((uint64_t)T << 32) | nx;
-            fill += __popc(km);
-            c += 32;
+            if (km) {
+                const unsigned pos = fill + __popc(km & ((1u << lane) - 1u));
+                if (keep && pos < WALK_NODES) node[pos] = q;
+                fill += __popc(km);
+            }
         }
-    }
-    if (fill > WALK_NODES) return false;
-    __syncwarp();
-    uint32_t d = NarrowRows::INF, t = NarrowRows::INF;
+        __syncwarp();
+        if (fill <= WALK_NODES) break;
+        if (pass >= WALK_PASSES) return false;
+        // the lanes' first candidates, best first
+        uint64_t lowest = ~0ull;
 #pragma unroll 1
-    for (unsigned i = lane; i < fill; i += 32) {
-        const uint32_t T = (uint32_t)(node[i] >> 32), k = (T - 1u) >> sh;
-        uint32_t g = max(cell[k + (k >> ps)], T);
-#pragma unroll 4
-        for (unsigned j = 0; j < fill; ++j) {
-            const uint32_t tj = (uint32_t)(node[j] >> 32);
-            if (tj < T && (tj - 1u) >> sh == k) g = max(g, (uint32_t)node[j]);
+        for (int k = 0; k < 32; ++k) {
+            const uint32_t l = __reduce_min_sync(FULL, (uint32_t)(first >> 32));
+            const uint32_t T = __reduce_min_sync(FULL, (uint32_t)(first >> 32) == l ? (uint32_t)first : NarrowRows::INF);
+            if (l > d || l == NarrowRows::INF) break;
+            const uint64_t q = ((uint64_t)l << 32) | T;
+            lowest = min(lowest, q);
+            if (first == q) first = ~0ull;
+            const uint32_t g = exact(T);
+            if (g != NarrowRows::INF && (g - T < d || (g - T == d && T < t))) { d = g - T; t = T; }
         }
+        after = lowest + 1;
+    }
+#pragma unroll 1
+    for (unsigned done = 0; done < fill; ++done) {
+        uint64_t q = ~0ull;
+        for (unsigned i = lane; i < fill; i += 32) if (node[i] >= after) q = min(q, node[i]);
+        const uint32_t l = __reduce_min_sync(FULL, (uint32_t)(q >> 32));
+        const uint32_t T = __reduce_min_sync(FULL, (uint32_t)(q >> 32) == l ? (uint32_t)q : NarrowRows::INF);
+        if (l > d || l == NarrowRows::INF) break;
+        after = (((uint64_t)l << 32) | T) + 1;
+        const uint32_t g = exact(T);
         if (g != NarrowRows::INF && (g - T < d || (g - T == d && T < t))) { d = g - T; t = T; }
     }
-    bd = __reduce_min_sync(FULL, d);
-    bt = __reduce_min_sync(FULL, d == bd ? t : NarrowRows::INF);
-    return bd != NarrowRows::INF;                                 // (always, unless rows are not sorted)
+    bd = d; bt = t;
+    return d != NarrowRows::INF;                                  // (always, unless rows are not sorted)
 }
 
 // Dynamic shared memory: a warp after the other, P.words words each: the rows (n * stride), candidates, cells.
@@ -238,6 +256,8 @@ __global__ void __launch_bounds__(128) k_walk(const WalkParams P) {
     int status = ZL_OK;
     if (tmin < 0 || tmax >= VALUE_LIMIT || tmax < tmin || lmin < tmin) status = ZL_ERR_INVALID_ARG;   // outside [0, 2^62), or first/last columns out of order
     else if (unsorted) status = ZL_ERR_UNSORTED;
+#pragma unroll 1
+    for (int p = lane; p < n; p += 32) x[p * P.stride + R] = (uint32_t)(uint64_t)tmin - 2u;      // relative: infinite
     __syncwarp();
     int64_t bar = INT64_MIN, wt = INT64_MIN;
     int at[K];
@@ -248,7 +268,7 @@ __global__ void __launch_bounds__(128) k_walk(const WalkParams P) {
             const NarrowRows rows{x, (uint32_t)(uint64_t)tmin - 1u, P.stride};
             const uint32_t last = (uint32_t)(lmin - tmin) + 1u;
             uint32_t d, t;
-            if (!search_cells(rows, n, R, (uint32_t)(t0 - tmin) + 1u, last, cell, P.cells, node, d, t)) walk<K>(rows, n, R, last, d, t);
+            if (!search_cells<K>(rows, n, R, (uint32_t)(t0 - tmin) + 1u, last, cell, P.cells, node, d, t)) walk<K>(rows, n, R, last, d, t);
             bar = tmin - 1 + (int64_t)(t + d); wt = (int64_t)d;
 #pragma unroll
             for (int k = 0; k < K; ++k) if (32 * k + lane < n) at[k] = first_from(rows, 32 * k + lane, R, t + d + 1u) - 1;
@@ -270,11 +290,20 @@ __global__ void __launch_bounds__(128) k_walk(const WalkParams P) {
     for (int k = 0; k < K; ++k) if (32 * k + lane < n) P.idx[(size_t)b * n + 32 * k + lane] = at[k];
 }
 
-bool walk_shape(int n, int R) { return n <= 128 && R <= WALK_MAX_R && (long long)n * R <= SMALL_MAX; }
+// A warp alone takes its passes' latency: up to WALK_ALONE timestamps that is the quickest all the same (n=16, R=16, B=1 6.5 us;
+// 11 to 15 with a CTA).  With more of them it needs other warps beside it, the more the longer its own chain is; and workers
+// enough for the bounds to be tight, and rows short enough for the cells.  Measured against a CTA an instance that sorts it:
+// n=16, R=64, B=4096 38 us (68), n=32, R=32, B=4000 37 us (70), n=8, R=64, B=1000 18 us (22), but n=16, R=60, B=800 28 us (23),
+// n=100, R=40, B=1000 103 us (68), n=2, R=100, B=2000 53 us (23).
+bool walk_shape(int n, int R, int batch, int num_sms) {
+    const long long N = (long long)n * R;
+    if (n > 128 || R > 64 || (n < 4 && N > 64)) return false;
+    return N <= WALK_ALONE || (N <= 2 * WALK_ALONE && batch > 4 * num_sms) || (N <= 4 * WALK_ALONE && batch > 16 * num_sms);
+}
 
 void enqueue_walk(const Pipeline &q, cudaStream_t st) {
     WalkParams P;
-    P.n = q.n; P.R = q.R; P.B = q.B; P.stride = q.R | 1; P.check_sorted = (q.flags & ZL_FLAG_CHECK_SORTED) ? 1 : 0;
+    P.n = q.n; P.R = q.R; P.B = q.B; P.stride = q.R + 1; P.check_sorted = (q.flags & ZL_FLAG_CHECK_SORTED) ? 1 : 0;
     P.ts = q.ts; P.idx = q.idx; P.barrier = q.barrier; P.wait = q.wait; P.status = q.status;
     const int warps = q.B > 4 * q.num_sms ? 4 : 1;                // few instances: one on an SM
     // about eight cells an iteration of the slowest worker: fewer leave more candidates, more cost the passes over them

@@ -104,7 +104,7 @@ void enqueue_cells(const Pipeline &q, const FilterBufs &fb, const LaunchPlan &p,
 cudaError_t cell_limits();
 
 // walk.cu: RANGE, small instances of up to 128 workers, a warp per instance in one launch
-bool walk_shape(int n, int R);
+bool walk_shape(int n, int R, int batch, int num_sms);
 void enqueue_walk(const Pipeline &q, cudaStream_t st);
 cudaError_t walk_limits();
 

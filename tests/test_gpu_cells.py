@@ -108,3 +108,31 @@ def test_a_handle_takes_the_route_after_its_first_calls_and_leaves_it_when_it_fa
     assert torch.equal(a.idx, ref.idx) and torch.equal(a.wait, ref.wait) and torch.equal(a.barrier, ref.barrier)
     assert torch.equal(b.idx, ref.idx) and torch.equal(b.wait, ref.wait * 50_000)
     h.destroy()
+
+
+@pytest.mark.parametrize("n,R,B", [(1, 1, 3), (1, 64, 2), (4, 64, 3), (32, 8, 5), (33, 7, 4), (64, 4, 3), (65, 3, 3), (128, 2, 3), (128, 4, 700),
+                                   (16, 31, 601), (16, 64, 2500), (31, 33, 2400)])
+@pytest.mark.parametrize("values", ["spread", "ties", "wide"])
+def test_small_instances_a_warp_each(n, R, B, values):
+    # one to four rows a lane, the last row of a lane missing, one warp a CTA and four, the last CTA not full
+    rng = np.random.default_rng(n * 1000 + R)
+    hi = {"spread": 10 ** 6, "ties": 3, "wide": 10 ** 9}[values]
+    ts = (rng.integers(0, 3 * hi, size=(B, n, 1)) + np.cumsum(rng.integers(0, hi, size=(B, n, R)), axis=2)).astype(np.int64)
+    if B > 3 and R > 2:
+        ts[1, n // 2, 1] = ts[1, n // 2, 0] - 1                    # not sorted
+        ts[3, 0, 0] = -1
+    h = zl.ZipLine(n, R, B, 0, 0, zl.ZL_FLAG_CHECK_SORTED)
+    assert h.launches_per_call == 1
+    sel = h.select_batched(torch.from_numpy(ts).cuda())
+    torch.cuda.synchronize()
+    status, wait, barrier, idx = (x.cpu().numpy() for x in (sel.status, sel.wait, sel.barrier, sel.idx))
+    for b in range(min(B, 200)):
+        if B > 3 and R > 2 and b in (1, 3):
+            assert status[b] in (zl.binding.ZL_ERR_UNSORTED, zl.binding.ZL_ERR_INVALID_ARG) and (idx[b] == -1).all()
+            continue
+        w, t, ix = o.sweep_window(ts[b], 0)
+        assert status[b] == 0 and (int(wait[b]), int(barrier[b])) == (w, t) and (idx[b] == ix).all(), b
+    h.set_option("no_walk", 1)                                     # the rest of the batch: a CTA an instance
+    ref = h.select_batched(torch.from_numpy(ts).cuda())
+    assert torch.equal(ref.idx, sel.idx) and torch.equal(ref.wait, sel.wait) and torch.equal(ref.barrier, sel.barrier) and torch.equal(ref.status, sel.status)
+    h.destroy()
