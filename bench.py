@@ -362,7 +362,7 @@ def main():
     peak, peak_kind = measured_peak_gbs()
     names = STAGES[3] if h_launches == 1 else ("k_cells", "-", "-", "k_cell_rest") if h_launches == 2 else STAGES[route]
 
-    def dominant(pr):
+    def dominant(pr, names):
         stages = {}
         for nm, v in zip(names, (pr["ms_prologue"], pr["ms_filter"], pr["ms_sweep"], pr["ms_finalize"])):
             if nm != "-":
@@ -374,9 +374,9 @@ def main():
         gbs = nbytes / (ms * 1e-3) / 1e9
         return {"GB/s": gbs, "frac_of_measured": gbs / peak, "frac_of_nominal_8000": gbs / NOMINAL_GBS}
 
-    dom, dom_ms, stage_ms = dominant(t_prof["prof"])
+    dom, dom_ms, stage_ms = dominant(t_prof["prof"], names)
     ach = examined * 8 / (dom_ms * 1e-3) / 1e9
-    dom_f, dom_ms_f, stage_ms_f = dominant(t_fprof["prof"])
+    dom_f, dom_ms_f, stage_ms_f = dominant(t_fprof["prof"], STAGES[route])
     ach_f = nts * 8 / (dom_ms_f * 1e-3) / 1e9
     model = ("8 B per timestamp not after the first exhausted row (the search stops there)" if route == 1 else "8 B per timestamp")
     roofline = {"bound": "hbm", "kernel": dom, "achieved": ach, "peak": peak, "unit": "GB/s", "frac": ach / peak,

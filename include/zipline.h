@@ -155,10 +155,11 @@ zl_status zl_gridscan_batched(const int64_t *d_ts, int32_t B, int32_t n, int32_t
 /*
  * The same search with HOST buffers (same shapes and meaning as above):
  * copies the input to the device, runs the kernels, copies the results back
- * and waits for them.  Staging buffers are allocated by the first such call
- * on a handle (so that call allocates; later ones do not).  h_status may be
- * NULL.  Pinned host memory makes the copies asynchronous to the host until
- * the final wait; pageable memory works too.
+ * and waits for them.  Staging buffers are allocated by the first call on a
+ * handle that needs them (so that call allocates; later ones do not).  h_status
+ * may be NULL.  Timestamps in pinned host memory are read in place, and only as
+ * far as the search needs them, where the shape allows; otherwise they are copied
+ * to the device first.  Pageable memory works too.
  */
 zl_status zl_select_batched_host(zl_handle *h, const int64_t *h_ts, int32_t B,
                                  int32_t *h_idx, int64_t *h_barrier, int64_t *h_wait,

@@ -940,6 +940,7 @@ static void enqueue_cells_t(const Pipeline &q, const FilterBufs &fb, const Launc
     };
     launch(k_cells<OBJ, SRC>, dim3(s.cluster, q.B), s.threads, s.smem, s.cluster, src, P);
     if (ev) for (int k = 1; k < 4; ++k) cudaEventRecord(ev[k], st);
+    if (q.cells == 2) return;                                     // the caller looks at the flags itself
     SweepParams sp;
     sp.ts = q.ts; sp.meta = q.meta; sp.seg = q.seg;
     sp.n = q.n; sp.R = q.R; sp.B = q.B; sp.nseg = p.nseg; sp.nres = q.nres; sp.G = p.G_rest; sp.cap = p.cap;
