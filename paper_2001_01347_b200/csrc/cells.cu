@@ -562,21 +562,29 @@ __global__ void __launch_bounds__(1024, 1) k_cells(const SRC src, const CellPara
             ub = 0;
 #pragma unroll 1
             for (int r = 0; r < G; ++r) ub += sh.exs[r];
-            // times past lm at which the exhausted rows alone wait longer than that are left out: the first of 32 trial
-            // times (closer together near lm) where they do
-            const uint64_t past = min(ub, (uint64_t)(tend - lm));
-            const uint32_t trial = lm + (uint32_t)((past * (uint64_t)((lane + 1) * (lane + 1))) >> 10);
-            uint64_t e = 0;
-#pragma unroll 1
-            for (int p = warp; p < n; p += nw) { const uint32_t last = ends[p].y; e += trial > last ? trial - last : 0u; }
-            unsigned long long *es = (unsigned long long *)sh.node;              // (32 words, not in use yet)
-            if (warp == 0) es[lane] = 0;
+            // times past lm at which the exhausted rows alone wait longer than that are left out: the first of 32 trial times
+            // where they do (closer together near lm), then the first of 32 more between that one and the one before it
+            unsigned long long *es = (unsigned long long *)sh.node;              // (64 words, not in use yet)
+            if (tid < 64) es[tid] = 0;
             if (tid == 0) sh.acc = 0;
-            __syncthreads();
-            atomicAdd(&es[lane], (unsigned long long)e);
-            __syncthreads();
-            const unsigned over = __ballot_sync(FULL, es[lane] > ub);
-            const uint32_t stop = over ? __shfl_sync(FULL, trial, __ffs(over) - 1) : tend;
+            uint32_t below = lm, stop = lm + (uint32_t)min(ub, (uint64_t)(tend - lm));
+#pragma unroll 1
+            for (int part = 0; part < 2; ++part, es += 32) {
+                __syncthreads();
+                const uint64_t k = part ? 32ull * (lane + 1) : (uint64_t)((lane + 1) * (lane + 1));
+                const uint32_t trial = below + (uint32_t)(((uint64_t)(stop - below) * k) >> 10);
+                uint64_t e = 0;
+#pragma unroll 1
+                for (int p = warp; p < n; p += nw) { const uint32_t last = ends[p].y; e += trial > last ? trial - last : 0u; }
+                atomicAdd(&es[lane], (unsigned long long)e);
+                __syncthreads();
+                const unsigned over = __ballot_sync(FULL, es[lane] > ub);
+                const int first = over ? __ffs(over) - 1 : 32;
+                const uint32_t at = __shfl_sync(FULL, trial, min(first, 31)), before = __shfl_sync(FULL, trial, max(first - 1, 0));
+                if (first > 0) below = before;
+                if (first < 32) stop = at;
+                else { stop = part ? stop : tend; below = stop; }
+            }
             lo = t0;
             hi = max(lo, min(stop, tend)) + 1u;
             // n cell widths are the looseness of a cell's bounds; the wait itself spreads over time by about sqrt(n) times
@@ -832,7 +840,8 @@ __global__ void __launch_bounds__(1024, 1) k_cells(const SRC src, const CellPara
             sh.order[at] = (unsigned short)k;
         }
         __syncthreads();
-        const int batch = max(4, min(CELL_BATCH, 2 * nt / P.rpc));
+        // (SUM: a cell whose bound does not exceed d nearly always has to be looked at)
+        const int batch = OBJ == ZL_OBJ_SUM ? 8 : max(4, min(CELL_BATCH, 2 * nt / P.rpc));
 #pragma unroll 1
         for (int from = 0; from < ns && fits; from += batch) {
             if (sh.lb[sh.order[from]] > sh.best.d) break;
@@ -893,12 +902,13 @@ struct CellShape { int cluster, threads, cap; size_t smem; };
 
 static CellShape cell_shape(int n, int R, int B, int objective, int num_sms) {
     CellShape s;
-    // CTAs: as many as there are SMs, each with 16 rows at least to ask; clusters of 16 only for the largest instances, of
+    // CTAs: as many as there are SMs (SUM: two an SM), each with 16 rows at least to ask; clusters of 16 only for the largest instances, of
     // which few fill the GPU.  Threads: as many as an SM holds (clusters of 16: for two CTAs an SM, or not all of eight
     // clusters find room at once), one to so many timestamps (RANGE looks through an eighth of them).
     const int most = (long long)n * R >= (1 << 22) ? CELL_CLUSTER : 8;
+    const long long per_sm_ctas = objective == ZL_OBJ_RANGE ? 1 : 2;      // (SUM n=1024, R=1024, B=64: 236 us with one, 206 with two)
     s.cluster = 1;
-    while (s.cluster < most && (long long)B * s.cluster * 2 <= num_sms && n / (s.cluster * 2) >= 16) s.cluster *= 2;
+    while (s.cluster < most && (long long)B * s.cluster * 2 <= per_sm_ctas * num_sms && n / (s.cluster * 2) >= 16) s.cluster *= 2;
     const long long ctas = (long long)B * s.cluster;
     s.threads = ctas > 4LL * num_sms ? 128 : ctas > 2LL * num_sms ? 256 : ctas > num_sms || s.cluster > 8 ? 512 : 1024;
     const int per_thread = 32 * (objective == ZL_OBJ_RANGE ? 48 : 16);
