@@ -75,6 +75,8 @@ using zl::Pipeline;
 using zl::pow2_ceil;
 using zl::pow2_floor;
 constexpr int PROF_EVENTS = 5;
+constexpr long long MAPPED_MIN = 1 << 18;      // timestamps from which rows in pinned host memory are read in place (fewer: one copy is over sooner
+                                               // than the chain of reads across the bus)
 constexpr int CELLS_AFTER = 8;                 // calls of a handle before it tries the cell route
 constexpr int CELLS_MIN_WORKERS = 8;           // fewer workers: their few elements are sorted as cheaply, and the bounds of a cell are loose
 constexpr size_t CANARY_BYTES = 64;
@@ -146,7 +148,13 @@ void enqueue(const Pipeline &q, const LaunchPlan &p, cudaStream_t st, cudaEvent_
     if (ev) cudaEventRecord(ev[4], st);
 }
 
-cudaError_t raise_shared_memory_limits() {
+std::mutex g_limits_mutex;
+unsigned long long g_limits_done;                              // bit d: done for device d (devices beyond the 64th: every time)
+
+// More than the default 48 KB of dynamic shared memory for the kernels that take it: once a device, not with every handle.
+cudaError_t raise_shared_memory_limits(int device) {
+    std::lock_guard<std::mutex> lock(g_limits_mutex);
+    if (device < 64 && (g_limits_done >> device) & 1ull) return cudaSuccess;
     cudaError_t e = zl::prologue_limits();
     if (e == cudaSuccess) e = zl::range_limits();
     if (e == cudaSuccess) e = zl::small_limits();
@@ -157,6 +165,7 @@ cudaError_t raise_shared_memory_limits() {
     if (e == cudaSuccess) e = zl::range_rest_limits();
     if (e == cudaSuccess) e = zl::bucket_route_limits();
     if (e == cudaSuccess) e = zl::sweep_limits();
+    if (e == cudaSuccess && device < 64) g_limits_done |= 1ull << device;
     return e;
 }
 
@@ -360,7 +369,7 @@ zl_status zl_create(const zl_config *cfg, zl_handle **out) {
     if (e == cudaSuccess) e = alloc((void **)&h->d_seg, seg_b);
     const size_t pred_b = (cfg->flags & ZL_FLAG_PREDICTOR) ? (size_t)cfg->max_batch * cfg->n_workers * cfg->lookahead_R * 8 : 0;
     if (e == cudaSuccess && pred_b) e = alloc((void **)&h->d_pred, pred_b);
-    if (e == cudaSuccess) e = raise_shared_memory_limits();   // more than the default 48 KB of dynamic shared memory
+    if (e == cudaSuccess) e = raise_shared_memory_limits(cfg->device);
     if (e != cudaSuccess) {
         zl_status st = cuda_fail(nullptr, e);
         cudaFree(h->d_meta); cudaFree(h->d_seg); cudaFree(h->d_pred); cudaFree(h->d_cflags);
@@ -600,8 +609,9 @@ static void fill_pipeline(Pipeline &q, const zl_handle *h, int B) {
 // pinned memory that the device can reach, and no recent call for which that did not work out (after one the next calls copy,
 // twice as many after every such call).  The sortedness check reads every row anyway, and SUM enough of them for the bus to be
 // slower in pieces than in one copy (n=1024, R=1024, B=64: 20.7 ms against 11.6; RANGE 3.0 against 9.8).
-static const int64_t *mapped_rows(zl_handle *h, const int64_t *h_ts) {
+static const int64_t *mapped_rows(zl_handle *h, const int64_t *h_ts, int B) {
     if (h->cfg.objective != ZL_OBJ_RANGE || !cells_allowed(h) || (h->cfg.flags & ZL_FLAG_CHECK_SORTED)) return nullptr;
+    if ((long long)B * h->cfg.n_workers * h->cfg.lookahead_R < MAPPED_MIN) return nullptr;
     if (h->mapped_wait > 0) { --h->mapped_wait; return nullptr; }
     cudaPointerAttributes a;
     if (cudaPointerGetAttributes(&a, h_ts) != cudaSuccess) { cudaGetLastError(); return nullptr; }
@@ -748,7 +758,7 @@ zl_status zl_select_batched_host(zl_handle *h, const int64_t *h_ts, int32_t B, i
         h->staging_bytes += mb * n * 4 + mb * 20;
     }
     cudaStream_t st = h->s_stream;
-    if (const int64_t *in_place = mapped_rows(h, h_ts)) {
+    if (const int64_t *in_place = mapped_rows(h, h_ts, B)) {
         // The cell route reads a part of the rows only, so it reads them where they are, across the bus, instead of having
         // all of them copied first.  What it leaves over takes the copy below.
         Pipeline q;
@@ -843,7 +853,7 @@ zl_status zl_select_batched_noalloc(int32_t n_workers, int32_t lookahead_R, int3
             void *ptr = nullptr;
             cudaError_t e = cudaGetSymbolAddress((void **)&ptr, g_noalloc_scratch);
             if (e == cudaSuccess) e = cudaDeviceGetAttribute(&g_noalloc_sms[dev], cudaDevAttrMultiProcessorCount, dev);
-            if (e == cudaSuccess) e = raise_shared_memory_limits();
+            if (e == cudaSuccess) e = raise_shared_memory_limits(dev);
             if (e != cudaSuccess || !ptr) return ZL_ERR_CUDA;
             g_noalloc_ptr[dev] = ptr;
         }
