@@ -47,7 +47,7 @@ constexpr int CELL_SLACK = 4;             // elements by which a row may be off 
 constexpr int GUARD_BINS = 64;            // rows by their span, eight bins to a factor of two below the longest
 constexpr float GUARD_IRREGULAR = 32.f;   // bins by which more rows are looked through, to a unit of their gaps' relative deviation above 0.1
 constexpr float RANGE_CELLS = 100.f;      // RANGE: cells to the longest mean iteration
-constexpr float SUM_WIDTH = 0.23f;        // SUM: n cell widths against the spread of the wait over time (see k_cells)
+constexpr float SUM_WIDTH = 0.12f;        // SUM: n cell widths against the spread of the wait over time (see k_cells)
 
 // ------------------------------------------------------------------------------ rows
 // Relative times of an instance's rows, 32 bits: elements before the first are at time 0 (before everything), those behind
@@ -588,7 +588,8 @@ __global__ void __launch_bounds__(1024, 1) k_cells(const SRC src, const CellPara
             lo = t0;
             hi = max(lo, min(stop, tend)) + 1u;
             // n cell widths are the looseness of a cell's bounds; the wait itself spreads over time by about sqrt(n) times
-            // 0.29 iterations, an iteration being about twice the mean wait of a worker
+            // 0.29 iterations, an iteration being about twice the mean wait of a worker.  (n=17, R=700, B=20: half the factor
+            // 73 us, twice the factor 840, with six instances left over; n=32, R=400, B=20 41, 39 and 68.)
             width = SUM_WIDTH * (float)ub / ((float)n * sqrtf((float)n));
             __syncthreads();                                      // es has been read
         }
@@ -914,9 +915,9 @@ static CellShape cell_shape(int n, int R, int B, int objective, int num_sms) {
     const int per_thread = 32 * (objective == ZL_OBJ_RANGE ? 48 : 16);
     s.threads = (int)std::min<long long>(s.threads, std::max<long long>(128, 32 * (((long long)n * R / s.cluster + per_thread - 1) / per_thread)));
     // Cells an instance can use.  RANGE: RANGE_CELLS to an iteration of the slowest row, of which there are rarely more than
-    // half R before the first row runs out.  SUM: see SUM_WIDTH, 3 to 6 sqrt(n) cells an iteration.  No more than lets the
+    // half R before the first row runs out.  SUM: see SUM_WIDTH, 6 to 12 sqrt(n) cells an iteration.  No more than lets the
     // CTAs of the call (up to eight an SM) be resident together: they are bound by latency, not by what they move.
-    double want = objective == ZL_OBJ_RANGE ? RANGE_CELLS * 0.5 * R : 6.0 * R * std::sqrt((double)n);
+    double want = objective == ZL_OBJ_RANGE ? RANGE_CELLS * 0.5 * R : 12.0 * R * std::sqrt((double)n);
     want = std::max(256.0, std::min(want, (double)(1 << 18)));
     const long long per_sm = s.cluster > 8 ? 2 : std::max<long long>(1, std::min<long long>(8, (ctas + num_sms - 1) / num_sms));
     const double cell_bytes = objective == ZL_OBJ_RANGE ? 4.0 : 4.125;

@@ -78,7 +78,6 @@ constexpr int PROF_EVENTS = 5;
 constexpr long long MAPPED_MIN = 1 << 18;      // timestamps from which rows in pinned host memory are read in place (fewer: one copy is over sooner
                                                // than the chain of reads across the bus)
 constexpr int CELLS_AFTER = 8;                 // calls of a handle before it tries the cell route
-constexpr int CELLS_MIN_WORKERS = 8;           // fewer workers: their few elements are sorted as cheaply, and the bounds of a cell are loose
 constexpr size_t CANARY_BYTES = 64;
 constexpr int CANARY_BYTE = 0xC5;
 
@@ -542,9 +541,21 @@ static int rest_split_now(const zl_handle *h) {
 // examined, self-checks, a tuning knob of the other routes).
 static bool cells_allowed(const zl_handle *h) {
     return h->d_cflags && !h->opt_no_filter && !(h->cfg.flags & (ZL_FLAG_FULL_SWEEP | ZL_FLAG_DEBUG_CHECKS | ZL_FLAG_FORCE_FILTER)) &&
-           (long long)h->cfg.n_workers * h->cfg.lookahead_R > zl::SMALL_MAX && h->cfg.n_workers >= CELLS_MIN_WORKERS &&
+           (long long)h->cfg.n_workers * h->cfg.lookahead_R > zl::SMALL_MAX && h->cfg.n_workers >= 4 &&
            !h->opt_filter_bulk && !h->opt_rest_split && !h->opt_filter_round && !h->opt_filter_threads &&
            !h->opt_filter_rows && !h->opt_cluster && !h->opt_tail_cap && !h->opt_tail_threads && !h->opt_prologue_threads && !h->opt_no_cells;
+}
+// The shapes it takes by itself.  RANGE: all (n=4, R=4000, B=8 77 us against 156, n=7, R=1218, B=34 55 against 224)
+// but a handful of workers with a very long lookahead, where whole instances may be left over (n=8, R=16384, B=4: one of the
+// four, 1.1 ms against 0.4; n=16, R=65536 none).
+// SUM: the sum over the workers is smooth enough for few cells to be left only where there are many workers (n=17, R=700,
+// B=20 67 us against 53 on the bucket route), and a long lookahead has so many cells of nearly the least wait that some
+// instances keep more than the list holds (n=100, R=1500, B=64 up to 5 of them and 2.4 ms against 0.27; none at n=256 and
+// above up to R=2000, 170 us against 1000).  With a short one the cells cannot pay for the cluster's dozen barriers unless
+// the instances fill the GPU (n=3000, R=10, B=6 73 us against 57; n=256, R=24, B=64 40 against 66).
+static bool cells_shape(int objective, int n, int R, int B) {
+    if (objective == ZL_OBJ_RANGE) return n >= 16 || R <= 4096;
+    return n >= 64 && R >= (B >= 32 ? 24 : 40) && R <= (n >= 256 ? 2048 : 1024);
 }
 // Whether the next call takes it.  A handle's first calls go down the other routes, whose time depends little on how the
 // timestamps fall; then the cells are tried, and stay for as long as they leave nothing over.  A call that did leave some
@@ -553,6 +564,7 @@ static bool cells_allowed(const zl_handle *h) {
 static bool cells_now(const zl_handle *h) {
     if (!cells_allowed(h)) return false;
     if (h->opt_cells) return true;
+    if (!cells_shape(h->cfg.objective, h->cfg.n_workers, h->cfg.lookahead_R, h->cfg.max_batch)) return false;
     if (h->cells_last && ((volatile const uint32_t *)h->h_hint)[1] != 0) return false;
     return h->cells_wait == 0;
 }
@@ -879,7 +891,8 @@ zl_status zl_select_batched_noalloc(int32_t n_workers, int32_t lookahead_R, int3
     q.filter_threads = q.filter_rows = q.filter_round = 0; q.pdl_off = 0; q.prologue_threads = q.tail_threads = 0; q.cluster = q.filter_stages = 0; q.checks_off = 0; q.filter_bulk = 0; q.tail_cap = 0; q.rest_per_sm = 0; q.max_rounds = 0; q.rest_split = 0; q.small = (long long)n_workers * lookahead_R <= zl::SMALL_MAX && B <= 4 * std::max(1, tmp.num_sms) ? 1 : 0;
     q.idx = d_idx; q.barrier = d_barrier; q.wait = d_wait; q.status = d_status;
     q.walk = objective == ZL_OBJ_RANGE && !(flags & ZL_FLAG_FULL_SWEEP) && zl::walk_shape(n_workers, lookahead_R, B, std::max(1, tmp.num_sms)) ? 1 : 0;
-    q.cells = (long long)n_workers * lookahead_R > zl::SMALL_MAX && !(flags & ZL_FLAG_FULL_SWEEP) && n_workers >= CELLS_MIN_WORKERS ? 1 : 0;
+    q.cells = (long long)n_workers * lookahead_R > zl::SMALL_MAX && !(flags & ZL_FLAG_FULL_SWEEP) && n_workers >= 4 &&
+              cells_shape(objective, n_workers, lookahead_R, B) ? 1 : 0;
     q.cflags = (uint32_t *)((unsigned char *)g_noalloc_ptr[dev] + NOALLOC_META_BYTES); q.epoch = tmp.cells_epoch;
     enqueue(q, p, (cudaStream_t)cuda_stream, nullptr, zl::MatBatch{d_ts});
     return cudaGetLastError() == cudaSuccess ? ZL_OK : ZL_ERR_CUDA;
