@@ -623,11 +623,16 @@ static void fill_pipeline(Pipeline &q, const zl_handle *h, int B) {
 // slower in pieces than in one copy (n=1024, R=1024, B=64: 20.7 ms against 11.6; RANGE 3.0 against 9.8).
 static const int64_t *mapped_rows(zl_handle *h, const int64_t *h_ts, int B) {
     if (h->cfg.objective != ZL_OBJ_RANGE || !cells_allowed(h) || (h->cfg.flags & ZL_FLAG_CHECK_SORTED)) return nullptr;
-    if ((long long)B * h->cfg.n_workers * h->cfg.lookahead_R < MAPPED_MIN) return nullptr;
+    const long long total = (long long)B * h->cfg.n_workers * h->cfg.lookahead_R;
+    if (total < MAPPED_MIN || !cells_shape(ZL_OBJ_RANGE, h->cfg.n_workers, h->cfg.lookahead_R, B)) return nullptr;
     if (h->mapped_wait > 0) { --h->mapped_wait; return nullptr; }
-    cudaPointerAttributes a;
-    if (cudaPointerGetAttributes(&a, h_ts) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+    cudaPointerAttributes a, z;                                   // of the first timestamp and of the last one
+    if (cudaPointerGetAttributes(&a, h_ts) != cudaSuccess || cudaPointerGetAttributes(&z, h_ts + total - 1) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
     if (a.type != cudaMemoryTypeHost || !a.devicePointer || ((uintptr_t)a.devicePointer & 7)) return nullptr;
+    if (z.type != cudaMemoryTypeHost || z.devicePointer != (void *)((const int64_t *)a.devicePointer + total - 1)) return nullptr;
     return (const int64_t *)a.devicePointer;
 }
 

@@ -47,6 +47,12 @@ def test_shapes_around_the_pieces_slices_and_clusters(n, R, B, objective):
     assert_oracle(ts, objective, sel)
 
 
+@pytest.mark.parametrize("n,R,B", [(4, 300, 40), (5, 2000, 3), (7, 1025, 34)])
+def test_a_handful_of_workers(n, R, B):
+    ts = zi.generate(zi.CONFIGS["c4"].with_(B=B, n=n, R=R))
+    assert_oracle(ts, 0, select(ts, 0)[0])
+
+
 @pytest.mark.parametrize("objective", [0, 1])
 def test_ties_flat_rows_and_far_from_arithmetic(objective):
     rng = np.random.default_rng(5 + objective)
@@ -107,6 +113,21 @@ def test_a_handle_takes_the_route_after_its_first_calls_and_leaves_it_when_it_fa
     torch.cuda.synchronize()
     assert torch.equal(a.idx, ref.idx) and torch.equal(a.wait, ref.wait) and torch.equal(a.barrier, ref.barrier)
     assert torch.equal(b.idx, ref.idx) and torch.equal(b.wait, ref.wait * 50_000)
+    h.destroy()
+
+
+@pytest.mark.parametrize("pinned", [True, False])
+@pytest.mark.parametrize("wide", [False, True])
+def test_host_rows_read_in_place_or_copied(pinned, wide):
+    # just above 2^18 timestamps; a batch with an instance that the cells leave over is copied after all
+    n, R, B = 65, 257, 16
+    ts = zi.generate(zi.CONFIGS["c4"].with_(B=B, n=n, R=R))
+    if wide:
+        ts[3] *= 50_000
+    t = torch.from_numpy(ts).pin_memory() if pinned else torch.from_numpy(ts)
+    h = zl.ZipLine(n, R, B, 0)
+    for _ in range(2):
+        assert_oracle(ts, 0, h.select_batched_host(t))
     h.destroy()
 
 
