@@ -47,7 +47,7 @@ def test_shapes_around_the_pieces_slices_and_clusters(n, R, B, objective):
     assert_oracle(ts, objective, sel)
 
 
-@pytest.mark.parametrize("n,R,B", [(4, 300, 40), (5, 2000, 3), (7, 1025, 34)])
+@pytest.mark.parametrize("n,R,B", [(4, 1025, 40), (5, 2000, 3), (7, 1218, 34)])
 def test_a_handful_of_workers(n, R, B):
     ts = zi.generate(zi.CONFIGS["c4"].with_(B=B, n=n, R=R))
     assert_oracle(ts, 0, select(ts, 0)[0])
