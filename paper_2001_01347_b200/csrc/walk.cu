@@ -13,7 +13,7 @@
 
 namespace zl {
 
-constexpr int WALK_ALONE = 256;
+constexpr int WALK_ALONE = 256;            // timestamps of an instance whose passes take a microsecond or two
 constexpr int WALK_MAX_CELLS = 512;
 constexpr int WALK_PASSES = 24;            // most passes that take a single candidate
 constexpr unsigned WALK_NODES = 128;       // room for candidates
@@ -114,7 +114,9 @@ __device__ __forceinline__ bool search_cells(const NarrowRows &rows, int n, int 
         }
     }
     __syncwarp();
-    // ... and then a lower bound of G inside it: the exclusive prefix maximum
+    // ... and then a lower bound of G inside it: the exclusive prefix maximum; the most promising cell is the one where that
+    // exceeds the cell's end by least
+    uint32_t best = NarrowRows::INF, start = 0;
     {
         uint32_t run = 0;
         uint32_t *mine = cell + lane * (per + 1);
@@ -125,9 +127,36 @@ __device__ __forceinline__ bool search_cells(const NarrowRows &rows, int n, int 
         run = __shfl_up_sync(FULL, run, 1);
         run = lane == 0 ? t0 : max(run, t0);
 #pragma unroll 4
-        for (int j = 0; j < per; ++j) { const uint32_t v = mine[j]; mine[j] = run; run = max(run, v); }
+        for (int j = 0; j < per; ++j) {
+            const uint32_t v = mine[j], c = (uint32_t)(lane * per + j);
+            const uint32_t end = (uint32_t)(((uint64_t)lmin * (c + 1u)) >> (ps + 5)) + 1u;
+            const uint32_t l = run > end ? run - end : 0u;
+            if (l < best) { best = l; start = (uint32_t)(((uint64_t)lmin * c) >> (ps + 5)) + 1u; }
+            mine[j] = run;
+            run = max(run, v);
+        }
     }
     __syncwarp();
+    // a d that is attained: the rows' first elements at or after that cell's start (about: any time up to lmin will do).  With no
+    // more than a few hundred elements the passes below have few candidates as it is.
+    uint32_t d = NarrowRows::INF, t = NarrowRows::INF;
+    if (n * R > WALK_ALONE) {
+        const uint32_t l = __reduce_min_sync(FULL, best);
+        const int owner = __ffs(__ballot_sync(FULL, best == l)) - 1;
+        start = min(__shfl_sync(FULL, start, owner), lmin);
+        uint32_t g = 0, m = NarrowRows::INF;
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            const int p = 32 * k + lane;
+            if (p < n) {
+                const int i = first_from(rows, p, R, start);
+                const uint32_t T = i < R ? rows.at(p, i) : NarrowRows::INF;
+                g = max(g, T); m = min(m, T);
+            }
+        }
+        g = __reduce_max_sync(FULL, g); m = __reduce_min_sync(FULL, m);
+        if (g != NarrowRows::INF) { d = g - m; t = m; }
+    }
     // d of the element at time T: all rows' first elements at or after it
     auto exact = [&](uint32_t T) {
         uint32_t g = T;
@@ -140,7 +169,6 @@ __device__ __forceinline__ bool search_cells(const NarrowRows &rows, int n, int 
     };
     // Best first: (bound, time) of the elements, in that order.  A pass over the elements collects those behind the last one
     // evaluated whose bound does not exceed d; while there are more than there is room for, only the first of them is taken.
-    uint32_t d = NarrowRows::INF, t = NarrowRows::INF;
     uint64_t after = 0;
     unsigned fill = 0;
 #pragma unroll 1
@@ -290,15 +318,17 @@ __global__ void __launch_bounds__(128) k_walk(const WalkParams P) {
     for (int k = 0; k < K; ++k) if (32 * k + lane < n) P.idx[(size_t)b * n + 32 * k + lane] = at[k];
 }
 
-// A warp alone takes its passes' latency: up to WALK_ALONE timestamps that is the quickest all the same (n=16, R=16, B=1 6.5 us;
-// 11 to 15 with a CTA).  With more of them it needs other warps beside it, the more the longer its own chain is; and workers
-// enough for the bounds to be tight, and rows short enough for the cells.  Measured against a CTA an instance that sorts it:
-// n=16, R=64, B=4096 38 us (68), n=32, R=32, B=4000 37 us (70), n=8, R=64, B=1000 18 us (22), but n=16, R=60, B=800 28 us (23),
-// n=100, R=40, B=1000 103 us (68), n=2, R=100, B=2000 53 us (23).
+// A warp's passes over the elements and its few evaluations are one chain: the more elements, the more other warps it needs
+// beside it to be worth more than a CTA that sorts the instance, and the rows must be short and not too few for the bounds to
+// be tight.  Measured in us, this kernel / a CTA an instance: n=16, R=16, B=1 6.2 / 11; n=4, R=80 10 / 17 (B=1), 22 / 50 (4800);
+// n=16, R=30 13 / 23 (100), 13 / 21 (600), 22 / 58 (4800); n=32, R=32 14 / 24 (1), 19 / 23 (600), 38 / 84 (4800); n=100, R=10 18 / 15
+// (1), 25 / 17 (100), 27 / 34 (600); n=16, R=100 32 / 29 (600), 37 / 40 (1200), 62 / 116 (4800); n=60, R=50 44 / 42 (600), 45 / 68
+// (1200); n=128, R=20 57 / 77 (1200); but n=64, R=64 93 / 75 (1200), n=16, R=128 45 / 43 (1200), n=4, R=200 53 / 30 (1200).
 bool walk_shape(int n, int R, int batch, int num_sms) {
     const long long N = (long long)n * R;
-    if (n > 128 || R > 64 || (n < 4 && N > 64)) return false;
-    return N <= WALK_ALONE || (N <= 2 * WALK_ALONE && batch > 4 * num_sms) || (N <= 4 * WALK_ALONE && batch > 16 * num_sms);
+    if (n > 128 || R > 100 || (n < 4 && N > 64)) return false;
+    return N <= 2 * WALK_ALONE || (N <= 4 * WALK_ALONE && R <= 64 && (n <= 32 || batch > 4 * num_sms)) ||
+           (N <= (R <= 64 ? 12 : 8) * WALK_ALONE && n >= 8 && batch > 8 * num_sms);
 }
 
 void enqueue_walk(const Pipeline &q, cudaStream_t st) {

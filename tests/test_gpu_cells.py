@@ -132,7 +132,7 @@ def test_host_rows_read_in_place_or_copied(pinned, wide):
 
 
 @pytest.mark.parametrize("n,R,B", [(1, 1, 3), (1, 64, 2), (4, 64, 3), (32, 8, 5), (33, 7, 4), (64, 4, 3), (65, 3, 3), (128, 2, 3), (128, 4, 700),
-                                   (16, 31, 601), (16, 64, 2500), (31, 33, 2400)])
+                                   (16, 31, 601), (16, 64, 2500), (31, 33, 2400), (5, 100, 3), (32, 32, 5), (65, 47, 1300), (128, 24, 1200), (20, 100, 1201)])
 @pytest.mark.parametrize("values", ["spread", "ties", "wide"])
 def test_small_instances_a_warp_each(n, R, B, values):
     # one to four rows a lane, the last row of a lane missing, one warp a CTA and four, the last CTA not full
