@@ -253,6 +253,7 @@ const char *zl_status_string(zl_status s) {
 
 int32_t zl_max_workers(void) { return zl::MAX_WORKERS; }
 
+static bool walk_route(const zl_handle *h);
 zl_status zl_create(const zl_config *cfg, zl_handle **out) {
     if (!cfg || !out) return ZL_ERR_INVALID_ARG;
     *out = nullptr;
@@ -354,7 +355,7 @@ zl_status zl_create(const zl_config *cfg, zl_handle **out) {
             memset(&f, 0, sizeof(f));
         }
     }
-    if ((cfg->objective == ZL_OBJ_RANGE && !range_small) || (long long)cfg->n_workers * cfg->lookahead_R > zl::SMALL_MAX) {
+    if ((cfg->objective == ZL_OBJ_RANGE && !range_small) || !walk_route(h)) {
         // cell route, and the words by which a call tells the next one how it went
         if (e == cudaSuccess) e = alloc((void **)&h->d_cflags, 128);
         filter_b += 128;
@@ -537,25 +538,31 @@ static int rest_split_now(const zl_handle *h) {
     return h->h_hint && *(volatile const uint32_t *)h->h_hint != 0;
 }
 
-// The cell route: every shape above the one-launch sizes, unless the handle asks for another route (every timestamp
+// The cell route: every shape that a warp an instance does not take, unless the handle asks for another route (every timestamp
 // examined, self-checks, a tuning knob of the other routes).
 static bool cells_allowed(const zl_handle *h) {
     return h->d_cflags && !h->opt_no_filter && !(h->cfg.flags & (ZL_FLAG_FULL_SWEEP | ZL_FLAG_DEBUG_CHECKS | ZL_FLAG_FORCE_FILTER)) &&
-           (long long)h->cfg.n_workers * h->cfg.lookahead_R > zl::SMALL_MAX && h->cfg.n_workers >= 4 &&
+           !walk_route(h) && h->cfg.n_workers >= 4 &&
            !h->opt_filter_bulk && !h->opt_rest_split && !h->opt_filter_round && !h->opt_filter_threads &&
            !h->opt_filter_rows && !h->opt_cluster && !h->opt_tail_cap && !h->opt_tail_threads && !h->opt_prologue_threads && !h->opt_no_cells;
 }
-// The shapes it takes by itself.  RANGE: all (n=4, R=4000, B=8 77 us against 156, n=7, R=1218, B=34 55 against 224)
-// but a handful of workers with a very long lookahead, where whole instances may be left over (n=8, R=16384, B=4: one of the
-// four, 1.1 ms against 0.4; n=16, R=65536 none).
-// SUM: the sum over the workers is smooth enough for few cells to be left only where there are many workers (n=17, R=700,
-// B=20 67 us against 53 on the bucket route), and a long lookahead has so many cells of nearly the least wait that some
-// instances keep more than the list holds (n=100, R=1500, B=64 up to 5 of them and 2.4 ms against 0.27; none at n=256 and
-// above up to R=2000, 170 us against 1000).  With a short one the cells cannot pay for the cluster's dozen barriers unless
-// the instances fill the GPU (n=3000, R=10, B=6 73 us against 57; n=256, R=24, B=64 40 against 66).
-static bool cells_shape(int objective, int n, int R, int B) {
-    if (objective == ZL_OBJ_RANGE) return n >= 16 || R <= 4096;
-    return n >= 64 && R >= (B >= 32 ? 24 : 40) && R <= (n >= 256 ? 2048 : 1024);
+// The shapes it takes by itself, where it is the faster one (us, cells / the other route).
+// RANGE: rows of 16 timestamps and more (n=64, R=64 15 / 24 (B=1), 29 / 70 (500), 44 / 89 (1500); n=4, R=4000, B=8 77 / 156), with
+// many workers and instances of 8 (n=300, R=13, B=500 47 / 58, but B=1 23 / 21 and n=4000, R=6, B=10 135 / 46), but not a handful
+// of workers with a very long lookahead, where whole instances may be left over (n=8, R=16384, B=4: one of the four, 1.1 ms /
+// 0.4; n=16, R=65536 none).
+// SUM, instances of the one-launch sizes: n=10, R=15 14 / 19; n=10, R=50 15 / 40; n=64, R=64 24 / 44 (B=1), 36 / 117 (500); n=8,
+// R=200, B=100 34 / 32.  In larger batches, and larger instances, the sum is smooth enough for few cells to be left only where
+// there are many workers (n=17, R=700, B=20 67 / 53; n=32, R=32, B=4000 108 / 88; n=64, R=64, B=1500 76 / 126), and a long
+// lookahead has so many cells of nearly the least wait that some instances keep more than the list holds (n=100, R=1500, B=64 up
+// to 5 of them, 2.4 ms / 0.27; none at n=256 and above up to R=2000, 170 / 1000).  With a short one the cells cannot pay for the
+// cluster's dozen barriers unless the instances fill the GPU (n=3000, R=10, B=6 73 / 57; n=256, R=24, B=64 40 / 66; n=100, R=10,
+// B=3000 94 / 108; n=1000, R=4, B=1000 210 / 138).
+static bool cells_shape(int objective, int n, int R, int B, int num_sms) {
+    const bool many = B > 4 * num_sms;
+    if (objective == ZL_OBJ_RANGE) return (R >= 16 || (R >= 8 && n >= 256 && B >= 100)) && (n >= 16 || R <= 4096);
+    if ((long long)n * R <= zl::SMALL_MAX && !many) return n >= 6 && R >= 12;
+    return n >= 64 && R >= (many ? 10 : B >= 32 ? 24 : 40) && R <= (n >= 256 ? 2048 : 1024);
 }
 // Whether the next call takes it.  A handle's first calls go down the other routes, whose time depends little on how the
 // timestamps fall; then the cells are tried, and stay for as long as they leave nothing over.  A call that did leave some
@@ -564,7 +571,7 @@ static bool cells_shape(int objective, int n, int R, int B) {
 static bool cells_now(const zl_handle *h) {
     if (!cells_allowed(h)) return false;
     if (h->opt_cells) return true;
-    if (!cells_shape(h->cfg.objective, h->cfg.n_workers, h->cfg.lookahead_R, h->cfg.max_batch)) return false;
+    if (!cells_shape(h->cfg.objective, h->cfg.n_workers, h->cfg.lookahead_R, h->cfg.max_batch, std::max(1, h->num_sms))) return false;
     if (h->cells_last && ((volatile const uint32_t *)h->h_hint)[1] != 0) return false;
     return h->cells_wait == 0;
 }
@@ -582,15 +589,15 @@ static bool cells_take(zl_handle *h) {
     return now;
 }
 static void set_cells(Pipeline &q, zl_handle *h) {
-    q.cells = !q.small && cells_take(h) ? 1 : 0;
+    q.cells = cells_take(h) ? 1 : 0;
     q.cflags = h->d_cflags;
     q.epoch = ++h->cells_epoch;
 }
 
 int32_t zl_launches_per_call(const zl_handle *h) {
     if (!h) return 0;
-    if (small_route(h) || walk_route(h)) return 1;
     if (cells_now(h)) return 2;
+    if (small_route(h) || walk_route(h)) return 1;
     const bool filter = h->cfg.objective == ZL_OBJ_RANGE && !h->opt_no_filter && h->fb.table != nullptr;
     const bool sumfast = !filter && !h->opt_no_filter && h->fb.scap != 0;
     return (filter ? (rest_split_now(h) ? 9 : 4) : 3) + (sumfast ? (h->fb.scells ? 3 : 2) : 0) + ((h->cfg.flags & ZL_FLAG_CHECK_SORTED) ? 1 : 0);
@@ -624,7 +631,7 @@ static void fill_pipeline(Pipeline &q, const zl_handle *h, int B) {
 static const int64_t *mapped_rows(zl_handle *h, const int64_t *h_ts, int B) {
     if (h->cfg.objective != ZL_OBJ_RANGE || !cells_allowed(h) || (h->cfg.flags & ZL_FLAG_CHECK_SORTED)) return nullptr;
     const long long total = (long long)B * h->cfg.n_workers * h->cfg.lookahead_R;
-    if (total < MAPPED_MIN || !cells_shape(ZL_OBJ_RANGE, h->cfg.n_workers, h->cfg.lookahead_R, B)) return nullptr;
+    if (total < MAPPED_MIN || !cells_shape(ZL_OBJ_RANGE, h->cfg.n_workers, h->cfg.lookahead_R, B, std::max(1, h->num_sms))) return nullptr;
     if (h->mapped_wait > 0) { --h->mapped_wait; return nullptr; }
     cudaPointerAttributes a, z;                                   // of the first timestamp and of the last one
     if (cudaPointerGetAttributes(&a, h_ts) != cudaSuccess || cudaPointerGetAttributes(&z, h_ts + total - 1) != cudaSuccess) {
@@ -896,8 +903,8 @@ zl_status zl_select_batched_noalloc(int32_t n_workers, int32_t lookahead_R, int3
     q.filter_threads = q.filter_rows = q.filter_round = 0; q.pdl_off = 0; q.prologue_threads = q.tail_threads = 0; q.cluster = q.filter_stages = 0; q.checks_off = 0; q.filter_bulk = 0; q.tail_cap = 0; q.rest_per_sm = 0; q.max_rounds = 0; q.rest_split = 0; q.small = (long long)n_workers * lookahead_R <= zl::SMALL_MAX && B <= 4 * std::max(1, tmp.num_sms) ? 1 : 0;
     q.idx = d_idx; q.barrier = d_barrier; q.wait = d_wait; q.status = d_status;
     q.walk = objective == ZL_OBJ_RANGE && !(flags & ZL_FLAG_FULL_SWEEP) && zl::walk_shape(n_workers, lookahead_R, B, std::max(1, tmp.num_sms)) ? 1 : 0;
-    q.cells = (long long)n_workers * lookahead_R > zl::SMALL_MAX && !(flags & ZL_FLAG_FULL_SWEEP) && n_workers >= 4 &&
-              cells_shape(objective, n_workers, lookahead_R, B) ? 1 : 0;
+    q.cells = !q.walk && !(flags & ZL_FLAG_FULL_SWEEP) && n_workers >= 4 &&
+              cells_shape(objective, n_workers, lookahead_R, B, std::max(1, tmp.num_sms)) ? 1 : 0;
     q.cflags = (uint32_t *)((unsigned char *)g_noalloc_ptr[dev] + NOALLOC_META_BYTES); q.epoch = tmp.cells_epoch;
     enqueue(q, p, (cudaStream_t)cuda_stream, nullptr, zl::MatBatch{d_ts});
     return cudaGetLastError() == cudaSuccess ? ZL_OK : ZL_ERR_CUDA;

@@ -36,7 +36,7 @@ def assert_oracle(ts, objective, sel):
 @pytest.mark.parametrize("objective", [0, 1])
 @pytest.mark.parametrize("n,R,B", [(8, 513, 3), (8, 5000, 2), (15, 300, 5), (17, 257, 160), (31, 133, 9), (33, 129, 2), (63, 67, 700),
                                    (97, 211, 40), (128, 33, 20), (255, 65, 1), (257, 64, 7), (1000, 15, 1), (1025, 9, 3), (4096, 2, 2),
-                                   (4095, 130, 1)])
+                                   (4095, 130, 1), (10, 150, 3), (64, 64, 700), (300, 13, 600), (129, 8, 2)])
 def test_shapes_around_the_pieces_slices_and_clusters(n, R, B, objective):
     # rows of odd length and start (pieces of eight elements on 32-byte boundaries), row counts around the CTAs of a
     # cluster, batches that change its size; spread workers with rare long iterations, so that estimates are off
