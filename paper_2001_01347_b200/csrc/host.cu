@@ -547,22 +547,28 @@ static bool cells_allowed(const zl_handle *h) {
            !h->opt_filter_rows && !h->opt_cluster && !h->opt_tail_cap && !h->opt_tail_threads && !h->opt_prologue_threads && !h->opt_no_cells;
 }
 // The shapes it takes by itself, where it is the faster one (us, cells / the other route).
-// RANGE: rows of 16 timestamps and more (n=64, R=64 15 / 24 (B=1), 29 / 70 (500), 44 / 89 (1500); n=4, R=4000, B=8 77 / 156), with
-// many workers and instances of 8 (n=300, R=13, B=500 47 / 58, but B=1 23 / 21 and n=4000, R=6, B=10 135 / 46), but not a handful
-// of workers with a very long lookahead, where whole instances may be left over (n=8, R=16384, B=4: one of the four, 1.1 ms /
-// 0.4; n=16, R=65536 none).
+// RANGE: rows of 20 timestamps and more (n=64, R=64 15 / 24 (B=1), 29 / 70 (500), 44 / 89 (1500); n=7, R=1218, B=34 55 / 224); with
+// more workers than one CTA's few dozen guards only longer rows (n=292, R=26, B=15 33 / 26; n=652, R=62, B=17 45 / 33) unless the
+// instances fill the GPU (n=300, R=12, B=1500 65 / 146, but n=410, R=9, B=192 47 / 27).  Not four or five workers (n=4, R=966,
+// B=386 465 / 158), nor a handful of them with a very long lookahead, where whole instances may be left over (n=8, R=16384,
+// B=4: one of the four, 1.1 ms / 0.4; n=16, R=65536 none).
 // SUM, instances of the one-launch sizes: n=10, R=15 14 / 19; n=10, R=50 15 / 40; n=64, R=64 24 / 44 (B=1), 36 / 117 (500); n=8,
 // R=200, B=100 34 / 32.  In larger batches, and larger instances, the sum is smooth enough for few cells to be left only where
 // there are many workers (n=17, R=700, B=20 67 / 53; n=32, R=32, B=4000 108 / 88; n=64, R=64, B=1500 76 / 126), and a long
 // lookahead has so many cells of nearly the least wait that some instances keep more than the list holds (n=100, R=1500, B=64 up
-// to 5 of them, 2.4 ms / 0.27; none at n=256 and above up to R=2000, 170 / 1000).  With a short one the cells cannot pay for the
+// to 5 of them, 2.4 ms / 0.27; none at n=256 and above up to R=2000, 170 / 1000), the more so where many instances share an SM and
+// each has fewer cells (n=74, R=501, B=242 1100 / 233; n=332, R=1107, B=79 1420 / 990; n=937, R=21, B=1606 2440 / 1230).  With a short one the cells cannot pay for the
 // cluster's dozen barriers unless the instances fill the GPU (n=3000, R=10, B=6 73 / 57; n=256, R=24, B=64 40 / 66; n=100, R=10,
 // B=3000 94 / 108; n=1000, R=4, B=1000 210 / 138).
 static bool cells_shape(int objective, int n, int R, int B, int num_sms) {
     const bool many = B > 4 * num_sms;
-    if (objective == ZL_OBJ_RANGE) return (R >= 16 || (R >= 8 && n >= 256 && B >= 100)) && (n >= 16 || R <= 4096);
-    if ((long long)n * R <= zl::SMALL_MAX && !many) return n >= 6 && R >= 12;
-    return n >= 64 && R >= (many ? 10 : B >= 32 ? 24 : 40) && R <= (n >= 256 ? 2048 : 1024);
+    if (objective == ZL_OBJ_RANGE) {
+        if (n < 6 || (n < 16 && R > 4096)) return false;
+        return n <= 128 ? R >= 20 || (many && R >= 8) : R >= 96 || (R >= 32 && B >= 64) || (R >= 16 && B >= 256) || (R >= 8 && many);
+    }
+    if ((long long)n * R <= zl::SMALL_MAX && !many) return n >= 10 && R >= 12;
+    if (n < 64 || R < (many ? 10 : B >= 32 ? 24 : 40) || (B >= 256 && n > 512)) return false;
+    return R <= (n >= 256 ? (B <= 64 ? 2048 : 512) : B <= 32 ? 512 : 256);
 }
 // Whether the next call takes it.  A handle's first calls go down the other routes, whose time depends little on how the
 // timestamps fall; then the cells are tried, and stay for as long as they leave nothing over.  A call that did leave some

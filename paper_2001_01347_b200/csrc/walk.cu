@@ -323,11 +323,12 @@ __global__ void __launch_bounds__(128) k_walk(const WalkParams P) {
 // be tight.  Measured in us, this kernel / a CTA an instance: n=16, R=16, B=1 6.2 / 11; n=4, R=80 10 / 17 (B=1), 22 / 50 (4800);
 // n=16, R=30 13 / 23 (100), 13 / 21 (600), 22 / 58 (4800); n=32, R=32 14 / 24 (1), 19 / 23 (600), 38 / 84 (4800); n=100, R=10 18 / 15
 // (1), 25 / 17 (100), 27 / 34 (600); n=16, R=100 32 / 29 (600), 37 / 40 (1200), 62 / 116 (4800); n=60, R=50 44 / 42 (600), 45 / 68
-// (1200); n=128, R=20 57 / 77 (1200); but n=64, R=64 93 / 75 (1200), n=16, R=128 45 / 43 (1200), n=4, R=200 53 / 30 (1200).
+// (1200); n=128, R=20 57 / 77 (1200); but n=64, R=64 93 / 75 (1200), n=16, R=128 45 / 43 (1200), n=4, R=200 53 / 30 (1200), n=97, R=4 19 / 15 (6), n=2,
+// R=28 11 / 7 (522).
 bool walk_shape(int n, int R, int batch, int num_sms) {
     const long long N = (long long)n * R;
-    if (n > 128 || R > 100 || (n < 4 && N > 64)) return false;
-    return N <= 2 * WALK_ALONE || (N <= 4 * WALK_ALONE && R <= 64 && (n <= 32 || batch > 4 * num_sms)) ||
+    if (n > 128 || R > 100 || (n < 4 && N > 32)) return false;
+    return N <= WALK_ALONE || (N <= 2 * WALK_ALONE && (n <= 64 || batch > 4 * num_sms)) || (N <= 4 * WALK_ALONE && R <= 64 && (n <= 32 || batch > 4 * num_sms)) ||
            (N <= (R <= 64 ? 12 : 8) * WALK_ALONE && n >= 8 && batch > 8 * num_sms);
 }
 
