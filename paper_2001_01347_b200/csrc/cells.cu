@@ -368,11 +368,14 @@ __device__ __noinline__ bool evaluate_cells(CellShared &sh, int from, int ns, co
 // cells the scan before them and the smallest lower bound among them [cap / 128] two u64.
 template <int OBJ, class SRC>
 __global__ void __launch_bounds__(1024, 1) k_cells(const SRC src, const CellParams P) {
-    grid_dep_wait();
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ CellShared sh;
     cg::cluster_group cl = cg::this_cluster();
     const int b = blockIdx.y, rank = blockIdx.x, G = gridDim.x;
+    // A CTA's shared memory may be written by the others only once it runs: everybody says so here, and waits for the rest
+    // with the columns read, before the first store into another CTA.
+    if (G > 1) cl.barrier_arrive();
+    grid_dep_wait();
     const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
     const int n = P.n, R = P.R;
     uint32_t *cell = (uint32_t *)smem;
@@ -399,9 +402,7 @@ __global__ void __launch_bounds__(1024, 1) k_cells(const SRC src, const CellPara
             }
             const uint64_t ux = (uint64_t)x ^ (1ull << 63), uy = (uint64_t)y ^ (1ull << 63);
             q[0] = min(q[0], ux); q[1] = max(q[1], ux); q[2] = min(q[2], uy); q[3] = max(q[3], uy);
-            const uint2 e = make_uint2((uint32_t)(uint64_t)x, (uint32_t)(uint64_t)y);
-#pragma unroll 1
-            for (int r = 0; r < G; ++r) cl.map_shared_rank(ends, r)[r0 + p] = e;
+            ends[r0 + p] = make_uint2((uint32_t)(uint64_t)x, (uint32_t)(uint64_t)y);
         }
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
@@ -420,6 +421,16 @@ __global__ void __launch_bounds__(1024, 1) k_cells(const SRC src, const CellPara
 #pragma unroll 1
         for (int k = tid; k < GUARD_BINS; k += nt) sh.hist[k] = 0;
         __syncthreads();
+        if (G > 1) {
+            cl.barrier_wait();
+#pragma unroll 1
+            for (int r = 0; r < G; ++r) {
+                if (r == rank) continue;
+                uint2 *to = cl.map_shared_rank(ends, r);
+#pragma unroll 1
+                for (int p = tid; p < nrows; p += nt) to[r0 + p] = ends[r0 + p];
+            }
+        }
         if (tid < 4 * G) {
             const int k = tid & 3, r = tid >> 2;
             unsigned long long v = sh.red[k][0];
