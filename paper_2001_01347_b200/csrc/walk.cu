@@ -96,7 +96,8 @@ __device__ __forceinline__ bool search_cells(const NarrowRows &rows, int n, int 
                                              uint32_t &bd, uint32_t &bt) {
     const int lane = threadIdx.x & 31, N = n * rows.stride;       // all words of the rows, one after the other
     const int per = most / 32, ps = __ffs(per) - 1;               // a run of cells a lane; cell c sits at c + c / per (no bank conflicts)
-    // (T - 1) < lmin for every T <= lmin, so its cell ((T - 1) * scale) >> 32 is below `most`
+    // T - 1 < lmin, so its cell ((T - 1) * scale) >> 32 is below `most`.  (T = 0, a time before the first elements, is only met in
+    // rows that are not sorted; such an element belongs to no cell.)
     const uint32_t scale = (uint32_t)min((uint64_t)0xffffffffu, ((uint64_t)most << 32) / lmin);
     auto cell_at = [&](uint32_t T) { const uint32_t k = __umulhi(T - 1u, scale); return cell + k + (k >> ps); };
 #pragma unroll 1
@@ -107,7 +108,7 @@ __device__ __forceinline__ bool search_cells(const NarrowRows &rows, int n, int 
 #pragma unroll 4
         for (int f = lane; f < N; f += 32) {
             const uint32_t T = rows.at(0, f), nx = rows.at(0, f + 1);
-            if (T <= lmin) {
+            if (T - 1u < lmin) {
                 uint32_t *w = cell_at(T);
                 if (*w < nx) atomicMax(w, nx);
             }
@@ -181,7 +182,7 @@ __device__ __forceinline__ bool search_cells(const NarrowRows &rows, int n, int 
             uint64_t q = ~0ull;
             if (f0 + lane < N) {
                 const uint32_t T = rows.at(0, f0 + lane), nx = rows.at(0, f0 + lane + 1);
-                if (T <= lmin) {
+                if (T - 1u < lmin) {
                     const uint32_t g = max(*cell_at(T), T), l = g - T;
                     q = ((uint64_t)l << 32) | T;
                     keep = nx > g && l <= d && q >= after;

@@ -157,3 +157,22 @@ def test_small_instances_a_warp_each(n, R, B, values):
     ref = h.select_batched(torch.from_numpy(ts).cuda())
     assert torch.equal(ref.idx, sel.idx) and torch.equal(ref.wait, sel.wait) and torch.equal(ref.barrier, sel.barrier) and torch.equal(ref.status, sel.status)
     h.destroy()
+
+
+@pytest.mark.parametrize("n,R,B", [(4, 8, 3), (16, 64, 700), (33, 20, 700), (100, 10, 3)])
+def test_small_instances_with_a_time_before_every_first_element(n, R, B):
+    # rows that are not sorted, and not checked to be: what an instance's result is is not defined, but it stays within its own
+    # buffers, and the others are right
+    rng = np.random.default_rng(n)
+    ts = (1000 + np.cumsum(rng.integers(1, 10 ** 6, size=(B, n, R)), axis=2)).astype(np.int64)
+    broken = ts.copy()
+    for back in (1, 2, 1 << 20):
+        broken[1] = ts[1]
+        broken[1, n - 1, 1:-1] = ts[1, :, 0].min() - back
+        h = zl.ZipLine(n, R, B, 0)
+        assert h.launches_per_call == 1
+        sel = h.select_batched(torch.from_numpy(broken).cuda())
+        torch.cuda.synchronize()
+        keep = [0] + list(range(2, min(B, 60)))
+        assert_oracle(ts[keep], 0, zl.Selection(sel.idx[keep], sel.barrier[keep], sel.wait[keep], sel.status[keep]))
+        h.destroy()
