@@ -18,6 +18,7 @@
 //   cells.cu      the cell route: branch and bound over time cells (both objectives, all but the smallest instances), and what it
 //                 leaves over; the routes above serve a handle's first calls and those the cells do not work out for.
 //   baselines.cu  GridScan / FullGridScan, the predictor, the per-position trace.
+#include <cuda.h>
 #include <cuda_runtime.h>
 #include <stddef.h>
 #include <stdint.h>
@@ -630,6 +631,23 @@ static void fill_pipeline(Pipeline &q, const zl_handle *h, int B) {
     q.cells = 0; q.cflags = nullptr; q.epoch = 0; q.idx = nullptr; q.barrier = q.wait = nullptr; q.status = nullptr;
 }
 
+// The identity of the allocation or registration that a pinned pointer belongs to, as the driver counts them (0: none, or unknown).
+static unsigned long long pinned_buffer_id(const void *p) {
+    typedef CUresult (*GetAttribute)(void *, CUpointer_attribute, CUdeviceptr);
+    static const GetAttribute get = [] {
+        void *f = nullptr;
+        cudaDriverEntryPointQueryResult found = cudaDriverEntryPointSymbolNotFound;
+        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttribute", &f, 12000, cudaEnableDefault, &found) != cudaSuccess ||
+            found != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            f = nullptr;
+        }
+        return (GetAttribute)f;
+    }();
+    unsigned long long id = 0;
+    return get && get(&id, CU_POINTER_ATTRIBUTE_BUFFER_ID, (CUdeviceptr)(uintptr_t)p) == CUDA_SUCCESS ? id : 0;
+}
+
 // The device's view of pinned host rows when a host-buffer call should read them in place: the cell route's shapes, rows in
 // pinned memory that the device can reach, and no recent call for which that did not work out (after one the next calls copy,
 // twice as many after every such call).  The sortedness check reads every row anyway, and SUM enough of them for the bus to be
@@ -646,6 +664,9 @@ static const int64_t *mapped_rows(zl_handle *h, const int64_t *h_ts, int B) {
     }
     if (a.type != cudaMemoryTypeHost || !a.devicePointer || ((uintptr_t)a.devicePointer & 7)) return nullptr;
     if (z.type != cudaMemoryTypeHost || z.devicePointer != (void *)((const int64_t *)a.devicePointer + total - 1)) return nullptr;
+    // ... of one piece: between two registrations there may be memory that the device cannot read
+    const unsigned long long id = pinned_buffer_id(h_ts);
+    if (!id || pinned_buffer_id(h_ts + total - 1) != id) return nullptr;
     return (const int64_t *)a.devicePointer;
 }
 

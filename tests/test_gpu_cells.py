@@ -126,8 +126,10 @@ def test_host_rows_read_in_place_or_copied(pinned, wide):
         ts[3] *= 50_000
     t = torch.from_numpy(ts).pin_memory() if pinned else torch.from_numpy(ts)
     h = zl.ZipLine(n, R, B, 0)
+    before = h.workspace_bytes
     for _ in range(2):
         assert_oracle(ts, 0, h.select_batched_host(t))
+    assert (h.workspace_bytes - before >= ts.nbytes) == (wide or not pinned)       # the staging buffer of the copy
     h.destroy()
 
 
@@ -176,3 +178,32 @@ def test_small_instances_with_a_time_before_every_first_element(n, R, B):
         keep = [0] + list(range(2, min(B, 60)))
         assert_oracle(ts[keep], 0, zl.Selection(sel.idx[keep], sel.barrier[keep], sel.wait[keep], sel.status[keep]))
         h.destroy()
+
+
+def test_host_rows_in_two_pinned_regions_are_not_read_in_place():
+    # the first and the last pages are registered, what lies between is not: the rows are copied (or the copy is refused), and the
+    # staging buffer of the copy exists afterwards
+    import mmap
+    n, R, B = 65, 257, 16
+    ts = zi.generate(zi.CONFIGS["c4"].with_(B=B, n=n, R=R))
+    page, size = mmap.PAGESIZE, ts.nbytes
+    total = -(-size // page) * page
+    m = mmap.mmap(-1, total)
+    a = np.frombuffer(m, dtype=np.int64, count=ts.size).reshape(ts.shape)
+    a[...] = ts
+    t = torch.from_numpy(a)
+    rt = torch.cuda.cudart()
+    ends = ((t.data_ptr(), 4 * page), (t.data_ptr() + total - 4 * page, 4 * page))
+    for p, k in ends:
+        assert int(rt.cudaHostRegister(p, k, 0)) == 0
+    h = zl.ZipLine(n, R, B, 0)
+    before = h.workspace_bytes
+    try:
+        assert_oracle(ts, 0, h.select_batched_host(t))
+    except zl.ZipLineError as e:
+        assert e.code == zl.binding.ZL_ERR_CUDA
+    finally:
+        assert h.workspace_bytes - before >= size
+        h.destroy()
+        for p, _ in ends:
+            assert int(rt.cudaHostUnregister(p)) == 0
