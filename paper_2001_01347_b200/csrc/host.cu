@@ -213,6 +213,7 @@ LaunchPlan make_plan(const zl_handle *h, int B) {
 
 zl_status cuda_fail(zl_handle *h, cudaError_t e) {
     if (h) h->last_cuda_error = (int)e;
+    cudaGetLastError();                                           // reported here: not again by the next call that looks
     return e == cudaErrorMemoryAllocation ? ZL_ERR_NOMEM : ZL_ERR_CUDA;
 }
 

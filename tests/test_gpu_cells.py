@@ -204,6 +204,7 @@ def test_host_rows_in_two_pinned_regions_are_not_read_in_place():
         assert e.code == zl.binding.ZL_ERR_CUDA
     finally:
         assert h.workspace_bytes - before >= size
+        assert_oracle(ts, 0, h.select_batched(torch.from_numpy(ts).cuda()))    # (a refused copy is not reported once more)
         h.destroy()
         for p, _ in ends:
             assert int(rt.cudaHostUnregister(p)) == 0
