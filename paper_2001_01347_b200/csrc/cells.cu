@@ -273,6 +273,12 @@ struct CellShared {
     SegResult best;                               // (in every CTA) the smallest objective so far
 };
 
+// A cell's last time; `limit` is where the timeline (or a CTA's slice of it) ends.  Formed from what is left of it behind the
+// cell's start: start + width would pass 2^32 in the last cell of a timeline that ends just below.
+__device__ __forceinline__ uint32_t cell_end(uint32_t start, uint32_t shift, uint32_t limit) {
+    return start + min((1u << shift) - 1u, limit - 1u - start);
+}
+
 __device__ __forceinline__ float warp_sum(float x) {
 #pragma unroll
     for (int d = 16; d > 0; d >>= 1) x += __shfl_xor_sync(FULL, x, d);
@@ -293,7 +299,7 @@ __device__ __noinline__ bool evaluate_cells(CellShared &sh, int from, int ns, co
         const int k = q / nrows, p = q - k * nrows;
         const int x = sh.order[from + k];
         const uint32_t a = lo + (sh.cell[x] << shift);
-        const uint32_t e = min(a + ((1u << shift) - 1u), hi - 1u);            // the cell's last time
+        const uint32_t e = cell_end(a, shift, hi);
         const uint64_t base = sh.base[x];
         const uint2 en = ends[r0 + p];
         int i = first_at_or_after(rd, r0 + p, R, a, en.x, en.y);
@@ -713,7 +719,7 @@ __global__ void __launch_bounds__(1024, 1) k_cells(const SRC src, const CellPara
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     const int c = 128 * k + 4 * lane + j;
-                    const uint32_t end = min(a + ((uint32_t)(c + 1) << shift) - 1u, bnd - 1u);
+                    const uint32_t end = cell_end(a + ((uint32_t)c << shift), shift, bnd);
                     const uint64_t q = (uint64_t)(g[j] > end ? g[j] - end : 0u) << 24 | (c0 + (uint32_t)c + 1u);      // never 0
                     if (c < m && g[j] != INF32 && q > low && q < key) { key = q; kbase = g[j]; }
                 }
@@ -738,7 +744,7 @@ __global__ void __launch_bounds__(1024, 1) k_cells(const SRC src, const CellPara
                 for (int j = 0; j < 4; ++j) {
                     const int c = 128 * k + 4 * lane + j;
                     if (dv[j] != 0u) {
-                        const uint32_t start = a + ((uint32_t)c << shift), end = min(start + ((1u << shift) - 1u), bnd - 1u);
+                        const uint32_t start = a + ((uint32_t)c << shift), end = cell_end(start, shift, bnd);
                         const uint64_t u = nn * end - S[j], l = nn * start > S[j] ? nn * start - S[j] : 0ull;
                         lbm = min(lbm, l);
                         const uint64_t q = min(u, (uint64_t)0xffffffffffull) << 24 | (c0 + (uint32_t)c + 1u);
@@ -802,7 +808,7 @@ __global__ void __launch_bounds__(1024, 1) k_cells(const SRC src, const CellPara
                 const uint32_t g[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    const uint32_t end = min(a + ((uint32_t)(c + j + 1) << shift) - 1u, bnd - 1u);
+                    const uint32_t end = cell_end(a + ((uint32_t)(c + j) << shift), shift, bnd);
                     const uint64_t l = g[j] > end ? (uint64_t)(g[j] - end) : 0ull;
                     if (c + j < m && l <= d && (l << 24 | (c0 + (uint32_t)(c + j) + 1u)) > low) keep(c0 + (uint32_t)(c + j), g[j], l);
                 }
@@ -823,7 +829,7 @@ __global__ void __launch_bounds__(1024, 1) k_cells(const SRC src, const CellPara
                 for (int j = 0; j < 4; ++j) {
                     const uint32_t c = (uint32_t)(128 * k + 4 * lane + j);
                     if (dv[j] != 0u) {
-                        const uint32_t start = a + (c << shift), end = min(start + ((1u << shift) - 1u), bnd - 1u);
+                        const uint32_t start = a + (c << shift), end = cell_end(start, shift, bnd);
                         const uint64_t st = (uint64_t)n * start, l = st > S[j] ? st - S[j] : 0ull;
                         const uint64_t q = min((uint64_t)n * end - S[j], (uint64_t)0xffffffffffull) << 24 | (c0 + c + 1u);
                         if (l <= d && q > low) keep(c0 + c, S[j] - dv[j], l);

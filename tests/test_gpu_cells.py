@@ -208,3 +208,26 @@ def test_host_rows_in_two_pinned_regions_are_not_read_in_place():
         h.destroy()
         for p, _ in ends:
             assert int(rt.cudaHostUnregister(p)) == 0
+
+
+@pytest.mark.parametrize("objective", [0, 1])
+@pytest.mark.parametrize("short", [0, 16, 999, 1 << 18, (1 << 20) + 7])
+@pytest.mark.parametrize("n,R", [(64, 128), (300, 40), (20, 300)])
+def test_the_last_cell_of_a_timeline_that_ends_just_below_32_bits(n, R, short, objective):
+    # every row ends at the same time, up to the largest that 32 bits hold: the optimum (0) is the last element, in the cell
+    # that 2^32 cuts.  One row has an element shortly before, so that no cell before it sees the last one as its first.
+    end = (1 << 32) - 4 - short
+    rng = np.random.default_rng(n + short)
+    inner = np.sort(rng.integers(1, end - (1 << 21), size=(3, n, R - 2)), axis=2)
+    first, last = np.arange(3 * n).reshape(3, n, 1) % 7, np.full((3, n, 1), end)
+    first[:, 0] = 0
+    ts = np.concatenate([first, inner, last], axis=2).astype(np.int64)
+    ts[:, 1, R - 2] = end - (6 << 16)
+    assert (np.diff(ts, axis=2) >= 0).all()
+    assert_oracle(ts, objective, select(ts, objective)[0])
+    ts += 12_345
+    d = torch.from_numpy(ts).cuda()
+    out = zl.Selection(torch.empty((3, n), dtype=torch.int32, device="cuda"), *(torch.empty(3, dtype=t, device="cuda") for t in (torch.int64, torch.int64, torch.int32)))
+    zl.zl_select_batched_noalloc(d, out, objective)
+    torch.cuda.synchronize()
+    assert_oracle(ts, objective, out)
