@@ -50,8 +50,8 @@ struct zl_handle {
     // options (0 = automatic)
     int opt_threads, opt_lanes, opt_segments, opt_round_factor, opt_no_filter, opt_filter_threads, opt_filter_rows, opt_pdl_off, opt_prologue_threads, opt_tail_threads, opt_filter_round, opt_cluster, opt_filter_stages, opt_checks_off, opt_filter_bulk, opt_tail_cap, opt_max_rounds, opt_no_small, opt_rest_split, opt_no_cells, opt_cells, opt_no_walk;
     int epoch;               // calls so far: the two sets of per-call flags alternate
+    int last_B;              // instances of the last call (0: none yet)
     int last_cuda_error;
-    int launches;
     // optional per-kernel timing: PROF_EVENTS events per recorded call
     cudaEvent_t *prof_ev;
     int prof_cap, prof_calls;
@@ -255,7 +255,7 @@ const char *zl_status_string(zl_status s) {
 
 int32_t zl_max_workers(void) { return zl::MAX_WORKERS; }
 
-static bool walk_route(const zl_handle *h);
+static bool walk_route(const zl_handle *h, int B);
 zl_status zl_create(const zl_config *cfg, zl_handle **out) {
     if (!cfg || !out) return ZL_ERR_INVALID_ARG;
     *out = nullptr;
@@ -357,7 +357,7 @@ zl_status zl_create(const zl_config *cfg, zl_handle **out) {
             memset(&f, 0, sizeof(f));
         }
     }
-    if ((cfg->objective == ZL_OBJ_RANGE && !range_small) || !walk_route(h)) {
+    if ((cfg->objective == ZL_OBJ_RANGE && !range_small) || !walk_route(h, cfg->max_batch)) {
         // cell route, and the words by which a call tells the next one how it went
         if (e == cudaSuccess) e = alloc((void **)&h->d_cflags, 128);
         filter_b += 128;
@@ -526,9 +526,10 @@ static bool small_route(const zl_handle *h) {
            !h->opt_no_filter && !h->opt_no_small && !(h->cfg.flags & ZL_FLAG_FORCE_FILTER);
 }
 
-// RANGE, small instances of few workers, whatever the batch: a warp each (walk.cu).
-static bool walk_route(const zl_handle *h) {
-    return h->cfg.objective == ZL_OBJ_RANGE && zl::walk_shape(h->cfg.n_workers, h->cfg.lookahead_R, h->cfg.max_batch, std::max(1, h->num_sms)) && !h->opt_no_filter && !h->opt_no_small &&
+// RANGE, small instances of few workers: a warp each (walk.cu).  By the instances of the call, not by what the handle has room for
+// (n=64, R=48 on a handle for 4096, one instance: 23 us on the bucket route, 35 with a warp).
+static bool walk_route(const zl_handle *h, int B) {
+    return h->cfg.objective == ZL_OBJ_RANGE && zl::walk_shape(h->cfg.n_workers, h->cfg.lookahead_R, B, std::max(1, h->num_sms)) && !h->opt_no_filter && !h->opt_no_small &&
            !h->opt_no_walk && !(h->cfg.flags & (ZL_FLAG_FORCE_FILTER | ZL_FLAG_FULL_SWEEP | ZL_FLAG_DEBUG_CHECKS));
 }
 
@@ -542,9 +543,9 @@ static int rest_split_now(const zl_handle *h) {
 
 // The cell route: every shape that a warp an instance does not take, unless the handle asks for another route (every timestamp
 // examined, self-checks, a tuning knob of the other routes).
-static bool cells_allowed(const zl_handle *h) {
+static bool cells_allowed(const zl_handle *h, int B) {
     return h->d_cflags && !h->opt_no_filter && !(h->cfg.flags & (ZL_FLAG_FULL_SWEEP | ZL_FLAG_DEBUG_CHECKS | ZL_FLAG_FORCE_FILTER)) &&
-           !walk_route(h) && h->cfg.n_workers >= 4 &&
+           !walk_route(h, B) && h->cfg.n_workers >= 4 &&
            !h->opt_filter_bulk && !h->opt_rest_split && !h->opt_filter_round && !h->opt_filter_threads &&
            !h->opt_filter_rows && !h->opt_cluster && !h->opt_tail_cap && !h->opt_tail_threads && !h->opt_prologue_threads && !h->opt_no_cells;
 }
@@ -562,31 +563,36 @@ static bool cells_allowed(const zl_handle *h) {
 // each has fewer cells (n=74, R=501, B=242 1100 / 233; n=332, R=1107, B=79 1420 / 990; n=937, R=21, B=1606 2440 / 1230).  With a short one the cells cannot pay for the
 // cluster's dozen barriers unless the instances fill the GPU (n=3000, R=10, B=6 73 / 57; n=256, R=24, B=64 40 / 66; n=100, R=10,
 // B=3000 94 / 108; n=1000, R=4, B=1000 210 / 138).
-static bool cells_shape(int objective, int n, int R, int B, int num_sms) {
-    const bool many = B > 4 * num_sms;
+// one_launch: what the call would take otherwise is the one-launch kernel.  The bucket route, which serves such instances on a handle
+// for more of them, is the faster one for few (SUM n=300, R=12, B=64 45 / 32, n=64, R=64 26 / 27; RANGE n=8, R=200, B=64 25 / 23).
+static bool cells_shape(int objective, int n, int R, int B, int num_sms, bool one_launch) {
+    const bool many = B > 4 * num_sms, small = (long long)n * R <= zl::SMALL_MAX;
     if (objective == ZL_OBJ_RANGE) {
-        if (n < 6 || (n < 16 && R > 4096)) return false;
+        if (n < 6 || (n < 16 && (R > 4096 || (small && !one_launch)))) return false;
         return n <= 128 ? R >= 20 || (many && R >= 8) : R >= 96 || (R >= 32 && B >= 64) || (R >= 16 && B >= 256) || (R >= 8 && many);
     }
-    if ((long long)n * R <= zl::SMALL_MAX && !many) return n >= 10 && R >= 12;
+    if (small && !many) return one_launch && n >= 10 && R >= 12;
     if (n < 64 || R < (many ? 10 : B >= 32 ? 24 : 40) || (B >= 256 && n > 512)) return false;
     return R <= (n >= 256 ? (B <= 64 ? 2048 : 512) : B <= 32 ? 512 : 256);
+}
+static bool cells_fit(const zl_handle *h, int B) {
+    return cells_shape(h->cfg.objective, h->cfg.n_workers, h->cfg.lookahead_R, B, std::max(1, h->num_sms), small_route(h));
 }
 // Whether the next call takes it.  A handle's first calls go down the other routes, whose time depends little on how the
 // timestamps fall; then the cells are tried, and stay for as long as they leave nothing over.  A call that did leave some
 // instance to the segment sweep (the word in pinned memory says so) sends the next ones down the other routes again, twice
 // as many after every such call.
-static bool cells_now(const zl_handle *h) {
-    if (!cells_allowed(h)) return false;
+static bool cells_now(const zl_handle *h, int B) {
+    if (!cells_allowed(h, B)) return false;
     if (h->opt_cells) return true;
-    if (!cells_shape(h->cfg.objective, h->cfg.n_workers, h->cfg.lookahead_R, h->cfg.max_batch, std::max(1, h->num_sms))) return false;
+    if (!cells_fit(h, B)) return false;
     if (h->cells_last && ((volatile const uint32_t *)h->h_hint)[1] != 0) return false;
     return h->cells_wait == 0;
 }
 // The decision at a call, and its bookkeeping.
-static bool cells_take(zl_handle *h) {
-    const bool now = cells_now(h);
-    if (h->cells_last && !now && cells_allowed(h)) {
+static bool cells_take(zl_handle *h, int B) {
+    const bool now = cells_now(h, B);
+    if (h->cells_last && !now && cells_allowed(h, B) && cells_fit(h, B)) {
         ((volatile uint32_t *)h->h_hint)[1] = 0;
         ++h->cells_fails;
         h->cells_wait = CELLS_AFTER << std::min(h->cells_fails, 8);
@@ -597,15 +603,16 @@ static bool cells_take(zl_handle *h) {
     return now;
 }
 static void set_cells(Pipeline &q, zl_handle *h) {
-    q.cells = cells_take(h) ? 1 : 0;
+    q.cells = cells_take(h, q.B) ? 1 : 0;
     q.cflags = h->d_cflags;
     q.epoch = ++h->cells_epoch;
 }
 
 int32_t zl_launches_per_call(const zl_handle *h) {
     if (!h) return 0;
-    if (cells_now(h)) return 2;
-    if (small_route(h) || walk_route(h)) return 1;
+    const int B = h->last_B ? h->last_B : h->cfg.max_batch;
+    if (cells_now(h, B)) return 2;
+    if (small_route(h) || walk_route(h, B)) return 1;
     const bool filter = h->cfg.objective == ZL_OBJ_RANGE && !h->opt_no_filter && h->fb.table != nullptr;
     const bool sumfast = !filter && !h->opt_no_filter && h->fb.scap != 0;
     return (filter ? (rest_split_now(h) ? 9 : 4) : 3) + (sumfast ? (h->fb.scells ? 3 : 2) : 0) + ((h->cfg.flags & ZL_FLAG_CHECK_SORTED) ? 1 : 0);
@@ -628,7 +635,7 @@ static void fill_pipeline(Pipeline &q, const zl_handle *h, int B) {
     q.prologue_threads = h->opt_prologue_threads; q.tail_threads = h->opt_tail_threads;
     if (h->opt_no_filter) { q.fb.table = nullptr; q.fb.scap = 0; }
     q.cluster = h->opt_cluster; q.filter_stages = h->opt_filter_stages;
-    q.checks_off = h->opt_checks_off; q.filter_bulk = h->opt_filter_bulk; q.tail_cap = h->opt_tail_cap; q.rest_per_sm = 0; q.max_rounds = h->opt_max_rounds; q.small = small_route(h) ? 1 : 0; q.walk = walk_route(h) ? 1 : 0; q.rest_split = rest_split_now(h) ? 1 : 2;
+    q.checks_off = h->opt_checks_off; q.filter_bulk = h->opt_filter_bulk; q.tail_cap = h->opt_tail_cap; q.rest_per_sm = 0; q.max_rounds = h->opt_max_rounds; q.small = small_route(h) ? 1 : 0; q.walk = walk_route(h, B) ? 1 : 0; q.rest_split = rest_split_now(h) ? 1 : 2;
     q.cells = 0; q.cflags = nullptr; q.epoch = 0; q.idx = nullptr; q.barrier = q.wait = nullptr; q.status = nullptr;
 }
 
@@ -654,9 +661,9 @@ static unsigned long long pinned_buffer_id(const void *p) {
 // twice as many after every such call).  The sortedness check reads every row anyway, and SUM enough of them for the bus to be
 // slower in pieces than in one copy (n=1024, R=1024, B=64: 20.7 ms against 11.6; RANGE 3.0 against 9.8).
 static const int64_t *mapped_rows(zl_handle *h, const int64_t *h_ts, int B) {
-    if (h->cfg.objective != ZL_OBJ_RANGE || !cells_allowed(h) || (h->cfg.flags & ZL_FLAG_CHECK_SORTED)) return nullptr;
+    if (h->cfg.objective != ZL_OBJ_RANGE || !cells_allowed(h, B) || (h->cfg.flags & ZL_FLAG_CHECK_SORTED)) return nullptr;
     const long long total = (long long)B * h->cfg.n_workers * h->cfg.lookahead_R;
-    if (total < MAPPED_MIN || !cells_shape(ZL_OBJ_RANGE, h->cfg.n_workers, h->cfg.lookahead_R, B, std::max(1, h->num_sms))) return nullptr;
+    if (total < MAPPED_MIN || !cells_fit(h, B)) return nullptr;
     if (h->mapped_wait > 0) { --h->mapped_wait; return nullptr; }
     cudaPointerAttributes a, z;                                   // of the first timestamp and of the last one
     if (cudaPointerGetAttributes(&a, h_ts) != cudaSuccess || cudaPointerGetAttributes(&z, h_ts + total - 1) != cudaSuccess) {
@@ -694,7 +701,7 @@ zl_status zl_select_batched(zl_handle *h, const int64_t *d_ts, int32_t B, int32_
         ++h->epoch;
     }
     q.idx = d_idx; q.barrier = d_barrier; q.wait = d_wait; q.status = d_status;
-    h->launches += zl_launches_per_call(h);
+    h->last_B = B;
     set_cells(q, h);
     enqueue(q, p, st, ev, zl::MatBatch{d_ts});
     if (ev) ++h->prof_calls;
@@ -762,7 +769,7 @@ zl_status zl_predict_select_batched(zl_handle *h, const int64_t *d_last, const i
     if (!h || !h->d_pred) return ZL_ERR_INVALID_ARG;
     if (B < 1 || B > h->cfg.max_batch) return ZL_ERR_INVALID_ARG;
     if (!on_device(h->cfg.device)) return ZL_ERR_INVALID_ARG;
-    if ((h->cfg.objective == ZL_OBJ_RANGE && h->fb.table != nullptr) || cells_now(h)) {
+    if ((h->cfg.objective == ZL_OBJ_RANGE && h->fb.table != nullptr) || cells_now(h, B)) {
         // the cell route, or (RANGE) the filter route and its fallback, on generated rows: the predicted matrix is never written
         if (!d_last || !d_interval || !d_idx || !d_barrier || !d_wait) return ZL_ERR_INVALID_ARG;
         if (((uintptr_t)d_last & 7) || ((uintptr_t)d_interval & 7) || ((uintptr_t)d_barrier & 7) || ((uintptr_t)d_wait & 7) ||
@@ -781,7 +788,7 @@ zl_status zl_predict_select_batched(zl_handle *h, const int64_t *d_last, const i
             ++h->epoch;
         }
         q.idx = d_idx; q.barrier = d_barrier; q.wait = d_wait; q.status = d_status;
-        h->launches += zl_launches_per_call(h);
+        h->last_B = B;
         set_cells(q, h);
         enqueue(q, p, (cudaStream_t)cuda_stream, ev, zl::AriBatch{d_last, d_interval});
         if (ev) ++h->prof_calls;
@@ -790,7 +797,6 @@ zl_status zl_predict_select_batched(zl_handle *h, const int64_t *d_last, const i
     }
     zl_status rc = zl_predict_batched(d_last, d_interval, B, h->cfg.n_workers, h->cfg.lookahead_R, h->d_pred, cuda_stream);
     if (rc != ZL_OK) return rc;
-    ++h->launches;
     return zl_select_batched(h, h->d_pred, B, d_idx, d_barrier, d_wait, d_status, cuda_stream);
 }
 
@@ -821,7 +827,6 @@ zl_status zl_select_batched_host(zl_handle *h, const int64_t *h_ts, int32_t B, i
         q.cflags = h->d_cflags; q.epoch = ++h->cells_epoch;
         uint32_t words[8];
         enqueue(q, make_plan(h, B), st, nullptr, zl::MatBatch{in_place});
-        ++h->launches;
         ZL_CUDA(h, cudaGetLastError());
         ZL_CUDA(h, cudaMemcpyAsync(h_idx, h->s_idx, (size_t)B * n * 4, cudaMemcpyDeviceToHost, st));
         ZL_CUDA(h, cudaMemcpyAsync(h_barrier, h->s_barrier, (size_t)B * 8, cudaMemcpyDeviceToHost, st));
@@ -932,7 +937,7 @@ zl_status zl_select_batched_noalloc(int32_t n_workers, int32_t lookahead_R, int3
     q.idx = d_idx; q.barrier = d_barrier; q.wait = d_wait; q.status = d_status;
     q.walk = objective == ZL_OBJ_RANGE && !(flags & ZL_FLAG_FULL_SWEEP) && zl::walk_shape(n_workers, lookahead_R, B, std::max(1, tmp.num_sms)) ? 1 : 0;
     q.cells = !q.walk && !(flags & ZL_FLAG_FULL_SWEEP) && n_workers >= 4 &&
-              cells_shape(objective, n_workers, lookahead_R, B, std::max(1, tmp.num_sms)) ? 1 : 0;
+              cells_shape(objective, n_workers, lookahead_R, B, std::max(1, tmp.num_sms), q.small != 0) ? 1 : 0;
     q.cflags = (uint32_t *)((unsigned char *)g_noalloc_ptr[dev] + NOALLOC_META_BYTES); q.epoch = tmp.cells_epoch;
     enqueue(q, p, (cudaStream_t)cuda_stream, nullptr, zl::MatBatch{d_ts});
     return cudaGetLastError() == cudaSuccess ? ZL_OK : ZL_ERR_CUDA;

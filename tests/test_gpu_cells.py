@@ -231,3 +231,24 @@ def test_the_last_cell_of_a_timeline_that_ends_just_below_32_bits(n, R, short, o
     zl.zl_select_batched_noalloc(d, out, objective)
     torch.cuda.synchronize()
     assert_oracle(ts, objective, out)
+
+
+@pytest.mark.parametrize("objective,n,R,few,many", [(0, 64, 48, 5, 1), (0, 128, 20, 5, 1), (0, 300, 12, 5, 2), (1, 300, 12, 5, 2)])
+def test_the_route_follows_the_instances_of_the_call(objective, n, R, few, many):
+    # one instance on a handle with room for 4096: the kernels that are best for one (the bucket route's, or the cells where
+    # they are), not those that are best for 4096
+    ts = zi.generate(zi.CONFIGS["c3"].with_(B=1300, n=n, R=R))
+    d = torch.from_numpy(ts).cuda()
+    h = zl.ZipLine(n, R, 4096, objective)
+    for _ in range(10):
+        one = h.select_batched(d[:1].contiguous())
+    assert h.launches_per_call == few
+    assert_oracle(ts[:1], objective, one)
+    for _ in range(10):
+        sel = h.select_batched(d)
+    assert h.launches_per_call == many
+    assert_oracle(ts[:40], objective, zl.Selection(sel.idx[:40], sel.barrier[:40], sel.wait[:40], sel.status[:40]))
+    one = h.select_batched(d[:1].contiguous())
+    assert h.launches_per_call == few
+    assert torch.equal(one.idx[0], sel.idx[0]) and one.wait[0] == sel.wait[0]
+    h.destroy()
