@@ -241,7 +241,7 @@ struct CellParams {
     InstMeta *meta;
     uint32_t epoch;                  // number of the call: a word of `flags` is raised when it holds this
     uint32_t *flags;                 // [1] some instance needs the segment sweep, [2] some instance's outputs are missing,
-                                     // [3] some instance was left to the segment sweep for want of room, [4], [5] grid_barrier
+                                     // [3] the calls to come should rather not take this route, [4], [5] grid_barrier
     int32_t *idx; int64_t *barrier; int64_t *wait; int32_t *status;
 };
 
@@ -492,7 +492,7 @@ __global__ void __launch_bounds__(1024, 1) k_cells(const SRC src, const CellPara
         if (rank == 0 && tid == 0) {
             P.meta[b] = M;
             P.flags[2] = P.epoch;                                 // the last kernel writes this instance's outputs
-            if (M.status == ZL_OK) P.flags[1] = P.epoch;
+            if (M.status == ZL_OK) P.flags[1] = P.flags[3] = P.epoch;
         }
         return;
     }
@@ -903,7 +903,7 @@ __global__ void __launch_bounds__(CELL_REST_THREADS) k_cell_rest(const SRC src, 
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ SweepShared sh;
     const uint4 fl = __ldcg(reinterpret_cast<const uint4 *>(P.flags));
-    if (F.hint && fl.w == P.epoch && blockIdx.x == 0 && threadIdx.x == 0) F.hint[1] = 1u;      // for the host's next calls
+    if (F.hint && fl.w == P.epoch && blockIdx.x == 0 && threadIdx.x == 0) F.hint[1] = P.epoch; // for the host's next calls
     if (fl.y != P.epoch && fl.z != P.epoch) return;               // every instance is finished
     bool ok = true;
     if (fl.y == P.epoch) {

@@ -34,6 +34,19 @@
 #include "zl_host.h"
 
 // ================================================================================== host side
+namespace {
+constexpr int CELLS_AFTER = 8;                 // calls of a handle before it tries the cell route
+constexpr int BACKOFF_MOST = 8;                // failures beyond which the wait does not grow
+
+// When a way of doing a call that may not work out is tried again: after a failure the next 16 calls leave it, twice as many after
+// every further one; as many good calls in a row as it last waited take one failure back.
+struct Backoff {
+    int fails, wait, good;
+    void failed() { fails = fails < BACKOFF_MOST ? fails + 1 : BACKOFF_MOST; wait = CELLS_AFTER << fails; good = 0; }
+    void worked() { if (fails > 0 && ++good >= CELLS_AFTER << fails) { --fails; good = 0; } }
+};
+}  // namespace
+
 struct zl_handle {
     zl_config cfg;
     int num_sms;
@@ -62,11 +75,11 @@ struct zl_handle {
     // more survivors than one CTA finishes?); the next call reads it, without waiting, to choose the form of its last stage
     uint32_t *h_hint, *d_hint;
     // cell route
-    uint32_t *d_cflags;      // eight words, then the word last written to the hint
-    uint32_t cells_epoch;    // calls on the cell route
-    int cells_last;          // the previous call took the cell route
-    int cells_fails, cells_wait;   // calls it did not work out for so far; calls left until it is tried (again)
-    int mapped_fails, mapped_wait; // the same for host-buffer calls that read the caller's memory in place
+    uint32_t *d_cflags;      // [0..7] the route's words (see CellParams); [16] the word last written to the hint of the RANGE filter route
+    uint32_t cells_epoch;    // number of the last call (any route)
+    uint32_t cells_since;    // number of the call with which the present run of calls on the cell route began
+    int cells_last;          // the last call of a shape it takes was on it
+    Backoff cells, mapped;   // the cell route; host-buffer calls that read the caller's memory in place
 };
 
 namespace {
@@ -78,7 +91,6 @@ using zl::pow2_floor;
 constexpr int PROF_EVENTS = 5;
 constexpr long long MAPPED_MIN = 1 << 18;      // timestamps from which rows in pinned host memory are read in place (fewer: one copy is over sooner
                                                // than the chain of reads across the bus)
-constexpr int CELLS_AFTER = 8;                 // calls of a handle before it tries the cell route
 constexpr size_t CANARY_BYTES = 64;
 constexpr int CANARY_BYTE = 0xC5;
 
@@ -271,7 +283,7 @@ zl_status zl_create(const zl_config *cfg, zl_handle **out) {
     if (!h) return ZL_ERR_NOMEM;
     memset(h, 0, sizeof(*h));
     h->cfg = *cfg;
-    h->cells_wait = CELLS_AFTER;
+    h->cells.wait = CELLS_AFTER;
     DeviceScope scope(cfg->device);                               // the caller's device is current again on return
     cudaError_t e = scope.err;
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, cfg->device);
@@ -578,34 +590,39 @@ static bool cells_shape(int objective, int n, int R, int B, int num_sms, bool on
 static bool cells_fit(const zl_handle *h, int B) {
     return cells_shape(h->cfg.objective, h->cfg.n_workers, h->cfg.lookahead_R, B, std::max(1, h->num_sms), small_route(h));
 }
+// Whether a call of the present run of calls on the cell route has left some instance to the segment sweep, as far as its word has
+// arrived (the read does not wait).  The word holds the call's number: one that was enqueued before the run began, or that a
+// replayed graph repeats, says nothing about it.
+static bool cells_failed(const zl_handle *h) {
+    const uint32_t w = ((volatile const uint32_t *)h->h_hint)[1];
+    return h->cells_last && w != 0 && (int32_t)(w - h->cells_since) >= 0;
+}
 // Whether the next call takes it.  A handle's first calls go down the other routes, whose time depends little on how the
 // timestamps fall; then the cells are tried, and stay for as long as they leave nothing over.  A call that did leave some
-// instance to the segment sweep (the word in pinned memory says so) sends the next ones down the other routes again, twice
-// as many after every such call.
+// instance to the segment sweep sends the next ones down the other routes again (see Backoff).
 static bool cells_now(const zl_handle *h, int B) {
     if (!cells_allowed(h, B)) return false;
     if (h->opt_cells) return true;
-    if (!cells_fit(h, B)) return false;
-    if (h->cells_last && ((volatile const uint32_t *)h->h_hint)[1] != 0) return false;
-    return h->cells_wait == 0;
+    return cells_fit(h, B) && !cells_failed(h) && h->cells.wait == 0;
 }
-// The decision at a call, and its bookkeeping.
-static bool cells_take(zl_handle *h, int B) {
+// The decision at a call, and its bookkeeping; `epoch` is the call's number.
+static bool cells_take(zl_handle *h, int B, uint32_t epoch) {
     const bool now = cells_now(h, B);
-    if (h->cells_last && !now && cells_allowed(h, B) && cells_fit(h, B)) {
-        ((volatile uint32_t *)h->h_hint)[1] = 0;
-        ++h->cells_fails;
-        h->cells_wait = CELLS_AFTER << std::min(h->cells_fails, 8);
-    } else if (!now && h->cells_wait > 0) {
-        --h->cells_wait;
+    if (!cells_allowed(h, B) || !(h->opt_cells || cells_fit(h, B))) return false;       // not a shape it takes: nothing to learn
+    if (now) {
+        if (!h->cells_last) h->cells_since = epoch; else h->cells.worked();
+    } else if (cells_failed(h)) {
+        h->cells.failed();
+    } else if (h->cells.wait > 0) {
+        --h->cells.wait;
     }
     h->cells_last = now;
     return now;
 }
 static void set_cells(Pipeline &q, zl_handle *h) {
-    q.cells = cells_take(h, q.B) ? 1 : 0;
     q.cflags = h->d_cflags;
     q.epoch = ++h->cells_epoch;
+    q.cells = cells_take(h, q.B, q.epoch) ? 1 : 0;
 }
 
 int32_t zl_launches_per_call(const zl_handle *h) {
@@ -664,7 +681,7 @@ static const int64_t *mapped_rows(zl_handle *h, const int64_t *h_ts, int B) {
     if (h->cfg.objective != ZL_OBJ_RANGE || !cells_allowed(h, B) || (h->cfg.flags & ZL_FLAG_CHECK_SORTED)) return nullptr;
     const long long total = (long long)B * h->cfg.n_workers * h->cfg.lookahead_R;
     if (total < MAPPED_MIN || !cells_fit(h, B)) return nullptr;
-    if (h->mapped_wait > 0) { --h->mapped_wait; return nullptr; }
+    if (h->mapped.wait > 0) { --h->mapped.wait; return nullptr; }
     cudaPointerAttributes a, z;                                   // of the first timestamp and of the last one
     if (cudaPointerGetAttributes(&a, h_ts) != cudaSuccess || cudaPointerGetAttributes(&z, h_ts + total - 1) != cudaSuccess) {
         cudaGetLastError();
@@ -834,8 +851,11 @@ zl_status zl_select_batched_host(zl_handle *h, const int64_t *h_ts, int32_t B, i
         if (h_status) ZL_CUDA(h, cudaMemcpyAsync(h_status, h->s_status, (size_t)B * 4, cudaMemcpyDeviceToHost, st));
         ZL_CUDA(h, cudaMemcpyAsync(words, h->d_cflags, sizeof(words), cudaMemcpyDeviceToHost, st));
         ZL_CUDA(h, cudaStreamSynchronize(st));
-        if (words[1] != q.epoch && words[2] != q.epoch) return ZL_OK;
-        h->mapped_wait = CELLS_AFTER << std::min(++h->mapped_fails, 8);
+        if (words[1] != q.epoch && words[2] != q.epoch) {
+            h->mapped.worked();
+            return ZL_OK;
+        }
+        h->mapped.failed();
     }
     if (!h->s_ts) {
         ZL_CUDA(h, cudaMalloc((void **)&h->s_ts, mb * n * R * 8));

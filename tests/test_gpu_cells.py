@@ -99,20 +99,49 @@ def test_predicted_rows(objective):
         h.destroy()
 
 
-def test_a_handle_takes_the_route_after_its_first_calls_and_leaves_it_when_it_fails():
-    n, R = 64, 128
-    good = torch.from_numpy(zi.generate(zi.CONFIGS["c3"].with_(B=4, n=n, R=R))).cuda()
-    wide = good * 50_000                                           # every instance is left to the segment sweep
-    h = zl.ZipLine(n, R, 4, 0)
-    ref = h.select_batched(good)
-    for _ in range(9):
-        h.select_batched(good)
-    assert h.launches_per_call == 2
-    a = h.select_batched(good)
-    b = h.select_batched(wide)
+def periodic(n, R, B, seed=3):
+    """Workers that all take exactly as long: every period holds a selection of nearly the least wait, far more cells than there
+    is room for are left, and the instance goes to the segment sweep."""
+    rng = np.random.default_rng(seed)
+    return (rng.integers(0, 100_000, size=(B, n, 1)) + 100_000 * np.arange(1, R + 1)).astype(np.int64)
+
+
+@pytest.mark.parametrize("bad_rows", ["periodic", "wide"])
+@pytest.mark.parametrize("objective", [0, 1])
+def test_a_handle_takes_the_route_after_its_first_calls_and_leaves_it_when_it_fails(objective, bad_rows):
+    n, R, B = 64, 512, 4
+    ts = zi.generate(zi.CONFIGS["c3"].with_(B=B, n=n, R=R))
+    rows = periodic(n, R, B) if bad_rows == "periodic" else ts * 50_000           # lists that overflow; spans beyond 32 bits
+    good, bad = torch.from_numpy(ts).cuda(), torch.from_numpy(rows).cuda()
+    if bad_rows == "periodic":
+        assert max(select(rows, objective)[1]) == 1
+    h = zl.ZipLine(n, R, B, objective)
+
+    def calls(k, on_cells):
+        for _ in range(k):
+            assert (h.launches_per_call == 2) == on_cells
+            assert_oracle(ts, objective, h.select_batched(good))
+    calls(8, False)
+    for _ in range(2):                                             # the second failure waits as long as the first: it was made good
+        calls(3, True)
+        for _ in range(10):                                        # several are under way when the first one's word arrives
+            sel = h.select_batched(bad)
+        assert_oracle(rows, objective, sel)
+        torch.cuda.synchronize()
+        assert h.launches_per_call != 2
+        while h.launches_per_call != 2:
+            h.select_batched(good)
+        calls(1, True)
+        torch.cuda.synchronize()
+        calls(40, True)                                            # the late words are not booked against the new run of calls
+    h.select_batched(bad)
     torch.cuda.synchronize()
-    assert torch.equal(a.idx, ref.idx) and torch.equal(a.wait, ref.wait) and torch.equal(a.barrier, ref.barrier)
-    assert torch.equal(b.idx, ref.idx) and torch.equal(b.wait, ref.wait * 50_000)
+    calls(17, False)                                               # the call that sees the word, then the 16 of a first failure
+    calls(1, True)
+    h.select_batched(bad)                                          # a second failure in a row waits twice as long
+    torch.cuda.synchronize()
+    calls(33, False)
+    calls(1, True)
     h.destroy()
 
 
