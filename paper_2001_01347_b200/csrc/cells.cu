@@ -967,7 +967,7 @@ static void enqueue_cells_t(const Pipeline &q, const FilterBufs &fb, const Launc
         cfg.attrs = attr; cfg.numAttrs = cluster > 1 ? 2 : 1;
         cudaLaunchKernelEx(&cfg, kernel, args...);
     };
-    launch(k_cells<OBJ, SRC>, dim3(s.cluster, q.B), s.threads, s.smem, s.cluster, src, P);
+    if (q.cells != 3) launch(k_cells<OBJ, SRC>, dim3(s.cluster, q.B), s.threads, s.smem, s.cluster, src, P);
     if (ev) for (int k = 1; k < 4; ++k) cudaEventRecord(ev[k], st);
     if (q.cells == 2) return;                                     // the caller looks at the flags itself
     SweepParams sp;

@@ -842,18 +842,22 @@ zl_status zl_select_batched_host(zl_handle *h, const int64_t *h_ts, int32_t B, i
         q.idx = h->s_idx; q.barrier = h->s_barrier; q.wait = h->s_wait; q.status = h->s_status;
         q.small = q.walk = 0; q.cells = 2;
         q.cflags = h->d_cflags; q.epoch = ++h->cells_epoch;
-        uint32_t words[8];
-        enqueue(q, make_plan(h, B), st, nullptr, zl::MatBatch{in_place});
-        ZL_CUDA(h, cudaGetLastError());
-        ZL_CUDA(h, cudaMemcpyAsync(h_idx, h->s_idx, (size_t)B * n * 4, cudaMemcpyDeviceToHost, st));
-        ZL_CUDA(h, cudaMemcpyAsync(h_barrier, h->s_barrier, (size_t)B * 8, cudaMemcpyDeviceToHost, st));
-        ZL_CUDA(h, cudaMemcpyAsync(h_wait, h->s_wait, (size_t)B * 8, cudaMemcpyDeviceToHost, st));
-        if (h_status) ZL_CUDA(h, cudaMemcpyAsync(h_status, h->s_status, (size_t)B * 4, cudaMemcpyDeviceToHost, st));
-        ZL_CUDA(h, cudaMemcpyAsync(words, h->d_cflags, sizeof(words), cudaMemcpyDeviceToHost, st));
-        ZL_CUDA(h, cudaStreamSynchronize(st));
-        if (words[1] != q.epoch && words[2] != q.epoch) {
-            h->mapped.worked();
-            return ZL_OK;
+        for (;;) {
+            uint32_t words[8];
+            enqueue(q, make_plan(h, B), st, nullptr, zl::MatBatch{in_place});
+            ZL_CUDA(h, cudaGetLastError());
+            ZL_CUDA(h, cudaMemcpyAsync(h_idx, h->s_idx, (size_t)B * n * 4, cudaMemcpyDeviceToHost, st));
+            ZL_CUDA(h, cudaMemcpyAsync(h_barrier, h->s_barrier, (size_t)B * 8, cudaMemcpyDeviceToHost, st));
+            ZL_CUDA(h, cudaMemcpyAsync(h_wait, h->s_wait, (size_t)B * 8, cudaMemcpyDeviceToHost, st));
+            if (h_status) ZL_CUDA(h, cudaMemcpyAsync(h_status, h->s_status, (size_t)B * 4, cudaMemcpyDeviceToHost, st));
+            ZL_CUDA(h, cudaMemcpyAsync(words, h->d_cflags, sizeof(words), cudaMemcpyDeviceToHost, st));
+            ZL_CUDA(h, cudaStreamSynchronize(st));
+            if (words[1] == q.epoch) break;                       // some instance has to be swept: over a copy of the rows
+            if (words[2] != q.epoch || q.cells == 3) {
+                h->mapped.worked();
+                return ZL_OK;
+            }
+            q.cells = 3;                                          // instances in error, nothing else: their outputs take no rows
         }
         h->mapped.failed();
     }

@@ -37,7 +37,7 @@ struct Pipeline {
     int max_rounds;                                               // 0: automatic; else the segment sweep's round limit
     int rest_per_sm;                                              // CTAs of k_range_rest resident per SM (0: ask the runtime)
     int checks_off;                                               // debug handle: unchecked kernels, clock stamps still taken
-    int cells;                                                    // 1: the cell route; 2: its search only, without the kernel for what it leaves over
+    int cells;                                                    // 1: the cell route; 2: its search only, without the kernel for what it leaves over; 3: that kernel only
     uint32_t *cflags, epoch;                                      // its eight words; the number of the call
     int32_t *idx; int64_t *barrier; int64_t *wait; int32_t *status;
 };

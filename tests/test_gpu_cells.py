@@ -148,7 +148,8 @@ def test_a_handle_takes_the_route_after_its_first_calls_and_leaves_it_when_it_fa
 @pytest.mark.parametrize("pinned", [True, False])
 @pytest.mark.parametrize("wide", [False, True])
 def test_host_rows_read_in_place_or_copied(pinned, wide):
-    # just above 2^18 timestamps; a batch with an instance that the cells leave over is copied after all
+    # just above 2^18 timestamps; a batch with an instance that the cells leave over is copied after all, one with an instance in
+    # error is not
     n, R, B = 65, 257, 16
     ts = zi.generate(zi.CONFIGS["c4"].with_(B=B, n=n, R=R))
     if wide:
@@ -158,6 +159,12 @@ def test_host_rows_read_in_place_or_copied(pinned, wide):
     before = h.workspace_bytes
     for _ in range(2):
         assert_oracle(ts, 0, h.select_batched_host(t))
+    t[5, 0, 0] = -1
+    for _ in range(2):
+        sel = h.select_batched_host(t)
+        keep = [b for b in range(B) if b != 5]
+        assert sel.status[5] == zl.binding.ZL_ERR_INVALID_ARG and (sel.idx[5] == -1).all() and sel.wait[5] == np.iinfo(np.int64).min
+        assert_oracle(ts[keep], 0, zl.Selection(sel.idx[keep], sel.barrier[keep], sel.wait[keep], sel.status[keep]))
     assert (h.workspace_bytes - before >= ts.nbytes) == (wide or not pinned)       # the staging buffer of the copy
     h.destroy()
 
