@@ -42,7 +42,19 @@ constexpr int CELL_NODES = 1024;          // most elements in those
 constexpr int CELL_CLUSTER = 16;          // most CTAs of a cluster
 constexpr long long CELL_ASK = 4;         // asking a row for a cell costs about as much as looking through this many of its elements, all cells of a
                                           // batch at once (n=1024, R=1024, B=64, mean of ten seeds 69 us with 16 and half the batch, 63 with 4)
-constexpr int CELL_ROUNDS = 48;           // most cells evaluated one by one before an instance is given up
+constexpr int CELL_ROUNDS = 4;            // rounds after the first in which more cells may be left than there is room for (regular rows need one or two, SUM
+                                          // up to four; with 48, rows of equal periods, n=64, R=128, took 0.5 ms before they were given up)
+constexpr int CELL_HOPELESS = 2 * CELL_ALIVE;    // ... and so many are never worth a further round
+// Cells evaluated, and eight for every round, beyond which the handle's next calls leave the route: regular rows, over 300 random shapes, need up
+// to 33 (RANGE) and 87 (SUM); where many cells tie the other routes are the faster ones (RANGE, times rounded to half a mean iteration, n=93, R=211,
+// B=64 494 us / 99).
+constexpr int CELL_ASKED_RANGE = 48, CELL_ASKED_SUM = 112;
+constexpr int CELL_IDLE = 32;             // elements of a row in one cell that cannot matter, from which on the row is taken to stand still (one timestamp
+                                          // everywhere, n=1024, R=1024, B=8 511 us / 58 on the filter route: one thread goes through them)
+constexpr float CELL_OFF = 64.f;          // RANGE: elements by which a row's middle is off its estimate, root mean square, from which on the rows are far from
+                                          // arithmetic: what the estimate misses is read by one thread, eight elements after the other (gaps with a power-law
+                                          // tail, n=1024, R=1024, B=8 305 us / 60 on the filter route, bursts of iterations 301 / 70; but iterations that grow
+                                          // fivefold, R=256 and 43 off, n=128, B=256 65 / 284)
 constexpr int CELL_FEW = 8;               // so many cells are asked for in any case
 constexpr int CELL_SLACK = 4;             // elements by which a row may be off its estimate before a further piece is read
 constexpr int GUARD_BINS = 64;            // rows by their span, eight bins to a factor of two below the longest
@@ -113,9 +125,9 @@ __device__ __forceinline__ uint32_t element(const RD &rd, int row, int i) { retu
 // Rows are close to arithmetic, so which pieces a row needs is estimated from its ends; where the estimate falls short on
 // either side the thread of the first or last piece reads on.  act(T) gets nine consecutive times, eight pairs of
 // neighbours: every pair with one of its elements in the range, and the pair that straddles a, comes exactly once; others
-// may come.  The caller leaves out rows without an element in the range.
+// may come.  The caller leaves out rows without an element in the range.  Returns the number of pieces.
 template <class RD, class ACT>
-__device__ __forceinline__ void stream_rows(const RD &rd, int R, int row, bool have, uint32_t e0, uint32_t eR, uint32_t a, uint32_t b, ACT act) {
+__device__ __forceinline__ int stream_rows(const RD &rd, int R, int row, bool have, uint32_t e0, uint32_t eR, uint32_t a, uint32_t b, ACT act) {
     const int lane = threadIdx.x & 31;
     int s0 = 0, np = 0;
     if (have) {
@@ -168,6 +180,7 @@ __device__ __forceinline__ void stream_rows(const RD &rd, int R, int row, bool h
             }
         }
     }
+    return total;
 }
 
 // Index of a row's first element at or after time t, by one thread: windows of eight elements (and the one before them), the
@@ -256,6 +269,7 @@ struct CellShared {
     unsigned long long acc, total, key, kbase;
     uint32_t hist[GUARD_BINS];
     float span;                                   // RANGE: rows of at least this span are guards
+    unsigned int pieces;                          // RANGE: pieces of eight elements that the slice took
     unsigned long long later;                     // RANGE: about how many timestamps of the other rows lie in the range
     // the cells to evaluate (in every CTA), and the order in which that is done
     uint32_t cell[CELL_ALIVE];
@@ -268,8 +282,10 @@ struct CellShared {
     uint32_t gmax[CELL_BATCH], gmin[CELL_BATCH];  // RANGE: ... of all rows'
     uint64_t node[CELL_NODES];                    // the elements in the cells: time << 32 | RANGE the row's next element, SUM the element less the row's previous one
     unsigned int nnodes;
+    int asked;                                    // (in every CTA) cells evaluated, see CELL_ASKED_*
     uint64_t tmp[34];
     unsigned int sstatus;
+    unsigned int slow;                            // (in every CTA) rows far from arithmetic, or standing still
     SegResult best;                               // (in every CTA) the smallest objective so far
 };
 
@@ -308,6 +324,7 @@ __device__ __noinline__ bool evaluate_cells(CellShared &sh, int from, int ns, co
             if (T > sh.gmaxl[k]) atomicMax(&sh.gmaxl[k], T);
             if (T < sh.gminl[k]) atomicMin(&sh.gminl[k], T);
         }
+        int idle = 0;
 #pragma unroll 1
         for (; i < R && T <= e; ++i) {
             const uint32_t nx = element(rd, r0 + p, i + 1);
@@ -316,6 +333,8 @@ __device__ __noinline__ bool evaluate_cells(CellShared &sh, int from, int ns, co
             if (OBJ == ZL_OBJ_RANGE ? (uint64_t)nx > base : pay != 0u) {
                 const unsigned pos = atomicAdd(&ld.nnodes, 1u);
                 if (pos < CELL_NODES) ld.node[pos] = ((uint64_t)T << 32) | pay;
+            } else if (++idle == CELL_IDLE) {
+                sh.slow = 1;
             }
             pv = T; T = nx;
         }
@@ -420,7 +439,7 @@ __global__ void __launch_bounds__(1024, 1) k_cells(const SRC src, const CellPara
             if (lane == 0) sh.tmp[warp] = (uint64_t)__float_as_uint(irr);
         }
         if (tid == 0) {
-            sh.acc = 0; sh.total = 0; sh.key = ~0ull; sh.ncells = 0; sh.nnodes = 0; sh.sstatus = 0; sh.later = 0;
+            sh.acc = 0; sh.total = 0; sh.key = ~0ull; sh.ncells = 0; sh.nnodes = 0; sh.sstatus = 0; sh.later = 0; sh.pieces = 0; sh.slow = 0; sh.asked = 0;
             sh.best.d = sh.best.t = ~0ull; sh.best.valid = 0; sh.best.status = 0;
         }
         if (tid < CELL_BATCH) { sh.gmax[tid] = sh.gmaxl[tid] = 0; sh.gmin[tid] = sh.gminl[tid] = INF32; }
@@ -547,6 +566,7 @@ __global__ void __launch_bounds__(1024, 1) k_cells(const SRC src, const CellPara
 #pragma unroll 1
                 for (int r = 0; r < G; ++r) irr += sh.exi[r];
                 const float dev = sqrtf(irr / (float)((n + (n + 31) / 32 - 1) / ((n + 31) / 32)));
+                if (lane == 0 && dev * sqrtf((float)R) > 2.f * CELL_OFF) sh.slow = 1;      // (dev * sqrt(R) / 2 elements in the middle)
                 k += 1 + (int)(GUARD_IRREGULAR * max(0.f, min(1.f, dev) - 0.1f));
                 k = max(k, __reduce_min_sync(FULL, n0 >= least ? 2 * lane : n1 >= least ? 2 * lane + 1 : GUARD_BINS));
                 if (lane == 0) sh.span = k >= min(GUARD_BINS - 1, top) ? 0.f : __int_as_float((top - k) << 20);
@@ -642,7 +662,7 @@ __global__ void __launch_bounds__(1024, 1) k_cells(const SRC src, const CellPara
                         have = false;
                     }
                 }
-                stream_rows(rd, R, row, have, e.x, e.y, a, bnd, [&](const uint32_t (&T)[9]) {
+                const int pieces = stream_rows(rd, R, row, have, e.x, e.y, a, bnd, [&](const uint32_t (&T)[9]) {
                     if (OBJ == ZL_OBJ_RANGE) {
                         // cell[k] becomes a lower bound of G at the start of cell k (before the prefix maximum): an element
                         // says that G is at least its successor for the cells after its own.  Elements before the slice
@@ -672,6 +692,7 @@ __global__ void __launch_bounds__(1024, 1) k_cells(const SRC src, const CellPara
                         total += in; carry += before;
                     }
                 });
+                if (OBJ == ZL_OBJ_RANGE && lane == 0) atomicAdd(&sh.pieces, (unsigned)pieces);
             }
             if (OBJ == ZL_OBJ_SUM) {
                 carry = warp_reduce(carry, OpAdd());
@@ -790,8 +811,11 @@ __global__ void __launch_bounds__(1024, 1) k_cells(const SRC src, const CellPara
         __syncthreads();
         fits = evaluate_cells<OBJ>(sh, 0, 1, rd, ends, n, R, r0, nrows, lo, hi, shift);
         if (!fits) break;
-        // ---- the cells that may still hold a smaller one, or the same one earlier
+        if (tid == 0) sh.asked += 8;
+        // ---- the cells that may still hold a smaller one, or the same one earlier: only cells before the best one's
         const uint64_t d = sh.best.d;
+        const uint32_t cb = ((uint32_t)sh.best.t - lo) >> shift;
+        const uint64_t limit = d < INF32 ? d << 24 | (cb + 1u) : ~0ull;      // RANGE: the best one's key, as of a cell whose bound is attained
         CellShared &ld = *cl.map_shared_rank(&sh, 0);
         auto keep = [&](uint32_t c, uint64_t base, uint64_t l) {
             const unsigned pos = atomicAdd(&ld.ncells, 1u);
@@ -810,7 +834,8 @@ __global__ void __launch_bounds__(1024, 1) k_cells(const SRC src, const CellPara
                 for (int j = 0; j < 4; ++j) {
                     const uint32_t end = cell_end(a + ((uint32_t)(c + j) << shift), shift, bnd);
                     const uint64_t l = g[j] > end ? (uint64_t)(g[j] - end) : 0ull;
-                    if (c + j < m && l <= d && (l << 24 | (c0 + (uint32_t)(c + j) + 1u)) > low) keep(c0 + (uint32_t)(c + j), g[j], l);
+                    const uint64_t q = l << 24 | (c0 + (uint32_t)(c + j) + 1u);
+                    if (c + j < m && q > low && q < limit) keep(c0 + (uint32_t)(c + j), g[j], l);
                 }
             }
         } else {
@@ -832,7 +857,7 @@ __global__ void __launch_bounds__(1024, 1) k_cells(const SRC src, const CellPara
                         const uint32_t start = a + (c << shift), end = cell_end(start, shift, bnd);
                         const uint64_t st = (uint64_t)n * start, l = st > S[j] ? st - S[j] : 0ull;
                         const uint64_t q = min((uint64_t)n * end - S[j], (uint64_t)0xffffffffffull) << 24 | (c0 + c + 1u);
-                        if (l <= d && q > low) keep(c0 + c, S[j] - dv[j], l);
+                        if ((l < d || (l == d && c0 + c < cb)) && q > low) keep(c0 + c, S[j] - dv[j], l);
                     }
                 }
             }
@@ -846,16 +871,17 @@ __global__ void __launch_bounds__(1024, 1) k_cells(const SRC src, const CellPara
             continue;                                             // (a cluster barrier follows before the length is touched again)
         }
         if (ns > CELL_ALIVE) {                                    // more than there is room for: the next best cell may discard them
-            fits = round < CELL_ROUNDS;
+            fits = round < CELL_ROUNDS && ns <= CELL_HOPELESS;
             if (fits) continue;
             break;
         }
 #pragma unroll 1
-        for (int k = tid; k < ns; k += nt) {                      // most promising first
+        for (int k = tid; k < ns; k += nt) {                      // most promising first, of equal ones the earliest
             const uint64_t l = sh.lb[k];
+            const uint32_t c = sh.cell[k];
             int at = 0;
 #pragma unroll 1
-            for (int i = 0; i < ns; ++i) at += sh.lb[i] < l || (sh.lb[i] == l && i < k);
+            for (int i = 0; i < ns; ++i) at += sh.lb[i] < l || (sh.lb[i] == l && sh.cell[i] < c);
             sh.order[at] = (unsigned short)k;
         }
         __syncthreads();
@@ -863,11 +889,18 @@ __global__ void __launch_bounds__(1024, 1) k_cells(const SRC src, const CellPara
         const int batch = OBJ == ZL_OBJ_SUM ? 8 : max(4, min(CELL_BATCH, 4 * nt / P.rpc));
 #pragma unroll 1
         for (int from = 0; from < ns && fits; from += batch) {
-            if (sh.lb[sh.order[from]] > sh.best.d) break;
+            const int x = sh.order[from];
+            if (sh.lb[x] > sh.best.d || (sh.lb[x] == sh.best.d && sh.cell[x] >= ((uint32_t)sh.best.t - lo) >> shift)) break;
+            if (tid == 0) sh.asked += min(batch, ns - from);
             fits = evaluate_cells<OBJ>(sh, from, min(batch, ns - from), rd, ends, n, R, r0, nrows, lo, hi, shift);
         }
         break;
     }
+    // Rows that the route is not made for: many evaluations, rows that stand still, RANGE rows far off their estimates or far more of
+    // them in one slice than its share.  The result is as good as any, but the handle's next calls are better off elsewhere.
+    if (tid == 0 && (sh.slow || sh.asked > (OBJ == ZL_OBJ_RANGE ? CELL_ASKED_RANGE : CELL_ASKED_SUM) ||
+                     (OBJ == ZL_OBJ_RANGE && G > 1 && streamed == 0 && 16ll * G * ((long long)sh.pieces - 2 * n) > 3ll * n * R)))
+        P.flags[3] = P.epoch;
     cl.sync();                                                    // no CTA leaves while another may still read its memory
     // (a result above the wait known to be attained means rows that are not sorted: the sweep decides)
     if (!fits || !sh.best.valid || sh.best.d > ub) {

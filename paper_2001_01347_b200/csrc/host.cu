@@ -590,7 +590,8 @@ static bool cells_shape(int objective, int n, int R, int B, int num_sms, bool on
 static bool cells_fit(const zl_handle *h, int B) {
     return cells_shape(h->cfg.objective, h->cfg.n_workers, h->cfg.lookahead_R, B, std::max(1, h->num_sms), small_route(h));
 }
-// Whether a call of the present run of calls on the cell route has left some instance to the segment sweep, as far as its word has
+// Whether the cell route did not work out for a call of the present run of calls on it - some instance was left to the segment sweep,
+// or took many more evaluations than rows of the kind that the route is made for -, as far as its word has
 // arrived (the read does not wait).  The word holds the call's number: one that was enqueued before the run began, or that a
 // replayed graph repeats, says nothing about it.
 static bool cells_failed(const zl_handle *h) {
@@ -598,8 +599,8 @@ static bool cells_failed(const zl_handle *h) {
     return h->cells_last && w != 0 && (int32_t)(w - h->cells_since) >= 0;
 }
 // Whether the next call takes it.  A handle's first calls go down the other routes, whose time depends little on how the
-// timestamps fall; then the cells are tried, and stay for as long as they leave nothing over.  A call that did leave some
-// instance to the segment sweep sends the next ones down the other routes again (see Backoff).
+// timestamps fall; then the cells are tried, and stay for as long as they work out.  A call for which they did
+// not sends the next ones down the other routes again (see Backoff).
 static bool cells_now(const zl_handle *h, int B) {
     if (!cells_allowed(h, B)) return false;
     if (h->opt_cells) return true;
@@ -854,7 +855,7 @@ zl_status zl_select_batched_host(zl_handle *h, const int64_t *h_ts, int32_t B, i
             ZL_CUDA(h, cudaStreamSynchronize(st));
             if (words[1] == q.epoch) break;                       // some instance has to be swept: over a copy of the rows
             if (words[2] != q.epoch || q.cells == 3) {
-                h->mapped.worked();
+                if (words[3] == q.epoch) h->mapped.failed(); else h->mapped.worked();
                 return ZL_OK;
             }
             q.cells = 3;                                          // instances in error, nothing else: their outputs take no rows
