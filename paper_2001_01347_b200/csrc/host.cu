@@ -79,7 +79,9 @@ struct zl_handle {
     uint32_t cells_epoch;    // number of the last call (any route)
     uint32_t cells_since;    // number of the call with which the present run of calls on the cell route began
     int cells_last;          // the last call of a shape it takes was on it
-    Backoff cells, mapped;   // the cell route; host-buffer calls that read the caller's memory in place
+    uint32_t walk_since;     // the same two for the warp-per-instance kernel
+    int walk_last;
+    Backoff cells, walk, mapped;   // the cell route; the warp-per-instance kernel; host-buffer calls that read the caller's memory in place
 };
 
 namespace {
@@ -267,7 +269,6 @@ const char *zl_status_string(zl_status s) {
 
 int32_t zl_max_workers(void) { return zl::MAX_WORKERS; }
 
-static bool walk_route(const zl_handle *h, int B);
 zl_status zl_create(const zl_config *cfg, zl_handle **out) {
     if (!cfg || !out) return ZL_ERR_INVALID_ARG;
     *out = nullptr;
@@ -369,8 +370,8 @@ zl_status zl_create(const zl_config *cfg, zl_handle **out) {
             memset(&f, 0, sizeof(f));
         }
     }
-    if ((cfg->objective == ZL_OBJ_RANGE && !range_small) || !walk_route(h, cfg->max_batch)) {
-        // cell route, and the words by which a call tells the next one how it went
+    {
+        // the cell route's words, and those by which a call tells the next ones how it went
         if (e == cudaSuccess) e = alloc((void **)&h->d_cflags, 128);
         filter_b += 128;
         if (e == cudaSuccess) e = cudaMemset(h->d_cflags, 0, 128);
@@ -590,6 +591,27 @@ static bool cells_shape(int objective, int n, int R, int B, int num_sms, bool on
 static bool cells_fit(const zl_handle *h, int B) {
     return cells_shape(h->cfg.objective, h->cfg.n_workers, h->cfg.lookahead_R, B, std::max(1, h->num_sms), small_route(h));
 }
+// Whether the warp-per-instance kernel takes the next call: it leaves the instances it is not made for to the other routes as the cell
+// route does (below), but is tried from a handle's first call on.
+static bool walk_now(const zl_handle *h, int B) {
+    if (!walk_route(h, B)) return false;
+    const uint32_t w = ((volatile const uint32_t *)h->h_hint)[2];
+    return !(h->walk_last && w != 0 && (int32_t)(w - h->walk_since) >= 0) && h->walk.wait == 0;
+}
+static bool walk_take(zl_handle *h, int B, uint32_t epoch) {
+    if (!walk_route(h, B)) return false;
+    const bool now = walk_now(h, B);
+    if (now) {
+        if (!h->walk_last) h->walk_since = epoch; else h->walk.worked();
+    } else if (h->walk_last) {
+        h->walk.failed();
+    } else {
+        --h->walk.wait;
+    }
+    h->walk_last = now;
+    return now;
+}
+
 // Whether the cell route did not work out for a call of the present run of calls on it - some instance was left to the segment sweep,
 // or took many more evaluations than rows of the kind that the route is made for -, as far as its word has
 // arrived (the read does not wait).  The word holds the call's number: one that was enqueued before the run began, or that a
@@ -624,13 +646,14 @@ static void set_cells(Pipeline &q, zl_handle *h) {
     q.cflags = h->d_cflags;
     q.epoch = ++h->cells_epoch;
     q.cells = cells_take(h, q.B, q.epoch) ? 1 : 0;
+    q.walk = q.ts && walk_take(h, q.B, q.epoch) ? 1 : 0;
 }
 
 int32_t zl_launches_per_call(const zl_handle *h) {
     if (!h) return 0;
     const int B = h->last_B ? h->last_B : h->cfg.max_batch;
     if (cells_now(h, B)) return 2;
-    if (small_route(h) || walk_route(h, B)) return 1;
+    if (small_route(h) || walk_now(h, B)) return 1;
     const bool filter = h->cfg.objective == ZL_OBJ_RANGE && !h->opt_no_filter && h->fb.table != nullptr;
     const bool sumfast = !filter && !h->opt_no_filter && h->fb.scap != 0;
     return (filter ? (rest_split_now(h) ? 9 : 4) : 3) + (sumfast ? (h->fb.scells ? 3 : 2) : 0) + ((h->cfg.flags & ZL_FLAG_CHECK_SORTED) ? 1 : 0);
@@ -653,7 +676,7 @@ static void fill_pipeline(Pipeline &q, const zl_handle *h, int B) {
     q.prologue_threads = h->opt_prologue_threads; q.tail_threads = h->opt_tail_threads;
     if (h->opt_no_filter) { q.fb.table = nullptr; q.fb.scap = 0; }
     q.cluster = h->opt_cluster; q.filter_stages = h->opt_filter_stages;
-    q.checks_off = h->opt_checks_off; q.filter_bulk = h->opt_filter_bulk; q.tail_cap = h->opt_tail_cap; q.rest_per_sm = 0; q.max_rounds = h->opt_max_rounds; q.small = small_route(h) ? 1 : 0; q.walk = walk_route(h, B) ? 1 : 0; q.rest_split = rest_split_now(h) ? 1 : 2;
+    q.checks_off = h->opt_checks_off; q.filter_bulk = h->opt_filter_bulk; q.tail_cap = h->opt_tail_cap; q.rest_per_sm = 0; q.max_rounds = h->opt_max_rounds; q.small = small_route(h) ? 1 : 0; q.walk = 0; q.rest_split = rest_split_now(h) ? 1 : 2;
     q.cells = 0; q.cflags = nullptr; q.epoch = 0; q.idx = nullptr; q.barrier = q.wait = nullptr; q.status = nullptr;
 }
 
@@ -960,7 +983,7 @@ zl_status zl_select_batched_noalloc(int32_t n_workers, int32_t lookahead_R, int3
     memset(&q.fb, 0, sizeof(q.fb));
     q.filter_threads = q.filter_rows = q.filter_round = 0; q.pdl_off = 0; q.prologue_threads = q.tail_threads = 0; q.cluster = q.filter_stages = 0; q.checks_off = 0; q.filter_bulk = 0; q.tail_cap = 0; q.rest_per_sm = 0; q.max_rounds = 0; q.rest_split = 0; q.small = (long long)n_workers * lookahead_R <= zl::SMALL_MAX && B <= 4 * std::max(1, tmp.num_sms) ? 1 : 0;
     q.idx = d_idx; q.barrier = d_barrier; q.wait = d_wait; q.status = d_status;
-    q.walk = objective == ZL_OBJ_RANGE && !(flags & ZL_FLAG_FULL_SWEEP) && zl::walk_shape(n_workers, lookahead_R, B, std::max(1, tmp.num_sms)) ? 1 : 0;
+    q.walk = objective == ZL_OBJ_RANGE && !(flags & ZL_FLAG_FULL_SWEEP) && zl::walk_shape_alone(n_workers, lookahead_R) ? 1 : 0;
     q.cells = !q.walk && !(flags & ZL_FLAG_FULL_SWEEP) && n_workers >= 4 &&
               cells_shape(objective, n_workers, lookahead_R, B, std::max(1, tmp.num_sms), q.small != 0) ? 1 : 0;
     q.cflags = (uint32_t *)((unsigned char *)g_noalloc_ptr[dev] + NOALLOC_META_BYTES); q.epoch = tmp.cells_epoch;

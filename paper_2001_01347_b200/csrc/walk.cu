@@ -17,11 +17,15 @@ constexpr int WALK_ALONE = 256;            // timestamps of an instance whose pa
 constexpr int WALK_MAX_CELLS = 512;
 constexpr int WALK_PASSES = 24;            // most passes that take a single candidate
 constexpr unsigned WALK_NODES = 128;       // room for candidates
+constexpr int WALK_PASSES_FINE = 1;        // passes that take single candidates, beyond which the handle's next calls leave the kernel (regular
+                                           // instances need none)
 
 struct WalkParams {
     int n, R, B, stride, cells, words, check_sorted;      // stride: words between rows in shared memory: R and one that reads as infinite
     const int64_t *ts;
     int32_t *idx; int64_t *barrier; int64_t *wait; int32_t *status;
+    uint32_t *slow, epoch;                                // pinned host memory, or nullptr: set to the call's number by an instance that this
+                                                          // kernel is not made for (many equal or nearly equal waits, spans of 2^32 and more)
 };
 
 // Relative times as 32-bit words in shared memory, or (spans of 2^32 and more) 64-bit values straight from the rows.
@@ -93,7 +97,7 @@ __device__ __forceinline__ int first_from(const ROWS &rows, int p, int R, typena
 // the warp's.  False: more candidates than there is room for.
 template <int K>
 __device__ __forceinline__ bool search_cells(const NarrowRows &rows, int n, int R, uint32_t t0, uint32_t lmin, uint32_t *cell, int most, uint64_t *node,
-                                             uint32_t &bd, uint32_t &bt) {
+                                             uint32_t &bd, uint32_t &bt, int &passes) {
     const int lane = threadIdx.x & 31, N = n * rows.stride;       // all words of the rows, one after the other
     const int per = most / 32, ps = __ffs(per) - 1;               // a run of cells a lane; cell c sits at c + c / per (no bank conflicts)
     // T - 1 < lmin, so its cell ((T - 1) * scale) >> 32 is below `most`.  (T = 0, a time before the first elements, is only met in
@@ -169,7 +173,7 @@ __device__ __forceinline__ bool search_cells(const NarrowRows &rows, int n, int 
         return __reduce_max_sync(FULL, g);
     };
     // Best first: (bound, time) of the elements, in that order.  A pass over the elements collects those behind the last one
-    // evaluated whose bound does not exceed d; while there are more than there is room for, only the first of them is taken.
+    // evaluated whose bound is below d (or d itself, at an earlier time); while there are more than there is room for, only the first of them is taken.
     uint64_t after = 0;
     unsigned fill = 0;
 #pragma unroll 1
@@ -185,7 +189,7 @@ __device__ __forceinline__ bool search_cells(const NarrowRows &rows, int n, int 
                 if (T - 1u < lmin) {
                     const uint32_t g = max(*cell_at(T), T), l = g - T;
                     q = ((uint64_t)l << 32) | T;
-                    keep = nx > g && l <= d && q >= after;
+                    keep = nx > g && (l < d || (l == d && T < t)) && q >= after;
                 }
             }
             if (keep) first = min(first, q);
@@ -197,6 +201,7 @@ __device__ __forceinline__ bool search_cells(const NarrowRows &rows, int n, int 
             }
         }
         __syncwarp();
+        passes = pass;
         if (fill <= WALK_NODES) break;
         if (pass >= WALK_PASSES) return false;
         // the lanes' first candidates, best first
@@ -289,7 +294,7 @@ __global__ void __launch_bounds__(128) k_walk(const WalkParams P) {
     for (int p = lane; p < n; p += 32) x[p * P.stride + R] = (uint32_t)(uint64_t)tmin - 2u;      // relative: infinite
     __syncwarp();
     int64_t bar = INT64_MIN, wt = INT64_MIN;
-    int at[K];
+    int at[K], passes = 0;
 #pragma unroll
     for (int k = 0; k < K; ++k) at[k] = -1;
     if (status == ZL_OK) {
@@ -297,13 +302,14 @@ __global__ void __launch_bounds__(128) k_walk(const WalkParams P) {
             const NarrowRows rows{x, (uint32_t)(uint64_t)tmin - 1u, P.stride};
             const uint32_t last = (uint32_t)(lmin - tmin) + 1u;
             uint32_t d, t;
-            if (!search_cells<K>(rows, n, R, (uint32_t)(t0 - tmin) + 1u, last, cell, P.cells, node, d, t)) walk<K>(rows, n, R, last, d, t);
+            if (!search_cells<K>(rows, n, R, (uint32_t)(t0 - tmin) + 1u, last, cell, P.cells, node, d, t, passes)) walk<K>(rows, n, R, last, d, t);
             bar = tmin - 1 + (int64_t)(t + d); wt = (int64_t)d;
 #pragma unroll
             for (int k = 0; k < K; ++k) if (32 * k + lane < n) at[k] = first_from(rows, 32 * k + lane, R, t + d + 1u) - 1;
         } else {
             const WideRows rows{ts, tmin, R};
             uint64_t d, t;
+            passes = WALK_PASSES;
             walk<K>(rows, n, R, (uint64_t)(lmin - tmin) + 1, d, t);
             bar = tmin - 1 + (int64_t)(t + d); wt = (int64_t)d;
 #pragma unroll
@@ -311,6 +317,7 @@ __global__ void __launch_bounds__(128) k_walk(const WalkParams P) {
         }
     }
     if (lane == 0) {
+        if (passes > WALK_PASSES_FINE && P.slow) *(volatile uint32_t *)P.slow = P.epoch;
         P.wait[b] = wt;
         P.barrier[b] = bar;
         if (P.status) P.status[b] = status;
@@ -321,11 +328,15 @@ __global__ void __launch_bounds__(128) k_walk(const WalkParams P) {
 
 // A warp's passes over the elements and its few evaluations are one chain: the more elements, the more other warps it needs
 // beside it to be worth more than a CTA that sorts the instance, and the rows must be short and not too few for the bounds to
-// be tight.  Measured in us, this kernel / a CTA an instance: n=16, R=16, B=1 6.2 / 11; n=4, R=80 10 / 17 (B=1), 22 / 50 (4800);
+// be tight.  (Instances with many equal or nearly equal waits cost it 5 to 20 times what a CTA that sorts them takes, n=16, R=64 B=1 335-650 us,
+// B=1500 340-710, against 30-50: a handle leaves the kernel after such a call, and without a handle only instances of
+// at most WALK_ALONE timestamps are given to it.)  Measured in us, this kernel / a CTA an instance: n=16, R=16, B=1 6.2 / 11; n=4, R=80 10 / 17 (B=1), 22 / 50 (4800);
 // n=16, R=30 13 / 23 (100), 13 / 21 (600), 22 / 58 (4800); n=32, R=32 14 / 24 (1), 19 / 23 (600), 38 / 84 (4800); n=100, R=10 18 / 15
 // (1), 25 / 17 (100), 27 / 34 (600); n=16, R=100 32 / 29 (600), 37 / 40 (1200), 62 / 116 (4800); n=60, R=50 44 / 42 (600), 45 / 68
 // (1200); n=128, R=20 57 / 77 (1200); but n=64, R=64 93 / 75 (1200), n=16, R=128 45 / 43 (1200), n=4, R=200 53 / 30 (1200), n=97, R=4 19 / 15 (6), n=2,
 // R=28 11 / 7 (522).
+bool walk_shape_alone(int n, int R) { return (long long)n * R <= WALK_ALONE && walk_shape(n, R, 1, 1); }
+
 bool walk_shape(int n, int R, int batch, int num_sms) {
     const long long N = (long long)n * R;
     if (n > 128 || R > 100 || (n < 4 && N > 32)) return false;
@@ -336,6 +347,7 @@ bool walk_shape(int n, int R, int batch, int num_sms) {
 void enqueue_walk(const Pipeline &q, cudaStream_t st) {
     WalkParams P;
     P.n = q.n; P.R = q.R; P.B = q.B; P.stride = q.R + 1; P.check_sorted = (q.flags & ZL_FLAG_CHECK_SORTED) ? 1 : 0;
+    P.slow = q.fb.hint && q.epoch ? q.fb.hint + 2 : nullptr; P.epoch = q.epoch;
     P.ts = q.ts; P.idx = q.idx; P.barrier = q.barrier; P.wait = q.wait; P.status = q.status;
     const int warps = q.B > 4 * q.num_sms ? 4 : 1;                // few instances: one on an SM
     // about eight cells an iteration of the slowest worker: fewer leave more candidates, more cost the passes over them

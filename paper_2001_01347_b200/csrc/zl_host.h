@@ -105,6 +105,7 @@ cudaError_t cell_limits();
 
 // walk.cu: RANGE, small instances of up to 128 workers, a warp per instance in one launch
 bool walk_shape(int n, int R, int batch, int num_sms);
+bool walk_shape_alone(int n, int R);      // ... whatever the rows hold
 void enqueue_walk(const Pipeline &q, cudaStream_t st);
 cudaError_t walk_limits();
 

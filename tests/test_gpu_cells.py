@@ -269,7 +269,7 @@ def test_the_last_cell_of_a_timeline_that_ends_just_below_32_bits(n, R, short, o
     assert_oracle(ts, objective, out)
 
 
-@pytest.mark.parametrize("objective,n,R,few,many", [(0, 64, 48, 5, 1), (0, 128, 20, 5, 1), (0, 300, 12, 5, 2), (1, 300, 12, 5, 2)])
+@pytest.mark.parametrize("objective,n,R,few,many", [(0, 64, 48, 2, 1), (0, 128, 20, 2, 1), (0, 300, 12, 5, 2), (1, 300, 12, 5, 2)])
 def test_the_route_follows_the_instances_of_the_call(objective, n, R, few, many):
     # one instance on a handle with room for 4096: the kernels that are best for one (the bucket route's, or the cells where
     # they are), not those that are best for 4096

@@ -91,3 +91,42 @@ def test_many_selections_of_the_least_wait(n, R, B, objective, kind):
 @pytest.mark.parametrize("n,R,B", [(300, 1023, 3), (1024, 1024, 8)])
 def test_rows_far_from_arithmetic(n, R, B, kind):
     compare(rows(kind, n, R, B), 0, 2.0)
+
+
+@pytest.mark.parametrize("kind", ["identical rows", "equal periods", "coarse clock", "small numbers", "wide"])
+@pytest.mark.parametrize("n,R,B", [(16, 64, 1500), (16, 64, 2), (33, 24, 700)])
+def test_small_instances_with_many_selections_of_the_least_wait(n, R, B, kind):
+    ts = rows("coarse clock", n, R, B) * 50_000 if kind == "wide" else rows(kind, n, R, B)
+    compare(ts, 0, 1.5)
+
+
+def test_regular_small_instances_stay_with_a_warp_each():
+    import zl_inputs as zi
+    for recipe in ("c2", "c3", "c4"):
+        for n, R in ((16, 64), (32, 32), (20, 100)):
+            ts = torch.from_numpy(zi.generate(zi.CONFIGS[recipe].with_(B=4096, n=n, R=R))).cuda()
+            h = zl.ZipLine(n, R, 4096, 0)
+            for _ in range(3):
+                h.select_batched(ts)
+                torch.cuda.synchronize()
+            assert h.launches_per_call == 1                        # (4 on the bucket route)
+            h.destroy()
+
+
+def test_small_instances_without_a_handle():
+    # no state to learn from: at most twice what a CTA an instance takes, whatever the rows hold
+    for n, R, B in ((16, 64, 2), (16, 16, 2), (32, 32, 8)):
+        for kind in ("equal periods", "identical rows", "coarse clock"):
+            ts = torch.from_numpy(rows(kind, n, R, B)).cuda()
+            out = zl.Selection(torch.empty((B, n), dtype=torch.int32, device="cuda"),
+                               *(torch.empty(B, dtype=t, device="cuda") for t in (torch.int64, torch.int64, torch.int32)))
+            zl.zl_select_batched_noalloc(ts, out, 0)
+            check(ts.cpu().numpy(), 0, out)
+            h = zl.ZipLine(n, R, B, 0)
+            h.set_option("no_cells", 1)
+            h.set_option("no_walk", 1)
+            sel = h.select_batched(ts)
+            plain = us(lambda: h.select_batched(ts, sel))
+            t = us(lambda: zl.zl_select_batched_noalloc(ts, out, 0))
+            assert t <= 2 * plain + 30, (n, R, kind, t, plain)
+            h.destroy()
