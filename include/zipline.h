@@ -96,6 +96,10 @@ zl_status zl_create(const zl_config *cfg, zl_handle **out);
  *             allocates or synchronises.  The caller owns every buffer.  The current
  *             device must be the handle's (cfg.device): ZL_ERR_INVALID_ARG otherwise.
  *
+ * A handle's first eight calls take kernels whose time depends little on how the timestamps fall; after that (small RANGE
+ * instances: from the first call on) it tries the ones that are made for rows of fairly regular iterations, 1.5 to 10 times
+ * faster on such rows, and goes back for a while after a call for which they did not work out.  The results are the same.
+ *
  * Result definition: wait is the minimum of d_Z over all R^n selections;
  * barrier is the smallest max(Z) among the minimisers; idx[p] is the largest i
  * with e^p_i <= barrier.  Returns host-detectable errors only.
@@ -198,11 +202,13 @@ zl_status zl_trace_batched(const int64_t *d_ts, int32_t B, int32_t n, int32_t R,
  * point keeps the scratch it needs (per-instance summaries and per-segment partial
  * results) in a fixed array compiled into the library instead, zl_noalloc_scratch_bytes()
  * bytes (about 400 KB) that every GPU using the library holds until the process exits.
- * It calls no cudaMalloc, cudaFree or other allocating routine.  Instances of at most
- * 4096 timestamps in batches of up to four per SM run the one-launch kernel, which needs
- * no scratch at all; everything else runs the segment sweep.  The faster filter route of
- * the RANGE objective needs buffers of about the size of the input and is only available
- * through a handle.
+ * It calls no cudaMalloc, cudaFree or other allocating routine.  Where the sizes allow it searches
+ * over time cells, which needs no buffers; instances of at most 4096 timestamps in batches of up
+ * to four per SM otherwise run the one-launch kernel, which needs no scratch at all; everything
+ * else, and what the cells leave over, runs the segment sweep.  (Nothing is learnt from one call
+ * for the next here: rows far from regular - equal periods, one timestamp everywhere - cost up to
+ * three times the sweep alone.)  The filter route of the RANGE objective and the bucket route need
+ * buffers of about the size of the input and are only available through a handle.
  *
  * Arguments are those of zl_create's configuration (n_workers, lookahead_R, objective,
  * flags) followed by those of zl_select_batched, with the same meaning, layout and
