@@ -256,12 +256,14 @@ def main():
             call()
         torch.cuda.synchronize()
         if inner is None:
+            # of the calls to come: a handle's first eight take other routes than these (warm-up or not)
             a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-            a.record()
-            for _ in range(8):
-                call()
-            b.record()
-            torch.cuda.synchronize()
+            for calls in (0 if host else 16, 8):
+                a.record()
+                for _ in range(calls):
+                    call()
+                b.record()
+                torch.cuda.synchronize()
             est_ms = a.elapsed_time(b) / 8
             inner = 1 if host else max(1, int(np.ceil(1.3 * MIN_TIMED_MS / (steps * est_ms))))
         if world > 1:
