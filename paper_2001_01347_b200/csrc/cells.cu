@@ -39,7 +39,17 @@ constexpr uint32_t INF32 = 0xffffffffu;
 constexpr int CELL_ALIVE = 128;           // most cells of an instance that the bounds may leave
 constexpr int CELL_BATCH = 16;            // most cells that the rows are asked for at once
 constexpr int CELL_NODES = 1024;          // most elements in those
+constexpr int CELL_PAIRS = 256;            // answers that a batch of cells should give, from what the last ones gave
 constexpr int CELL_CLUSTER = 16;          // most CTAs of a cluster
+// Most threads of a CTA, and so registers a thread: 96, or (RANGE) 80 where three CTAs share an SM or rows are very short and many do
+// (n=200, R=100, B=400 36 us with 80, 44 with 96; n=809, R=8, B=865 59 / 71; but n=1024, R=1024, B=64 48 / 44, n=128, R=256, B=1024 49 / 46).  With
+// 72 or 64 registers values are spilled inside the loops, and what is spilled has often left the L1 cache, past which the rows
+// stream, by the time it is wanted back: n=1024, R=1024, B=64 55 and 74 us.
+constexpr int CELL_THREADS = 640, CELL_THREADS_MANY = 768;
+constexpr int CELL_FIRST = 4;             // most runs of cells that a round asks for at first
+// Cells next to one another are asked for as one: the eight elements that a row is looked at for hold what it has in several cells as well.
+// RUN: most cells of a run (a power of two); two cells of the list belong to one if there are at most RUN / 2 others between them.
+template <int OBJ> constexpr uint32_t CELL_RUN = OBJ == ZL_OBJ_SUM ? 32 : 8;
 constexpr long long CELL_ASK = 4;         // asking a row for a cell costs about as much as looking through this many of its elements, all cells of a
                                           // batch at once (n=1024, R=1024, B=64, mean of ten seeds 69 us with 16 and half the batch, 63 with 4)
 constexpr int CELL_ROUNDS = 4;            // rounds after the first in which more cells may be left than there is room for (regular rows need one or two, SUM
@@ -56,7 +66,8 @@ constexpr float CELL_OFF = 64.f;          // RANGE: elements by which a row's mi
                                           // tail, n=1024, R=1024, B=8 305 us / 60 on the filter route, bursts of iterations 301 / 70; but iterations that grow
                                           // fivefold, R=256 and 43 off, n=128, B=256 65 / 284)
 constexpr int CELL_FEW = 8;               // so many cells are asked for in any case
-constexpr int CELL_SLACK = 4;             // elements by which a row may be off its estimate before a further piece is read
+constexpr int CELL_SLACK = 4;             // elements by which a row may be off its estimate before it is read on, at least
+constexpr int EXPECTED_BINS = 2;
 constexpr int GUARD_BINS = 64;            // rows by their span, eight bins to a factor of two below the longest
 constexpr float GUARD_IRREGULAR = 32.f;   // bins by which more rows are looked through, to a unit of their gaps' relative deviation above 0.1
 constexpr float RANGE_CELLS = 100.f;      // RANGE: cells to the longest mean iteration
@@ -64,153 +75,268 @@ constexpr float SUM_WIDTH = 0.12f;        // SUM: n cell widths against the spre
 
 // ------------------------------------------------------------------------------ rows
 // Relative times of an instance's rows, 32 bits: elements before the first are at time 0 (before everything), those behind
-// the last infinite.  in(): one element known to exist.  eight(): T[0] = element i - 1, T[k] = element i + k - 1, with i as
-// given by align() (a 32-byte boundary of memory): two 32-byte loads and a single one, all under way together.
+// the last infinite.  in(): one element known to exist.  load(): elements i .. i + 7 as they are stored, with i as given by
+// align() (a 32-byte boundary of memory: two 32-byte loads), which rel() makes times of, and trim() sees to what lies
+// outside the row.  load() has no branch - one whose sides meet again in the same registers makes the loads in it wait for
+// each other -: pieces that the matrix does not have the memory for, at its very ends, are !whole() and hold something else.
 template <class SRC> struct RowReader;
 template <> struct RowReader<MatBatch> {
-    const int64_t *inst; int R; uint32_t tminlo;
-    __device__ __forceinline__ RowReader(const MatBatch &s, int b, int n, int R_, int64_t tmin)
-        : inst(s.ts + (size_t)b * n * R_), R(R_), tminlo((uint32_t)(uint64_t)tmin - 1u) {}
+    const int64_t *inst; int R; uint32_t tminlo; int first, last;     // the piece that starts at element i + row * R exists from `first` to `last`
+    __device__ __forceinline__ RowReader(const MatBatch &s, int b, int B, int n, int R_, int64_t tmin)
+        : inst(s.ts + (size_t)b * n * R_), R(R_), tminlo((uint32_t)(uint64_t)tmin - 1u) {
+        const int off = (int)(((uintptr_t)inst >> 3) & 3u);           // elements from the boundary before the instance to its first
+        first = b > 0 ? -off : off ? 4 - off : 0;
+        last = (int)min((long long)(B - b) * n * R_ - 8, 0x7ffffff0ll);
+        last -= (last + off) & 3;                                     // (a matrix of fewer than eight elements: last < first)
+    }
     __device__ __forceinline__ uint32_t in(int row, int i) const { return (uint32_t)(uint64_t)ldg64(inst + (size_t)row * R + i) - tminlo; }
-    __device__ __forceinline__ void eight(int row, int i, uint32_t (&T)[9]) const {
-        const int64_t *p = inst + (size_t)row * R + i;
-        uint64_t v[9];
-        v[0] = tminlo;
-        if (i > 0) v[0] = (uint64_t)ldg64(p - 1);
-        if (i >= 0 && i + 8 <= R) {
-            asm volatile("ld.global.nc.v4.u64 {%0, %1, %2, %3}, [%4];" : "=l"(v[1]), "=l"(v[2]), "=l"(v[3]), "=l"(v[4]) : "l"(p));
-            asm volatile("ld.global.nc.v4.u64 {%0, %1, %2, %3}, [%4];" : "=l"(v[5]), "=l"(v[6]), "=l"(v[7]), "=l"(v[8]) : "l"(p + 4));
-        } else {
-#pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                v[k + 1] = i + k < 0 ? (uint64_t)tminlo : (uint64_t)tminlo - 1u;
-                if ((unsigned)(i + k) < (unsigned)R) v[k + 1] = (uint64_t)ldg64(p + k);
-            }
-        }
-#pragma unroll
-        for (int k = 0; k < 9; ++k) T[k] = (uint32_t)v[k] - tminlo;
+    __device__ __forceinline__ uint32_t rel(uint64_t x) const { return (uint32_t)x - tminlo; }
+    __device__ __forceinline__ bool whole(int row, int i) const { return row * R + i >= first && row * R + i <= last; }      // n * R is below 2^31
+    __device__ __forceinline__ void load(int row, int i, uint64_t (&v)[8]) const {
+        if (last < first) return;
+        const int64_t *p = inst + min(max(row * R + i, first), last);
+        asm volatile("ld.global.nc.v4.u64 {%0, %1, %2, %3}, [%4];" : "=l"(v[0]), "=l"(v[1]), "=l"(v[2]), "=l"(v[3]) : "l"(p));
+        asm volatile("ld.global.nc.v4.u64 {%0, %1, %2, %3}, [%4];" : "=l"(v[4]), "=l"(v[5]), "=l"(v[6]), "=l"(v[7]) : "l"(p + 4));
     }
     __device__ __forceinline__ int align(int row, int i) const { return i - (int)(((uintptr_t)(inst + (size_t)row * R + i) >> 3) & 3u); }
     __device__ __forceinline__ void prefetch(int row, int i) const {
-        const int64_t *p = inst + (size_t)row * R + i;
-        if (i >= 0 && i + 8 <= R) {
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(p + 4));
-        }
+        if (last < first) return;
+        const int64_t *p = inst + min(max(row * R + i, first), last);
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(p + 4));
     }
 };
 template <> struct RowReader<AriBatch> {
     const int64_t *last, *iv; int R; uint32_t tminlo;
-    __device__ __forceinline__ RowReader(const AriBatch &s, int b, int n, int R_, int64_t tmin)
+    __device__ __forceinline__ RowReader(const AriBatch &s, int b, int, int n, int R_, int64_t tmin)
         : last(s.last + (size_t)b * n), iv(s.iv + (size_t)b * n), R(R_), tminlo((uint32_t)(uint64_t)tmin - 1u) {}
     __device__ __forceinline__ uint32_t in(int row, int i) const {
         return (uint32_t)(uint64_t)ldg64(last + row) - tminlo + (uint32_t)(i + 1) * (uint32_t)(uint64_t)ldg64(iv + row);
     }
-    __device__ __forceinline__ void eight(int row, int i, uint32_t (&T)[9]) const {
-        const uint32_t v = (uint32_t)(uint64_t)ldg64(iv + row);
-        uint32_t t = in(row, i - 1);
+    __device__ __forceinline__ uint32_t rel(uint64_t x) const { return (uint32_t)x; }
+    __device__ __forceinline__ void load(int row, int i, uint64_t (&v)[8]) const {
+        const uint32_t d = (uint32_t)(uint64_t)ldg64(iv + row);
+        uint32_t t = in(row, i);
 #pragma unroll
-        for (int k = 0; k < 9; ++k, t += v) T[k] = i + k - 1 < 0 ? 0u : i + k - 1 < R ? t : INF32;
+        for (int k = 0; k < 8; ++k, t += d) v[k] = t;
     }
+    __device__ __forceinline__ bool whole(int, int) const { return true; }
     __device__ __forceinline__ int align(int, int i) const { return i; }
     __device__ __forceinline__ void prefetch(int, int) const {}
 };
 template <class RD>
 __device__ __forceinline__ uint32_t element(const RD &rd, int row, int i) { return i < 0 ? 0u : i < rd.R ? rd.in(row, i) : INF32; }
+// Element i - 1 and the eight from i on, whatever is there.
+template <class RD>
+__device__ __forceinline__ void nine(const RD &rd, int row, int i, uint32_t (&T)[9]) {
+#pragma unroll
+    for (int k = 0; k < 9; ++k) T[k] = element(rd, row, i - 1 + k);
+}
+// T[1] to T[8] of eight loaded elements, i the first of them.
+template <class RD>
+__device__ __forceinline__ void trim(const RD &rd, int i, const uint64_t (&v)[8], uint32_t (&T)[9]) {
+#pragma unroll
+    for (int k = 0; k < 8; ++k) T[k + 1] = rd.rel(v[k]);
+    if (i < 0 || i + 8 > rd.R) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) { if (i + k < 0) T[k + 1] = 0u; if (i + k >= rd.R) T[k + 1] = INF32; }
+    }
+}
 
-// The elements of up to 32 rows (a row a lane: `row`, its first and last element) that the time range [a, b) needs, by the
-// whole warp.  A row is taken in pieces of eight elements, a piece a thread; the pieces of the warp's rows are dealt out to
-// its lanes one after the other, whatever their rows.  (A warp on one row at a time, two elements a lane, spends its
-// instructions on lanes outside the range and on bookkeeping: n=1024, R=1024, B=64 80 us instead of 41 for this pass.)
-// Rows are close to arithmetic, so which pieces a row needs is estimated from its ends; where the estimate falls short on
-// either side the thread of the first or last piece reads on.  act(T) gets nine consecutive times, eight pairs of
-// neighbours: every pair with one of its elements in the range, and the pair that straddles a, comes exactly once; others
-// may come.  The caller leaves out rows without an element in the range.  Returns the number of pieces.
-template <class RD, class ACT>
-__device__ __forceinline__ int stream_rows(const RD &rd, int R, int row, bool have, uint32_t e0, uint32_t eR, uint32_t a, uint32_t b, ACT act) {
+// ------------------------------------------------------------------------------ reductions of a warp
+// 64 bits as two 32-bit reductions of the hardware (five shuffle steps of two registers take several times as long).
+__device__ __forceinline__ uint64_t warp_min64(uint64_t v) {
+    const uint32_t h = __reduce_min_sync(FULL, (uint32_t)(v >> 32));
+    return (uint64_t)h << 32 | __reduce_min_sync(FULL, (uint32_t)(v >> 32) == h ? (uint32_t)v : INF32);
+}
+__device__ __forceinline__ uint64_t warp_max64(uint64_t v) {
+    const uint32_t h = __reduce_max_sync(FULL, (uint32_t)(v >> 32));
+    return (uint64_t)h << 32 | __reduce_max_sync(FULL, (uint32_t)(v >> 32) == h ? (uint32_t)v : 0u);
+}
+// (pieces of 26, 26 and 12 bits: a sum of 32 of them fits)
+__device__ __forceinline__ uint64_t warp_sum64(uint64_t v) {
+    const uint32_t m = (1u << 26) - 1u;
+    return (uint64_t)__reduce_add_sync(FULL, (uint32_t)v & m) + ((uint64_t)__reduce_add_sync(FULL, (uint32_t)(v >> 26) & m) << 26) +
+           ((uint64_t)__reduce_add_sync(FULL, (uint32_t)(v >> 52)) << 52);
+}
+__device__ __forceinline__ float warp_sum(float x) {              // the same value in every lane
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) x += __shfl_xor_sync(FULL, x, d);
+    return x;
+}
+
+// ------------------------------------------------------------------------------ looking through rows
+// The rows that have elements in the time range [a, b) of interest, and the pieces of eight elements that each of them needs:
+// a row's pieces are sb + 8 q with q from excl up to the next row's.  In shared memory, a batch of rows at a time.
+constexpr int LIST_ROWS = 1024;
+struct RowList {
+    uint32_t excl[LIST_ROWS];
+    int sb[LIST_ROWS];
+    unsigned short row[LIST_ROWS];
+};
+
+// A row (a lane; `have`: it counts) goes to the list.  Which pieces it needs is estimated from its ends, `slack` elements more on
+// either side: rows are close to arithmetic.  fill: rows and pieces so far, in one word of 32 bits where pieces are sure to fit
+// into 20 of them (64-bit atomics on shared memory are loops).  The warp's lanes call together.
+struct ListFill { uint32_t packed; unsigned long long wide; };
+constexpr int LIST_BITS = 20;
+__device__ __forceinline__ bool list_packed(int n, int R) { return (long long)min(n, LIST_ROWS) * (R / 8 + 3) < (1 << LIST_BITS); }
+template <class RD>
+__device__ __forceinline__ void list_rows(RowList &L, ListFill &fill, bool packed, const RD &rd, int R, int row, bool have, uint32_t e0, uint32_t eR,
+                                          uint32_t a, uint32_t b, int slack) {
     const int lane = threadIdx.x & 31;
-    int s0 = 0, np = 0;
+    const unsigned who = __ballot_sync(FULL, have);
+    if (!who) return;
+    int s0 = 0;
+    uint32_t np = 0;
     if (have) {
         const float f = eR > e0 ? (float)(R - 1) / (float)(eR - e0) : 0.f;
-        if (a > e0) s0 = max(0, min((int)((float)(a - e0) * f) - CELL_SLACK, R - 1));
+        if (a > e0) s0 = max(0, min((int)((float)(a - e0) * f) - slack, R - 1));
         s0 = rd.align(row, s0);
-        const int last = b > eR ? R : min((int)((float)(b - e0) * f) + 1 + CELL_SLACK, R);
-        np = max(1, (last - s0 + 8) >> 3);
+        const int last = b > eR ? R : min((int)((float)(b - e0) * f) + 1 + slack, R);
+        np = (uint32_t)max(1, (last - s0 + 8) >> 3);
     }
-    int incl = np;
+    uint32_t incl = np;
 #pragma unroll
-    for (int d = 1; d < 32; d <<= 1) { const int y = __shfl_up_sync(FULL, incl, d); if (lane >= d) incl += y; }
-    const int total = __shfl_sync(FULL, incl, 31);
-    const int sb = s0 - 8 * (incl - np);                          // piece q of the warp starts at element sb + 8 q of its row
-    // the lane's piece of the 32 from q0 on: its row, its first element, whether it is its row's first or last one
-    int r = 0, ns = 0;
-    unsigned edge = 0;
-    auto assign = [&](int q0) {
-        const int q = min(q0 + lane, total - 1);
-        int j = 0;                                                // the lane whose row piece q belongs to
-#pragma unroll
-        for (int d = 16; d > 0; d >>= 1) if (__shfl_sync(FULL, incl, j + d - 1) <= q) j += d;
-        const int end = __shfl_sync(FULL, incl, j), first = end - __shfl_sync(FULL, np, j);
-        r = __shfl_sync(FULL, row, j);
-        ns = __shfl_sync(FULL, sb, j) + 8 * q;
-        edge = (q == first ? 1u : 0u) | (q == end - 1 ? 2u : 0u);
-    };
-    if (total > 0) assign(0);
-#pragma unroll 1
-    for (int q0 = 0; q0 < total; q0 += 32) {
-        const bool mine = q0 + lane < total;
-        const int row_q = r;
-        int s = ns;
-        int back = (edge & 1u) ? s : 0, fwd = (edge & 2u) ? s + 8 : R + 1;     // where the row may have to be read on
-        if (q0 + 32 < total) {                                    // the next piece on its way to the L2 while this one is worked on
-            assign(q0 + 32);
-            if (q0 + 32 + lane < total) rd.prefetch(r, ns);
+    for (int d = 1; d < 32; d <<= 1) { const uint32_t y = __shfl_up_sync(FULL, incl, d); if (lane >= d) incl += y; }
+    uint32_t rows = 0, q = 0;
+    if (lane == 31) {
+        if (packed) {
+            const uint32_t at = atomicAdd(&fill.packed, (uint32_t)__popc(who) << LIST_BITS | incl);
+            rows = at >> LIST_BITS; q = at & ((1u << LIST_BITS) - 1u);
+        } else {
+            const unsigned long long at = atomicAdd(&fill.wide, (unsigned long long)__popc(who) << 40 | incl);
+            rows = (uint32_t)(at >> 40); q = (uint32_t)at;
         }
-        if (mine) {
+    }
+    rows = __shfl_sync(FULL, rows, 31); q = __shfl_sync(FULL, q, 31);
+    if (have) {
+        const int pos = (int)rows + __popc(who & ((1u << lane) - 1u));
+        q += incl - np;
+        L.excl[pos] = q; L.sb[pos] = (int)((uint32_t)s0 - 8u * q); L.row[pos] = (unsigned short)row;
+    }
+}
+
+// The CTA looks through the listed rows: the pieces are dealt out evenly to its warps, each a run of them, a piece a lane.
+// (Rows dealt out instead, 32 to a warp, leave the warps with the most guards twice as long at it as the others: n=1024, R=1024,
+// B=64 14 to 25 us for this pass.)  While one is worked on, the lane's next is on its way to the L2.  Where the estimate of a row's pieces falls short on either side its first or last piece leaves a
+// bit, and all such rows are read on by the whole CTA at the end (one access after the other by the lane itself, with its
+// warp waiting, takes half as long again where single gaps are long).  act(T) gets nine consecutive times, eight pairs of
+// neighbours: every pair with one of its elements in the range, and the pair that straddles a, comes exactly once; others
+// may come.
+template <class RD, class ACT>
+__device__ __forceinline__ void stream_list(const RowList &L, uint32_t (*more)[LIST_ROWS / 32], int rows, uint32_t pieces, const RD &rd, int R, uint32_t a, uint32_t b, ACT act) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const uint32_t share = (pieces + nw - 1) / nw, p0 = min(share * warp, pieces), p1 = min(p0 + share, pieces);
+    if (p0 < p1) {
+        // the row that piece p0 belongs to: the last one that starts at or before it, two steps of 32
+        int j0;
+        {
+            const int per = (rows + 31) / 32;
+            const unsigned m = __ballot_sync(FULL, lane * per < rows && L.excl[min(lane * per, rows - 1)] <= p0);
+            j0 = (__popc(m) - 1) * per;
+            const unsigned k = __ballot_sync(FULL, lane < per && j0 + lane < rows && L.excl[min(j0 + lane, rows - 1)] <= p0);
+            j0 += __popc(k) - 1;                                      // LIST_ROWS <= 32 * 32
+        }
+        // piece q + lane: its entry of the list, its first element, whether it is its row's first (1) or last (2) one
+        auto assign = [&](uint32_t q, int &entry, int &s, unsigned &edge) {
+            const int j = j0 + lane;
+            const uint32_t h = (j < rows ? L.excl[j] : pieces) - q;   // where the lane's entry starts; entry j0 at or before q
+            const unsigned heads = __reduce_or_sync(FULL, h < 32u ? 1u << h : 0u);      // (bit 0: entry j0 starts with piece q)
+            const int k = __popc((heads & ~1u) & (FULL >> (31 - lane))), behind = j0 + __popc(heads & ~1u) + 1;
+            const bool next = (behind < rows ? L.excl[behind] : pieces) == q + 32u;     // a row, or the end, right behind these 32
+            entry = min(j0 + k, rows - 1);
+            s = (int)((uint32_t)L.sb[entry] + 8u * (q + lane));
+            edge = ((heads >> lane) & 1u) | ((lane < 31 ? (heads >> (lane + 1)) & 1u : next ? 1u : 0u) << 1);
+            j0 = behind - (next ? 0 : 1);
+        };
+        int entry, s;
+        unsigned edge;
+        assign(p0, entry, s, edge);
+        uint32_t carry = rd.in(L.row[entry], max(s - 1, 0));          // (lane 0) the element before the first of these pieces
 #pragma unroll 1
-            for (;;) {
-                uint32_t T[9];
-                rd.eight(row_q, s, T);
+        for (uint32_t q = p0; q < p1; q += 32u) {
+            const uint32_t x = q + lane;
+            const bool mine = x < p1;
+            const int row = L.row[entry];
+            uint64_t v[8];
+            if (mine) rd.load(row, s, v);
+            int nentry, ns;
+            unsigned nedge;
+            if (q + 32u < p1) {                                       // the next piece on its way to the L2 while this one is worked on
+                assign(q + 32u, nentry, ns, nedge);
+                if (x + 32u < p1) rd.prefetch(L.row[nentry], ns);
+            }
+            uint32_t T[9];
+            trim(rd, s, v, T);
+            if (mine && !rd.whole(row, s)) nine(rd, row, s, T);       // (seldom)
+            const uint32_t up = __shfl_up_sync(FULL, T[8], 1);
+            T[0] = (edge & 1u) ? (s > 0 ? T[1] : 0u) : lane == 0 ? carry : up;      // (a row's first piece starts with no gap: see below)
+            carry = __shfl_sync(FULL, T[8], 31);
+            if (mine) {
                 act(T);
-                if (s <= back && (s <= 0 || T[0] < a)) back = 0;  // the row's start of the range is covered
-                if (s + 8 >= fwd && T[8] >= b) fwd = R + 1;       // ... and its end
-                if (back > 0) s = back = back - 8;
-                else if (fwd <= R) { s = fwd; fwd += 8; }
-                else break;
+                if ((edge & 1u) && s > 0 && T[1] >= a) atomicOr(&more[0][entry >> 5], 1u << (entry & 31));
+                if ((edge & 2u) && s + 8 <= R && T[8] < b) atomicOr(&more[1][entry >> 5], 1u << (entry & 31));
+            }
+            entry = nentry; s = ns; edge = nedge;
+        }
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int i = threadIdx.x; i < 2 * LIST_ROWS; i += blockDim.x) {
+        const int right = i >= LIST_ROWS ? 1 : 0, j = i & (LIST_ROWS - 1);
+        if (j < rows && (more[right][j >> 5] >> (j & 31) & 1u)) {
+            const int row = L.row[j];
+            int s = (int)((uint32_t)L.sb[j] + 8u * (right ? (j + 1 < rows ? L.excl[j + 1] : pieces) - 1u : L.excl[j]));
+            if (!right) ++s;                                      // to the left the pair of the piece's first element and the one before it comes along
+            bool on = true;
+#pragma unroll 1
+            while (on) {
+                uint32_t U[9];
+                s += right ? 8 : -8;
+                nine(rd, row, s, U);
+                act(U);
+                on = right ? s + 8 <= R && U[8] < b : s > 0 && U[0] >= a;
             }
         }
     }
-    return total;
 }
 
-// Index of a row's first element at or after time t, by one thread: windows of eight elements (and the one before them), the
-// first around the place that the row's ends suggest, the next ones where the mean interval puts t from the end of the
-// window nearest to it; then doubling steps and bisection.
+// Where the eight elements that are looked at first for time t start: t's place by the row's ends, a little before it.
+template <class RD>
+__device__ __forceinline__ int window_at(const RD &rd, int row, int R, uint32_t t, uint32_t e0, float inv) {
+    return rd.align(row, min(max((t > e0 ? (int)min((float)(t - e0) * inv, (float)R) : 0) - 2, 0), R - 1));
+}
+__device__ __forceinline__ float per_time(int R, uint32_t e0, uint32_t eR) { return eR > e0 ? (float)(R - 1) / (float)(eR - e0) : 0.f; }
+// They start at s and do not hold the first element at or after a, or not the one before it, or not all up to what is asked for: where the
+// next eight start, by how far off these are.
+template <class RD>
+__device__ __forceinline__ int window_next(const RD &rd, int row, int R, int s, uint32_t T1, uint32_t T8, uint32_t a, float inv) {
+    const int off = (int)min((float)(T1 >= a ? T1 - a : T8 < a ? a - T8 : 0u) * inv, (float)R);
+    return rd.align(row, min(max(T1 >= a ? s - 3 - off : T8 < a ? s + 5 + off : s + 4, 0), R - 1));
+}
+
+// Index of a row's first element at or after time t, by one thread: eight elements around the place that the row's ends suggest, then
+// where the mean interval puts t from the nearest of those; then bisection.
 template <class RD>
 __device__ __noinline__ int first_at_or_after(const RD rd, int row, int R, uint32_t t, uint32_t e0, uint32_t eR) {
     if (t <= e0) return 0;
     if (t > eR) return R;
-    const float inv = (float)(R - 1) / (float)(eR - e0);          // e0 < t <= eR
-    int lo = 0, hi = R - 1;                                       // element lo is before t, element hi is not
-    int g = (int)((float)(t - e0) * inv);
+    int lo = 0, hi = R - 1;                                       // element lo is before t, element hi is not (e0 < t <= eR)
+    const float inv = per_time(R, e0, eR);
+    int s = window_at(rd, row, R, t, e0, inv);
 #pragma unroll 1
-    for (int it = 0; it < 4; ++it) {
-        const int s = rd.align(row, min(max(g - 2, 0), R - 1));
+    for (int it = 0; it < 4 && rd.whole(row, s); ++it) {
+        uint64_t v[8];
         uint32_t T[9];
-        rd.eight(row, s, T);
+        rd.load(row, s, v);
+        trim(rd, s, v, T);
         int c = 0;
 #pragma unroll
-        for (int k = 0; k < 9; ++k) c += T[k] < t ? 1 : 0;        // sorted: the first c of them
-        if (c > 0 && c < 9) return s - 1 + c;
-        if (c == 0) { hi = min(hi, s - 1); g = s - 1 - (int)min((float)(T[0] - t) * inv, (float)R); }
-        else { lo = max(lo, s + 7); g = s + 8 + (int)min((float)(t - T[8]) * inv, (float)R); }
-        g = min(max(g, lo), hi);
-    }
-    const bool up = g - lo < hi - g;
-#pragma unroll 1
-    for (int step = 8; hi - lo > 1; step <<= 1) {
-        const int q = up ? min(lo + step, hi - 1) : max(hi - step, lo + 1);
-        if (rd.in(row, q) < t) { lo = q; if (!up) break; } else { hi = q; if (up) break; }
+        for (int k = 1; k < 9; ++k) c += T[k] < t ? 1 : 0;        // sorted: the first c of them
+        if (c < 8 && (c > 0 || s <= lo + 1)) return s + c;
+        if (c == 0) hi = min(hi, s); else lo = max(lo, s + 7);
+        s = rd.align(row, min(max(window_next(rd, row, R, s, T[1], T[8], t, inv), lo), hi));
     }
 #pragma unroll 1
     while (hi - lo > 1) {
@@ -220,26 +346,27 @@ __device__ __noinline__ int first_at_or_after(const RD rd, int row, int R, uint3
     return hi;
 }
 
-// Whether one of `rows` consecutive rows decreases somewhere: a warp a row, four elements a lane and step.
+// Whether one of `rows` consecutive rows decreases somewhere: their elements one after the other, whatever rows they belong
+// to, 256 a warp and step.  (A warp a row: the next row's loads wait for this one's, n=93, R=211 5.6 us.)
 static __device__ bool rows_unsorted(const int64_t *ts, int rows, int R) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const long long N = (long long)rows * R;
     bool bad = false;
 #pragma unroll 1
-    for (int r = warp; r < rows; r += nw) {
-        const int64_t *row = ts + (size_t)r * R;
-        int64_t tail = INT64_MIN;
-#pragma unroll 1
-        for (int i0 = 0; i0 < R; i0 += 128) {
-            int64_t v[4];
+    for (long long f0 = 256ll * warp; f0 < N; f0 += 256ll * nw) {
+        int64_t v[8], before = 0;
+        if (lane == 0 && f0 > 0) before = ldg64(ts + f0 - 1);
 #pragma unroll
-            for (int k = 0; k < 4; ++k) { const int i = i0 + 32 * k + lane; v[k] = i < R ? ldg64(row + i) : INT64_MAX; }
+        for (int k = 0; k < 8; ++k) { const long long f = f0 + 32 * k + lane; v[k] = f < N ? ldg64(ts + f) : INT64_MAX; }
+        int c = (int)((uint32_t)(f0 + lane) % (uint32_t)R);       // the column (n * R is below 2^31)
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                int64_t p = (int64_t)shfl_up((uint64_t)v[k], 1);
-                if (lane == 0) p = tail;
-                bad |= v[k] < p;
-                tail = (int64_t)shfl_idx((uint64_t)v[k], 31);
-            }
+        for (int k = 0; k < 8; ++k) {
+            int64_t p = (int64_t)shfl_up((uint64_t)v[k], 1);
+            if (lane == 0) p = before;
+            bad |= c != 0 && v[k] < p;
+            before = (int64_t)shfl_idx((uint64_t)v[k], 31);
+            c += 32;
+            while (c >= R) c -= R;
         }
     }
     return bad;
@@ -258,6 +385,13 @@ struct CellParams {
     int32_t *idx; int64_t *barrier; int64_t *wait; int32_t *status;
 };
 
+// What the rows answer when they are asked for cells.  A cluster has three of them: what the own rows answered, and what arrived from
+// every CTA (its share of the room each), twice, used in turn: the next answers may arrive while these are worked on.
+struct Answers {
+    uint64_t node[CELL_NODES];                    // the elements in the cells: time << 32 | RANGE the row's next element, SUM the element less the row's previous one
+    unsigned char slot[CELL_NODES];               // ... which of the cells
+};
+
 struct CellShared {
     // from every CTA of the cluster (each array is written by the others before one cluster barrier and read after it, so no
     // two exchanges share one): minima and maxima of its rows' ends; whether one of its rows decreases; SUM its rows' wait at
@@ -265,28 +399,45 @@ struct CellShared {
     unsigned long long ex[4][CELL_CLUSTER];
     float exi[CELL_CLUSTER];                      // RANGE: how irregular its rows are (sum over a few of them, see k_cells)
     unsigned long long exc[CELL_CLUSTER], exs[CELL_CLUSTER], exv[CELL_CLUSTER], exb[CELL_CLUSTER];
-    unsigned long long red[4][32];
-    unsigned long long acc, total, key, kbase;
+    unsigned long long red[4][32], keys[32], kbases[32];
+    // of Answers: how many from every CTA; RANGE latest and earliest of the rows' first elements at or after the cell's start
+    struct { uint32_t gmax[CELL_BATCH], gmin[CELL_BATCH]; uint32_t count[CELL_CLUSTER]; } heard[2];
+    uint32_t gmax[CELL_BATCH], gmin[CELL_BATCH];  // ... of the own rows'
+    unsigned int nnodes;
+    ListFill fill;
+    unsigned long long acc, total;
     uint32_t hist[GUARD_BINS];
-    float span;                                   // RANGE: rows of at least this span are guards
-    unsigned int pieces;                          // RANGE: pieces of eight elements that the slice took
     unsigned long long later;                     // RANGE: about how many timestamps of the other rows lie in the range
     // the cells to evaluate (in every CTA), and the order in which that is done
     uint32_t cell[CELL_ALIVE];
-    uint64_t base[CELL_ALIVE];                    // RANGE: a lower bound of G at the cell's start, SUM: S there
-    uint64_t lb[CELL_ALIVE];                      // lower bound of the objective in the cell
+    union {
+        struct {
+            uint64_t base[CELL_ALIVE];            // RANGE: a lower bound of G at the cell's start, SUM: S there
+            uint64_t lb[CELL_ALIVE];              // lower bound of the objective in the cell
+        };
+        uint32_t more[2][LIST_ROWS / 32];         // (while rows are looked through: which of them have to be read on, to the left, to the right)
+    };
     unsigned short order[CELL_ALIVE];
     unsigned int ncells;
-    uint32_t gmaxl[CELL_BATCH], gminl[CELL_BATCH];   // RANGE: latest and earliest of the own rows' first elements at or after the cell's start
-    // in the first CTA: what the rows answered
-    uint32_t gmax[CELL_BATCH], gmin[CELL_BATCH];  // RANGE: ... of all rows'
-    uint64_t node[CELL_NODES];                    // the elements in the cells: time << 32 | RANGE the row's next element, SUM the element less the row's previous one
-    unsigned int nnodes;
-    int asked;                                    // (in every CTA) cells evaluated, see CELL_ASKED_*
-    uint64_t tmp[34];
-    unsigned int sstatus;
+    // the ones that the rows are being asked for: first and last time, G or S as above
+    uint32_t ca[CELL_BATCH], ce[CELL_BATCH];
+    uint64_t cb[CELL_BATCH];
+    uint2 asked_run[CELL_FIRST * (CELL_ROUNDS + 2)];      // first and last cell of the runs evaluated before the list was made
+    // the list's runs, in the order of their first cells: first and last cell, G or S at the start, smallest lower bound
+    uint2 run[CELL_ALIVE];
+    uint64_t run_base[CELL_ALIVE];
+    unsigned long long run_lb[CELL_ALIVE];
+    uint32_t exf[CELL_CLUSTER];                   // (exchanged with exv, exb) first cell of the run around the most promising one
+    int runs;
+    uint64_t bestd[32]; uint32_t bestt[32];
+    // what is the same in all threads and needed now and then: shared memory, not a register each (the compiler spills some sixty of
+    // them otherwise, and what is spilled has often left the L1 cache by the time it is wanted back: n=1024, R=1024, B=64 72 us)
+    int64_t tmin;
+    uint64_t ub, bd;                              // SUM: a wait that is attained; the smallest objective so far and its time
+    uint32_t bt, t0, lmin, tend, lo, hi, shift, c0, m, a, bnd, gap, expected, took, longest;
+    float span, width;                            // RANGE: rows of at least this span are guards; what a cell may span
+    int slack, firsts, around, ndone, asked, per_cell;
     unsigned int slow;                            // (in every CTA) rows far from arithmetic, or standing still
-    SegResult best;                               // (in every CTA) the smallest objective so far
 };
 
 // A cell's last time; `limit` is where the timeline (or a CTA's slice of it) ends.  Formed from what is left of it behind the
@@ -295,117 +446,309 @@ __device__ __forceinline__ uint32_t cell_end(uint32_t start, uint32_t shift, uin
     return start + min((1u << shift) - 1u, limit - 1u - start);
 }
 
-__device__ __forceinline__ float warp_sum(float x) {
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) x += __shfl_xor_sync(FULL, x, d);
-    return x;
+__device__ __noinline__ bool was_asked(const uint2 *runs, int n, uint32_t c) {
+    bool is = false;
+#pragma unroll 1
+    for (int k = 0; k < n; ++k) is |= runs[k].x <= c && c <= runs[k].y;
+    return is;
 }
 
-// The exact minimum over `ns` listed cells, from sh.order[from] on (in every CTA of the cluster the same): every CTA asks
-// its rows, the first one evaluates and hands the result to the others.  Every thread of the cluster calls; two cluster
-// barriers.  False: more elements than there is room for.
-template <int OBJ, class RD>
-__device__ __noinline__ bool evaluate_cells(CellShared &sh, int from, int ns, const RD rd, const uint2 *ends, int n, int R, int r0, int nrows,
-                                            uint32_t lo, uint32_t hi, uint32_t shift) {
+struct Best { uint64_t d; uint32_t t; };          // smallest objective and its time, the first of equal ones; the same in every thread of the cluster
+__device__ __forceinline__ Best warp_best(uint64_t d, uint32_t t) {
+    const uint64_t m = warp_min64(d);
+    return Best{m, __reduce_min_sync(FULL, d == m ? t : INF32)};
+}
+
+// The exact minimum over the `ns` cells of sh.ca, sh.ce, sh.cb (in every CTA of the cluster the same): every CTA asks its rows
+// and sends what they answer to all CTAs, and behind one cluster barrier every CTA (with a few dozen answers every
+// warp, without a further barrier) evaluates all of it.  Every thread of the cluster calls.  Returns the number of answers: more than CELL_NODES,
+// and there was no room for them.
+//
+// A (cell, row) pair a lane, a warp on one cell: eight elements around the place that the row's ends suggest are loaded, then,
+// by how far off they were, eight others, until they hold the first element at or after the cell's start and all that
+// follow in it.  (Searched for the first element, then asked for its successor and the next ones: three to five accesses one
+// after the other, n=1024, R=1024, B=64 7 us, eight cells of SUM 17 us.)
+template <int OBJ, class SRC>
+__device__ __forceinline__ int evaluate_cells(CellShared &sh, Answers *answers, const uint2 *ends, const SRC &src, int B, int n, int R, int rpc, int turn, int ns) {
     cg::cluster_group cl = cg::this_cluster();
-    const int tid = threadIdx.x, nt = blockDim.x, G = (int)cl.num_blocks(), rank = (int)cl.block_rank();
-    CellShared &ld = *cl.map_shared_rank(&sh, 0);
+    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5, G = gridDim.x;
+    const int r0 = min((int)blockIdx.x * rpc, n), nrows = min(rpc, n - r0);
+    const RowReader<SRC> rd(src, blockIdx.y, B, n, R, sh.tmin);
+    Answers *an = answers;
+    auto put = [&](int k, uint32_t T, uint32_t pay) {
+        const unsigned pos = atomicAdd(&sh.nnodes, 1u);
+        if (pos < CELL_NODES) { an->node[pos] = (uint64_t)T << 32 | pay; an->slot[pos] = (unsigned char)k; }
+    };
+    const int chunks = (rpc + 31) >> 5, items = ns * chunks;
 #pragma unroll 1
-    for (int q = tid; q < ns * nrows; q += nt) {                  // a (cell, row) pair a thread
-        const int k = q / nrows, p = q - k * nrows;
-        const int x = sh.order[from + k];
-        const uint32_t a = lo + (sh.cell[x] << shift);
-        const uint32_t e = cell_end(a, shift, hi);
-        const uint64_t base = sh.base[x];
-        const uint2 en = ends[r0 + p];
-        int i = first_at_or_after(rd, r0 + p, R, a, en.x, en.y);
-        uint32_t T = element(rd, r0 + p, i), pv = OBJ == ZL_OBJ_SUM ? element(rd, r0 + p, i - 1) : 0u;
+    for (int it = warp; it < items; it += nw) {
+        const int k = it / chunks, p = 32 * (it - k * chunks) + lane, row = r0 + p;
+        const uint32_t a = sh.ca[k], e = sh.ce[k];
+        const uint64_t base = sh.cb[k];
+        uint32_t first = 0, last = INF32;                         // RANGE: of the row, for the latest and the earliest
+        if (p < nrows) {
+            const uint2 en = ends[row];
+            const float inv = per_time(R, en.x, en.y);
+            int s = window_at(rd, row, R, a, en.x, inv);
+            uint32_t T[9];
+            bool open = true;
+#pragma unroll 1
+            for (int step = 0; step < 4 && open; ++step) {
+                uint64_t v[8];
+                rd.load(row, s, v);
+                trim(rd, s, v, T);
+                if (!rd.whole(row, s)) break;
+                open = !((T[1] < a || s <= 0) && T[8] > e);
+                if (open) s = window_next(rd, row, R, s, T[1], T[8], a, inv);
+            }
+            if (!open) {
+                T[0] = 0;
+                uint32_t f = T[8];
+                unsigned in = 0;                                  // which of the eight are answers
+#pragma unroll
+                for (int j = 7; j > 0; --j) {
+                    if (T[j] >= a) f = T[j];
+                    // (RANGE: an element that does not raise the running maximum cannot matter)
+                    if (T[j] - a <= e - a && (OBJ == ZL_OBJ_RANGE ? (uint64_t)T[j + 1] > base : T[j] != T[j - 1])) in |= 1u << j;
+                }
+                first = last = f;
+#pragma unroll 1
+                for (; in; in &= in - 1u) {
+                    const int j = __ffs(in) - 1;
+                    uint32_t x = 0, y = 0;                        // RANGE elements j and j + 1, SUM j and j - 1
+#pragma unroll
+                    for (int i = 1; i < 8; ++i) if (i == j) { x = T[i]; y = T[OBJ == ZL_OBJ_RANGE ? i + 1 : i - 1]; }
+                    put(k, x, OBJ == ZL_OBJ_RANGE ? y : x - y);
+                }
+            } else {
+                int i = first_at_or_after(rd, row, R, a, en.x, en.y);
+                uint32_t X = element(rd, row, i), pv = OBJ == ZL_OBJ_SUM ? element(rd, row, i - 1) : 0u;
+                first = last = X;
+                int idle = 0;
+#pragma unroll 1
+                for (; i < R && X <= e; ++i) {
+                    const uint32_t nx = element(rd, row, i + 1);
+                    const uint32_t pay = OBJ == ZL_OBJ_RANGE ? nx : X - pv;
+                    if (OBJ == ZL_OBJ_RANGE ? (uint64_t)nx > base : pay != 0u) put(k, X, pay);
+                    else if (++idle == CELL_IDLE) sh.slow = 1;
+                    pv = X; X = nx;
+                }
+            }
+        }
         if (OBJ == ZL_OBJ_RANGE) {
-            if (T > sh.gmaxl[k]) atomicMax(&sh.gmaxl[k], T);
-            if (T < sh.gminl[k]) atomicMin(&sh.gminl[k], T);
+            first = __reduce_max_sync(FULL, first);
+            last = __reduce_min_sync(FULL, last);
+            if (lane == 0) { atomicMax(&sh.gmax[k], first); atomicMin(&sh.gmin[k], last); }
         }
-        int idle = 0;
+    }
+    __syncthreads();
+    int m = (int)sh.nnodes, mine_k = 0;
+    uint64_t mine_x = 0;
+    const uint32_t *gmax = sh.gmax, *gmin = sh.gmin;
+    if (G > 1) {
+        const int rank = blockIdx.x, room = CELL_NODES / G, sent = min(m, room);
+        auto &heard = sh.heard[turn];
+        Answers *in = answers + 1 + turn;
+        gmax = heard.gmax; gmin = heard.gmin;
 #pragma unroll 1
-        for (; i < R && T <= e; ++i) {
-            const uint32_t nx = element(rd, r0 + p, i + 1);
-            const uint32_t pay = OBJ == ZL_OBJ_RANGE ? nx : T - pv;
-            // (RANGE: an element that does not raise the running maximum cannot matter)
-            if (OBJ == ZL_OBJ_RANGE ? (uint64_t)nx > base : pay != 0u) {
-                const unsigned pos = atomicAdd(&ld.nnodes, 1u);
-                if (pos < CELL_NODES) ld.node[pos] = ((uint64_t)T << 32) | pay;
-            } else if (++idle == CELL_IDLE) {
-                sh.slow = 1;
+        for (int r = warp; r < G; r += nw) {                      // to CTA r
+            Answers *to = cl.map_shared_rank(in, r);
+            for (int i = lane; i < sent; i += 32) { to->node[rank * room + i] = an->node[i]; to->slot[rank * room + i] = an->slot[i]; }
+            auto *h = cl.map_shared_rank(&heard, r);
+            if (lane == 0) h->count[rank] = (uint32_t)m;
+            if (OBJ == ZL_OBJ_RANGE && lane < ns) { atomicMax(&h->gmax[lane], sh.gmax[lane]); atomicMin(&h->gmin[lane], sh.gmin[lane]); }
+        }
+        cl.sync();
+        const int c = lane < G ? (int)heard.count[min(lane, G - 1)] : 0;
+        int incl = c;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) { const int y = __shfl_up_sync(FULL, incl, d); if (lane >= d) incl += y; }
+        m = __shfl_sync(FULL, incl, 31);
+        const bool over = __any_sync(FULL, c > room);            // more from one CTA than its share: they are fetched from where they were put
+        if (m <= 32 && !over) {
+            // a lane each: from which CTA, and which of its answers
+            int at = lane;
+#pragma unroll 1
+            for (int r = 0; r + 1 < G; ++r) { const int p = __shfl_sync(FULL, incl, r); if (lane >= p) at = (r + 1) * room + lane - p; }
+            if (lane < m) { mine_x = in->node[at]; mine_k = in->slot[at]; }
+        } else if (m <= CELL_NODES) {
+            Answers *to = over ? in : an;
+#pragma unroll 1
+            for (int r = warp; r < G; r += nw) {
+                const int count = __shfl_sync(FULL, c, r), at = __shfl_sync(FULL, incl, r) - count;
+                const Answers *from = over ? cl.map_shared_rank(an, r) : in;
+                const int first = over ? 0 : r * room;
+                for (int i = lane; i < count; i += 32) { to->node[at + i] = from->node[first + i]; to->slot[at + i] = from->slot[first + i]; }
             }
-            pv = T; T = nx;
+            if (over) cl.sync(); else __syncthreads();
+            an = to;
+        }
+    } else if (lane < m && m <= 32) {
+        mine_x = an->node[lane]; mine_k = an->slot[lane];
+    }
+    uint64_t d = sh.bd;
+    uint32_t t = sh.bt;
+    if (OBJ == ZL_OBJ_RANGE && m <= CELL_NODES && lane < ns && gmax[lane] != INF32 && gmin[lane] < sh.hi) {
+        // the first element at or after the cell's start, wherever it is
+        const uint64_t w = (uint64_t)(gmax[lane] - gmin[lane]);
+        if (w < d || (w == d && gmin[lane] < t)) { d = w; t = gmin[lane]; }
+    }
+    // the exact objective of an answer: the sweep over its cell's answers up to it.  Up to 32 of them: a lane each, every warp for itself.
+    const bool few = m <= 32;
+    if (few) {
+        const uint32_t T = (uint32_t)(mine_x >> 32), pay = (uint32_t)mine_x;
+        uint64_t v = lane < m ? (OBJ == ZL_OBJ_RANGE ? (uint64_t)gmax[mine_k] : sh.cb[mine_k]) : 0ull;
+        // (RANGE: what G has at the start already does not raise it)
+        const bool counts = lane < m && (OBJ == ZL_OBJ_SUM || pay > v);
+        unsigned left = __ballot_sync(FULL, counts);
+#pragma unroll 2
+        for (; left; left &= left - 1u) {
+            const int j = __ffs(left) - 1, k = __shfl_sync(FULL, mine_k, j);
+            const uint32_t o = __shfl_sync(FULL, T, j), y = __shfl_sync(FULL, pay, j);
+            if (OBJ == ZL_OBJ_RANGE) { if (k == mine_k && o < T) v = max(v, (uint64_t)y); }      // max(Z): latest next of the earlier elements
+            else if (k == mine_k && o <= T) v += y;                                              // S: every delta up to T
+        }
+        const uint64_t w = OBJ == ZL_OBJ_SUM ? (uint64_t)n * T - v : v >= INF32 ? ~0ull : v - T;
+        if (counts && w != ~0ull && (w < d || (w == d && T < t))) { d = w; t = T; }
+    } else if (m <= CELL_NODES) {
+#pragma unroll 1
+        for (int i = tid; i < m; i += nt) {
+            const uint64_t x = an->node[i];
+            const uint32_t T = (uint32_t)(x >> 32);
+            const int k = an->slot[i];
+            uint64_t v = OBJ == ZL_OBJ_RANGE ? (uint64_t)gmax[k] : sh.cb[k];
+#pragma unroll 8
+            for (int j = 0; j < m; ++j) {
+                const uint64_t y = an->node[j];
+                const uint32_t o = (uint32_t)(y >> 32), pay = (uint32_t)y;
+                const bool same = an->slot[j] == k;
+                if (OBJ == ZL_OBJ_RANGE) { if (same && o < T) v = max(v, (uint64_t)pay); }
+                else if (same && o <= T) v += pay;
+            }
+            const uint64_t w = OBJ == ZL_OBJ_SUM ? (uint64_t)n * T - v : v >= INF32 ? ~0ull : v - T;
+            if (w != ~0ull && (w < d || (w == d && T < t))) { d = w; t = T; }
         }
     }
-    if (OBJ == ZL_OBJ_RANGE) {
+    Best best = warp_best(d, t);
+    if (!few && m <= CELL_NODES) {
+        if (lane == 0) { sh.bestd[warp] = best.d; sh.bestt[warp] = best.t; }
         __syncthreads();
-        if (tid < ns) {
-            atomicMax(&ld.gmax[tid], sh.gmaxl[tid]); atomicMin(&ld.gmin[tid], sh.gminl[tid]);
-            sh.gmaxl[tid] = 0; sh.gminl[tid] = INF32;
-        }
+        best = warp_best(lane < nw ? sh.bestd[lane] : ~0ull, lane < nw ? sh.bestt[lane] : INF32);
     }
-    cl.sync();
-    if (rank == 0) {
-        const int m = (int)sh.nnodes;
-        uint64_t bd = ~0ull, bt = ~0ull;
-        if (m <= CELL_NODES) {
+    __syncthreads();                                              // everybody has read the answers
+    if (tid == 0) { sh.nnodes = 0; sh.bd = best.d; sh.bt = best.t; sh.per_cell = max(1, m / ns); sh.asked += m / (OBJ == ZL_OBJ_RANGE ? 16 : 64); }
+    if (tid < CELL_BATCH) { sh.gmax[tid] = sh.heard[turn].gmax[tid] = 0; sh.gmin[tid] = sh.heard[turn].gmin[tid] = INF32; }
+    __syncthreads();
+    return m;
+}
+
+// The elements of the slice's rows into its cells: RANGE of the guards (stage 0) or of the other rows (stage 1), SUM of all rows.
+template <int OBJ, class SRC>
+__device__ __forceinline__ void look_through(CellShared &sh, uint32_t *cell, Answers *answers, const uint2 *ends, const SRC &src, int B, int n, int R, int stage) {
+    const RowReader<SRC> rd(src, blockIdx.y, B, n, R, sh.tmin);
+    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
+    const uint32_t a = sh.a, bnd = sh.bnd, shift = sh.shift, gap = sh.gap, m = sh.m, w = bnd - a;
+    uint64_t carry = 0, total = 0;                        // SUM: the rows' last elements before a, and all deltas in the slice
+    RowList &list = *reinterpret_cast<RowList *>(answers);
+    const bool packed = list_packed(n, R);
 #pragma unroll 1
-            for (int i = tid; i < m; i += nt) {
-                const uint32_t T = (uint32_t)(sh.node[i] >> 32), c = (T - lo) >> shift;
-                uint64_t v = 0;
+    for (int from = 0; from < n && m > 0; from += LIST_ROWS) {
+        if (from > 0) __syncthreads();
+        if (tid < LIST_ROWS / 32) sh.more[0][tid] = sh.more[1][tid] = 0;
 #pragma unroll 1
-                for (int k = 0; k < ns; ++k) {
-                    const int x = sh.order[from + k];
-                    if (sh.cell[x] == c) v = OBJ == ZL_OBJ_RANGE ? (uint64_t)sh.gmax[k] : sh.base[x];
+        for (int g = warp; 32 * g < min(LIST_ROWS, n - from); g += nw) {
+            const int row = from + 32 * g + lane;
+            uint2 e = make_uint2(0u, 0u);
+            bool have = row < n;
+            if (have) {
+                e = ends[row];
+                if (OBJ == ZL_OBJ_RANGE) have = ((float)(e.y - e.x) >= sh.span) == (stage == 0);
+                if (e.x >= bnd || e.y < a) {              // no element of the row in the slice
+                    if (OBJ == ZL_OBJ_SUM && have && e.y < a) carry += e.y;
+                    have = false;
                 }
-#pragma unroll 4
-                for (int k = 0; k < m; ++k) {
-                    const uint32_t t = (uint32_t)(sh.node[k] >> 32), pay = (uint32_t)sh.node[k];
-                    if ((t - lo) >> shift != c) continue;
-                    if (OBJ == ZL_OBJ_RANGE) { if (t < T) v = max(v, (uint64_t)pay); }       // max(Z): latest next of the earlier elements
-                    else if (t <= T) v += pay;                                               // S: every delta up to T
-                }
-                const uint64_t d = OBJ == ZL_OBJ_SUM ? (uint64_t)n * T - v : v >= INF32 ? ~0ull : v - T;
-                if (d != ~0ull && (d < bd || (d == bd && (uint64_t)T < bt))) { bd = d; bt = T; }
             }
-            if (OBJ == ZL_OBJ_RANGE && tid < ns && sh.gmax[tid] != INF32 && sh.gmin[tid] < hi) {
-                // the first element at or after the cell's start, wherever it is
-                const uint64_t d = (uint64_t)(sh.gmax[tid] - sh.gmin[tid]), t = sh.gmin[tid];
-                if (d < bd || (d == bd && t < bt)) { bd = d; bt = t; }
-            }
+            list_rows(list, sh.fill, packed, rd, R, row, have, e.x, e.y, a, bnd, sh.slack);
         }
-        if (tid == 0 && (sh.best.d < bd || (sh.best.d == bd && sh.best.t < bt))) { bd = sh.best.d; bt = sh.best.t; }
         __syncthreads();
-        block_best_to_result(bd, bt, ZL_OK, sh.tmp, &sh.sstatus, sh.best);
-        if (tid == 0) { if (m > CELL_NODES) sh.best.valid = 0; sh.nnodes = 0; }
-        if (tid < CELL_BATCH) { sh.gmax[tid] = 0; sh.gmin[tid] = INF32; }
+        const int rows = (int)(packed ? sh.fill.packed >> LIST_BITS : sh.fill.wide >> 40);
+        const uint32_t pieces = packed ? sh.fill.packed & ((1u << LIST_BITS) - 1u) : (uint32_t)sh.fill.wide;
+        if (rows > 0) stream_list(list, sh.more, rows, pieces, rd, R, a, bnd, [&](const uint32_t (&T)[9]) {
+            if (OBJ == ZL_OBJ_RANGE) {
+                // cell[k] becomes a lower bound of G at the start of cell k (before the prefix maximum): an element
+                // says that G is at least its successor for the cells after its own.  Elements before the slice
+                // count for its first cell; those in its last cell or behind it go to cell[m], which is not looked
+                // at.  A gap of at most `gap` cannot push a cell's bound, G less the cell's end, beyond that: it discards no cell.
+                uint32_t longer = 0;
+#pragma unroll
+                for (int j = 0; j < 8; ++j) longer = max(longer, T[j + 1] - T[j]);
+                if (longer > gap) {
+#pragma unroll
+                    for (int h = 0; h < 8; h += 4) {
+                        uint32_t k[4], v[4];
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            k[j] = T[h + j] < a ? 0u : min(((T[h + j] - a) >> shift) + 1u, m);
+                            v[j] = cell[k[j]];
+                        }
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) if (T[h + j + 1] - T[h + j] > gap && v[j] < T[h + j + 1]) atomicMax(&cell[k[j]], T[h + j + 1]);
+                    }
+                }
+            } else {
+                uint32_t in = 0;
+#pragma unroll
+                for (int j = 1; j < 9; ++j) {
+                    const uint32_t d = T[j] - a, delta = T[j] - T[j - 1];
+                    if (d < w) { atomicAdd(cell + (d >> shift), delta); in += delta; }
+                }
+                total += in;
+                if (T[0] < a && T[8] >= a) {              // the row's last element before the slice
+                    uint32_t before = T[0];
+#pragma unroll
+                    for (int j = 1; j < 8; ++j) if (T[j] < a) before = T[j];
+                    carry += before;
+                }
+            }
+        });
         __syncthreads();
-        const SegResult r = sh.best;
-        if (tid > 0 && tid < G) cl.map_shared_rank(&sh, tid)->best = r;
+        if (tid == 0) { sh.fill.packed = 0; sh.fill.wide = 0; if (stage == 0) sh.took += pieces; }
     }
-    cl.sync();
-    return sh.best.valid != 0;
+    if (OBJ == ZL_OBJ_SUM) {
+        carry = warp_sum64(carry);
+        total = warp_sum64(total);
+        if (lane == 0) { atomicAdd(&sh.acc, (unsigned long long)carry); atomicAdd(&sh.total, (unsigned long long)total); }
+    }
 }
 
 // Dynamic shared memory: the slice's cells [cap + 4] u32 | rows' first and last element, relative [n] uint2 | SUM: per 128
-// cells the scan before them and the smallest lower bound among them [cap / 128] two u64.
-template <int OBJ, class SRC>
-__global__ void __launch_bounds__(1024, 1) k_cells(const SRC src, const CellParams P) {
+// cells the scan before them and the smallest lower bound among them [cap / 128] two u64 | one Answers (three in a cluster),
+// over which the list of rows to look through lies.
+template <int OBJ, class SRC, int MT>
+__global__ void __launch_bounds__(MT, 1) k_cells(const SRC src, const CellParams P) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ CellShared sh;
     cg::cluster_group cl = cg::this_cluster();
     const int b = blockIdx.y, rank = blockIdx.x, G = gridDim.x;
-    // A CTA's shared memory may be written by the others only once it runs: everybody says so here, and waits for the rest
-    // with the columns read, before the first store into another CTA.
-    if (G > 1) cl.barrier_arrive();
-    grid_dep_wait();
     const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
     const int n = P.n, R = P.R;
     uint32_t *cell = (uint32_t *)smem;
     uint2 *ends = (uint2 *)(cell + P.cap + 4);
     uint64_t *blk_before = (uint64_t *)(ends + n), *blk_lb = blk_before + P.cap / 128;
+    Answers *answers = (Answers *)(OBJ == ZL_OBJ_SUM ? blk_lb + P.cap / 128 : blk_before);
+    // A CTA's shared memory may be written by the others only once it runs: everybody says so here, and waits for the rest
+    // with the columns read, before the first store into another CTA.
+    if (G > 1) cl.barrier_arrive();
+    // What takes no input comes before the wait for the kernel in front.
+#pragma unroll 1
+    for (int c = tid; c <= P.cap / 4; c += nt) reinterpret_cast<uint4 *>(cell)[c] = make_uint4(0, 0, 0, 0);
+    if (tid == 0) { sh.acc = 0; sh.total = 0; sh.ncells = 0; sh.later = 0; sh.slow = 0; sh.gap = 0; sh.nnodes = 0; sh.fill.packed = 0; sh.fill.wide = 0; }
+    if (tid < CELL_BATCH) {
+        sh.gmax[tid] = sh.heard[0].gmax[tid] = sh.heard[1].gmax[tid] = 0;
+        sh.gmin[tid] = sh.heard[0].gmin[tid] = sh.heard[1].gmin[tid] = INF32;
+    }
+    for (int k = tid; k < GUARD_BINS; k += nt) sh.hist[k] = 0;
+    grid_dep_wait();
     const int r0 = min(rank * P.rpc, n), nrows = min(P.rpc, n - r0);
     if (b == 0 && rank == 0 && tid < 2) P.flags[4 + tid] = 0;      // (used by the last kernel only)
     // ---- columns of the own rows; everybody gets everybody's minima and maxima and the low words of the rows' ends
@@ -417,12 +760,13 @@ __global__ void __launch_bounds__(1024, 1) k_cells(const SRC src, const CellPara
 #pragma unroll 1
         for (int p = tid; p < nrows; p += nt) {
             const auto row = rows.row(r0 + p);
-            const int64_t x = row.at(0), y = row.at(R - 1);
-            if (OBJ == ZL_OBJ_RANGE && R > 2 && (r0 + p) % step == 0) {
+            const int h = (R - 1) / 2;
+            const bool probe = OBJ == ZL_OBJ_RANGE && R > 2 && (r0 + p) % step == 0;
+            const int64_t x = row.at(0), y = row.at(R - 1), z = probe ? row.at(h) : 0;
+            if (probe) {
                 // RANGE, a few dozen rows: how far the row's middle element is from where a row of equal gaps has it, in gaps: after h of R - 1
                 // gaps with a standard deviation of s (in gaps) that is s * sqrt(h * (R - 1 - h) / (R - 1)) on average
-                const int h = (R - 1) / 2;
-                const float span = (float)(y - x), off = (float)(row.at(h) - x) * (float)(R - 1) - span * (float)h;
+                const float span = (float)(y - x), off = (float)(z - x) * (float)(R - 1) - span * (float)h;
                 if (span > 0.f) irr += off * off / (span * span) * ((float)(R - 1) / ((float)h * (float)(R - 1 - h)));
             }
             const uint64_t ux = (uint64_t)x ^ (1ull << 63), uy = (uint64_t)y ^ (1ull << 63);
@@ -431,20 +775,13 @@ __global__ void __launch_bounds__(1024, 1) k_cells(const SRC src, const CellPara
         }
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            q[k] = (k & 1) ? warp_reduce(q[k], OpMax()) : warp_reduce(q[k], OpMin());
+            q[k] = (k & 1) ? warp_max64(q[k]) : warp_min64(q[k]);
             if (lane == 0) sh.red[k][warp] = q[k];
         }
         if (OBJ == ZL_OBJ_RANGE) {
             irr = warp_sum(irr);
-            if (lane == 0) sh.tmp[warp] = (uint64_t)__float_as_uint(irr);
+            if (lane == 0) sh.keys[warp] = (uint64_t)__float_as_uint(irr);
         }
-        if (tid == 0) {
-            sh.acc = 0; sh.total = 0; sh.key = ~0ull; sh.ncells = 0; sh.nnodes = 0; sh.sstatus = 0; sh.later = 0; sh.pieces = 0; sh.slow = 0; sh.asked = 0;
-            sh.best.d = sh.best.t = ~0ull; sh.best.valid = 0; sh.best.status = 0;
-        }
-        if (tid < CELL_BATCH) { sh.gmax[tid] = sh.gmaxl[tid] = 0; sh.gmin[tid] = sh.gminl[tid] = INF32; }
-#pragma unroll 1
-        for (int k = tid; k < GUARD_BINS; k += nt) sh.hist[k] = 0;
         __syncthreads();
         if (G > 1) {
             cl.barrier_wait();
@@ -456,38 +793,36 @@ __global__ void __launch_bounds__(1024, 1) k_cells(const SRC src, const CellPara
                 for (int p = tid; p < nrows; p += nt) to[r0 + p] = ends[r0 + p];
             }
         }
-        if (tid < 4 * G) {
-            const int k = tid & 3, r = tid >> 2;
-            unsigned long long v = sh.red[k][0];
 #pragma unroll 1
-            for (int w = 1; w < nw; ++w) v = (k & 1) ? max(v, sh.red[k][w]) : min(v, sh.red[k][w]);
-            cl.map_shared_rank(&sh, r)->ex[k][rank] = v;
-            if (OBJ == ZL_OBJ_RANGE && k == 0) {
-                float v = 0.f;
-#pragma unroll 1
-                for (int w = 0; w < nw; ++w) v += __uint_as_float((uint32_t)sh.tmp[w]);
-                cl.map_shared_rank(&sh, r)->exi[rank] = v;
+        for (int k = warp; k < (OBJ == ZL_OBJ_RANGE ? 5 : 4); k += nw) {
+            if (k < 4) {
+                uint64_t v = lane < nw ? sh.red[k][lane] : (k & 1) ? 0ull : ~0ull;
+                v = (k & 1) ? warp_max64(v) : warp_min64(v);
+                if (lane < G) cl.map_shared_rank(&sh, lane)->ex[k][rank] = v;
+            } else {
+                const float v = warp_sum(lane < nw ? __uint_as_float((uint32_t)sh.keys[lane]) : 0.f);
+                if (lane < G) cl.map_shared_rank(&sh, lane)->exi[rank] = v;
             }
         }
     }
-#pragma unroll 1
-    for (int c = tid; c <= P.cap / 4; c += nt) reinterpret_cast<uint4 *>(cell)[c] = make_uint4(0, 0, 0, 0);
     if constexpr (std::is_same<SRC, MatBatch>::value) if (P.check_sorted) {
         const bool bad = rows_unsorted(src.ts + ((size_t)b * n + r0) * R, nrows, R);
         const int any = __syncthreads_or(bad);
         if (tid < G) cl.map_shared_rank(&sh, tid)->exc[rank] = any ? 1ull : 0ull;
     }
     cl.sync();
+    int64_t tmin;
+    {
     InstMeta M;
     {
         uint64_t q[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            q[k] = sh.ex[k][0];
-#pragma unroll 1
-            for (int r = 1; r < G; ++r) q[k] = (k & 1) ? max(q[k], (uint64_t)sh.ex[k][r]) : min(q[k], (uint64_t)sh.ex[k][r]);
+            q[k] = lane < G ? (uint64_t)sh.ex[k][lane] : (k & 1) ? 0ull : ~0ull;
+            q[k] = (k & 1) ? warp_max64(q[k]) : warp_min64(q[k]);
         }
-        const int64_t tmin = (int64_t)(q[0] ^ (1ull << 63)), t0 = (int64_t)(q[1] ^ (1ull << 63));
+        tmin = (int64_t)(q[0] ^ (1ull << 63));
+        const int64_t t0 = (int64_t)(q[1] ^ (1ull << 63));
         const int64_t lmin = (int64_t)(q[2] ^ (1ull << 63)), tmax = (int64_t)(q[3] ^ (1ull << 63));
         M.tmin = tmin; M.status = ZL_OK;
         M.cscale = 0; M.fscale = 0; M.count = 0; M.count2 = 0; M.overflow = 0; M.dmin = 0;
@@ -501,28 +836,23 @@ __global__ void __launch_bounds__(1024, 1) k_cells(const SRC src, const CellPara
             M.use32 = M.tend < 0xfffffffeull;
             if (OBJ == ZL_OBJ_SUM && M.tend > (uint64_t)INT64_MAX / (uint64_t)n) M.status = ZL_ERR_UNSUPPORTED;
         }
-        if (P.check_sorted && M.status == ZL_OK) {
-#pragma unroll 1
-            for (int r = 0; r < G; ++r) if (sh.exc[r]) M.status = ZL_ERR_UNSORTED;
-        }
+        if (P.check_sorted && M.status == ZL_OK && __any_sync(FULL, lane < G && sh.exc[min(lane, G - 1)])) M.status = ZL_ERR_UNSORTED;
         M.cscale = M.status == ZL_OK && M.use32 ? 1u : 0u;
+        if (rank == 0 && tid == 0) P.meta[b] = M;
     }
     if (!M.cscale) {                                              // the same in the whole cluster
         if (rank == 0 && tid == 0) {
-            P.meta[b] = M;
             P.flags[2] = P.epoch;                                 // the last kernel writes this instance's outputs
             if (M.status == ZL_OK) P.flags[1] = P.flags[3] = P.epoch;
         }
         return;
     }
-    const RowReader<SRC> rd(src, b, n, R, M.tmin);
-    const uint32_t t0 = (uint32_t)M.t0, lmin = (uint32_t)M.lmin, tend = (uint32_t)M.tend, tminlo = (uint32_t)(uint64_t)M.tmin - 1u;
-    uint32_t lo = 1, hi = lmin + 1, shift;
-    uint64_t ub = ~0ull;                                          // SUM: a wait that is attained
-    float width;                                                  // what a cell may span, in time units
+    if (tid == 0) { sh.tmin = M.tmin; sh.t0 = (uint32_t)M.t0; sh.lmin = (uint32_t)M.lmin; sh.tend = (uint32_t)M.tend; }
+    }
     {
         uint32_t longest = 0;
-#pragma unroll 1
+        const uint32_t tminlo = (uint32_t)(uint64_t)tmin - 1u;
+#pragma unroll 2
         for (int p = tid; p < n; p += nt) {
             uint2 e = ends[p];
             e.x -= tminlo; e.y -= tminlo;
@@ -531,198 +861,156 @@ __global__ void __launch_bounds__(1024, 1) k_cells(const SRC src, const CellPara
         }
         longest = __reduce_max_sync(FULL, longest);
         if (lane == 0) sh.red[0][warp] = longest;
+    }
+    __syncthreads();
+    if (OBJ == ZL_OBJ_RANGE) {
+        // Guards: the rows that can set G near the optimum.  At a random time row i's next element is uniform in its mean
+        // gap m_i away, so all are within x with probability prod(x / m_i) over the rows with m_i > x; the smallest d of
+        // about N = n * R tries is the x where sum(log(m_i / x)) reaches log(N), and rows with gaps shorter than that
+        // hardly matter.  With the rows counted by the logarithm of their span that is a prefix sum of a prefix sum.  Rows
+        // a bin shorter are taken along, and more of them where single gaps are much longer than the row's mean.  (A fifth
+        // to a half of the rows on the workloads at hand.  A fixed fifth leaves dozens of cells where single gaps are
+        // long: n=1024, R=1024, B=64 87 us; a fixed half costs n=128, R=256, B=1024 68 us instead of 53.)
+        const uint32_t longest = __reduce_max_sync(FULL, lane < nw ? (uint32_t)sh.red[0][lane] : 0u);
+        const int top = __float_as_int((float)longest) >> 20;
+#pragma unroll 2
+        for (int p = tid; p < n; p += nt) {
+            const uint2 e = ends[p];
+            atomicAdd(&sh.hist[min(GUARD_BINS - 1, top - (__float_as_int((float)(e.y - e.x)) >> 20))], 1u);
+        }
         __syncthreads();
-        longest = (uint32_t)sh.red[0][0];
-#pragma unroll 1
-        for (int w = 1; w < nw; ++w) longest = max(longest, (uint32_t)sh.red[0][w]);
-        if (OBJ == ZL_OBJ_RANGE) {
-            // Guards: the rows that can set G near the optimum.  At a random time row i's next element is uniform in its mean
-            // gap m_i away, so all are within x with probability prod(x / m_i) over the rows with m_i > x; the smallest d of
-            // about N = n * R tries is the x where sum(log(m_i / x)) reaches log(N), and rows with gaps shorter than that
-            // hardly matter.  With the rows counted by the logarithm of their span that is a prefix sum of a prefix sum.  Rows
-            // a bin shorter are taken along, and more of them where single gaps are much longer than the row's mean.  (A fifth
-            // to a half of the rows on the workloads at hand.  A fixed fifth leaves dozens of cells where single gaps are
-            // long: n=1024, R=1024, B=64 87 us; a fixed half costs n=128, R=256, B=1024 68 us instead of 53.)
-            const int top = __float_as_int((float)longest) >> 20;
-#pragma unroll 1
-            for (int p = tid; p < n; p += nt) {
-                const uint2 e = ends[p];
-                atomicAdd(&sh.hist[min(GUARD_BINS - 1, top - (__float_as_int((float)(e.y - e.x)) >> 20))], 1u);
-            }
-            __syncthreads();
-            if (warp == 0) {
-                const uint32_t x0 = sh.hist[2 * lane], x1 = sh.hist[2 * lane + 1];
-                uint32_t inc = x0 + x1;                           // rows in the bins up to the lane's second one
+        float span;
+        {                                                         // every warp by itself
+            const uint32_t x0 = sh.hist[2 * lane], x1 = sh.hist[2 * lane + 1];
+            uint32_t inc = x0 + x1;                               // rows in the bins up to the lane's second one
 #pragma unroll
-                for (int d = 1; d < 32; d <<= 1) { const uint32_t y = __shfl_up_sync(FULL, inc, d); if (lane >= d) inc += y; }
-                const uint32_t n0 = inc - x1, n1 = inc;           // rows up to bin 2 lane, 2 lane + 1
-                uint32_t dep = n0 + n1;                           // sum of these over the bins: (bin - own bin) over the rows, from the next bin on
+            for (int d = 1; d < 32; d <<= 1) { const uint32_t y = __shfl_up_sync(FULL, inc, d); if (lane >= d) inc += y; }
+            const uint32_t n0 = inc - x1, n1 = inc;               // rows up to bin 2 lane, 2 lane + 1
+            uint32_t dep = n0 + n1;                               // sum of these over the bins: (bin - own bin) over the rows, from the next bin on
 #pragma unroll
-                for (int d = 1; d < 32; d <<= 1) { const uint32_t y = __shfl_up_sync(FULL, dep, d); if (lane >= d) dep += y; }
-                const uint32_t d0 = dep - n0 - n1, d1 = dep - n1; // that sum at bin 2 lane, 2 lane + 1
-                const uint32_t tries = (uint32_t)(8.f * log2f((float)n * (float)R)), least = (uint32_t)min(n, 8);
-                int k = __reduce_min_sync(FULL, d0 >= tries ? 2 * lane : d1 >= tries ? 2 * lane + 1 : GUARD_BINS);
-                float irr = 0.f;
-#pragma unroll 1
-                for (int r = 0; r < G; ++r) irr += sh.exi[r];
-                const float dev = sqrtf(irr / (float)((n + (n + 31) / 32 - 1) / ((n + 31) / 32)));
-                if (lane == 0 && dev * sqrtf((float)R) > 2.f * CELL_OFF) sh.slow = 1;      // (dev * sqrt(R) / 2 elements in the middle)
-                k += 1 + (int)(GUARD_IRREGULAR * max(0.f, min(1.f, dev) - 0.1f));
-                k = max(k, __reduce_min_sync(FULL, n0 >= least ? 2 * lane : n1 >= least ? 2 * lane + 1 : GUARD_BINS));
-                if (lane == 0) sh.span = k >= min(GUARD_BINS - 1, top) ? 0.f : __int_as_float((top - k) << 20);
+            for (int d = 1; d < 32; d <<= 1) { const uint32_t y = __shfl_up_sync(FULL, dep, d); if (lane >= d) dep += y; }
+            const uint32_t d0 = dep - n0 - n1, d1 = dep - n1;     // that sum at bin 2 lane, 2 lane + 1
+            const uint32_t tries = (uint32_t)(8.f * log2f((float)n * (float)R)), least = (uint32_t)min(n, 8);
+            const int at = __reduce_min_sync(FULL, d0 >= tries ? 2 * lane : d1 >= tries ? 2 * lane + 1 : GUARD_BINS);
+            const float irr = warp_sum(lane < G ? sh.exi[min(lane, G - 1)] : 0.f);
+            const float dev = sqrtf(irr / (float)((n + (n + 31) / 32 - 1) / ((n + 31) / 32)));
+            int k = at + 1 + (int)(GUARD_IRREGULAR * max(0.f, min(1.f, dev) - 0.1f));
+            k = max(k, __reduce_min_sync(FULL, n0 >= least ? 2 * lane : n1 >= least ? 2 * lane + 1 : GUARD_BINS));
+            span = k >= min(GUARD_BINS - 1, top) ? 0.f : __int_as_float((top - k) << 20);
+            if (tid == 0) {
+                if (dev * sqrtf((float)R) > 2.f * CELL_OFF) sh.slow = 1;      // (dev * sqrt(R) / 2 elements in the middle)
+                sh.span = span;
+                sh.slack = CELL_SLACK + (int)min(32.f, 0.5f * dev * sqrtf((float)R));
+                // gaps that are shorter than the smallest d that is to be expected hardly matter
+                sh.gap = at < GUARD_BINS && top - at > EXPECTED_BINS ? (uint32_t)(__int_as_float((top - at - EXPECTED_BINS) << 20) / (float)max(R - 1, 1)) : 0u;
+                sh.width = R > 1 ? (float)longest / ((float)(R - 1) * RANGE_CELLS) : 0.f;
+                sh.lo = 1; sh.hi = sh.lmin + 1u; sh.ub = ~0ull;
             }
-            __syncthreads();
-            const float span = sh.span;
-            float el = 0.f;
-#pragma unroll 1
-            for (int p = tid; p < n; p += nt) {
-                const float w = (float)(ends[p].y - ends[p].x);
-                if (w < span) el += min(1.f, (float)(lmin - min(lmin, ends[p].x)) / w) * (float)R;
-            }
-            el = warp_sum(el);
-            if (lane == 0) atomicAdd(&sh.later, (unsigned long long)el);
-            width = R > 1 ? (float)longest / ((float)(R - 1) * RANGE_CELLS) : 0.f;
-        } else {
-            // the wait at one time between the last worker's start and the first row's end
-            const uint32_t lm = max(lmin, t0), t = t0 + (lm - t0) / 2;
+        }
+        float el = 0.f;
+        const uint32_t lmin = sh.lmin;
+#pragma unroll 2
+        for (int p = tid; p < n; p += nt) {
+            const float w = (float)(ends[p].y - ends[p].x);
+            if (w < span) el += min(1.f, (float)(lmin - min(lmin, ends[p].x)) / w) * (float)R;
+        }
+        el = warp_sum(el);
+        if (lane == 0) atomicAdd(&sh.later, (unsigned long long)el);
+    } else {
+        // the wait at one time between the last worker's start and the first row's end
+        const uint32_t t0 = sh.t0, lm = max(sh.lmin, t0);
+        {
+            const uint32_t t = t0 + (lm - t0) / 2;
+            const RowReader<SRC> rd(src, b, P.B, n, R, sh.tmin);
             uint64_t acc = 0;
 #pragma unroll 1
             for (int p = tid; p < nrows; p += nt) {
                 const uint2 e = ends[r0 + p];
-                const int i = first_at_or_after(rd, r0 + p, R, t + 1u, e.x, e.y);
-                acc += t - rd.in(r0 + p, max(0, i - 1));
+                acc += t - rd.in(r0 + p, max(0, first_at_or_after(rd, r0 + p, R, t + 1u, e.x, e.y) - 1));
             }
-            acc = warp_reduce(acc, OpAdd());
+            acc = warp_sum64(acc);
             if (lane == 0) atomicAdd(&sh.acc, (unsigned long long)acc);
+        }
+        unsigned long long *es = (unsigned long long *)answers;   // (64 words, not in use yet)
+        if (tid < 64) es[tid] = 0;
+        __syncthreads();
+        if (tid < G) cl.map_shared_rank(&sh, tid)->exs[rank] = sh.acc;
+        cl.sync();
+        const uint64_t ub = warp_sum64(lane < G ? (uint64_t)sh.exs[min(lane, G - 1)] : 0ull);
+        // times past lm at which the exhausted rows alone wait longer than that are left out: the first of 32 trial times
+        // where they do (closer together near lm), then the first of 32 more between that one and the one before it
+        const uint32_t tend = sh.tend;
+        uint32_t below = lm, stop = lm + (uint32_t)min(ub, (uint64_t)(tend - lm));
+#pragma unroll 1
+        for (int part = 0; part < 2; ++part, es += 32) {
+            const uint64_t k = part ? 32ull * (lane + 1) : (uint64_t)((lane + 1) * (lane + 1));
+            const uint32_t trial = below + (uint32_t)(((uint64_t)(stop - below) * k) >> 10);
+            uint64_t e = 0;
+#pragma unroll 4
+            for (int p = warp; p < n; p += nw) { const uint32_t last = ends[p].y; e += trial > last ? trial - last : 0u; }
+            atomicAdd(&es[lane], (unsigned long long)e);
             __syncthreads();
-            if (tid < G) cl.map_shared_rank(&sh, tid)->exs[rank] = sh.acc;
-            cl.sync();
-            ub = 0;
-#pragma unroll 1
-            for (int r = 0; r < G; ++r) ub += sh.exs[r];
-            // times past lm at which the exhausted rows alone wait longer than that are left out: the first of 32 trial times
-            // where they do (closer together near lm), then the first of 32 more between that one and the one before it
-            unsigned long long *es = (unsigned long long *)sh.node;              // (64 words, not in use yet)
-            if (tid < 64) es[tid] = 0;
-            if (tid == 0) sh.acc = 0;
-            uint32_t below = lm, stop = lm + (uint32_t)min(ub, (uint64_t)(tend - lm));
-#pragma unroll 1
-            for (int part = 0; part < 2; ++part, es += 32) {
-                __syncthreads();
-                const uint64_t k = part ? 32ull * (lane + 1) : (uint64_t)((lane + 1) * (lane + 1));
-                const uint32_t trial = below + (uint32_t)(((uint64_t)(stop - below) * k) >> 10);
-                uint64_t e = 0;
-#pragma unroll 1
-                for (int p = warp; p < n; p += nw) { const uint32_t last = ends[p].y; e += trial > last ? trial - last : 0u; }
-                atomicAdd(&es[lane], (unsigned long long)e);
-                __syncthreads();
-                const unsigned over = __ballot_sync(FULL, es[lane] > ub);
-                const int first = over ? __ffs(over) - 1 : 32;
-                const uint32_t at = __shfl_sync(FULL, trial, min(first, 31)), before = __shfl_sync(FULL, trial, max(first - 1, 0));
-                if (first > 0) below = before;
-                if (first < 32) stop = at;
-                else { stop = part ? stop : tend; below = stop; }
-            }
-            lo = t0;
-            hi = max(lo, min(stop, tend)) + 1u;
+            const unsigned over = __ballot_sync(FULL, es[lane] > ub);
+            const int first = over ? __ffs(over) - 1 : 32;
+            const uint32_t at = __shfl_sync(FULL, trial, min(first, 31)), before = __shfl_sync(FULL, trial, max(first - 1, 0));
+            if (first > 0) below = before;
+            if (first < 32) stop = at;
+            else { stop = part ? stop : tend; below = stop; }
+        }
+        if (tid == 0) {
+            sh.acc = 0;
+            sh.lo = t0; sh.hi = max(t0, min(stop, tend)) + 1u; sh.ub = ub; sh.slack = CELL_SLACK; sh.span = 0.f;
             // n cell widths are the looseness of a cell's bounds; the wait itself spreads over time by about sqrt(n) times
             // 0.29 iterations, an iteration being about twice the mean wait of a worker.  (n=17, R=700, B=20: half the factor
             // 73 us, twice the factor 840, with six instances left over; n=32, R=400, B=20 41, 39 and 68.)
-            width = SUM_WIDTH * (float)ub / ((float)n * sqrtf((float)n));
-            __syncthreads();                                      // es has been read
+            sh.width = SUM_WIDTH * (float)ub / ((float)n * sqrtf((float)n));
         }
     }
-    shift = width >= 2.f ? (uint32_t)min(31, (__float_as_int(width) >> 23) - 127) : 0u;
-    while (((hi - lo - 1u) >> shift) >= (uint32_t)(G * P.cap)) ++shift;
-    const uint32_t ncells = ((hi - lo - 1u) >> shift) + 1u;
-    const uint32_t per = ((ncells + G - 1) / G + 3u) & ~3u;       // cells of a CTA (cap is a multiple of 128, so they fit)
-    const uint32_t c0 = min((uint32_t)rank * per, ncells), c1 = min(c0 + per, ncells);
-    const int m = (int)(c1 - c0), nblk = (m + 127) >> 7;
-    const uint32_t a = lo + (c0 << shift), bnd = c1 == ncells ? hi : lo + (c1 << shift);
+    if (tid == 0) {
+        // the cells, and the CTA's slice of them
+        const uint32_t lo = sh.lo, hi = sh.hi;
+        uint32_t shift = sh.width >= 2.f ? (uint32_t)min(31, (__float_as_int(sh.width) >> 23) - 127) : 0u;
+        while (((hi - lo - 1u) >> shift) >= (uint32_t)(G * P.cap)) ++shift;
+        const uint32_t ncells = ((hi - lo - 1u) >> shift) + 1u;
+        const uint32_t per = ((ncells + G - 1) / G + 3u) & ~3u;   // cells of a CTA (cap is a multiple of 128, so they fit)
+        const uint32_t c0 = min((uint32_t)rank * per, ncells), c1 = min(c0 + per, ncells);
+        sh.shift = shift; sh.c0 = c0; sh.m = c1 - c0;
+        sh.a = lo + (c0 << shift); sh.bnd = c1 == ncells ? hi : lo + (c1 << shift);
+        // cells asked for at first: the most promising one of every CTA, as far as the answers cost the warps no second turn
+        sh.firsts = max(1, min(min(CELL_FIRST, G), nw / ((P.rpc + 31) >> 5)));
+        // with a few cells on either side of it: SUM so many as give about a dozen answers
+        sh.around = OBJ == ZL_OBJ_RANGE ? 1 : (int)max(2u, min(8u, (uint32_t)(8ull * ncells / ((unsigned long long)n * R))));
+        sh.bd = ~0ull; sh.bt = INF32; sh.ndone = 0; sh.asked = 0; sh.took = 0;
+    }
+    __syncthreads();
+    const int m = (int)sh.m, nblk = (m + 127) >> 7;
     bool fits = true;
-    uint32_t gap = 0;                                             // RANGE: no cell's bound is below this
-    uint64_t low = 0;                                             // cells with keys up to this have been evaluated
-    int stage = 0, streamed = -1;                                 // RANGE: 0 the guards, 1 (seldom) the other rows too
+    int stage = 0, streamed = -1, evaluated = 0;                  // RANGE: 0 the guards, 1 (seldom) the other rows too; evaluations
+    auto done = [&](uint32_t c) { return sh.ndone != 0 && was_asked(sh.asked_run, sh.ndone, c); };      // seldom called: for a cell that would be evaluated (once more)
 #pragma unroll 1
-    for (int round = 0;; ++round) {                               // a round: the most promising cell is evaluated, the rest counted
+    for (int round = 0;; ++round) {                               // a round: the most promising cells are evaluated, the rest counted
         // ---- the rows' elements in the slice
-        if (m > 0 && streamed != stage) {
-            uint64_t carry = 0, total = 0;                        // SUM: the rows' last elements before a, and all deltas in the slice
-            const uint32_t w = bnd - a;
-#pragma unroll 1
-            for (int base = warp; base < n; base += 32 * nw) {    // warp w takes rows w, w + nw, ..., a row a lane
-                const int row = base + lane * nw;
-                uint2 e = make_uint2(0u, 0u);
-                bool have = row < n;
-                if (have) {
-                    e = ends[row];
-                    if (OBJ == ZL_OBJ_RANGE) have = ((float)(e.y - e.x) >= sh.span) == (stage == 0);
-                    if (e.x >= bnd || e.y < a) {                  // no element of the row in the slice
-                        if (OBJ == ZL_OBJ_SUM && have && e.y < a) carry += e.y;
-                        have = false;
-                    }
-                }
-                const int pieces = stream_rows(rd, R, row, have, e.x, e.y, a, bnd, [&](const uint32_t (&T)[9]) {
-                    if (OBJ == ZL_OBJ_RANGE) {
-                        // cell[k] becomes a lower bound of G at the start of cell k (before the prefix maximum): an element
-                        // says that G is at least its successor for the cells after its own.  Elements before the slice
-                        // count for its first cell; those in its last cell or behind it go to cell[m], which is not looked
-                        // at.  A gap of at most `gap` cannot push a cell's bound, G less the cell's end, beyond that: it discards no cell.
-                        uint32_t longer = 0;
-#pragma unroll
-                        for (int j = 0; j < 8; ++j) longer = max(longer, T[j + 1] - T[j]);
-                        if (longer > gap) {
-                            uint32_t k[8], v[8];
-#pragma unroll
-                            for (int j = 0; j < 8; ++j) {
-                                k[j] = T[j] < a ? 0u : min(((T[j] - a) >> shift) + 1u, (uint32_t)m);
-                                v[j] = cell[k[j]];                // all eight under way; a value gone stale costs an update
-                            }
-#pragma unroll
-                            for (int j = 0; j < 8; ++j) if (T[j + 1] - T[j] > gap && v[j] < T[j + 1]) atomicMax(&cell[k[j]], T[j + 1]);
-                        }
-                    } else {
-                        uint32_t in = 0, before = 0;
-#pragma unroll
-                        for (int j = 0; j < 8; ++j) {
-                            const uint32_t d = T[j + 1] - a, delta = T[j + 1] - T[j];
-                            if (d < w) { atomicAdd(cell + (d >> shift), delta); in += delta; }
-                            if (T[j] < a && T[j + 1] >= a) before = T[j];
-                        }
-                        total += in; carry += before;
-                    }
-                });
-                if (OBJ == ZL_OBJ_RANGE && lane == 0) atomicAdd(&sh.pieces, (unsigned)pieces);
-            }
-            if (OBJ == ZL_OBJ_SUM) {
-                carry = warp_reduce(carry, OpAdd());
-                total = warp_reduce(total, OpAdd());
-                if (lane == 0) { atomicAdd(&sh.acc, (unsigned long long)carry); atomicAdd(&sh.total, (unsigned long long)total); }
-            }
-        }
+        if (streamed != stage) look_through<OBJ>(sh, cell, answers, ends, src, P.B, n, R, stage);
         streamed = stage;
-        __syncthreads();
         // ---- what the sweep knows at every cell's start; a warp takes a run of 128-cell blocks, four cells a lane
         const int bpw = (nblk + nw - 1) / nw, k0 = min(warp * bpw, nblk), k1 = min(k0 + bpw, nblk);
         typedef typename std::conditional<OBJ == ZL_OBJ_RANGE, uint32_t, uint64_t>::type ST;
         {
             ST t = 0;
-#pragma unroll 1
+#pragma unroll 2
             for (int k = k0; k < k1; ++k) {
                 const uint4 v = *reinterpret_cast<const uint4 *>(cell + 128 * k + 4 * lane);
                 if constexpr (OBJ == ZL_OBJ_RANGE) t = max(max(t, max(v.x, v.y)), max(v.z, v.w));
                 else t += (uint64_t)v.x + v.y + v.z + v.w;
             }
-            if constexpr (OBJ == ZL_OBJ_RANGE) t = __reduce_max_sync(FULL, t); else t = warp_reduce(t, OpAdd());
+            if constexpr (OBJ == ZL_OBJ_RANGE) t = __reduce_max_sync(FULL, t); else t = warp_sum64(t);
             if (lane == 0) sh.red[0][warp] = t;
         }
-        if (tid == 0) sh.key = ~0ull;
         __syncthreads();
         uint64_t key = ~0ull, kbase = 0;
+        const uint32_t a = sh.a, bnd = sh.bnd, shift = sh.shift, c0 = sh.c0;
         if constexpr (OBJ == ZL_OBJ_RANGE) {
-            uint32_t run = t0;
-#pragma unroll 1
-            for (int w = 0; w < warp; ++w) run = max(run, (uint32_t)sh.red[0][w]);
+            uint32_t run = max(sh.t0, __reduce_max_sync(FULL, lane < warp ? (uint32_t)sh.red[0][lane] : 0u));
 #pragma unroll 1
             for (int k = k0; k < k1; ++k) {
                 uint4 v = *reinterpret_cast<const uint4 *>(cell + 128 * k + 4 * lane);
@@ -742,13 +1030,16 @@ __global__ void __launch_bounds__(1024, 1) k_cells(const SRC src, const CellPara
                     const int c = 128 * k + 4 * lane + j;
                     const uint32_t end = cell_end(a + ((uint32_t)c << shift), shift, bnd);
                     const uint64_t q = (uint64_t)(g[j] > end ? g[j] - end : 0u) << 24 | (c0 + (uint32_t)c + 1u);      // never 0
-                    if (c < m && g[j] != INF32 && q > low && q < key) { key = q; kbase = g[j]; }
+                    if (c < m && g[j] != INF32 && q < key && !done(c0 + (uint32_t)c)) { key = q; kbase = g[j]; }
                 }
             }
         } else {
-            uint64_t run = sh.acc, all = 0;
-#pragma unroll 1
-            for (int w = 0; w < nw; ++w) { if (w < warp) run += sh.red[0][w]; all += sh.red[0][w]; }
+            uint64_t run, all;
+            {
+                const uint64_t x = lane < nw ? (uint64_t)sh.red[0][lane] : 0ull;
+                run = sh.acc + warp_sum64(lane < warp ? x : 0ull);
+                all = warp_sum64(x);
+            }
             const uint64_t nn = (uint64_t)n;
 #pragma unroll 1
             for (int k = k0; k < k1; ++k) {
@@ -758,21 +1049,30 @@ __global__ void __launch_bounds__(1024, 1) k_cells(const SRC src, const CellPara
 #pragma unroll
                 for (int d = 1; d < 32; d <<= 1) { const uint64_t y = shfl_up(inc, d); if (lane >= d) inc += y; }
                 const uint64_t before = run + inc - s4;
-                const uint64_t S[4] = {before + s1, before + s2, before + s3, before + s4};
-                const uint32_t dv[4] = {v.x, v.y, v.z, v.w};
+                const uint32_t c = 128u * k + 4u * lane, start = a + (c << shift);
                 uint64_t lbm = ~0ull;
+                if (s4 != 0) {
+                    // four cells together: none has a wait below the bound of the first one's start and all their elements
+                    const uint64_t l = nn * start > before + s4 ? nn * start - (before + s4) : 0ull;
+                    lbm = l;
+                    if (sh.ndone == 0) {
+                        // ... and the last one with elements in it attains at most this
+                        const uint32_t j = v.w ? 3u : v.z ? 2u : v.y ? 1u : 0u;
+                        const uint64_t u = nn * cell_end(start + (j << shift), shift, bnd) - (before + s4);
+                        const uint64_t q = min(u, (uint64_t)0xffffffffffull) << 24 | (c0 + c + j + 1u);
+                        if (q < key) { key = q; kbase = before + s4 - (j == 3u ? v.w : j == 2u ? v.z : j == 1u ? v.y : v.x); }
+                    } else {
+                        const uint64_t S[4] = {before + s1, before + s2, before + s3, before + s4};
+                        const uint32_t dv[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const int c = 128 * k + 4 * lane + j;
-                    if (dv[j] != 0u) {
-                        const uint32_t start = a + ((uint32_t)c << shift), end = cell_end(start, shift, bnd);
-                        const uint64_t u = nn * end - S[j], l = nn * start > S[j] ? nn * start - S[j] : 0ull;
-                        lbm = min(lbm, l);
-                        const uint64_t q = min(u, (uint64_t)0xffffffffffull) << 24 | (c0 + (uint32_t)c + 1u);
-                        if (q > low && q < key) { key = q; kbase = S[j] - dv[j]; }
+                        for (int j = 0; j < 4; ++j) {
+                            const uint64_t u = nn * cell_end(start + ((uint32_t)j << shift), shift, bnd) - S[j];
+                            const uint64_t q = min(u, (uint64_t)0xffffffffffull) << 24 | (c0 + c + (uint32_t)j + 1u);
+                            if (dv[j] != 0u && q < key && !done(c0 + c + (uint32_t)j)) { key = q; kbase = S[j] - dv[j]; }
+                        }
                     }
                 }
-                lbm = warp_reduce(lbm, OpMin());
+                lbm = warp_min64(lbm);
                 if (lane == 0) { blk_before[k] = run; blk_lb[k] = lbm; }
                 run += shfl_idx(inc, 31);
             }
@@ -780,151 +1080,224 @@ __global__ void __launch_bounds__(1024, 1) k_cells(const SRC src, const CellPara
             if (all != sh.total) fits = false;
         }
         {
-            const uint64_t mine = warp_reduce(key, OpMin());
-            if (lane == 0) atomicMin(&sh.key, (unsigned long long)mine);
+            const uint64_t mine = warp_min64(key);
+            if (key == mine) { sh.keys[warp] = mine; sh.kbases[warp] = kbase; }     // (keys are different, but where there is none)
             __syncthreads();
-            if (key != ~0ull && key == sh.key) sh.kbase = kbase;  // (keys are different)
-            __syncthreads();
-            if (tid < G) {
-                CellShared &to = *cl.map_shared_rank(&sh, tid);
-                to.exv[rank] = fits ? sh.key : 0ull;
-                to.exb[rank] = sh.kbase;
+            if (warp == 0) {
+                if (lane == 0) sh.ncells = 0;                     // (written to by the others behind the next cluster barriers)
+                const uint64_t x = lane < nw ? (uint64_t)sh.keys[lane] : ~0ull;
+                const uint64_t k = warp_min64(x);
+                uint64_t base = sh.kbases[__ffs(__ballot_sync(FULL, x == k)) - 1];
+                uint32_t first = 0;
+                if (k != ~0ull) {                                 // a few cells before it come along
+                    const int c = (int)((uint32_t)(k & 0xffffffu) - 1u - c0), from = max(c - sh.around, 0);
+                    first = c0 + (uint32_t)from;
+                    if constexpr (OBJ == ZL_OBJ_RANGE) base = cell[from];
+                    else base -= warp_sum64(lane < c - from ? (uint64_t)cell[min(from + lane, c)] : 0ull);
+                }
+                if (lane < G) {
+                    CellShared &to = *cl.map_shared_rank(&sh, lane);
+                    to.exv[rank] = fits ? k : 0ull;
+                    to.exb[rank] = base;
+                    to.exf[rank] = first;
+                }
             }
         }
         cl.sync();
-        uint64_t best_key = sh.exv[0];
-        int owner = 0;
+        // ---- the most promising cells: the best one of each CTA, in their order
+        int some = 0, listed = 0, from = 0;                       // runs of this evaluation; of the list (0: not made yet), and how many of them were evaluated
+        {
+            uint64_t x = lane < G ? (uint64_t)sh.exv[min(lane, G - 1)] : ~0ull;
+            if (__any_sync(FULL, x == 0ull)) fits = false;
+            if (!fits) break;
+            const int firsts = sh.firsts, ndone = sh.ndone;
 #pragma unroll 1
-        for (int r = 0; r < G; ++r) {
-            fits &= sh.exv[r] != 0ull;
-            if (sh.exv[r] < best_key) { best_key = sh.exv[r]; owner = r; }
-        }
-        if (!fits || best_key == ~0ull) { fits = false; break; }
-        // ---- the most promising cell exactly
-        if (OBJ == ZL_OBJ_RANGE && round == 0) gap = (uint32_t)(best_key >> 24);
-        low = best_key;
-        if (tid == 0) {
-            sh.cell[0] = (uint32_t)(best_key & 0xffffffu) - 1u; sh.order[0] = 0;
-            sh.base[0] = sh.exb[owner];
-            if (rank == 0) sh.ncells = 0;
-        }
-        __syncthreads();
-        fits = evaluate_cells<OBJ>(sh, 0, 1, rd, ends, n, R, r0, nrows, lo, hi, shift);
-        if (!fits) break;
-        if (tid == 0) sh.asked += 8;
-        // ---- the cells that may still hold a smaller one, or the same one earlier: only cells before the best one's
-        const uint64_t d = sh.best.d;
-        const uint32_t cb = ((uint32_t)sh.best.t - lo) >> shift;
-        const uint64_t limit = d < INF32 ? d << 24 | (cb + 1u) : ~0ull;      // RANGE: the best one's key, as of a cell whose bound is attained
-        CellShared &ld = *cl.map_shared_rank(&sh, 0);
-        auto keep = [&](uint32_t c, uint64_t base, uint64_t l) {
-            const unsigned pos = atomicAdd(&ld.ncells, 1u);
-            if (pos < CELL_ALIVE) {
-                // every CTA gets the list
-#pragma unroll 1
-                for (int r = 0; r < G; ++r) { CellShared &to = *cl.map_shared_rank(&sh, r); to.cell[pos] = c; to.base[pos] = base; to.lb[pos] = l; }
-            }
-        };
-        if constexpr (OBJ == ZL_OBJ_RANGE) {
-#pragma unroll 1
-            for (int c = 4 * tid; c < m; c += 4 * nt) {
-                const uint4 v = *reinterpret_cast<const uint4 *>(cell + c);
-                const uint32_t g[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const uint32_t end = cell_end(a + ((uint32_t)(c + j) << shift), shift, bnd);
-                    const uint64_t l = g[j] > end ? (uint64_t)(g[j] - end) : 0ull;
-                    const uint64_t q = l << 24 | (c0 + (uint32_t)(c + j) + 1u);
-                    if (c + j < m && q > low && q < limit) keep(c0 + (uint32_t)(c + j), g[j], l);
-                }
-            }
-        } else {
-#pragma unroll 1
-            for (int k = warp; k < nblk; k += nw) {
-                if (blk_lb[k] > d) continue;
-                const uint4 v = *reinterpret_cast<const uint4 *>(cell + 128 * k + 4 * lane);
-                const uint64_t s1 = v.x, s2 = s1 + v.y, s3 = s2 + v.z, s4 = s3 + v.w;
-                uint64_t inc = s4;
-#pragma unroll
-                for (int q = 1; q < 32; q <<= 1) { const uint64_t y = shfl_up(inc, q); if (lane >= q) inc += y; }
-                const uint64_t before = blk_before[k] + inc - s4;
-                const uint64_t S[4] = {before + s1, before + s2, before + s3, before + s4};
-                const uint32_t dv[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const uint32_t c = (uint32_t)(128 * k + 4 * lane + j);
-                    if (dv[j] != 0u) {
-                        const uint32_t start = a + (c << shift), end = cell_end(start, shift, bnd);
-                        const uint64_t st = (uint64_t)n * start, l = st > S[j] ? st - S[j] : 0ull;
-                        const uint64_t q = min((uint64_t)n * end - S[j], (uint64_t)0xffffffffffull) << 24 | (c0 + c + 1u);
-                        if ((l < d || (l == d && c0 + c < cb)) && q > low) keep(c0 + c, S[j] - dv[j], l);
+            for (; some < firsts; ++some) {
+                const uint64_t k = warp_min64(x);
+                if (k == ~0ull) break;
+                if (x == k) {
+                    x = ~0ull;
+                    if (warp == 0) {
+                        // with a few cells around it
+                        const uint32_t c = (uint32_t)(k & 0xffffffu) - 1u, first = sh.exf[lane], last = min(c + (uint32_t)sh.around, (sh.hi - 1u - sh.lo) >> shift);
+                        sh.asked_run[ndone + some] = make_uint2(first, last);
+                        sh.ca[some] = sh.lo + (first << shift); sh.ce[some] = cell_end(sh.lo + (last << shift), shift, sh.hi); sh.cb[some] = sh.exb[lane];
+                        // no cell's bound is below this: gaps of no more discard no cell
+                        if (some == 0 && OBJ == ZL_OBJ_RANGE && round == 0) sh.gap = max(sh.gap, (uint32_t)(k >> 24));
                     }
                 }
             }
+            if (some == 0) {                                      // none that has not been evaluated
+                if (round == 0) fits = false;
+                break;
+            }
         }
-        cl.sync();
-        const int ns = (int)ld.ncells;
-        if (ns == 0) break;
-        // asking every row for each of them, or looking through the other rows first?
-        if (OBJ == ZL_OBJ_RANGE && stage == 0 && sh.span > 0.f && (ns > CELL_ALIVE || (ns > CELL_FEW && (long long)ns * n * CELL_ASK > (long long)sh.later))) {
-            stage = 1; low = 0;
-            continue;                                             // (a cluster barrier follows before the length is touched again)
-        }
-        if (ns > CELL_ALIVE) {                                    // more than there is room for: the next best cell may discard them
-            fits = round < CELL_ROUNDS && ns <= CELL_HOPELESS;
-            if (fits) continue;
-            break;
-        }
+        bool again = false;
 #pragma unroll 1
-        for (int k = tid; k < ns; k += nt) {                      // most promising first, of equal ones the earliest
-            const uint64_t l = sh.lb[k];
-            const uint32_t c = sh.cell[k];
-            int at = 0;
+        for (;;) {
+            // ---- exactly
+            __syncthreads();
+            if (tid == 0) { if (listed == 0) { sh.ndone += some; sh.asked += 8; } else sh.asked += some; }
+            fits = evaluate_cells<OBJ>(sh, answers, ends, src, P.B, n, R, P.rpc, evaluated & 1, some) <= CELL_NODES;
+            ++evaluated;
+            if (!fits) break;
+            const uint64_t d = sh.bd;
+            const uint32_t cb = (sh.bt - sh.lo) >> shift;
+            if (listed == 0) {
+                // ---- the cells that may still hold a smaller one, or the same one earlier: only cells before the best one's
+                const uint64_t limit = d < INF32 ? d << 24 | (cb + 1u) : ~0ull;      // RANGE: the best one's key, as of a cell whose bound is attained
+                auto keep = [&](uint32_t c, uint64_t base, uint64_t l) {
+                    if (done(c)) return;
+                    // every CTA gets the list
 #pragma unroll 1
-            for (int i = 0; i < ns; ++i) at += sh.lb[i] < l || (sh.lb[i] == l && sh.cell[i] < c);
-            sh.order[at] = (unsigned short)k;
-        }
-        __syncthreads();
-        // (SUM: a cell whose bound does not exceed d nearly always has to be looked at)
-        const int batch = OBJ == ZL_OBJ_SUM ? 8 : max(4, min(CELL_BATCH, 4 * nt / P.rpc));
+                    for (int r = 0; r < G; ++r) {
+                        CellShared &to = *cl.map_shared_rank(&sh, r);
+                        const unsigned pos = atomicAdd(&to.ncells, 1u);
+                        if (pos < CELL_ALIVE) { to.cell[pos] = c; to.base[pos] = base; to.lb[pos] = l; }
+                    }
+                };
+                if constexpr (OBJ == ZL_OBJ_RANGE) {
 #pragma unroll 1
-        for (int from = 0; from < ns && fits; from += batch) {
-            const int x = sh.order[from];
-            if (sh.lb[x] > sh.best.d || (sh.lb[x] == sh.best.d && sh.cell[x] >= ((uint32_t)sh.best.t - lo) >> shift)) break;
-            if (tid == 0) sh.asked += min(batch, ns - from);
-            fits = evaluate_cells<OBJ>(sh, from, min(batch, ns - from), rd, ends, n, R, r0, nrows, lo, hi, shift);
+                    for (int c = 4 * tid; c < m; c += 4 * nt) {
+                        const uint4 v = *reinterpret_cast<const uint4 *>(cell + c);
+                        const uint32_t g[4] = {v.x, v.y, v.z, v.w};
+                        unsigned in = 0;
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            const uint32_t end = cell_end(a + ((uint32_t)(c + j) << shift), shift, bnd);
+                            const uint64_t q = (uint64_t)(g[j] > end ? g[j] - end : 0u) << 24 | (c0 + (uint32_t)(c + j) + 1u);
+                            if (c + j < m && q < limit) in |= 1u << j;
+                        }
+#pragma unroll 1
+                        for (; in; in &= in - 1u) {
+                            const int j = __ffs(in) - 1;
+                            const uint32_t x = j == 0 ? v.x : j == 1 ? v.y : j == 2 ? v.z : v.w, end = cell_end(a + ((uint32_t)(c + j) << shift), shift, bnd);
+                            keep(c0 + (uint32_t)(c + j), x, x > end ? (uint64_t)(x - end) : 0ull);
+                        }
+                    }
+                } else {
+#pragma unroll 1
+                    for (int k = warp; k < nblk; k += nw) {
+                        if (blk_lb[k] > d) continue;
+                        const uint4 v = *reinterpret_cast<const uint4 *>(cell + 128 * k + 4 * lane);
+                        const uint64_t s1 = v.x, s2 = s1 + v.y, s3 = s2 + v.z, s4 = s3 + v.w;
+                        uint64_t inc = s4;
+#pragma unroll
+                        for (int q = 1; q < 32; q <<= 1) { const uint64_t y = shfl_up(inc, q); if (lane >= q) inc += y; }
+                        uint64_t S = blk_before[k] + inc - s4;
+#pragma unroll 1
+                        for (int j = 0; j < 4; ++j) {
+                            const uint32_t c = (uint32_t)(128 * k + 4 * lane + j), x = cell[c];
+                            const uint64_t st = (uint64_t)n * (a + (c << shift)), l = st > S + x ? st - S - x : 0ull;
+                            if (x != 0u && (l < d || (l == d && c0 + c < cb))) keep(c0 + c, S, l);
+                            S += x;
+                        }
+                    }
+                }
+                cl.sync();
+                listed = (int)sh.ncells;
+                if (listed == 0) break;
+                if (OBJ == ZL_OBJ_RANGE && stage == 0 && sh.span > 0.f && listed > CELL_ALIVE) {      // the other rows may discard them
+                    stage = 1;
+                    again = true;                                 // (a cluster barrier follows before the list is written to again)
+                    break;
+                }
+                if (listed > CELL_ALIVE) {                        // more than there is room for: the next best cells may discard them
+                    fits = again = round < CELL_ROUNDS && listed <= CELL_HOPELESS;
+                    break;
+                }
+#pragma unroll 1
+                for (int k = tid; k < listed; k += nt) {          // in the order of time
+                    const uint32_t c = sh.cell[k];
+                    int at = 0;
+#pragma unroll 4
+                    for (int i = 0; i < listed; ++i) at += sh.cell[i] < c;
+                    sh.order[at] = (unsigned short)k;
+                }
+                __syncthreads();
+                if (warp == 0) {                                  // runs of them
+                    int runs = 0;
+#pragma unroll 1
+                    for (int i0 = 0; i0 < listed; i0 += 32) {
+                        const int i = i0 + lane, k = i < listed ? sh.order[i] : 0;
+                        const uint32_t c = sh.cell[k], before = i > 0 && i < listed ? sh.cell[sh.order[i - 1]] : 0u;
+                        const bool head = i < listed && (i == 0 || c - before > CELL_RUN<OBJ> / 2 + 1 || c / CELL_RUN<OBJ> != before / CELL_RUN<OBJ>);
+                        const unsigned heads = __ballot_sync(FULL, head);
+                        const int r = runs + __popc(heads & (FULL >> (31 - lane))) - 1;
+                        if (head) { sh.run[r] = make_uint2(c, c); sh.run_base[r] = sh.base[k]; sh.run_lb[r] = ~0ull; }
+                        __syncwarp();
+                        if (i < listed) { atomicMax(&sh.run[r].y, c); atomicMin(&sh.run_lb[r], (unsigned long long)sh.lb[k]); }
+                        __syncwarp();
+                        runs += __popc(heads);
+                    }
+                    if (lane == 0) sh.runs = runs;
+                }
+                __syncthreads();
+                listed = sh.runs;
+                // asking every row for each of them, or looking through the other rows first?
+                if (OBJ == ZL_OBJ_RANGE && stage == 0 && sh.span > 0.f && listed > CELL_FEW && (long long)listed * n * CELL_ASK > (long long)sh.later) {
+                    stage = 1;
+                    again = true;
+                    break;
+                }
+#pragma unroll 1
+                for (int k = tid; k < listed; k += nt) {          // most promising first, of equal ones the earliest
+                    const uint64_t l = sh.run_lb[k];
+                    int at = 0;
+#pragma unroll 2
+                    for (int i = 0; i < listed; ++i) at += sh.run_lb[i] < l || (sh.run_lb[i] == l && i < k);
+                    sh.order[at] = (unsigned short)k;
+                }
+                __syncthreads();
+            } else {
+                from += some;
+            }
+            // ---- the next runs of the list
+            if (from >= listed) break;
+            {
+                // (SUM: a cell whose bound does not exceed d nearly always has to be looked at; many answers a cell are compared with one another)
+                const int batch = OBJ == ZL_OBJ_SUM ? CELL_BATCH : max(4, min(CELL_BATCH, 4 * nt / P.rpc));
+                const int x = sh.order[from];
+                if (sh.run_lb[x] > d || (sh.run_lb[x] == d && sh.run[x].x >= cb)) break;
+                some = min(listed - from, max(4, min(batch, CELL_PAIRS / sh.per_cell)));
+                if (tid < some) {
+                    const int y = sh.order[from + tid];
+                    sh.ca[tid] = sh.lo + (sh.run[y].x << shift); sh.ce[tid] = cell_end(sh.lo + (sh.run[y].y << shift), shift, sh.hi); sh.cb[tid] = sh.run_base[y];
+                }
+            }
         }
-        break;
+        if (!again) break;
     }
+    // no CTA leaves while another may still write to its memory: everybody says here that it has done so for the last time
+    if (G > 1) cl.barrier_arrive();
+    const uint64_t d = sh.bd;
     // Rows that the route is not made for: many evaluations, rows that stand still, RANGE rows far off their estimates or far more of
     // them in one slice than its share.  The result is as good as any, but the handle's next calls are better off elsewhere.
     if (tid == 0 && (sh.slow || sh.asked > (OBJ == ZL_OBJ_RANGE ? CELL_ASKED_RANGE : CELL_ASKED_SUM) ||
-                     (OBJ == ZL_OBJ_RANGE && G > 1 && streamed == 0 && 16ll * G * ((long long)sh.pieces - 2 * n) > 3ll * n * R)))
+                     (OBJ == ZL_OBJ_RANGE && G > 1 && streamed == 0 && 16ll * G * ((long long)sh.took - 2 * n) > 3ll * n * R)))
         P.flags[3] = P.epoch;
-    cl.sync();                                                    // no CTA leaves while another may still read its memory
     // (a result above the wait known to be attained means rows that are not sorted: the sweep decides)
-    if (!fits || !sh.best.valid || sh.best.d > ub) {
+    if (!fits || d == ~0ull || d > sh.ub) {
         if (rank == 0 && tid == 0) {
-            M.overflow = 1;
-            P.meta[b] = M;
+            P.meta[b].overflow = 1;
             P.flags[1] = P.flags[2] = P.flags[3] = P.epoch;
         }
-        return;
-    }
-    const SegResult best = sh.best;
-    const uint32_t bar = (uint32_t)best.t + (OBJ == ZL_OBJ_RANGE ? (uint32_t)best.d : 0u);      // relative
-    if (rank == 0 && tid == 0) {
-        P.meta[b] = M;
-        P.wait[b] = (int64_t)best.d;
-        P.barrier[b] = M.tmin - 1 + (int64_t)bar;
-        if (P.status) P.status[b] = ZL_OK;
-    }
-    // ---- the indices of the own rows: the last element not after the barrier
+    } else {
+        const uint32_t bar = sh.bt + (OBJ == ZL_OBJ_RANGE ? (uint32_t)d : 0u);      // relative
+        if (rank == 0 && tid == 0) {
+            P.wait[b] = (int64_t)d;
+            P.barrier[b] = sh.tmin - 1 + (int64_t)bar;
+            if (P.status) P.status[b] = ZL_OK;
+        }
+        // ---- the indices of the own rows: the last element not after the barrier
+        const RowReader<SRC> rd(src, b, P.B, n, R, sh.tmin);
 #pragma unroll 1
-    for (int p = tid; p < nrows; p += nt) {
-        const uint2 e = ends[r0 + p];
-        P.idx[(size_t)b * n + r0 + p] = first_at_or_after(rd, r0 + p, R, bar + 1u, e.x, e.y) - 1;
+        for (int p = tid; p < nrows; p += nt) {
+            const uint2 e = ends[r0 + p];
+            P.idx[(size_t)b * n + r0 + p] = first_at_or_after(rd, r0 + p, R, bar + 1u, e.x, e.y) - 1;
+        }
     }
+    if (G > 1) cl.barrier_wait();
 }
 
 // ------------------------------------------------------------------------------ rest
@@ -950,33 +1323,37 @@ __global__ void __launch_bounds__(CELL_REST_THREADS) k_cell_rest(const SRC src, 
 
 // ------------------------------------------------------------------------------ host side
 // CTAs of an instance's cluster, their threads, and the cells each has room for.
-struct CellShape { int cluster, threads, cap; size_t smem; };
+struct CellShape { int cluster, threads, cap; bool many; size_t smem; };
 
 static CellShape cell_shape(int n, int R, int B, int objective, int num_sms) {
     CellShape s;
-    // CTAs: as many as there are SMs (SUM: two an SM), each with 16 rows at least to ask; clusters of 16 only for the largest instances, of
-    // which few fill the GPU.  Threads: as many as an SM holds (clusters of 16: for two CTAs an SM, or not all of eight
-    // clusters find room at once), one to so many timestamps (RANGE looks through an eighth of them).
-    const int most = (long long)n * R >= (1 << 22) ? CELL_CLUSTER : 8;
-    const long long per_sm_ctas = objective == ZL_OBJ_RANGE ? 1 : 2;      // (SUM n=1024, R=1024, B=64: 236 us with one, 206 with two)
+    // CTAs: as many as there are SMs, each with ten rows at least to ask.  More than eight only for the largest instances, of which
+    // few fill the GPU: as many as find room at once for every instance with an SM to each CTA (there is for 7 clusters of 16 and for 11
+    // of 10; n=4096, R=4096, B=8 161 us with 10, 187 with 16 CTAs of half the size).
     s.cluster = 1;
-    while (s.cluster < most && (long long)B * s.cluster * 2 <= per_sm_ctas * num_sms && n / (s.cluster * 2) >= 16) s.cluster *= 2;
+    while (s.cluster < 8 && (long long)B * s.cluster * 2 <= num_sms && n / (s.cluster * 2) >= 10) s.cluster *= 2;
+    if ((long long)n * R >= (1 << 22) && n >= 16 * CELL_CLUSTER && s.cluster == 8 && B <= 11) s.cluster = B <= 7 ? CELL_CLUSTER : 10;
     const long long ctas = (long long)B * s.cluster;
-    s.threads = ctas > 4LL * num_sms ? 128 : ctas > 2LL * num_sms ? 256 : ctas > num_sms || s.cluster > 8 ? 512 : 1024;
-    const int per_thread = 32 * (objective == ZL_OBJ_RANGE ? 48 : 16);
+    const int share = (int)std::max<long long>(1, std::min<long long>(8, (ctas + num_sms - 1) / num_sms));      // CTAs that share an SM
+    // threads: as many as an SM holds, whose registers CTAs get for four warps at a time
+    s.many = objective == ZL_OBJ_RANGE && (share == 3 || (share >= 6 && R < 16));
+    const int fours = (s.many ? CELL_THREADS_MANY : CELL_THREADS) / 128;
+    s.threads = 128 * std::max(1, fours / share);
+    const int per_thread = 32 * (objective == ZL_OBJ_RANGE ? 24 : 8);
     s.threads = (int)std::min<long long>(s.threads, std::max<long long>(128, 32 * (((long long)n * R / s.cluster + per_thread - 1) / per_thread)));
     // Cells an instance can use.  RANGE: RANGE_CELLS to an iteration of the slowest row, of which there are rarely more than
     // half R before the first row runs out.  SUM: see SUM_WIDTH, 6 to 12 sqrt(n) cells an iteration.  No more than lets the
     // CTAs of the call (up to eight an SM) be resident together: they are bound by latency, not by what they move.
     double want = objective == ZL_OBJ_RANGE ? RANGE_CELLS * 0.5 * R : 12.0 * R * std::sqrt((double)n);
     want = std::max(256.0, std::min(want, (double)(1 << 18)));
-    const long long per_sm = s.cluster > 8 ? 2 : std::max<long long>(1, std::min<long long>(8, (ctas + num_sms - 1) / num_sms));
+    const long long per_sm = std::max<long long>(1, std::min<long long>(objective == ZL_OBJ_RANGE ? 8 : CELL_THREADS / 128, (ctas + num_sms - 1) / num_sms));
     const double cell_bytes = objective == ZL_OBJ_RANGE ? 4.0 : 4.125;
-    const double room = (std::min(200.0, 224.0 / (double)per_sm) * 1024 - sizeof(CellShared) - 1024 - 8.0 * n - 64) / cell_bytes;
+    const size_t answers = (std::max((s.cluster > 1 ? 3 : 1) * sizeof(Answers), sizeof(RowList)) + 15) & ~(size_t)15;
+    const double room = (std::min(200.0, 224.0 / (double)per_sm) * 1024 - sizeof(CellShared) - 1024 - 8.0 * n - 64 - (double)answers) / cell_bytes;
     const int most_cells = std::max(2048, (int)room & ~127);
     s.cap = std::min(most_cells, ((int)(want / s.cluster) + 127) & ~127);
     s.cap = std::max(256, s.cap);
-    s.smem = (size_t)s.cap * 4 + 16 + (size_t)n * 8 + (objective == ZL_OBJ_RANGE ? 0 : (size_t)s.cap / 8);
+    s.smem = (size_t)s.cap * 4 + 16 + (size_t)n * 8 + (objective == ZL_OBJ_RANGE ? 0 : (size_t)s.cap / 8) + answers;
     return s;
 }
 
@@ -1000,7 +1377,11 @@ static void enqueue_cells_t(const Pipeline &q, const FilterBufs &fb, const Launc
         cfg.attrs = attr; cfg.numAttrs = cluster > 1 ? 2 : 1;
         cudaLaunchKernelEx(&cfg, kernel, args...);
     };
-    if (q.cells != 3) launch(k_cells<OBJ, SRC>, dim3(s.cluster, q.B), s.threads, s.smem, s.cluster, src, P);
+    if (q.cells != 3) {
+        auto kernel = k_cells<OBJ, SRC, CELL_THREADS>;
+        if constexpr (OBJ == ZL_OBJ_RANGE) if (s.many) kernel = k_cells<OBJ, SRC, CELL_THREADS_MANY>;
+        launch(kernel, dim3(s.cluster, q.B), s.threads, s.smem, s.cluster, src, P);
+    }
     if (ev) for (int k = 1; k < 4; ++k) cudaEventRecord(ev[k], st);
     if (q.cells == 2) return;                                     // the caller looks at the flags itself
     SweepParams sp;
@@ -1026,8 +1407,12 @@ void enqueue_cells(const Pipeline &q, const FilterBufs &fb, const LaunchPlan &p,
 template <int OBJ, class SRC>
 static cudaError_t cell_limits_t() {
     const int big = 200 * 1024;
-    cudaError_t e = cudaFuncSetAttribute(k_cells<OBJ, SRC>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_cells<OBJ, SRC>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    auto raise = [&](auto kernel) {
+        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
+        return e == cudaSuccess ? cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) : e;
+    };
+    cudaError_t e = raise(k_cells<OBJ, SRC, CELL_THREADS>);
+    if constexpr (OBJ == ZL_OBJ_RANGE) if (e == cudaSuccess) e = raise(k_cells<OBJ, SRC, CELL_THREADS_MANY>);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_cell_rest<OBJ, SRC>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
     return e;
 }

@@ -1,0 +1,63 @@
+"""The cell route's ways of reading rows and of passing answers on, at the sizes where they can go wrong, against the CPU oracle.
+Whole numbers: every comparison is exact."""
+import numpy as np
+import pytest
+import torch
+
+import oracle as o
+import zl_inputs as zi
+
+pytestmark = pytest.mark.gpu
+
+if torch.cuda.is_available():
+    import paper_2001_01347_b200 as zl
+
+
+def check(ts, objective, offset=0, instances=None):
+    """The cell route on rows that start `offset` timestamps behind a 32-byte boundary, with nothing allocated behind them."""
+    B, n, R = ts.shape
+    flat = torch.empty(offset + ts.size, dtype=torch.int64, device="cuda")
+    d = flat[offset:].view(B, n, R)
+    d.copy_(torch.from_numpy(ts))
+    h = zl.ZipLine(n, R, B, objective, 0)
+    h.set_option("cells", 1)
+    sel = h.select_batched(d)
+    torch.cuda.synchronize()
+    for b in range(B) if instances is None else instances:
+        w, t, idx = o.sweep_window(ts[b], objective)
+        assert (int(sel.status[b]), int(sel.wait[b]), int(sel.barrier[b])) == (0, w, t), b
+        assert (sel.idx[b].cpu().numpy() == idx).all(), b
+    h.destroy()
+
+
+@pytest.mark.parametrize("objective", [0, 1])
+@pytest.mark.parametrize("offset", [0, 1, 2, 3])
+@pytest.mark.parametrize("n,R,B", [(4, 1, 1), (4, 2, 1), (5, 3, 2), (7, 9, 1), (8, 8, 3), (33, 31, 2), (100, 150, 1)])
+def test_pieces_at_the_ends_of_the_matrix(n, R, B, offset, objective):
+    # eight elements on a 32-byte boundary may begin before the first row or end behind the last one
+    check(zi.generate(zi.CONFIGS["c4"].with_(B=B, n=n, R=R)), objective, offset)
+
+
+@pytest.mark.parametrize("objective", [0, 1])
+@pytest.mark.parametrize("n,R,B", [(1023, 40, 2), (1024, 40, 2), (1025, 40, 2), (2049, 33, 1), (1024, 8200, 1), (300, 14000, 8), (200, 100, 400), (64, 12, 1000)])
+def test_lists_of_rows_and_shapes_of_clusters(n, R, B, objective):
+    # one list of 1024 rows and more than one, counts of pieces beyond 20 bits, clusters of 16 and 10, three CTAs an SM, many of short rows
+    check(zi.generate(zi.CONFIGS["c4"].with_(B=B, n=n, R=R)), objective, 1, range(0, B, max(1, B // 3)))
+
+
+@pytest.mark.parametrize("objective", [0, 1])
+@pytest.mark.parametrize("share", [0.02, 0.2])
+def test_rows_far_off_their_estimates(share, objective):
+    # bursts: rows are read on to either side of what was estimated, one cell holds many elements of a row
+    rng = np.random.default_rng(3)
+    inc = np.where(rng.random((3, 200, 600)) < share, rng.integers(1, 100_000, (3, 200, 600)), rng.integers(1, 50, (3, 200, 600)))
+    check(np.cumsum(inc, axis=2).astype(np.int64), objective)
+
+
+@pytest.mark.parametrize("objective", [0, 1])
+@pytest.mark.parametrize("fast", [1, 20, 45])
+def test_more_answers_from_one_cta_than_its_share(fast, objective):
+    # the first CTA of the cluster has the fast workers, whose elements by the dozen lie in one run of cells
+    rng = np.random.default_rng(fast)
+    m = np.where(np.arange(160) < fast, 1000, 100_000)[None, :, None]
+    check(np.cumsum((m * (1 + 0.05 * rng.standard_normal((2, 160, 400)))).astype(np.int64), axis=2), objective)
