@@ -55,10 +55,10 @@ constexpr long long CELL_ASK = 4;         // asking a row for a cell costs about
 constexpr int CELL_ROUNDS = 4;            // rounds after the first in which more cells may be left than there is room for (regular rows need one or two, SUM
                                           // up to four; with 48, rows of equal periods, n=64, R=128, took 0.5 ms before they were given up)
 constexpr int CELL_HOPELESS = 2 * CELL_ALIVE;    // ... and so many are never worth a further round
-// Cells evaluated, and eight for every round, beyond which the handle's next calls leave the route: regular rows, over 300 random shapes, need up
-// to 33 (RANGE) and 87 (SUM); where many cells tie the other routes are the faster ones (RANGE, times rounded to half a mean iteration, n=93, R=211,
-// B=64 494 us / 99).
-constexpr int CELL_ASKED_RANGE = 48, CELL_ASKED_SUM = 112;
+// Runs of cells evaluated, eight for every round and one to sixteen answers (SUM 64), beyond which the handle's next calls leave the route:
+// regular rows need up to 50 (RANGE; predicted rows of a common kind, n=20, R=185, B=1356) and 87 (SUM); where many cells tie the other routes are the
+// faster ones (RANGE, times rounded to half a mean iteration, n=93, R=211, B=64 494 us / 99).
+constexpr int CELL_ASKED_RANGE = 72, CELL_ASKED_SUM = 112;
 constexpr int CELL_IDLE = 32;             // elements of a row in one cell that cannot matter, from which on the row is taken to stand still (one timestamp
                                           // everywhere, n=1024, R=1024, B=8 511 us / 58 on the filter route: one thread goes through them)
 constexpr float CELL_OFF = 64.f;          // RANGE: elements by which a row's middle is off its estimate, root mean square, from which on the rows are far from
@@ -347,26 +347,45 @@ __device__ __noinline__ int first_at_or_after(const RD rd, int row, int R, uint3
 }
 
 // Whether one of `rows` consecutive rows decreases somewhere: their elements one after the other, whatever rows they belong
-// to, 256 a warp and step.  (A warp a row: the next row's loads wait for this one's, n=93, R=211 5.6 us.)
+// to, 512 a warp and step with four 32-byte loads a lane under way.  (A warp a row: the next row's loads wait for this one's, n=93,
+// R=211 5.6 us; eight 8-byte loads a lane: n=1111, R=1072, B=44 134 us.)
 static __device__ bool rows_unsorted(const int64_t *ts, int rows, int R) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const long long N = (long long)rows * R;
+    const long long N = (long long)rows * R;                      // (n * R is below 2^31)
     bool bad = false;
+    // up to the first 32-byte boundary and behind the last whole 512 (or, rows shorter than eight, all): an element a thread
+    const int head = R < 8 ? (int)N : (int)min((long long)((4u - (unsigned)((uintptr_t)ts >> 3)) & 3u), N);
+    const int steps = (int)((N - head) >> 9);
+    for (long long f = threadIdx.x; f < N; f += blockDim.x) {
+        const long long end = head + 512ll * steps;
+        if (f >= head && f < end) {                               // (the steps' own)
+            f += (end - f) / blockDim.x * blockDim.x;
+            if (f < end) continue;
+            if (f >= N) break;
+        }
+        bad |= (uint32_t)f % (uint32_t)R != 0u && ldg64(ts + f) < ldg64(ts + f - 1);
+    }
 #pragma unroll 1
-    for (long long f0 = 256ll * warp; f0 < N; f0 += 256ll * nw) {
-        int64_t v[8], before = 0;
+    for (int k = warp; k < steps; k += nw) {
+        const int f0 = head + 512 * k;
+        int64_t v[2][8], before = 0;
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int64_t *p = ts + f0 + 256 * u + 8 * lane;
+            asm volatile("ld.global.nc.v4.u64 {%0, %1, %2, %3}, [%4];" : "=l"(v[u][0]), "=l"(v[u][1]), "=l"(v[u][2]), "=l"(v[u][3]) : "l"(p));
+            asm volatile("ld.global.nc.v4.u64 {%0, %1, %2, %3}, [%4];" : "=l"(v[u][4]), "=l"(v[u][5]), "=l"(v[u][6]), "=l"(v[u][7]) : "l"(p + 4));
+        }
         if (lane == 0 && f0 > 0) before = ldg64(ts + f0 - 1);
 #pragma unroll
-        for (int k = 0; k < 8; ++k) { const long long f = f0 + 32 * k + lane; v[k] = f < N ? ldg64(ts + f) : INT64_MAX; }
-        int c = (int)((uint32_t)(f0 + lane) % (uint32_t)R);       // the column (n * R is below 2^31)
+        for (int u = 0; u < 2; ++u) {
+            int64_t up = (int64_t)shfl_up((uint64_t)v[u][7], 1);
+            if (lane == 0) up = before;
+            before = (int64_t)shfl_idx((uint64_t)v[u][7], 31);
+            // which of the eight starts a row, and so follows nothing
+            const int c = (int)((uint32_t)(f0 + 256 * u + 8 * lane) % (uint32_t)R), first = c == 0 ? 0 : R - c;
+            bad |= first != 0 && v[u][0] < up;
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            int64_t p = (int64_t)shfl_up((uint64_t)v[k], 1);
-            if (lane == 0) p = before;
-            bad |= c != 0 && v[k] < p;
-            before = (int64_t)shfl_idx((uint64_t)v[k], 31);
-            c += 32;
-            while (c >= R) c -= R;
+            for (int j = 1; j < 8; ++j) bad |= first != j && v[u][j] < v[u][j - 1];
         }
     }
     return bad;
@@ -378,6 +397,7 @@ struct CellParams {
     int cap;                         // cells a CTA has room for (a multiple of 128)
     int rpc;                         // rows of a CTA when rows are asked
     int check_sorted;                // every row is read once to see that it does not decrease
+    int near;                        // the rows are in this GPU's memory (across the bus every timestamp read in vain costs more than reading on)
     InstMeta *meta;
     uint32_t epoch;                  // number of the call: a word of `flags` is raised when it holds this
     uint32_t *flags;                 // [1] some instance needs the segment sweep, [2] some instance's outputs are missing,
@@ -900,7 +920,7 @@ __global__ void __launch_bounds__(MT, 1) k_cells(const SRC src, const CellParams
             if (tid == 0) {
                 if (dev * sqrtf((float)R) > 2.f * CELL_OFF) sh.slow = 1;      // (dev * sqrt(R) / 2 elements in the middle)
                 sh.span = span;
-                sh.slack = CELL_SLACK + (int)min(32.f, 0.5f * dev * sqrtf((float)R));
+                sh.slack = CELL_SLACK + (P.near ? (int)min(32.f, 0.5f * dev * sqrtf((float)R)) : 0);
                 // gaps that are shorter than the smallest d that is to be expected hardly matter
                 sh.gap = at < GUARD_BINS && top - at > EXPECTED_BINS ? (uint32_t)(__int_as_float((top - at - EXPECTED_BINS) << 20) / (float)max(R - 1, 1)) : 0u;
                 sh.width = R > 1 ? (float)longest / ((float)(R - 1) * RANGE_CELLS) : 0.f;
@@ -1147,7 +1167,8 @@ __global__ void __launch_bounds__(MT, 1) k_cells(const SRC src, const CellParams
                 // ---- the cells that may still hold a smaller one, or the same one earlier: only cells before the best one's
                 const uint64_t limit = d < INF32 ? d << 24 | (cb + 1u) : ~0ull;      // RANGE: the best one's key, as of a cell whose bound is attained
                 auto keep = [&](uint32_t c, uint64_t base, uint64_t l) {
-                    if (done(c)) return;
+                    // (far too many already: how many more does not matter, and every CTA has been told of the same ones)
+                    if (*(volatile unsigned int *)&sh.ncells > (unsigned)CELL_HOPELESS || done(c)) return;
                     // every CTA gets the list
 #pragma unroll 1
                     for (int r = 0; r < G; ++r) {
@@ -1327,14 +1348,18 @@ struct CellShape { int cluster, threads, cap; bool many; size_t smem; };
 
 static CellShape cell_shape(int n, int R, int B, int objective, int num_sms) {
     CellShape s;
-    // CTAs: as many as there are SMs, each with ten rows at least to ask.  More than eight only for the largest instances, of which
+    // CTAs: as many as there are SMs, each with ten rows and a thousand timestamps at least (n=23, R=63, B=8 17 us
+    // with one CTA an instance, 21 with two).  More than eight only for the largest instances, of which
     // few fill the GPU: as many as find room at once for every instance with an SM to each CTA (there is for 7 clusters of 16 and for 11
     // of 10; n=4096, R=4096, B=8 161 us with 10, 187 with 16 CTAs of half the size).
     s.cluster = 1;
-    while (s.cluster < 8 && (long long)B * s.cluster * 2 <= num_sms && n / (s.cluster * 2) >= 10) s.cluster *= 2;
+    while (s.cluster < 8 && (long long)B * s.cluster * 2 <= num_sms && n / (s.cluster * 2) >= 10 && (long long)n * R >= 1024ll * 2 * s.cluster) s.cluster *= 2;
     if ((long long)n * R >= (1 << 22) && n >= 16 * CELL_CLUSTER && s.cluster == 8 && B <= 11) s.cluster = B <= 7 ? CELL_CLUSTER : 10;
     const long long ctas = (long long)B * s.cluster;
-    const int share = (int)std::max<long long>(1, std::min<long long>(8, (ctas + num_sms - 1) / num_sms));      // CTAs that share an SM
+    // CTAs that share an SM.  Clusters do not fill the GPU to the last SM: with an SM to each CTA there is room for 33 of 4 and 15 of 8
+    // (n=1286, R=136, B=16 46 us for two turns of clusters of 8, 32 with a cluster's CTAs two to an SM).
+    const int sms = s.cluster <= 2 || s.cluster > 8 ? num_sms : s.cluster == 4 ? num_sms * 9 / 10 : num_sms * 13 / 16;
+    const int share = (int)std::max<long long>(1, std::min<long long>(8, (ctas + sms - 1) / sms));
     // threads: as many as an SM holds, whose registers CTAs get for four warps at a time
     s.many = objective == ZL_OBJ_RANGE && (share == 3 || (share >= 6 && R < 16));
     const int fours = (s.many ? CELL_THREADS_MANY : CELL_THREADS) / 128;
@@ -1363,6 +1388,7 @@ static void enqueue_cells_t(const Pipeline &q, const FilterBufs &fb, const Launc
     CellParams P;
     P.n = q.n; P.R = q.R; P.B = q.B;
     P.cap = s.cap; P.rpc = (q.n + s.cluster - 1) / s.cluster; P.check_sorted = (q.flags & ZL_FLAG_CHECK_SORTED) ? 1 : 0;
+    P.near = q.cells != 2;
     P.meta = q.meta; P.flags = q.cflags; P.epoch = q.epoch;
     P.idx = q.idx; P.barrier = q.barrier; P.wait = q.wait; P.status = q.status;
     auto launch = [&](auto kernel, dim3 grid, int threads, size_t smem, int cluster, auto... args) {
