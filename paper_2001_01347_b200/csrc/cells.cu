@@ -6,11 +6,11 @@
 //   RANGE  The best Z whose minimum is at time t has max(Z) = G(t) = max over the rows of their first element at or after t,
 //          so d = G(T) - T, and every candidate of a cell has d >= G(start) - end.  G is set by the rows with long
 //          iterations: the slowest fifth to half of the rows ("guards": an eighth of the timestamps or so) give a lower bound of G
-//          at every cell's start - a maximum per cell, then a prefix maximum.  The cells with the smallest bounds are
-//          evaluated exactly (every row is asked for its elements in them: a search from the row's ends, a few loads); the
-//          smallest d discards nearly all other cells, and the ones it does not are evaluated the same way, most promising
-//          first.  Where the guards leave too many, the other rows are looked through for gaps longer than d: only those can
-//          discard a further cell.
+//          at every cell's start - a maximum per cell, then a prefix maximum; gaps much shorter than the smallest d that is to
+//          be expected are passed over.  The cells with the smallest bounds are evaluated exactly (every row is asked for
+//          its elements in them: eight elements where the row's ends suggest); the smallest d discards nearly all other cells,
+//          and the ones it does not are evaluated the same way, runs of neighbours together, most promising first.  Where the
+//          guards leave too many, the other rows are looked through for gaps longer than d: only those can discard a further cell.
 //   SUM    wait(T) = n T - S(T), S = sum of the workers' latest elements.  A sum of deltas per cell and a prefix sum give S
 //          at every cell's start, so every candidate of a cell has wait >= n start - S(end) and the cell's last element
 //          attains at most n end - S(end).  Cells whose lower bound exceeds a wait that is attained are discarded; the few
@@ -22,6 +22,10 @@
 // rows that count there), a share of the rows when rows are asked, and no global scratch.  k_cell_rest runs behind it: the
 // segment sweep for the instances it left over (spans of 2^32 or more, more surviving cells or elements than there is room
 // for) and the outputs of instances in error; it returns at once when there are none.
+//
+// What bounds it: a call of one instance, the chain of some dozen dependent steps (0.5 to 2 us each); many instances, the
+// instructions and latencies of looking through rows (2000 cycles for 32 pieces of eight elements with 20 warps an SM, n=1024,
+// R=1024, B=64 16 of 37 us in the kernel), not what it moves (2.8 TB/s there).
 //
 // Every CTA of a cluster passes the same cluster barriers: whatever a loop or a branch around one depends on is the same
 // value in the whole cluster (never the CTA's own number of rows or cells).
@@ -39,7 +43,7 @@ constexpr uint32_t INF32 = 0xffffffffu;
 constexpr int CELL_ALIVE = 128;           // most cells of an instance that the bounds may leave
 constexpr int CELL_BATCH = 16;            // most cells that the rows are asked for at once
 constexpr int CELL_NODES = 1024;          // most elements in those
-constexpr int CELL_PAIRS = 256;            // answers that a batch of cells should give, from what the last ones gave
+constexpr int CELL_PAIRS = 256;           // answers that a batch of cells should give, from what the last ones gave
 constexpr int CELL_CLUSTER = 16;          // most CTAs of a cluster
 // Most threads of a CTA, and so registers a thread: 96, or (RANGE) 80 where three CTAs share an SM or rows are very short and many do
 // (n=200, R=100, B=400 36 us with 80, 44 with 96; n=809, R=8, B=865 59 / 71; but n=1024, R=1024, B=64 48 / 44, n=128, R=256, B=1024 49 / 46).  With
@@ -67,7 +71,8 @@ constexpr float CELL_OFF = 64.f;          // RANGE: elements by which a row's mi
                                           // fivefold, R=256 and 43 off, n=128, B=256 65 / 284)
 constexpr int CELL_FEW = 8;               // so many cells are asked for in any case
 constexpr int CELL_SLACK = 4;             // elements by which a row may be off its estimate before it is read on, at least
-constexpr int EXPECTED_BINS = 2;
+constexpr int EXPECTED_BINS = 2;          // RANGE: bins below the d to be expected from which on gaps are passed over (n=1024, R=1024, B=64 44.5 us, 46.2 when none
+                                          // are, 43.8 with 0, but then n=1000, R=150, B=1 29 instead of 21: more cells are left)
 constexpr int GUARD_BINS = 64;            // rows by their span, eight bins to a factor of two below the longest
 constexpr float GUARD_IRREGULAR = 32.f;   // bins by which more rows are looked through, to a unit of their gaps' relative deviation above 0.1
 constexpr float RANGE_CELLS = 100.f;      // RANGE: cells to the longest mean iteration
@@ -219,11 +224,12 @@ __device__ __forceinline__ void list_rows(RowList &L, ListFill &fill, bool packe
 
 // The CTA looks through the listed rows: the pieces are dealt out evenly to its warps, each a run of them, a piece a lane.
 // (Rows dealt out instead, 32 to a warp, leave the warps with the most guards twice as long at it as the others: n=1024, R=1024,
-// B=64 14 to 25 us for this pass.)  While one is worked on, the lane's next is on its way to the L2.  Where the estimate of a row's pieces falls short on either side its first or last piece leaves a
-// bit, and all such rows are read on by the whole CTA at the end (one access after the other by the lane itself, with its
-// warp waiting, takes half as long again where single gaps are long).  act(T) gets nine consecutive times, eight pairs of
-// neighbours: every pair with one of its elements in the range, and the pair that straddles a, comes exactly once; others
-// may come.
+// B=64 14 to 25 us for this pass.  A run of pieces a thread scatters the loads: n=4096, R=4096, B=8 327 us a call instead of 161.)  While one
+// is worked on, the lane's next is on its way to the L2.  Where the estimate of a row's pieces falls short on either side its
+// first or last piece leaves a bit, and all such rows are read on by the whole CTA at the end (one access after the other by
+// the lane itself, with its warp waiting, takes half as long again where single gaps are long).  act(T) gets nine consecutive
+// times, eight pairs of neighbours: every pair with one of its elements in the range, and the pair that straddles a, comes
+// exactly once; others may come.
 template <class RD, class ACT>
 __device__ __forceinline__ void stream_list(const RowList &L, uint32_t (*more)[LIST_ROWS / 32], int rows, uint32_t pieces, const RD &rd, int R, uint32_t a, uint32_t b, ACT act) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -996,8 +1002,9 @@ __global__ void __launch_bounds__(MT, 1) k_cells(const SRC src, const CellParams
         const uint32_t c0 = min((uint32_t)rank * per, ncells), c1 = min(c0 + per, ncells);
         sh.shift = shift; sh.c0 = c0; sh.m = c1 - c0;
         sh.a = lo + (c0 << shift); sh.bnd = c1 == ncells ? hi : lo + (c1 << shift);
-        // cells asked for at first: the most promising one of every CTA, as far as the answers cost the warps no second turn
-        sh.firsts = max(1, min(min(CELL_FIRST, G), nw / ((P.rpc + 31) >> 5)));
+        // cells asked for at first: the most promising one of every CTA, as far as the answers cost the warps no second turn (one only
+        // across the bus: n=274, R=1062, B=8 from the host 226 us with four, 212 with one)
+        sh.firsts = P.near ? max(1, min(min(CELL_FIRST, G), nw / ((P.rpc + 31) >> 5))) : 1;
         // with a few cells on either side of it: SUM so many as give about a dozen answers
         sh.around = OBJ == ZL_OBJ_RANGE ? 1 : (int)max(2u, min(8u, (uint32_t)(8ull * ncells / ((unsigned long long)n * R))));
         sh.bd = ~0ull; sh.bt = INF32; sh.ndone = 0; sh.asked = 0; sh.took = 0;
@@ -1351,7 +1358,7 @@ static CellShape cell_shape(int n, int R, int B, int objective, int num_sms) {
     // CTAs: as many as there are SMs, each with ten rows and a thousand timestamps at least (n=23, R=63, B=8 17 us
     // with one CTA an instance, 21 with two).  More than eight only for the largest instances, of which
     // few fill the GPU: as many as find room at once for every instance with an SM to each CTA (there is for 7 clusters of 16 and for 11
-    // of 10; n=4096, R=4096, B=8 161 us with 10, 187 with 16 CTAs of half the size).
+    // of 10; n=4096, R=4096, B=8 149 us with 10, 187 with 16 CTAs of half the size).
     s.cluster = 1;
     while (s.cluster < 8 && (long long)B * s.cluster * 2 <= num_sms && n / (s.cluster * 2) >= 10 && (long long)n * R >= 1024ll * 2 * s.cluster) s.cluster *= 2;
     if ((long long)n * R >= (1 << 22) && n >= 16 * CELL_CLUSTER && s.cluster == 8 && B <= 11) s.cluster = B <= 7 ? CELL_CLUSTER : 10;
@@ -1368,10 +1375,11 @@ static CellShape cell_shape(int n, int R, int B, int objective, int num_sms) {
     s.threads = (int)std::min<long long>(s.threads, std::max<long long>(128, 32 * (((long long)n * R / s.cluster + per_thread - 1) / per_thread)));
     // Cells an instance can use.  RANGE: RANGE_CELLS to an iteration of the slowest row, of which there are rarely more than
     // half R before the first row runs out.  SUM: see SUM_WIDTH, 6 to 12 sqrt(n) cells an iteration.  No more than lets the
-    // CTAs of the call (up to eight an SM) be resident together: they are bound by latency, not by what they move.
+    // CTAs of the call be resident together (SUM as far as there are registers for; RANGE up to eight an SM: fewer cells are better where
+    // many instances share one, n=128, R=256, B=1024 46 us with 2800 cells, 51 with 4400).
     double want = objective == ZL_OBJ_RANGE ? RANGE_CELLS * 0.5 * R : 12.0 * R * std::sqrt((double)n);
     want = std::max(256.0, std::min(want, (double)(1 << 18)));
-    const long long per_sm = std::max<long long>(1, std::min<long long>(objective == ZL_OBJ_RANGE ? 8 : CELL_THREADS / 128, (ctas + num_sms - 1) / num_sms));
+    const int per_sm = std::min(objective == ZL_OBJ_RANGE ? 8 : CELL_THREADS / 128, share);
     const double cell_bytes = objective == ZL_OBJ_RANGE ? 4.0 : 4.125;
     const size_t answers = (std::max((s.cluster > 1 ? 3 : 1) * sizeof(Answers), sizeof(RowList)) + 15) & ~(size_t)15;
     const double room = (std::min(200.0, 224.0 / (double)per_sm) * 1024 - sizeof(CellShared) - 1024 - 8.0 * n - 64 - (double)answers) / cell_bytes;
