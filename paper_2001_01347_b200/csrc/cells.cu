@@ -831,12 +831,13 @@ __global__ void __launch_bounds__(MT, 1) k_cells(const SRC src, const CellParams
             }
         }
     }
+    auto sync_cluster = [&]() { if (G > 1) cl.sync(); else __syncthreads(); };      // (a cluster barrier of one CTA takes several times as long)
     if constexpr (std::is_same<SRC, MatBatch>::value) if (P.check_sorted) {
         const bool bad = rows_unsorted(src.ts + ((size_t)b * n + r0) * R, nrows, R);
         const int any = __syncthreads_or(bad);
         if (tid < G) cl.map_shared_rank(&sh, tid)->exc[rank] = any ? 1ull : 0ull;
     }
-    cl.sync();
+    sync_cluster();
     int64_t tmin;
     {
     InstMeta M;
@@ -961,7 +962,7 @@ __global__ void __launch_bounds__(MT, 1) k_cells(const SRC src, const CellParams
         if (tid < 64) es[tid] = 0;
         __syncthreads();
         if (tid < G) cl.map_shared_rank(&sh, tid)->exs[rank] = sh.acc;
-        cl.sync();
+        sync_cluster();
         const uint64_t ub = warp_sum64(lane < G ? (uint64_t)sh.exs[min(lane, G - 1)] : 0ull);
         // times past lm at which the exhausted rows alone wait longer than that are left out: the first of 32 trial times
         // where they do (closer together near lm), then the first of 32 more between that one and the one before it
@@ -1130,7 +1131,7 @@ __global__ void __launch_bounds__(MT, 1) k_cells(const SRC src, const CellParams
                 }
             }
         }
-        cl.sync();
+        sync_cluster();
         // ---- the most promising cells: the best one of each CTA, in their order
         int some = 0, listed = 0, from = 0;                       // runs of this evaluation; of the list (0: not made yet), and how many of them were evaluated
         {
@@ -1222,7 +1223,7 @@ __global__ void __launch_bounds__(MT, 1) k_cells(const SRC src, const CellParams
                         }
                     }
                 }
-                cl.sync();
+                sync_cluster();
                 listed = (int)sh.ncells;
                 if (listed == 0) break;
                 if (OBJ == ZL_OBJ_RANGE && stage == 0 && sh.span > 0.f && listed > CELL_ALIVE) {      // the other rows may discard them
