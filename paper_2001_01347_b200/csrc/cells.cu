@@ -1373,7 +1373,10 @@ static CellShape cell_shape(int n, int R, int B, int objective, int num_sms) {
     const int fours = (s.many ? CELL_THREADS_MANY : CELL_THREADS) / 128;
     s.threads = 128 * std::max(1, fours / share);
     const int per_thread = 32 * (objective == ZL_OBJ_RANGE ? 24 : 8);
-    s.threads = (int)std::min<long long>(s.threads, std::max<long long>(128, 32 * (((long long)n * R / s.cluster + per_thread - 1) / per_thread)));
+    // no more than one to so many timestamps, but enough for the passes over the cells where a CTA has an SM to itself (n=24, R=60, B=1 15.2 us
+    // with 128, 14.0 with 256; SUM n=100, R=150, B=1 21.7 with 256, 21.2 with 384)
+    const int least = share > 1 ? 128 : objective == ZL_OBJ_RANGE ? 256 : 384;
+    s.threads = (int)std::min<long long>(s.threads, std::max<long long>(least, 32 * (((long long)n * R / s.cluster + per_thread - 1) / per_thread)));
     // Cells an instance can use.  RANGE: RANGE_CELLS to an iteration of the slowest row, of which there are rarely more than
     // half R before the first row runs out.  SUM: see SUM_WIDTH, 6 to 12 sqrt(n) cells an iteration.  No more than lets the
     // CTAs of the call be resident together (SUM as far as there are registers for; RANGE up to eight an SM: fewer cells are better where
