@@ -259,7 +259,9 @@ __device__ __forceinline__ void stream_list(const RowList &L, uint32_t (*more)[L
         int entry, s;
         unsigned edge;
         assign(p0, entry, s, edge);
-        uint32_t carry = rd.in(L.row[entry], max(s - 1, 0));          // (lane 0) the element before the first of these pieces
+        // (lane 0) the element before the first of these pieces.  The other lanes may have no piece, and their s lies behind the row.
+        uint32_t carry = 0;
+        if (lane == 0) carry = rd.in(L.row[entry], max(s - 1, 0));
 #pragma unroll 1
         for (uint32_t q = p0; q < p1; q += 32u) {
             const uint32_t x = q + lane;
