@@ -42,14 +42,25 @@ namespace zl {
 constexpr uint32_t INF32 = 0xffffffffu;
 constexpr int CELL_ALIVE = 128;           // most cells of an instance that the bounds may leave
 constexpr int CELL_BATCH = 16;            // most cells that the rows are asked for at once
-constexpr int CELL_NODES = 1024;          // most elements in those
 constexpr int CELL_PAIRS = 256;           // answers that a batch of cells should give, from what the last ones gave
 constexpr int CELL_CLUSTER = 16;          // most CTAs of a cluster
-// Most threads of a CTA, and so registers a thread: 96, or (RANGE) 80 where three CTAs share an SM or rows are very short and many do
-// (n=200, R=100, B=400 36 us with 80, 44 with 96; n=809, R=8, B=865 59 / 71; but n=1024, R=1024, B=64 48 / 44, n=128, R=256, B=1024 49 / 46).  With
-// 72 or 64 registers values are spilled inside the loops, and what is spilled has often left the L1 cache, past which the rows
-// stream, by the time it is wanted back: n=1024, R=1024, B=64 55 and 74 us.
-constexpr int CELL_THREADS = 640, CELL_THREADS_MANY = 768;
+// The forms of the kernel.  ONE: an instance has one CTA, and what only clusters need falls away; THREADS: most threads of an SM, and so the
+// registers of a thread; ROWS: rows that are looked through at a time, NODES: most elements in the cells that the rows are asked for at once.
+// With 96 registers (640 threads) nothing is spilled, with 72 8 bytes outside the loops, with 64 72 bytes; a cluster's kernel with 72 or 64
+// spills inside the loops, and what is spilled has often left the L1 cache, past which the rows stream, by the time it is wanted back (n=1024, R=1024,
+// B=64 55 and 74 us, 44 with 96).  CTAs get registers for four warps at a time, so that 96 are good for five small CTAs an SM, 72 for seven: a thousand
+// instances are one turn instead of 1.4 (n=128, R=256, B=1024 53 us with 96, 40 with 72; n=181, R=18, B=1795 60 / 54; predicted n=131, R=41,
+// B=1760 44 / 37).  Three CTAs of 256 threads fit with 80 (n=350, R=157, B=373 53 us with 96 and 128 threads, 44 with 80), four with 64 (n=400, R=100,
+// B=480 48 us with 96 and 128 threads, 43 with 64; n=22, R=537, B=565 54 / 49; but instances of 128 threads' work: n=30, R=60, B=580 28 / 31).
+// With lists half as long (ROWS, NODES) there is room for 1400 cells more where seven CTAs share an SM.
+template <bool ONE_, int THREADS_, int ROWS_, int NODES_>
+struct CellForm { static constexpr bool ONE = ONE_; static constexpr int THREADS = THREADS_, ROWS = ROWS_, NODES = NODES_, CTAS = ONE_ ? 1 : CELL_CLUSTER; };
+typedef CellForm<false, 640, 1024, 1024> CellCluster;
+typedef CellForm<true, 640, 1024, 1024> CellAlone;        // up to two CTAs an SM, and SUM
+typedef CellForm<true, 768, 512, 512> CellThree;          // RANGE: three an SM,
+typedef CellForm<true, 1024, 512, 512> CellFour;          // four, or eight,
+typedef CellForm<true, 640, 512, 512> CellFive;           // four of 128 threads, or five,
+typedef CellForm<true, 896, 512, 512> CellSeven;          // six or seven (or eight)
 constexpr int CELL_FIRST = 4;             // most runs of cells that a round asks for at first
 // Cells next to one another are asked for as one: the eight elements that a row is looked at for hold what it has in several cells as well.
 // RUN: most cells of a run (a power of two); two cells of the list belong to one if there are at most RUN / 2 others between them.
@@ -173,11 +184,12 @@ __device__ __forceinline__ float warp_sum(float x) {              // the same va
 // ------------------------------------------------------------------------------ looking through rows
 // The rows that have elements in the time range [a, b) of interest, and the pieces of eight elements that each of them needs:
 // a row's pieces are sb + 8 q with q from excl up to the next row's.  In shared memory, a batch of rows at a time.
-constexpr int LIST_ROWS = 1024;
+template <int ROWS_>
 struct RowList {
-    uint32_t excl[LIST_ROWS];
-    int sb[LIST_ROWS];
-    unsigned short row[LIST_ROWS];
+    static constexpr int ROWS = ROWS_;
+    uint32_t excl[ROWS];
+    int sb[ROWS];
+    unsigned short row[ROWS];
 };
 
 // A row (a lane; `have`: it counts) goes to the list.  Which pieces it needs is estimated from its ends, `slack` elements more on
@@ -185,9 +197,9 @@ struct RowList {
 // into 20 of them (64-bit atomics on shared memory are loops).  The warp's lanes call together.
 struct ListFill { uint32_t packed; unsigned long long wide; };
 constexpr int LIST_BITS = 20;
-__device__ __forceinline__ bool list_packed(int n, int R) { return (long long)min(n, LIST_ROWS) * (R / 8 + 3) < (1 << LIST_BITS); }
-template <class RD>
-__device__ __forceinline__ void list_rows(RowList &L, ListFill &fill, bool packed, const RD &rd, int R, int row, bool have, uint32_t e0, uint32_t eR,
+__device__ __forceinline__ bool list_packed(int rows, int R) { return (long long)rows * (R / 8 + 3) < (1 << LIST_BITS); }
+template <class LIST, class RD>
+__device__ __forceinline__ void list_rows(LIST &L, ListFill &fill, bool packed, const RD &rd, int R, int row, bool have, uint32_t e0, uint32_t eR,
                                           uint32_t a, uint32_t b, int slack) {
     const int lane = threadIdx.x & 31;
     const unsigned who = __ballot_sync(FULL, have);
@@ -230,8 +242,8 @@ __device__ __forceinline__ void list_rows(RowList &L, ListFill &fill, bool packe
 // the lane itself, with its warp waiting, takes half as long again where single gaps are long).  act(T) gets nine consecutive
 // times, eight pairs of neighbours: every pair with one of its elements in the range, and the pair that straddles a, comes
 // exactly once; others may come.
-template <class RD, class ACT>
-__device__ __forceinline__ void stream_list(const RowList &L, uint32_t (*more)[LIST_ROWS / 32], int rows, uint32_t pieces, const RD &rd, int R, uint32_t a, uint32_t b, ACT act) {
+template <class LIST, class RD, class ACT>
+__device__ __forceinline__ void stream_list(const LIST &L, uint32_t (*more)[LIST::ROWS / 32], int rows, uint32_t pieces, const RD &rd, int R, uint32_t a, uint32_t b, ACT act) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const uint32_t share = (pieces + nw - 1) / nw, p0 = min(share * warp, pieces), p1 = min(p0 + share, pieces);
     if (p0 < p1) {
@@ -242,7 +254,7 @@ __device__ __forceinline__ void stream_list(const RowList &L, uint32_t (*more)[L
             const unsigned m = __ballot_sync(FULL, lane * per < rows && L.excl[min(lane * per, rows - 1)] <= p0);
             j0 = (__popc(m) - 1) * per;
             const unsigned k = __ballot_sync(FULL, lane < per && j0 + lane < rows && L.excl[min(j0 + lane, rows - 1)] <= p0);
-            j0 += __popc(k) - 1;                                      // LIST_ROWS <= 32 * 32
+            j0 += __popc(k) - 1;                                      // LIST::ROWS <= 32 * 32
         }
         // piece q + lane: its entry of the list, its first element, whether it is its row's first (1) or last (2) one
         auto assign = [&](uint32_t q, int &entry, int &s, unsigned &edge) {
@@ -269,8 +281,8 @@ __device__ __forceinline__ void stream_list(const RowList &L, uint32_t (*more)[L
             const int row = L.row[entry];
             uint64_t v[8];
             if (mine) rd.load(row, s, v);
-            int nentry, ns;
-            unsigned nedge;
+            int nentry = 0, ns = 0;
+            unsigned nedge = 0;
             if (q + 32u < p1) {                                       // the next piece on its way to the L2 while this one is worked on
                 assign(q + 32u, nentry, ns, nedge);
                 if (x + 32u < p1) rd.prefetch(L.row[nentry], ns);
@@ -291,8 +303,8 @@ __device__ __forceinline__ void stream_list(const RowList &L, uint32_t (*more)[L
     }
     __syncthreads();
 #pragma unroll 1
-    for (int i = threadIdx.x; i < 2 * LIST_ROWS; i += blockDim.x) {
-        const int right = i >= LIST_ROWS ? 1 : 0, j = i & (LIST_ROWS - 1);
+    for (int i = threadIdx.x; i < 2 * LIST::ROWS; i += blockDim.x) {
+        const int right = i >= LIST::ROWS ? 1 : 0, j = i & (LIST::ROWS - 1);
         if (j < rows && (more[right][j >> 5] >> (j & 31) & 1u)) {
             const int row = L.row[j];
             int s = (int)((uint32_t)L.sb[j] + 8u * (right ? (j + 1 < rows ? L.excl[j + 1] : pieces) - 1u : L.excl[j]));
@@ -415,21 +427,24 @@ struct CellParams {
 
 // What the rows answer when they are asked for cells.  A cluster has three of them: what the own rows answered, and what arrived from
 // every CTA (its share of the room each), twice, used in turn: the next answers may arrive while these are worked on.
+template <int NODES>
 struct Answers {
-    uint64_t node[CELL_NODES];                    // the elements in the cells: time << 32 | RANGE the row's next element, SUM the element less the row's previous one
-    unsigned char slot[CELL_NODES];               // ... which of the cells
+    uint64_t node[NODES];                         // the elements in the cells: time << 32 | RANGE the row's next element, SUM the element less the row's previous one
+    unsigned char slot[NODES];                    // ... which of the cells
 };
 
+template <int OBJ, class FORM>
 struct CellShared {
+    typedef typename std::conditional<OBJ == ZL_OBJ_RANGE, uint32_t, unsigned long long>::type Sum;      // RANGE: a time, SUM: a sum of times
     // from every CTA of the cluster (each array is written by the others before one cluster barrier and read after it, so no
     // two exchanges share one): minima and maxima of its rows' ends; whether one of its rows decreases; SUM its rows' wait at
     // the sample time; the key of its best cell, and G or S at its start
-    unsigned long long ex[4][CELL_CLUSTER];
-    float exi[CELL_CLUSTER];                      // RANGE: how irregular its rows are (sum over a few of them, see k_cells)
-    unsigned long long exc[CELL_CLUSTER], exs[CELL_CLUSTER], exv[CELL_CLUSTER], exb[CELL_CLUSTER];
+    unsigned long long ex[4][FORM::CTAS];
+    float exi[FORM::CTAS];                      // RANGE: how irregular its rows are (sum over a few of them, see k_cells)
+    unsigned long long exc[FORM::CTAS], exs[FORM::CTAS], exv[FORM::CTAS], exb[FORM::CTAS];
     unsigned long long red[4][32], keys[32], kbases[32];
     // of Answers: how many from every CTA; RANGE latest and earliest of the rows' first elements at or after the cell's start
-    struct { uint32_t gmax[CELL_BATCH], gmin[CELL_BATCH]; uint32_t count[CELL_CLUSTER]; } heard[2];
+    struct { uint32_t gmax[CELL_BATCH], gmin[CELL_BATCH]; uint32_t count[FORM::CTAS]; } heard[FORM::ONE ? 1 : 2];
     uint32_t gmax[CELL_BATCH], gmin[CELL_BATCH];  // ... of the own rows'
     unsigned int nnodes;
     ListFill fill;
@@ -440,10 +455,10 @@ struct CellShared {
     uint32_t cell[CELL_ALIVE];
     union {
         struct {
-            uint64_t base[CELL_ALIVE];            // RANGE: a lower bound of G at the cell's start, SUM: S there
-            uint64_t lb[CELL_ALIVE];              // lower bound of the objective in the cell
+            Sum base[CELL_ALIVE];                 // RANGE: a lower bound of G at the cell's start, SUM: S there
+            Sum lb[CELL_ALIVE];                   // lower bound of the objective in the cell
         };
-        uint32_t more[2][LIST_ROWS / 32];         // (while rows are looked through: which of them have to be read on, to the left, to the right)
+        uint32_t more[2][FORM::ROWS / 32];         // (while rows are looked through: which of them have to be read on, to the left, to the right)
     };
     unsigned short order[CELL_ALIVE];
     unsigned int ncells;
@@ -453,16 +468,16 @@ struct CellShared {
     uint2 asked_run[CELL_FIRST * (CELL_ROUNDS + 2)];      // first and last cell of the runs evaluated before the list was made
     // the list's runs, in the order of their first cells: first and last cell, G or S at the start, smallest lower bound
     uint2 run[CELL_ALIVE];
-    uint64_t run_base[CELL_ALIVE];
-    unsigned long long run_lb[CELL_ALIVE];
-    uint32_t exf[CELL_CLUSTER];                   // (exchanged with exv, exb) first cell of the run around the most promising one
+    Sum run_base[CELL_ALIVE];
+    unsigned long long run_lb[CELL_ALIVE];        // (64 bits in any case: with 32 the compiler spills twenty registers where it has 72)
+    uint32_t exf[FORM::CTAS];                   // (exchanged with exv, exb) first cell of the run around the most promising one
     int runs;
     uint64_t bestd[32]; uint32_t bestt[32];
     // what is the same in all threads and needed now and then: shared memory, not a register each (the compiler spills some sixty of
     // them otherwise, and what is spilled has often left the L1 cache by the time it is wanted back: n=1024, R=1024, B=64 72 us)
     int64_t tmin;
     uint64_t ub, bd;                              // SUM: a wait that is attained; the smallest objective so far and its time
-    uint32_t bt, t0, lmin, tend, lo, hi, shift, c0, m, a, bnd, gap, expected, took, longest;
+    uint32_t bt, t0, lmin, tend, lo, hi, shift, c0, m, a, bnd, gap, took;
     float span, width;                            // RANGE: rows of at least this span are guards; what a cell may span
     int slack, firsts, around, ndone, asked, per_cell;
     unsigned int slow;                            // (in every CTA) rows far from arithmetic, or standing still
@@ -481,6 +496,11 @@ __device__ __noinline__ bool was_asked(const uint2 *runs, int n, uint32_t c) {
     return is;
 }
 
+// The same variable in CTA `rank` of the cluster.  (ONE: the instance has one CTA.)
+template <bool ONE, class T> __device__ __forceinline__ T *map_shared_rank(T *x, int rank) {
+    if constexpr (ONE) return x; else return cg::this_cluster().map_shared_rank(x, rank);
+}
+
 struct Best { uint64_t d; uint32_t t; };          // smallest objective and its time, the first of equal ones; the same in every thread of the cluster
 __device__ __forceinline__ Best warp_best(uint64_t d, uint32_t t) {
     const uint64_t m = warp_min64(d);
@@ -489,23 +509,25 @@ __device__ __forceinline__ Best warp_best(uint64_t d, uint32_t t) {
 
 // The exact minimum over the `ns` cells of sh.ca, sh.ce, sh.cb (in every CTA of the cluster the same): every CTA asks its rows
 // and sends what they answer to all CTAs, and behind one cluster barrier every CTA (with a few dozen answers every
-// warp, without a further barrier) evaluates all of it.  Every thread of the cluster calls.  Returns the number of answers: more than CELL_NODES,
+// warp, without a further barrier) evaluates all of it.  Every thread of the cluster calls.  Returns the number of answers: more than FORM::NODES,
 // and there was no room for them.
 //
 // A (cell, row) pair a lane, a warp on one cell: eight elements around the place that the row's ends suggest are loaded, then,
 // by how far off they were, eight others, until they hold the first element at or after the cell's start and all that
 // follow in it.  (Searched for the first element, then asked for its successor and the next ones: three to five accesses one
 // after the other, n=1024, R=1024, B=64 7 us, eight cells of SUM 17 us.)
-template <int OBJ, class SRC>
-__device__ __forceinline__ int evaluate_cells(CellShared &sh, Answers *answers, const uint2 *ends, const SRC &src, int B, int n, int R, int rpc, int turn, int ns) {
+template <int OBJ, class SRC, class FORM>
+__device__ __forceinline__ int evaluate_cells(CellShared<OBJ, FORM> &sh, Answers<FORM::NODES> *answers, const uint2 *ends, const SRC &src, int B, int n, int R, int rpc, int turn, int ns) {
     cg::cluster_group cl = cg::this_cluster();
-    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5, G = gridDim.x;
-    const int r0 = min((int)blockIdx.x * rpc, n), nrows = min(rpc, n - r0);
+    constexpr bool ONE = FORM::ONE;
+    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5, G = ONE ? 1 : gridDim.x;
+    const int r0 = ONE ? 0 : min((int)blockIdx.x * rpc, n), nrows = ONE ? n : min(rpc, n - r0);
     const RowReader<SRC> rd(src, blockIdx.y, B, n, R, sh.tmin);
-    Answers *an = answers;
+    typedef Answers<FORM::NODES> Ans;
+    Ans *an = answers;
     auto put = [&](int k, uint32_t T, uint32_t pay) {
         const unsigned pos = atomicAdd(&sh.nnodes, 1u);
-        if (pos < CELL_NODES) { an->node[pos] = (uint64_t)T << 32 | pay; an->slot[pos] = (unsigned char)k; }
+        if (pos < FORM::NODES) { an->node[pos] = (uint64_t)T << 32 | pay; an->slot[pos] = (unsigned char)k; }
     };
     const int chunks = (rpc + 31) >> 5, items = ns * chunks;
 #pragma unroll 1
@@ -574,15 +596,15 @@ __device__ __forceinline__ int evaluate_cells(CellShared &sh, Answers *answers, 
     uint64_t mine_x = 0;
     const uint32_t *gmax = sh.gmax, *gmin = sh.gmin;
     if (G > 1) {
-        const int rank = blockIdx.x, room = CELL_NODES / G, sent = min(m, room);
+        const int rank = blockIdx.x, room = FORM::NODES / G, sent = min(m, room);
         auto &heard = sh.heard[turn];
-        Answers *in = answers + 1 + turn;
+        Ans *in = answers + 1 + turn;
         gmax = heard.gmax; gmin = heard.gmin;
 #pragma unroll 1
         for (int r = warp; r < G; r += nw) {                      // to CTA r
-            Answers *to = cl.map_shared_rank(in, r);
+            Ans *to = map_shared_rank<ONE>(in, r);
             for (int i = lane; i < sent; i += 32) { to->node[rank * room + i] = an->node[i]; to->slot[rank * room + i] = an->slot[i]; }
-            auto *h = cl.map_shared_rank(&heard, r);
+            auto *h = map_shared_rank<ONE>(&heard, r);
             if (lane == 0) h->count[rank] = (uint32_t)m;
             if (OBJ == ZL_OBJ_RANGE && lane < ns) { atomicMax(&h->gmax[lane], sh.gmax[lane]); atomicMin(&h->gmin[lane], sh.gmin[lane]); }
         }
@@ -599,12 +621,12 @@ __device__ __forceinline__ int evaluate_cells(CellShared &sh, Answers *answers, 
 #pragma unroll 1
             for (int r = 0; r + 1 < G; ++r) { const int p = __shfl_sync(FULL, incl, r); if (lane >= p) at = (r + 1) * room + lane - p; }
             if (lane < m) { mine_x = in->node[at]; mine_k = in->slot[at]; }
-        } else if (m <= CELL_NODES) {
-            Answers *to = over ? in : an;
+        } else if (m <= FORM::NODES) {
+            Ans *to = over ? in : an;
 #pragma unroll 1
             for (int r = warp; r < G; r += nw) {
                 const int count = __shfl_sync(FULL, c, r), at = __shfl_sync(FULL, incl, r) - count;
-                const Answers *from = over ? cl.map_shared_rank(an, r) : in;
+                const Ans *from = over ? map_shared_rank<ONE>(an, r) : in;
                 const int first = over ? 0 : r * room;
                 for (int i = lane; i < count; i += 32) { to->node[at + i] = from->node[first + i]; to->slot[at + i] = from->slot[first + i]; }
             }
@@ -616,7 +638,7 @@ __device__ __forceinline__ int evaluate_cells(CellShared &sh, Answers *answers, 
     }
     uint64_t d = sh.bd;
     uint32_t t = sh.bt;
-    if (OBJ == ZL_OBJ_RANGE && m <= CELL_NODES && lane < ns && gmax[lane] != INF32 && gmin[lane] < sh.hi) {
+    if (OBJ == ZL_OBJ_RANGE && m <= FORM::NODES && lane < ns && gmax[lane] != INF32 && gmin[lane] < sh.hi) {
         // the first element at or after the cell's start, wherever it is
         const uint64_t w = (uint64_t)(gmax[lane] - gmin[lane]);
         if (w < d || (w == d && gmin[lane] < t)) { d = w; t = gmin[lane]; }
@@ -638,7 +660,7 @@ __device__ __forceinline__ int evaluate_cells(CellShared &sh, Answers *answers, 
         }
         const uint64_t w = OBJ == ZL_OBJ_SUM ? (uint64_t)n * T - v : v >= INF32 ? ~0ull : v - T;
         if (counts && w != ~0ull && (w < d || (w == d && T < t))) { d = w; t = T; }
-    } else if (m <= CELL_NODES) {
+    } else if (m <= FORM::NODES) {
 #pragma unroll 1
         for (int i = tid; i < m; i += nt) {
             const uint64_t x = an->node[i];
@@ -658,33 +680,33 @@ __device__ __forceinline__ int evaluate_cells(CellShared &sh, Answers *answers, 
         }
     }
     Best best = warp_best(d, t);
-    if (!few && m <= CELL_NODES) {
+    if (!few && m <= FORM::NODES) {
         if (lane == 0) { sh.bestd[warp] = best.d; sh.bestt[warp] = best.t; }
         __syncthreads();
         best = warp_best(lane < nw ? sh.bestd[lane] : ~0ull, lane < nw ? sh.bestt[lane] : INF32);
     }
     __syncthreads();                                              // everybody has read the answers
     if (tid == 0) { sh.nnodes = 0; sh.bd = best.d; sh.bt = best.t; sh.per_cell = max(1, m / ns); sh.asked += m / (OBJ == ZL_OBJ_RANGE ? 16 : 64); }
-    if (tid < CELL_BATCH) { sh.gmax[tid] = sh.heard[turn].gmax[tid] = 0; sh.gmin[tid] = sh.heard[turn].gmin[tid] = INF32; }
+    if (tid < CELL_BATCH) { const int u = ONE ? 0 : turn; sh.gmax[tid] = sh.heard[u].gmax[tid] = 0; sh.gmin[tid] = sh.heard[u].gmin[tid] = INF32; }
     __syncthreads();
     return m;
 }
 
 // The elements of the slice's rows into its cells: RANGE of the guards (stage 0) or of the other rows (stage 1), SUM of all rows.
-template <int OBJ, class SRC>
-__device__ __forceinline__ void look_through(CellShared &sh, uint32_t *cell, Answers *answers, const uint2 *ends, const SRC &src, int B, int n, int R, int stage) {
+template <int OBJ, class SRC, class FORM>
+__device__ __forceinline__ void look_through(CellShared<OBJ, FORM> &sh, uint32_t *cell, Answers<FORM::NODES> *answers, const uint2 *ends, const SRC &src, int B, int n, int R, int stage) {
     const RowReader<SRC> rd(src, blockIdx.y, B, n, R, sh.tmin);
     const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
     const uint32_t a = sh.a, bnd = sh.bnd, shift = sh.shift, gap = sh.gap, m = sh.m, w = bnd - a;
     uint64_t carry = 0, total = 0;                        // SUM: the rows' last elements before a, and all deltas in the slice
-    RowList &list = *reinterpret_cast<RowList *>(answers);
-    const bool packed = list_packed(n, R);
+    RowList<FORM::ROWS> &list = *reinterpret_cast<RowList<FORM::ROWS> *>(answers);
+    const bool packed = list_packed(min(n, FORM::ROWS), R);
 #pragma unroll 1
-    for (int from = 0; from < n && m > 0; from += LIST_ROWS) {
+    for (int from = 0; from < n && m > 0; from += FORM::ROWS) {
         if (from > 0) __syncthreads();
-        if (tid < LIST_ROWS / 32) sh.more[0][tid] = sh.more[1][tid] = 0;
+        if (tid < FORM::ROWS / 32) sh.more[0][tid] = sh.more[1][tid] = 0;
 #pragma unroll 1
-        for (int g = warp; 32 * g < min(LIST_ROWS, n - from); g += nw) {
+        for (int g = warp; 32 * g < min(FORM::ROWS, n - from); g += nw) {
             const int row = from + 32 * g + lane;
             uint2 e = make_uint2(0u, 0u);
             bool have = row < n;
@@ -752,18 +774,20 @@ __device__ __forceinline__ void look_through(CellShared &sh, uint32_t *cell, Ans
 // Dynamic shared memory: the slice's cells [cap + 4] u32 | rows' first and last element, relative [n] uint2 | SUM: per 128
 // cells the scan before them and the smallest lower bound among them [cap / 128] two u64 | one Answers (three in a cluster),
 // over which the list of rows to look through lies.
-template <int OBJ, class SRC, int MT>
-__global__ void __launch_bounds__(MT, 1) k_cells(const SRC src, const CellParams P) {
+template <int OBJ, class SRC, class FORM>
+__global__ void __launch_bounds__(FORM::THREADS, 1) k_cells(const SRC src, const CellParams P) {
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ CellShared sh;
+    __shared__ CellShared<OBJ, FORM> sh;
+    constexpr bool ONE = FORM::ONE;
+    typedef typename CellShared<OBJ, FORM>::Sum Sum;
     cg::cluster_group cl = cg::this_cluster();
-    const int b = blockIdx.y, rank = blockIdx.x, G = gridDim.x;
+    const int b = blockIdx.y, rank = ONE ? 0 : blockIdx.x, G = ONE ? 1 : gridDim.x;
     const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
     const int n = P.n, R = P.R;
     uint32_t *cell = (uint32_t *)smem;
     uint2 *ends = (uint2 *)(cell + P.cap + 4);
     uint64_t *blk_before = (uint64_t *)(ends + n), *blk_lb = blk_before + P.cap / 128;
-    Answers *answers = (Answers *)(OBJ == ZL_OBJ_SUM ? blk_lb + P.cap / 128 : blk_before);
+    Answers<FORM::NODES> *answers = (Answers<FORM::NODES> *)(OBJ == ZL_OBJ_SUM ? blk_lb + P.cap / 128 : blk_before);
     // A CTA's shared memory may be written by the others only once it runs: everybody says so here, and waits for the rest
     // with the columns read, before the first store into another CTA.
     if (G > 1) cl.barrier_arrive();
@@ -772,12 +796,12 @@ __global__ void __launch_bounds__(MT, 1) k_cells(const SRC src, const CellParams
     for (int c = tid; c <= P.cap / 4; c += nt) reinterpret_cast<uint4 *>(cell)[c] = make_uint4(0, 0, 0, 0);
     if (tid == 0) { sh.acc = 0; sh.total = 0; sh.ncells = 0; sh.later = 0; sh.slow = 0; sh.gap = 0; sh.nnodes = 0; sh.fill.packed = 0; sh.fill.wide = 0; }
     if (tid < CELL_BATCH) {
-        sh.gmax[tid] = sh.heard[0].gmax[tid] = sh.heard[1].gmax[tid] = 0;
-        sh.gmin[tid] = sh.heard[0].gmin[tid] = sh.heard[1].gmin[tid] = INF32;
+        sh.gmax[tid] = sh.heard[0].gmax[tid] = sh.heard[ONE ? 0 : 1].gmax[tid] = 0;
+        sh.gmin[tid] = sh.heard[0].gmin[tid] = sh.heard[ONE ? 0 : 1].gmin[tid] = INF32;
     }
     for (int k = tid; k < GUARD_BINS; k += nt) sh.hist[k] = 0;
     grid_dep_wait();
-    const int r0 = min(rank * P.rpc, n), nrows = min(P.rpc, n - r0);
+    const int r0 = ONE ? 0 : min(rank * P.rpc, n), nrows = ONE ? n : min(P.rpc, n - r0);
     if (b == 0 && rank == 0 && tid < 2) P.flags[4 + tid] = 0;      // (used by the last kernel only)
     // ---- columns of the own rows; everybody gets everybody's minima and maxima and the low words of the rows' ends
     {
@@ -816,7 +840,7 @@ __global__ void __launch_bounds__(MT, 1) k_cells(const SRC src, const CellParams
 #pragma unroll 1
             for (int r = 0; r < G; ++r) {
                 if (r == rank) continue;
-                uint2 *to = cl.map_shared_rank(ends, r);
+                uint2 *to = map_shared_rank<ONE>(ends, r);
 #pragma unroll 1
                 for (int p = tid; p < nrows; p += nt) to[r0 + p] = ends[r0 + p];
             }
@@ -826,10 +850,10 @@ __global__ void __launch_bounds__(MT, 1) k_cells(const SRC src, const CellParams
             if (k < 4) {
                 uint64_t v = lane < nw ? sh.red[k][lane] : (k & 1) ? 0ull : ~0ull;
                 v = (k & 1) ? warp_max64(v) : warp_min64(v);
-                if (lane < G) cl.map_shared_rank(&sh, lane)->ex[k][rank] = v;
+                if (lane < G) map_shared_rank<ONE>(&sh, lane)->ex[k][rank] = v;
             } else {
                 const float v = warp_sum(lane < nw ? __uint_as_float((uint32_t)sh.keys[lane]) : 0.f);
-                if (lane < G) cl.map_shared_rank(&sh, lane)->exi[rank] = v;
+                if (lane < G) map_shared_rank<ONE>(&sh, lane)->exi[rank] = v;
             }
         }
     }
@@ -837,7 +861,7 @@ __global__ void __launch_bounds__(MT, 1) k_cells(const SRC src, const CellParams
     if constexpr (std::is_same<SRC, MatBatch>::value) if (P.check_sorted) {
         const bool bad = rows_unsorted(src.ts + ((size_t)b * n + r0) * R, nrows, R);
         const int any = __syncthreads_or(bad);
-        if (tid < G) cl.map_shared_rank(&sh, tid)->exc[rank] = any ? 1ull : 0ull;
+        if (tid < G) map_shared_rank<ONE>(&sh, tid)->exc[rank] = any ? 1ull : 0ull;
     }
     sync_cluster();
     int64_t tmin;
@@ -963,7 +987,7 @@ __global__ void __launch_bounds__(MT, 1) k_cells(const SRC src, const CellParams
         unsigned long long *es = (unsigned long long *)answers;   // (64 words, not in use yet)
         if (tid < 64) es[tid] = 0;
         __syncthreads();
-        if (tid < G) cl.map_shared_rank(&sh, tid)->exs[rank] = sh.acc;
+        if (tid < G) map_shared_rank<ONE>(&sh, tid)->exs[rank] = sh.acc;
         sync_cluster();
         const uint64_t ub = warp_sum64(lane < G ? (uint64_t)sh.exs[min(lane, G - 1)] : 0ull);
         // times past lm at which the exhausted rows alone wait longer than that are left out: the first of 32 trial times
@@ -1020,7 +1044,7 @@ __global__ void __launch_bounds__(MT, 1) k_cells(const SRC src, const CellParams
 #pragma unroll 1
     for (int round = 0;; ++round) {                               // a round: the most promising cells are evaluated, the rest counted
         // ---- the rows' elements in the slice
-        if (streamed != stage) look_through<OBJ>(sh, cell, answers, ends, src, P.B, n, R, stage);
+        if (streamed != stage) look_through<OBJ, SRC, FORM>(sh, cell, answers, ends, src, P.B, n, R, stage);
         streamed = stage;
         // ---- what the sweep knows at every cell's start; a warp takes a run of 128-cell blocks, four cells a lane
         const int bpw = (nblk + nw - 1) / nw, k0 = min(warp * bpw, nblk), k1 = min(k0 + bpw, nblk);
@@ -1126,7 +1150,7 @@ __global__ void __launch_bounds__(MT, 1) k_cells(const SRC src, const CellParams
                     else base -= warp_sum64(lane < c - from ? (uint64_t)cell[min(from + lane, c)] : 0ull);
                 }
                 if (lane < G) {
-                    CellShared &to = *cl.map_shared_rank(&sh, lane);
+                    auto &to = *map_shared_rank<ONE>(&sh, lane);
                     to.exv[rank] = fits ? k : 0ull;
                     to.exb[rank] = base;
                     to.exf[rank] = first;
@@ -1168,7 +1192,7 @@ __global__ void __launch_bounds__(MT, 1) k_cells(const SRC src, const CellParams
             // ---- exactly
             __syncthreads();
             if (tid == 0) { if (listed == 0) { sh.ndone += some; sh.asked += 8; } else sh.asked += some; }
-            fits = evaluate_cells<OBJ>(sh, answers, ends, src, P.B, n, R, P.rpc, evaluated & 1, some) <= CELL_NODES;
+            fits = evaluate_cells<OBJ, SRC, FORM>(sh, answers, ends, src, P.B, n, R, P.rpc, evaluated & 1, some) <= FORM::NODES;
             ++evaluated;
             if (!fits) break;
             const uint64_t d = sh.bd;
@@ -1176,13 +1200,13 @@ __global__ void __launch_bounds__(MT, 1) k_cells(const SRC src, const CellParams
             if (listed == 0) {
                 // ---- the cells that may still hold a smaller one, or the same one earlier: only cells before the best one's
                 const uint64_t limit = d < INF32 ? d << 24 | (cb + 1u) : ~0ull;      // RANGE: the best one's key, as of a cell whose bound is attained
-                auto keep = [&](uint32_t c, uint64_t base, uint64_t l) {
+                auto keep = [&](uint32_t c, Sum base, Sum l) {
                     // (far too many already: how many more does not matter, and every CTA has been told of the same ones)
                     if (*(volatile unsigned int *)&sh.ncells > (unsigned)CELL_HOPELESS || done(c)) return;
                     // every CTA gets the list
 #pragma unroll 1
                     for (int r = 0; r < G; ++r) {
-                        CellShared &to = *cl.map_shared_rank(&sh, r);
+                        auto &to = *map_shared_rank<ONE>(&sh, r);
                         const unsigned pos = atomicAdd(&to.ncells, 1u);
                         if (pos < CELL_ALIVE) { to.cell[pos] = c; to.base[pos] = base; to.lb[pos] = l; }
                     }
@@ -1203,7 +1227,7 @@ __global__ void __launch_bounds__(MT, 1) k_cells(const SRC src, const CellParams
                         for (; in; in &= in - 1u) {
                             const int j = __ffs(in) - 1;
                             const uint32_t x = j == 0 ? v.x : j == 1 ? v.y : j == 2 ? v.z : v.w, end = cell_end(a + ((uint32_t)(c + j) << shift), shift, bnd);
-                            keep(c0 + (uint32_t)(c + j), x, x > end ? (uint64_t)(x - end) : 0ull);
+                            keep(c0 + (uint32_t)(c + j), x, x > end ? x - end : 0u);
                         }
                     }
                 } else {
@@ -1220,7 +1244,7 @@ __global__ void __launch_bounds__(MT, 1) k_cells(const SRC src, const CellParams
                         for (int j = 0; j < 4; ++j) {
                             const uint32_t c = (uint32_t)(128 * k + 4 * lane + j), x = cell[c];
                             const uint64_t st = (uint64_t)n * (a + (c << shift)), l = st > S + x ? st - S - x : 0ull;
-                            if (x != 0u && (l < d || (l == d && c0 + c < cb))) keep(c0 + c, S, l);
+                            if (x != 0u && (l < d || (l == d && c0 + c < cb))) keep(c0 + c, (Sum)S, (Sum)l);
                             S += x;
                         }
                     }
@@ -1354,7 +1378,27 @@ __global__ void __launch_bounds__(CELL_REST_THREADS) k_cell_rest(const SRC src, 
 
 // ------------------------------------------------------------------------------ host side
 // CTAs of an instance's cluster, their threads, and the cells each has room for.
-struct CellShape { int cluster, threads, cap; bool many; size_t smem; };
+enum CellFormOf { FORM_CLUSTER, FORM_ALONE, FORM_THREE, FORM_FOUR, FORM_FIVE, FORM_SEVEN };
+struct CellShape { int cluster, threads, form, cap; size_t smem; };
+
+// What a form takes of an SM: most threads, shared memory that the kernel declares, and (`dynamic`) what lies behind the cells.
+struct CellRoom { int threads; size_t fixed, dynamic; };
+template <int OBJ, class FORM>
+static CellRoom cell_room_t() {
+    const size_t d = std::max((FORM::ONE ? 1 : 3) * sizeof(Answers<FORM::NODES>), sizeof(RowList<FORM::ROWS>));
+    return CellRoom{FORM::THREADS, sizeof(CellShared<OBJ, FORM>), (d + 15) & ~(size_t)15};
+}
+static CellRoom cell_room(int objective, int form) {
+    if (objective != ZL_OBJ_RANGE) return form == FORM_CLUSTER ? cell_room_t<ZL_OBJ_SUM, CellCluster>() : cell_room_t<ZL_OBJ_SUM, CellAlone>();
+    switch (form) {
+        case FORM_CLUSTER: return cell_room_t<ZL_OBJ_RANGE, CellCluster>();
+        case FORM_THREE: return cell_room_t<ZL_OBJ_RANGE, CellThree>();
+        case FORM_FOUR: return cell_room_t<ZL_OBJ_RANGE, CellFour>();
+        case FORM_FIVE: return cell_room_t<ZL_OBJ_RANGE, CellFive>();
+        case FORM_SEVEN: return cell_room_t<ZL_OBJ_RANGE, CellSeven>();
+        default: return cell_room_t<ZL_OBJ_RANGE, CellAlone>();
+    }
+}
 
 static CellShape cell_shape(int n, int R, int B, int objective, int num_sms) {
     CellShape s;
@@ -1370,10 +1414,26 @@ static CellShape cell_shape(int n, int R, int B, int objective, int num_sms) {
     // (n=1286, R=136, B=16 46 us for two turns of clusters of 8, 32 with a cluster's CTAs two to an SM).
     const int sms = s.cluster <= 2 || s.cluster > 8 ? num_sms : s.cluster == 4 ? num_sms * 9 / 10 : num_sms * 13 / 16;
     const int share = (int)std::max<long long>(1, std::min<long long>(8, (ctas + sms - 1) / sms));
+    const bool crowded = objective == ZL_OBJ_RANGE && share >= 3;
+    auto cells_in = [&](int form, double kb) {                     // cells that leave room for the CTAs that share an SM in so much shared memory
+        const CellRoom r = cell_room(objective, form);
+        const double left = std::min(200.0, kb / std::min(r.threads / 128, share)) * 1024 - (double)r.fixed - 1024 - 8.0 * n - 64 - (double)r.dynamic;
+        return std::max(2048, (int)(left / (objective == ZL_OBJ_RANGE ? 4.0 : 4.125)) & ~127);
+    };
+    // RANGE: the cells that two groups of equal workers need, of all the rows the most: about n / 6 an iteration of the slow ones (n=83, R=109, B=1177 58 us with
+    // 19 to each of R, 38 with 35; n=128, R=150, B=1024 74 with 16, 43 with 24; n=325, R=66, B=1366 93 with 44, 124 with 31); others do with less, but single instances of few workers (n=28, R=302,
+    // B=2129 95 us with 11, 440 with 9, where lists overflow).
+    const double need = R * std::min(0.5 * RANGE_CELLS, 6.0 + n / 6.0), least_cells = (n < 48 ? 1.2 : 0.7) * need;
+    // The form.  Eight CTAs an SM instead of seven where that saves a turn (n=124, R=20, B=1109 27 us with eight, 31 with seven; n=300, R=60, B=1150 53 /
+    // 62; but B=1363, two turns of either, n=62, R=93 55 / 53; n=565, R=34, B=1180 163 / 118), with as many cells; large instances that take
+    // several turns five of them, with more cells and no spills (n=74, R=200, B=1354 with long single gaps 63 / 70; n=117, R=338, B=1476 with stragglers 66 / 74, n=560, R=31, B=3431 215 / 231;
+    // but one turn of seven, n=128, R=256, B=1024 50 / 37).
+    auto turns = [&](int per_sm) { return (ctas + per_sm * num_sms - 1) / (per_sm * num_sms); };
+    const long long N = (long long)n * R;
+    s.form = s.cluster > 1 ? FORM_CLUSTER : !crowded ? FORM_ALONE : share == 3 ? FORM_THREE : share == 4 && N > 128 * 24 ? FORM_FOUR : share < 6 ? FORM_FIVE
+             : turns(8) < turns(7) && n <= 384 && cells_in(FORM_FOUR, 196.0) >= least_cells ? FORM_FOUR : N >= 12288 && turns(7) > 1 ? FORM_FIVE : FORM_SEVEN;
     // threads: as many as an SM holds, whose registers CTAs get for four warps at a time
-    s.many = objective == ZL_OBJ_RANGE && (share == 3 || (share >= 6 && R < 16));
-    const int fours = (s.many ? CELL_THREADS_MANY : CELL_THREADS) / 128;
-    s.threads = 128 * std::max(1, fours / share);
+    s.threads = 128 * std::max(1, cell_room(objective, s.form).threads / 128 / share);
     const int per_thread = 32 * (objective == ZL_OBJ_RANGE ? 24 : 8);
     // no more than one to so many timestamps, but enough for the passes over the cells where a CTA has an SM to itself (n=24, R=60, B=1 15.2 us
     // with 128, 14.0 with 256; SUM n=100, R=150, B=1 21.7 with 256, 21.2 with 384)
@@ -1381,18 +1441,20 @@ static CellShape cell_shape(int n, int R, int B, int objective, int num_sms) {
     s.threads = (int)std::min<long long>(s.threads, std::max<long long>(least, 32 * (((long long)n * R / s.cluster + per_thread - 1) / per_thread)));
     // Cells an instance can use.  RANGE: RANGE_CELLS to an iteration of the slowest row, of which there are rarely more than
     // half R before the first row runs out.  SUM: see SUM_WIDTH, 6 to 12 sqrt(n) cells an iteration.  No more than lets the
-    // CTAs of the call be resident together (SUM as far as there are registers for; RANGE up to eight an SM: fewer cells are better where
-    // many instances share one, n=128, R=256, B=1024 46 us with 2800 cells, 51 with 4400).
+    // CTAs of the call be resident together, as far as there are registers for them.
+    // RANGE, where three CTAs and more share an SM: cells that are not needed cost more than the passes over them, because what shared memory
+    // takes is gone from the L1 cache, past which the rows stream (n=218, R=213, B=700 78 us with 228 KB an SM in use, 61 with 196, 73
+    // again when the cells are as few but the memory is asked for all the same).  So 164 KB where that holds the cells (n=50, R=165, B=1313 with
+    // long single gaps 58 us, 65 with 196; not few workers: n=33, R=301, B=599 45 us with 164, 36 with 196), or 196, or 228 (predicted n=27, R=591, B=760 225
+    // us with 196, 56 with 228).  Few workers, whose bounds are less alike, never need 50 to each of R (n=27, R=151, B=398 33 us, 31 with 19).
     double want = objective == ZL_OBJ_RANGE ? RANGE_CELLS * 0.5 * R : 12.0 * R * std::sqrt((double)n);
+    if (crowded) want = std::min(want, R * (20.0 + n / 4.0));
     want = std::max(256.0, std::min(want, (double)(1 << 18)));
-    const int per_sm = std::min(objective == ZL_OBJ_RANGE ? 8 : CELL_THREADS / 128, share);
-    const double cell_bytes = objective == ZL_OBJ_RANGE ? 4.0 : 4.125;
-    const size_t answers = (std::max((s.cluster > 1 ? 3 : 1) * sizeof(Answers), sizeof(RowList)) + 15) & ~(size_t)15;
-    const double room = (std::min(200.0, 224.0 / (double)per_sm) * 1024 - sizeof(CellShared) - 1024 - 8.0 * n - 64 - (double)answers) / cell_bytes;
-    const int most_cells = std::max(2048, (int)room & ~127);
-    s.cap = std::min(most_cells, ((int)(want / s.cluster) + 127) & ~127);
+    double kb = 224.0;
+    if (crowded) kb = n >= 48 && cells_in(s.form, 164.0) >= need ? 164.0 : cells_in(s.form, 196.0) >= least_cells ? 196.0 : n < 48 || cells_in(s.form, 228.0) >= least_cells ? 228.0 : 196.0;
+    s.cap = std::min(cells_in(s.form, kb), ((int)(want / s.cluster) + 127) & ~127);
     s.cap = std::max(256, s.cap);
-    s.smem = (size_t)s.cap * 4 + 16 + (size_t)n * 8 + (objective == ZL_OBJ_RANGE ? 0 : (size_t)s.cap / 8) + answers;
+    s.smem = (size_t)s.cap * 4 + 16 + (size_t)n * 8 + (objective == ZL_OBJ_RANGE ? 0 : (size_t)s.cap / 8) + cell_room(objective, s.form).dynamic;
     return s;
 }
 
@@ -1418,8 +1480,13 @@ static void enqueue_cells_t(const Pipeline &q, const FilterBufs &fb, const Launc
         cudaLaunchKernelEx(&cfg, kernel, args...);
     };
     if (q.cells != 3) {
-        auto kernel = k_cells<OBJ, SRC, CELL_THREADS>;
-        if constexpr (OBJ == ZL_OBJ_RANGE) if (s.many) kernel = k_cells<OBJ, SRC, CELL_THREADS_MANY>;
+        auto kernel = s.form == FORM_CLUSTER ? k_cells<OBJ, SRC, CellCluster> : k_cells<OBJ, SRC, CellAlone>;
+        if constexpr (OBJ == ZL_OBJ_RANGE) {
+            if (s.form == FORM_THREE) kernel = k_cells<OBJ, SRC, CellThree>;
+            if (s.form == FORM_FOUR) kernel = k_cells<OBJ, SRC, CellFour>;
+            if (s.form == FORM_FIVE) kernel = k_cells<OBJ, SRC, CellFive>;
+            if (s.form == FORM_SEVEN) kernel = k_cells<OBJ, SRC, CellSeven>;
+        }
         launch(kernel, dim3(s.cluster, q.B), s.threads, s.smem, s.cluster, src, P);
     }
     if (ev) for (int k = 1; k < 4; ++k) cudaEventRecord(ev[k], st);
@@ -1451,8 +1518,14 @@ static cudaError_t cell_limits_t() {
         const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
         return e == cudaSuccess ? cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) : e;
     };
-    cudaError_t e = raise(k_cells<OBJ, SRC, CELL_THREADS>);
-    if constexpr (OBJ == ZL_OBJ_RANGE) if (e == cudaSuccess) e = raise(k_cells<OBJ, SRC, CELL_THREADS_MANY>);
+    cudaError_t e = raise(k_cells<OBJ, SRC, CellCluster>);
+    if (e == cudaSuccess) e = raise(k_cells<OBJ, SRC, CellAlone>);
+    if constexpr (OBJ == ZL_OBJ_RANGE) {
+        if (e == cudaSuccess) e = raise(k_cells<OBJ, SRC, CellThree>);
+        if (e == cudaSuccess) e = raise(k_cells<OBJ, SRC, CellFour>);
+        if (e == cudaSuccess) e = raise(k_cells<OBJ, SRC, CellFive>);
+        if (e == cudaSuccess) e = raise(k_cells<OBJ, SRC, CellSeven>);
+    }
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_cell_rest<OBJ, SRC>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
     return e;
 }

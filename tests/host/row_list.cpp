@@ -1,4 +1,4 @@
-// One CTA's reading of rows, as the cell route does it, on the CPU.  ROWS and LOOK are cut out of the kernel's source.
+// One CTA's reading of rows, as the cell route does it, on the CPU.  ROWS_FILE and LOOK_FILE are cut out of the kernel's source.
 #include "warp_on_cpu.h"
 
 enum { ZL_OBJ_RANGE = 0, ZL_OBJ_SUM = 1 };
@@ -8,9 +8,11 @@ static constexpr uint32_t INF32 = 0xffffffffu;
 static inline uint64_t shfl_up(uint64_t v, int d) { return __shfl_up_sync(FULL, v, d); }
 static inline uint64_t shfl_idx(uint64_t v, int i) { return __shfl_sync(FULL, v, i); }
 
-#include ROWS
+#include ROWS_FILE
 
-struct Answers { uint64_t words[2048]; };
+template <int ROWS_> struct Form { static constexpr int ROWS = ROWS_, NODES = 2048; };   // (NODES: room for the list)
+template <int NODES> struct Answers { uint64_t words[NODES]; };
+template <int OBJ, class FORM>
 struct CellShared {
     int64_t tmin;
     uint32_t a, bnd, shift, gap, m, took;
@@ -18,30 +20,34 @@ struct CellShared {
     int slack;
     ListFill fill;
     unsigned long long acc, total;
-    uint32_t more[2][LIST_ROWS / 32];
+    uint32_t more[2][FORM::ROWS / 32];
 };
 
-#include LOOK
+#include LOOK_FILE
 
 static void rows_are(const int64_t *ts, long long elements) { cpu::first = ts; cpu::end = ts + elements; cpu::bad = cpu::worst = 0; }
 static long verdict(int64_t *worst) { *worst = cpu::worst; return cpu::bad; }
 
-// A slice [a, bnd) of instance b in cells of 2^shift: what look_through makes of it with `threads` threads.  Returns the number of
-// loads from outside the matrix.
-extern "C" long look(int objective, const int64_t *ts, int B, int n, int R, int b, int64_t tmin, const uint32_t *ends, uint32_t a, uint32_t bnd, uint32_t shift, uint32_t m,
-                     uint32_t gap, float span, int slack, int stage, int threads, uint32_t *cell, uint64_t *sums, int64_t *worst) {
-    rows_are(ts, (long long)B * n * R);
-    static CellShared sh;
-    static Answers answers[3];
+template <int OBJ, class FORM>
+static void look_t(const MatBatch &src, int B, int n, int R, int64_t tmin, const uint32_t *ends, uint32_t a, uint32_t bnd, uint32_t shift, uint32_t m, uint32_t gap, float span,
+                   int slack, int stage, int threads, uint32_t *cell, uint64_t *sums) {
+    static CellShared<OBJ, FORM> sh;
+    static Answers<FORM::NODES> answers[3];
     memset(&sh, 0, sizeof sh);
     sh.tmin = tmin; sh.a = a; sh.bnd = bnd; sh.shift = shift; sh.gap = gap; sh.m = m; sh.span = span; sh.slack = slack;
-    blockIdx.y = b;
-    const MatBatch src{ts};
-    cpu::run(threads, [&] {
-        if (objective == ZL_OBJ_RANGE) look_through<ZL_OBJ_RANGE>(sh, cell, answers, (const uint2 *)ends, src, B, n, R, stage);
-        else look_through<ZL_OBJ_SUM>(sh, cell, answers, (const uint2 *)ends, src, B, n, R, stage);
-    });
+    cpu::run(threads, [&] { look_through<OBJ, MatBatch, FORM>(sh, cell, answers, (const uint2 *)ends, src, B, n, R, stage); });
     sums[0] = sh.acc; sums[1] = sh.total;
+}
+
+// A slice [a, bnd) of instance b in cells of 2^shift: what look_through makes of it with `threads` threads and lists of `rows` rows.
+// Returns the number of loads from outside the matrix.
+extern "C" long look(int objective, int rows, const int64_t *ts, int B, int n, int R, int b, int64_t tmin, const uint32_t *ends, uint32_t a, uint32_t bnd, uint32_t shift, uint32_t m,
+                     uint32_t gap, float span, int slack, int stage, int threads, uint32_t *cell, uint64_t *sums, int64_t *worst) {
+    rows_are(ts, (long long)B * n * R);
+    blockIdx.y = b;
+    auto *f = objective == ZL_OBJ_RANGE ? rows == 256 ? look_t<ZL_OBJ_RANGE, Form<256>> : rows == 512 ? look_t<ZL_OBJ_RANGE, Form<512>> : look_t<ZL_OBJ_RANGE, Form<1024>>
+                                        : rows == 256 ? look_t<ZL_OBJ_SUM, Form<256>> : rows == 512 ? look_t<ZL_OBJ_SUM, Form<512>> : look_t<ZL_OBJ_SUM, Form<1024>>;
+    f(MatBatch{ts}, B, n, R, tmin, ends, a, bnd, shift, m, gap, span, slack, stage, threads, cell, sums);
     return verdict(worst);
 }
 

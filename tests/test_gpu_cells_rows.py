@@ -61,3 +61,48 @@ def test_more_answers_from_one_cta_than_its_share(fast, objective):
     rng = np.random.default_rng(fast)
     m = np.where(np.arange(160) < fast, 1000, 100_000)[None, :, None]
     check(np.cumsum((m * (1 + 0.05 * rng.standard_normal((2, 160, 400)))).astype(np.int64), axis=2), objective)
+
+
+def on(route, ts, n, R, B, objective):
+    h = zl.ZipLine(n, R, B, objective, 0)
+    for option in route:
+        h.set_option(option, 1)
+    sel = h.select_batched(ts)
+    torch.cuda.synchronize()
+    launches, left = h.launches_per_call, h.filter_counts(B)[2]
+    h.destroy()
+    return sel, launches, left
+
+
+@pytest.mark.parametrize("recipe", ["c3", "c4"])
+@pytest.mark.parametrize("n,R,B", [(90, 60, 400), (40, 30, 500), (90, 60, 500), (90, 60, 700), (90, 60, 900), (90, 60, 1000), (120, 20, 1100),
+                                   (511, 12, 1000), (512, 12, 1000), (513, 12, 1000), (600, 25, 1200), (300, 60, 1150), (30, 600, 760)])
+def test_every_form_of_ctas_that_share_an_sm(n, R, B, recipe):
+    # three to eight CTAs an SM, few and many timestamps for their threads, one list of 512 rows and more than one, few rows
+    # with a long lookahead: every instance as the filter or bucket route has it, some as the oracle does
+    d = torch.from_numpy(zi.generate(zi.CONFIGS[recipe].with_(B=B, n=n, R=R))).cuda()
+    sel, launches, left = on(("cells", "no_walk"), d, n, R, B, 0)
+    assert launches == 2 and max(left) == 0
+    other, launches, _ = on(("no_cells", "no_walk"), d, n, R, B, 0)
+    assert launches != 2
+    for a, b in zip((sel.idx, sel.barrier, sel.wait, sel.status), (other.idx, other.barrier, other.wait, other.status)):
+        assert torch.equal(a, b)
+    for b in range(0, B, B // 4):
+        w, t, idx = o.sweep_window(d[b].cpu().numpy(), 0)
+        assert (int(sel.wait[b]), int(sel.barrier[b])) == (w, t), b
+        assert (sel.idx[b].cpu().numpy() == idx).all(), b
+
+
+def test_more_answers_than_a_crowded_cta_has_room_for():
+    # 200 workers fast enough for a run of cells to hold more than 512 elements: the sweep finishes what the cells leave over
+    n, R, B = 220, 100, 1000
+    rng = np.random.default_rng(4)
+    m = np.where(np.arange(n) < 200, 3_000, 100_000)[None, :, None]
+    ts = np.cumsum((m * (1 + 0.3 * rng.random((4, n, R)))).astype(np.int64), axis=2) + np.where(np.arange(n) < 200, 9_000_000, 0)[None, :, None]
+    d = torch.from_numpy(ts).cuda().repeat(B // 4, 1, 1)
+    sel, launches, _ = on(("cells", "no_walk"), d, n, R, B, 0)
+    assert launches == 2
+    for b in (0, 1, 2, 3, B - 1):
+        w, t, idx = o.sweep_window(ts[b % 4], 0)
+        assert (int(sel.status[b]), int(sel.wait[b]), int(sel.barrier[b])) == (0, w, t), b
+        assert (sel.idx[b].cpu().numpy() == idx).all(), b
