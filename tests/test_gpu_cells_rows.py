@@ -13,16 +13,20 @@ if torch.cuda.is_available():
     import paper_2001_01347_b200 as zl
 
 
-def check(ts, objective, offset=0, instances=None):
-    """The cell route on rows that start `offset` timestamps behind a 32-byte boundary, with nothing allocated behind them."""
+def check(ts, objective, offset=0, instances=None, leaves=0):
+    """The cell route, and nothing else, on rows that start `offset` timestamps behind a 32-byte boundary; `leaves`: instances that may be
+    left to the segment sweep.  (What lies outside the matrix is mapped here; tests/test_cells_rows_on_cpu.py looks at every load.)"""
     B, n, R = ts.shape
     flat = torch.empty(offset + ts.size, dtype=torch.int64, device="cuda")
     d = flat[offset:].view(B, n, R)
     d.copy_(torch.from_numpy(ts))
     h = zl.ZipLine(n, R, B, objective, 0)
     h.set_option("cells", 1)
+    h.set_option("no_walk", 1)
     sel = h.select_batched(d)
     torch.cuda.synchronize()
+    assert h.launches_per_call == 2
+    assert sum(x != 0 for x in h.filter_counts(B)[2]) <= leaves
     for b in range(B) if instances is None else instances:
         w, t, idx = o.sweep_window(ts[b], objective)
         assert (int(sel.status[b]), int(sel.wait[b]), int(sel.barrier[b])) == (0, w, t), b
@@ -39,7 +43,7 @@ def test_pieces_at_the_ends_of_the_matrix(n, R, B, offset, objective):
 
 
 @pytest.mark.parametrize("objective", [0, 1])
-@pytest.mark.parametrize("n,R,B", [(1023, 40, 2), (1024, 40, 2), (1025, 40, 2), (2049, 33, 1), (1024, 8200, 1), (300, 14000, 8), (200, 100, 400), (64, 12, 1000)])
+@pytest.mark.parametrize("n,R,B", [(1023, 40, 2), (1024, 40, 2), (1025, 40, 2), (2049, 33, 1), (1024, 8200, 1), (300, 14000, 8), (200, 100, 400), (64, 12, 1000), (300, 12, 1000)])
 def test_lists_of_rows_and_shapes_of_clusters(n, R, B, objective):
     # one list of 1024 rows and more than one, counts of pieces beyond 20 bits, clusters of 16 and 10, three CTAs an SM, many of short rows
     check(zi.generate(zi.CONFIGS["c4"].with_(B=B, n=n, R=R)), objective, 1, range(0, B, max(1, B // 3)))
@@ -51,16 +55,33 @@ def test_rows_far_off_their_estimates(share, objective):
     # bursts: rows are read on to either side of what was estimated, one cell holds many elements of a row
     rng = np.random.default_rng(3)
     inc = np.where(rng.random((3, 200, 600)) < share, rng.integers(1, 100_000, (3, 200, 600)), rng.integers(1, 50, (3, 200, 600)))
-    check(np.cumsum(inc, axis=2).astype(np.int64), objective)
+    # (SUM, the smaller share: two of the instances keep more cells than there is room for)
+    check(np.cumsum(inc, axis=2).astype(np.int64), objective, leaves=2 if objective == 1 and share == 0.02 else 0)
 
 
 @pytest.mark.parametrize("objective", [0, 1])
 @pytest.mark.parametrize("fast", [1, 20, 45])
-def test_more_answers_from_one_cta_than_its_share(fast, objective):
-    # the first CTA of the cluster has the fast workers, whose elements by the dozen lie in one run of cells
+def test_fast_workers_in_one_cta(fast, objective):
+    # the first CTA of the cluster has the fast workers; SUM: more than the 32 answers that a warp evaluates by itself
     rng = np.random.default_rng(fast)
     m = np.where(np.arange(160) < fast, 1000, 100_000)[None, :, None]
     check(np.cumsum((m * (1 + 0.05 * rng.standard_normal((2, 160, 400)))).astype(np.int64), axis=2), objective)
+
+
+@pytest.mark.parametrize("seed", [0, 1, 3])
+def test_more_answers_from_one_cta_than_its_share_sum(seed):
+    # bursts: one run of cells holds dozens of elements of a row (one to four exchanges an instance fetch answers from where they were put)
+    rng = np.random.default_rng(seed)
+    inc = np.where(rng.random((3, 200, 600)) < 0.03, rng.integers(1, 100_000, (3, 200, 600)), rng.integers(1, 50, (3, 200, 600)))
+    check(np.cumsum(inc, axis=2).astype(np.int64), 1)
+
+
+@pytest.mark.parametrize("jitter", [0, 0.0005])
+def test_more_answers_from_one_cta_than_its_share_range(jitter):
+    # the first CTA has the slow workers, all of one period and close together: forty answers to each of several runs of cells
+    rng = np.random.default_rng(1)
+    m = np.where(np.arange(320) < 40, 100_000, 3000)[None, :, None]
+    check(np.cumsum((m * (1 + jitter * rng.standard_normal((2, 320, 200)))).astype(np.int64), axis=2) + rng.integers(0, 1000, (2, 320, 1)), 0)
 
 
 def on(route, ts, n, R, B, objective):
@@ -72,6 +93,29 @@ def on(route, ts, n, R, B, objective):
     launches, left = h.launches_per_call, h.filter_counts(B)[2]
     h.destroy()
     return sel, launches, left
+
+
+@pytest.mark.parametrize("R", [7, 8, 9, 63, 64])
+@pytest.mark.parametrize("offset", [0, 1, 2, 3])
+def test_a_decrease_is_reported_wherever_it_is(R, offset):
+    # an instance for every place of the decrease, and one without
+    n = 9 if R < 63 else 5
+    places = [f for f in range(n * R) if f % R]
+    ts = np.tile(1000 + 2 * np.arange(1, R + 1), (len(places) + 1, n, 1)).astype(np.int64)
+    flat = ts.reshape(len(places) + 1, n * R)
+    for b, f in enumerate(places):
+        flat[b, f] = flat[b, f - 1] - 1
+    d = torch.empty(offset + ts.size, dtype=torch.int64, device="cuda")[offset:].view(ts.shape)
+    d.copy_(torch.from_numpy(ts))
+    for objective in (0, 1):
+        h = zl.ZipLine(n, R, len(ts), objective, 0, zl.ZL_FLAG_CHECK_SORTED)
+        h.set_option("cells", 1)
+        h.set_option("no_walk", 1)
+        sel = h.select_batched(d)
+        torch.cuda.synchronize()
+        assert h.launches_per_call == 2
+        assert sel.status.tolist() == [zl.binding.ZL_ERR_UNSORTED] * len(places) + [0], objective
+        h.destroy()
 
 
 @pytest.mark.parametrize("recipe", ["c3", "c4"])
@@ -93,15 +137,14 @@ def test_every_form_of_ctas_that_share_an_sm(n, R, B, recipe):
         assert (sel.idx[b].cpu().numpy() == idx).all(), b
 
 
-def test_more_answers_than_a_crowded_cta_has_room_for():
-    # 200 workers fast enough for a run of cells to hold more than 512 elements: the sweep finishes what the cells leave over
-    n, R, B = 220, 100, 1000
+def test_what_crowded_ctas_leave_over():
+    # workers in step: more answers, or more cells, than a CTA of seven an SM has room for; the segment sweep takes the instances
+    n, R, B = 1000, 20, 1000
     rng = np.random.default_rng(4)
-    m = np.where(np.arange(n) < 200, 3_000, 100_000)[None, :, None]
-    ts = np.cumsum((m * (1 + 0.3 * rng.random((4, n, R)))).astype(np.int64), axis=2) + np.where(np.arange(n) < 200, 9_000_000, 0)[None, :, None]
-    d = torch.from_numpy(ts).cuda().repeat(B // 4, 1, 1)
-    sel, launches, _ = on(("cells", "no_walk"), d, n, R, B, 0)
-    assert launches == 2
+    ts = 100_000 * np.arange(1, R + 1) + rng.integers(0, 500, (4, n, R)) + np.where(np.arange(n) < 200, 0, rng.integers(0, 100_000, n))[None, :, None]
+    ts = np.sort(ts.astype(np.int64), axis=2)
+    sel, launches, left = on(("cells", "no_walk"), torch.from_numpy(ts).cuda().repeat(B // 4, 1, 1), n, R, B, 0)
+    assert launches == 2 and max(left) == 1
     for b in (0, 1, 2, 3, B - 1):
         w, t, idx = o.sweep_window(ts[b % 4], 0)
         assert (int(sel.status[b]), int(sel.wait[b]), int(sel.barrier[b])) == (0, w, t), b
