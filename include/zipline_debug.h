@@ -70,6 +70,8 @@ zl_status zl_check_canaries(zl_handle *h, int32_t *buffers, int32_t *damaged);
  * record to h_record[0..3] (host) and clears it: [0] a code naming the access (0: no violation since the last
  * report), [1] the CTA, [2], [3] the low and high word of the offending index.  Covers the kernels of the
  * RANGE filter route that every call runs (k_range_head, k_filter / k_filter_arith, k_tail) and their ring variants.
+ * Such a handle does not take the cell route by itself; told to (option "cells"), it runs kernels there in which every load of the search from
+ * stored rows is compared with the instance or the matrix (not the sortedness check's, and not indices into shared memory).
  */
 zl_status zl_debug_report(zl_handle *h, uint32_t *h_record);
 

@@ -32,6 +32,7 @@
 #include <cmath>
 #include <cooperative_groups.h>
 
+#include "zl_guard.cuh"
 #include "zl_sweep.cuh"
 #include "zl_host.h"
 
@@ -410,6 +411,36 @@ static __device__ bool rows_unsorted(const int64_t *ts, int rows, int R) {
     }
     return bad;
 }
+
+// ------------------------------------------------------------------------------ checked rows
+// Stored rows, every load checked against the instance (single elements) or the matrix (pieces of eight): a bad index is recorded and the
+// load skipped.  For handles with ZL_FLAG_DEBUG_CHECKS that are told to take the route.
+struct MatChecked {
+    const int64_t *ts; uint32_t *record;
+    typedef MatRows Rows;
+    __device__ __forceinline__ MatRows inst(int b, int n, int R) const { return MatRows{ts + (size_t)b * n * R, R}; }
+};
+template <> struct RowReader<MatChecked> : RowReader<MatBatch> {
+    Guard<true> guard; long long before, own, all;                // elements of the matrix before the instance, of the instance, of the matrix
+    __device__ __forceinline__ RowReader(const MatChecked &s, int b, int B, int n, int R_, int64_t tmin)
+        : RowReader<MatBatch>(MatBatch{s.ts}, b, B, n, R_, tmin), guard{s.record, blockIdx.y * gridDim.x + blockIdx.x},
+          before((long long)b * n * R_), own((long long)n * R_), all((long long)B * n * R_) {}
+    __device__ __forceinline__ uint32_t in(int row, int i) const {
+        return guard.ok((uint64_t)((long long)row * R + i), (uint64_t)own, ACC_ROW) ? RowReader<MatBatch>::in(row, i) : 0u;
+    }
+    __device__ __forceinline__ void load(int row, int i, uint64_t (&v)[8]) const {
+        const long long at = before + min(max(row * R + i, first), last);
+        if (last >= first && guard.ok((uint64_t)at, (uint64_t)max(all - 7, 0ll), ACC_ROW_PIECE) &&
+            guard.ok((uintptr_t)(inst + (at - before)) & 31u, 1, ACC_ROW_ALIGN)) {
+            RowReader<MatBatch>::load(row, i, v);
+        } else {
+#pragma unroll
+            for (int k = 0; k < 8; ++k) v[k] = 0;
+        }
+    }
+};
+__host__ __device__ inline MatBatch plain_rows(const MatChecked &s) { return MatBatch{s.ts}; }
+template <class SRC> __host__ __device__ inline SRC plain_rows(const SRC &s) { return s; }
 
 // ------------------------------------------------------------------------------ the search
 struct CellParams {
@@ -858,7 +889,7 @@ __global__ void __launch_bounds__(FORM::THREADS, 1) k_cells(const SRC src, const
         }
     }
     auto sync_cluster = [&]() { if (G > 1) cl.sync(); else __syncthreads(); };      // (a cluster barrier of one CTA takes several times as long)
-    if constexpr (std::is_same<SRC, MatBatch>::value) if (P.check_sorted) {
+    if constexpr (!std::is_same<SRC, AriBatch>::value) if (P.check_sorted) {
         const bool bad = rows_unsorted(src.ts + ((size_t)b * n + r0) * R, nrows, R);
         const int any = __syncthreads_or(bad);
         if (tid < G) map_shared_rank<ONE>(&sh, tid)->exc[rank] = any ? 1ull : 0ull;
@@ -1458,6 +1489,21 @@ static CellShape cell_shape(int n, int R, int B, int objective, int num_sms) {
     return s;
 }
 
+// The kernel of a form.  (Forms with lists of the same length differ in their registers only: one of them is enough for checked rows.)
+template <int OBJ, class SRC>
+static auto cell_kernel(int form) {
+    auto kernel = form == FORM_CLUSTER ? k_cells<OBJ, SRC, CellCluster> : k_cells<OBJ, SRC, CellAlone>;
+    if constexpr (OBJ == ZL_OBJ_RANGE && std::is_same<SRC, MatChecked>::value) {
+        if (form != FORM_CLUSTER && form != FORM_ALONE) kernel = k_cells<OBJ, SRC, CellFive>;
+    } else if constexpr (OBJ == ZL_OBJ_RANGE) {
+        if (form == FORM_THREE) kernel = k_cells<OBJ, SRC, CellThree>;
+        if (form == FORM_FOUR) kernel = k_cells<OBJ, SRC, CellFour>;
+        if (form == FORM_FIVE) kernel = k_cells<OBJ, SRC, CellFive>;
+        if (form == FORM_SEVEN) kernel = k_cells<OBJ, SRC, CellSeven>;
+    }
+    return kernel;
+}
+
 template <int OBJ, class SRC>
 static void enqueue_cells_t(const Pipeline &q, const FilterBufs &fb, const LaunchPlan &p, cudaStream_t st, cudaEvent_t *ev, const SRC &src) {
     const CellShape s = cell_shape(q.n, q.R, q.B, OBJ, q.num_sms);
@@ -1480,14 +1526,7 @@ static void enqueue_cells_t(const Pipeline &q, const FilterBufs &fb, const Launc
         cudaLaunchKernelEx(&cfg, kernel, args...);
     };
     if (q.cells != 3) {
-        auto kernel = s.form == FORM_CLUSTER ? k_cells<OBJ, SRC, CellCluster> : k_cells<OBJ, SRC, CellAlone>;
-        if constexpr (OBJ == ZL_OBJ_RANGE) {
-            if (s.form == FORM_THREE) kernel = k_cells<OBJ, SRC, CellThree>;
-            if (s.form == FORM_FOUR) kernel = k_cells<OBJ, SRC, CellFour>;
-            if (s.form == FORM_FIVE) kernel = k_cells<OBJ, SRC, CellFive>;
-            if (s.form == FORM_SEVEN) kernel = k_cells<OBJ, SRC, CellSeven>;
-        }
-        launch(kernel, dim3(s.cluster, q.B), s.threads, s.smem, s.cluster, src, P);
+        launch(cell_kernel<OBJ, SRC>(s.form), dim3(s.cluster, q.B), s.threads, s.smem, s.cluster, src, P);
     }
     if (ev) for (int k = 1; k < 4; ++k) cudaEventRecord(ev[k], st);
     if (q.cells == 2) return;                                     // the caller looks at the flags itself
@@ -1500,12 +1539,19 @@ static void enqueue_cells_t(const Pipeline &q, const FilterBufs &fb, const Launc
     FilterBufs f = fb;
     f.tailcap = 0x7fffffff;                                       // what the route finished is finished: finalize leaves it alone
     const long long items = std::max<long long>((long long)p.nseg * q.B, ((long long)q.n * q.B + CELL_REST_THREADS - 1) / CELL_REST_THREADS);
-    launch(k_cell_rest<OBJ, SRC>, dim3((unsigned)std::max<long long>(1, std::min<long long>(q.num_sms, items))), CELL_REST_THREADS, p.smem, 1, src, sp, P, f);
+    launch(k_cell_rest<OBJ, decltype(plain_rows(src))>, dim3((unsigned)std::max<long long>(1, std::min<long long>(q.num_sms, items))), CELL_REST_THREADS, p.smem, 1, plain_rows(src), sp, P, f);
     if (ev) cudaEventRecord(ev[4], st);
 }
 
 void enqueue_cells(const Pipeline &q, const FilterBufs &fb, const LaunchPlan &p, cudaStream_t st, cudaEvent_t *ev, const MatBatch &src) {
-    if (q.objective == ZL_OBJ_RANGE) enqueue_cells_t<ZL_OBJ_RANGE>(q, fb, p, st, ev, src); else enqueue_cells_t<ZL_OBJ_SUM>(q, fb, p, st, ev, src);
+    const MatChecked checked{src.ts, q.guard};
+    if (q.guard) {
+        if (q.objective == ZL_OBJ_RANGE) enqueue_cells_t<ZL_OBJ_RANGE>(q, fb, p, st, ev, checked); else enqueue_cells_t<ZL_OBJ_SUM>(q, fb, p, st, ev, checked);
+    } else if (q.objective == ZL_OBJ_RANGE) {
+        enqueue_cells_t<ZL_OBJ_RANGE>(q, fb, p, st, ev, src);
+    } else {
+        enqueue_cells_t<ZL_OBJ_SUM>(q, fb, p, st, ev, src);
+    }
 }
 void enqueue_cells(const Pipeline &q, const FilterBufs &fb, const LaunchPlan &p, cudaStream_t st, cudaEvent_t *ev, const AriBatch &src) {
     if (q.objective == ZL_OBJ_RANGE) enqueue_cells_t<ZL_OBJ_RANGE>(q, fb, p, st, ev, src); else enqueue_cells_t<ZL_OBJ_SUM>(q, fb, p, st, ev, src);
@@ -1518,15 +1564,9 @@ static cudaError_t cell_limits_t() {
         const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
         return e == cudaSuccess ? cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) : e;
     };
-    cudaError_t e = raise(k_cells<OBJ, SRC, CellCluster>);
-    if (e == cudaSuccess) e = raise(k_cells<OBJ, SRC, CellAlone>);
-    if constexpr (OBJ == ZL_OBJ_RANGE) {
-        if (e == cudaSuccess) e = raise(k_cells<OBJ, SRC, CellThree>);
-        if (e == cudaSuccess) e = raise(k_cells<OBJ, SRC, CellFour>);
-        if (e == cudaSuccess) e = raise(k_cells<OBJ, SRC, CellFive>);
-        if (e == cudaSuccess) e = raise(k_cells<OBJ, SRC, CellSeven>);
-    }
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_cell_rest<OBJ, SRC>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
+    cudaError_t e = cudaSuccess;
+    for (int form : {FORM_CLUSTER, FORM_ALONE, FORM_THREE, FORM_FOUR, FORM_FIVE, FORM_SEVEN}) if (e == cudaSuccess) e = raise(cell_kernel<OBJ, SRC>(form));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_cell_rest<OBJ, decltype(plain_rows(std::declval<SRC>()))>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
     return e;
 }
 
@@ -1536,6 +1576,10 @@ cudaError_t cell_limits() {
     if (e == cudaSuccess) e = cell_limits_t<ZL_OBJ_SUM, MatBatch>();
     if (e == cudaSuccess) e = cell_limits_t<ZL_OBJ_SUM, AriBatch>();
     return e;
+}
+cudaError_t cell_checked_limits() {
+    const cudaError_t e = cell_limits_t<ZL_OBJ_RANGE, MatChecked>();
+    return e == cudaSuccess ? cell_limits_t<ZL_OBJ_SUM, MatChecked>() : e;
 }
 
 }  // namespace zl

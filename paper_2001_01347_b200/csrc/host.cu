@@ -75,7 +75,7 @@ struct zl_handle {
     // more survivors than one CTA finishes?); the next call reads it, without waiting, to choose the form of its last stage
     uint32_t *h_hint, *d_hint;
     // cell route
-    uint32_t *d_cflags;      // [0..7] the route's words (see CellParams); [16] the word last written to the hint of the RANGE filter route
+    uint32_t *d_cflags;      // [0..7] the route's words (see CellParams); [24..27] its record of bad indices (ZL_FLAG_DEBUG_CHECKS); [16] the word last written to the hint of the RANGE filter route
     uint32_t cells_epoch;    // number of the last call (any route)
     uint32_t cells_since;    // number of the call with which the present run of calls on the cell route began
     int cells_last;          // the last call of a shape it takes was on it
@@ -385,6 +385,7 @@ zl_status zl_create(const zl_config *cfg, zl_handle **out) {
     const size_t pred_b = (cfg->flags & ZL_FLAG_PREDICTOR) ? (size_t)cfg->max_batch * cfg->n_workers * cfg->lookahead_R * 8 : 0;
     if (e == cudaSuccess && pred_b) e = alloc((void **)&h->d_pred, pred_b);
     if (e == cudaSuccess) e = raise_shared_memory_limits(cfg->device);
+    if (e == cudaSuccess && canaries) e = zl::cell_checked_limits();
     if (e != cudaSuccess) {
         zl_status st = cuda_fail(nullptr, e);
         cudaFree(h->d_meta); cudaFree(h->d_seg); cudaFree(h->d_pred); cudaFree(h->d_cflags);
@@ -557,7 +558,8 @@ static int rest_split_now(const zl_handle *h) {
 // The cell route: every shape that a warp an instance does not take, unless the handle asks for another route (every timestamp
 // examined, self-checks, a tuning knob of the other routes).
 static bool cells_allowed(const zl_handle *h, int B) {
-    return h->d_cflags && !h->opt_no_filter && !(h->cfg.flags & (ZL_FLAG_FULL_SWEEP | ZL_FLAG_DEBUG_CHECKS | ZL_FLAG_FORCE_FILTER)) &&
+    return h->d_cflags && !h->opt_no_filter && !(h->cfg.flags & (ZL_FLAG_FULL_SWEEP | ZL_FLAG_FORCE_FILTER)) &&
+           (h->opt_cells || !(h->cfg.flags & ZL_FLAG_DEBUG_CHECKS)) &&
            !walk_route(h, B) && h->cfg.n_workers >= 4 &&
            !h->opt_filter_bulk && !h->opt_rest_split && !h->opt_filter_round && !h->opt_filter_threads &&
            !h->opt_filter_rows && !h->opt_cluster && !h->opt_tail_cap && !h->opt_tail_threads && !h->opt_prologue_threads && !h->opt_no_cells;
@@ -644,6 +646,7 @@ static bool cells_take(zl_handle *h, int B, uint32_t epoch) {
 }
 static void set_cells(Pipeline &q, zl_handle *h) {
     q.cflags = h->d_cflags;
+    if ((h->cfg.flags & ZL_FLAG_DEBUG_CHECKS) && !h->opt_checks_off) q.guard = h->d_cflags + 24;
     q.epoch = ++h->cells_epoch;
     q.cells = cells_take(h, q.B, q.epoch) ? 1 : 0;
     q.walk = q.ts && walk_take(h, q.B, q.epoch) ? 1 : 0;
@@ -677,7 +680,7 @@ static void fill_pipeline(Pipeline &q, const zl_handle *h, int B) {
     if (h->opt_no_filter) { q.fb.table = nullptr; q.fb.scap = 0; }
     q.cluster = h->opt_cluster; q.filter_stages = h->opt_filter_stages;
     q.checks_off = h->opt_checks_off; q.filter_bulk = h->opt_filter_bulk; q.tail_cap = h->opt_tail_cap; q.rest_per_sm = 0; q.max_rounds = h->opt_max_rounds; q.small = small_route(h) ? 1 : 0; q.walk = 0; q.rest_split = rest_split_now(h) ? 1 : 2;
-    q.cells = 0; q.cflags = nullptr; q.epoch = 0; q.idx = nullptr; q.barrier = q.wait = nullptr; q.status = nullptr;
+    q.cells = 0; q.cflags = q.guard = nullptr; q.epoch = 0; q.idx = nullptr; q.barrier = q.wait = nullptr; q.status = nullptr;
 }
 
 // The identity of the allocation or registration that a pinned pointer belongs to, as the driver counts them (0: none, or unknown).
@@ -702,7 +705,7 @@ static unsigned long long pinned_buffer_id(const void *p) {
 // twice as many after every such call).  The sortedness check reads every row anyway, and SUM enough of them for the bus to be
 // slower in pieces than in one copy (n=1024, R=1024, B=64: 20.7 ms against 11.6; RANGE 3.0 against 9.8).
 static const int64_t *mapped_rows(zl_handle *h, const int64_t *h_ts, int B) {
-    if (h->cfg.objective != ZL_OBJ_RANGE || !cells_allowed(h, B) || (h->cfg.flags & ZL_FLAG_CHECK_SORTED)) return nullptr;
+    if (h->cfg.objective != ZL_OBJ_RANGE || !cells_allowed(h, B) || (h->cfg.flags & (ZL_FLAG_CHECK_SORTED | ZL_FLAG_DEBUG_CHECKS))) return nullptr;
     const long long total = (long long)B * h->cfg.n_workers * h->cfg.lookahead_R;
     if (total < MAPPED_MIN || !cells_fit(h, B)) return nullptr;
     if (h->mapped.wait > 0) { --h->mapped.wait; return nullptr; }
@@ -781,12 +784,15 @@ zl_status zl_check_canaries(zl_handle *h, int32_t *buffers, int32_t *damaged) {
 zl_status zl_debug_report(zl_handle *h, uint32_t *h_record) {
     if (!h || !h_record) return ZL_ERR_INVALID_ARG;
     memset(h_record, 0, 4 * sizeof(uint32_t));
-    if (!h->fb.dbg) return ZL_OK;
+    if (!(h->cfg.flags & ZL_FLAG_DEBUG_CHECKS)) return ZL_OK;
     DeviceScope scope(h->cfg.device);
     ZL_CUDA(h, scope.err);
     ZL_CUDA(h, cudaDeviceSynchronize());
-    ZL_CUDA(h, cudaMemcpy(h_record, h->fb.dbg, 4 * sizeof(uint32_t), cudaMemcpyDeviceToHost));
-    ZL_CUDA(h, cudaMemset(h->fb.dbg, 0, 4 * sizeof(uint32_t)));
+    for (uint32_t *record : {h->fb.dbg, h->d_cflags + 24}) {      // of the filter route, and of the cell route
+        if (!record || h_record[0]) continue;
+        ZL_CUDA(h, cudaMemcpy(h_record, record, 4 * sizeof(uint32_t), cudaMemcpyDeviceToHost));
+        ZL_CUDA(h, cudaMemset(record, 0, 4 * sizeof(uint32_t)));
+    }
     return ZL_OK;
 }
 
@@ -986,6 +992,7 @@ zl_status zl_select_batched_noalloc(int32_t n_workers, int32_t lookahead_R, int3
     q.walk = objective == ZL_OBJ_RANGE && !(flags & ZL_FLAG_FULL_SWEEP) && zl::walk_shape_alone(n_workers, lookahead_R) ? 1 : 0;
     q.cells = !q.walk && !(flags & ZL_FLAG_FULL_SWEEP) && n_workers >= 4 &&
               cells_shape(objective, n_workers, lookahead_R, B, std::max(1, tmp.num_sms), q.small != 0) ? 1 : 0;
+    q.guard = nullptr;
     q.cflags = (uint32_t *)((unsigned char *)g_noalloc_ptr[dev] + NOALLOC_META_BYTES); q.epoch = tmp.cells_epoch;
     enqueue(q, p, (cudaStream_t)cuda_stream, nullptr, zl::MatBatch{d_ts});
     return cudaGetLastError() == cudaSuccess ? ZL_OK : ZL_ERR_CUDA;

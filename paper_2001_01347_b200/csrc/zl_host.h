@@ -39,6 +39,7 @@ struct Pipeline {
     int checks_off;                                               // debug handle: unchecked kernels, clock stamps still taken
     int cells;                                                    // 1: the cell route; 2: its search only, without the kernel for what it leaves over; 3: that kernel only
     uint32_t *cflags, epoch;                                      // its eight words; the number of the call
+    uint32_t *guard;                                              // its record of bad indices (nullptr: rows are read unchecked)
     int32_t *idx; int64_t *barrier; int64_t *wait; int32_t *status;
 };
 
@@ -102,6 +103,7 @@ cudaError_t bucket_route_limits();
 void enqueue_cells(const Pipeline &q, const FilterBufs &fb, const LaunchPlan &p, cudaStream_t st, cudaEvent_t *ev, const MatBatch &src);
 void enqueue_cells(const Pipeline &q, const FilterBufs &fb, const LaunchPlan &p, cudaStream_t st, cudaEvent_t *ev, const AriBatch &src);
 cudaError_t cell_limits();
+cudaError_t cell_checked_limits();                                // ... of the kernels that check their rows
 
 // walk.cu: RANGE, small instances of up to 128 workers, a warp per instance in one launch
 bool walk_shape(int n, int R, int batch, int num_sms);

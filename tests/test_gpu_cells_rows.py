@@ -84,6 +84,28 @@ def test_more_answers_from_one_cta_than_its_share_range(jitter):
     check(np.cumsum((m * (1 + jitter * rng.standard_normal((2, 320, 200)))).astype(np.int64), axis=2) + rng.integers(0, 1000, (2, 320, 1)), 0)
 
 
+@pytest.mark.parametrize("objective", [0, 1])
+@pytest.mark.parametrize("offset", [0, 1, 2, 3])
+@pytest.mark.parametrize("n,R,B", [(4, 2, 1), (7, 9, 2), (24, 60, 1), (128, 20, 100), (90, 60, 700), (1088, 64, 64), (1088, 128, 32), (1280, 32, 64), (300, 400, 2)])
+def test_every_load_of_the_rows_is_inside_them(n, R, B, offset, objective):
+    ts = zi.generate(zi.CONFIGS["c1"].with_(B=B, n=n, R=R))
+    d = torch.empty(offset + ts.size, dtype=torch.int64, device="cuda")[offset:].view(ts.shape)
+    d.copy_(torch.from_numpy(ts))
+    h = zl.ZipLine(n, R, B, objective, 0, zl.ZL_FLAG_DEBUG_CHECKS)
+    h.set_option("cells", 1)
+    h.set_option("no_walk", 1)
+    sel = h.select_batched(d)
+    torch.cuda.synchronize()
+    assert h.launches_per_call == 2 and max(h.filter_counts(B)[2]) == 0
+    assert h.debug_report() == (0, 0, 0)
+    assert h.check_canaries()[1] == 0
+    for b in (0, B - 1):
+        w, t, idx = o.sweep_window(ts[b], objective)
+        assert (int(sel.status[b]), int(sel.wait[b]), int(sel.barrier[b])) == (0, w, t), b
+        assert (sel.idx[b].cpu().numpy() == idx).all(), b
+    h.destroy()
+
+
 def on(route, ts, n, R, B, objective):
     h = zl.ZipLine(n, R, B, objective, 0)
     for option in route:
