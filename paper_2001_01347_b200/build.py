@@ -3,6 +3,7 @@ from __future__ import annotations
 
 import glob
 import os
+import re
 import shutil
 import subprocess
 from concurrent.futures import ThreadPoolExecutor
@@ -22,6 +23,12 @@ def sources() -> list[str]:
 def headers() -> list[str]:
     return sorted(glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(CSRC, "*.h"))
                   + glob.glob(os.path.join(INCLUDE, "*.h")))
+
+
+def _changed(src: str) -> float:
+    """When the source, or a source that it includes, was last changed."""
+    included = re.findall(r'^#include "(\w+\.cu)"', open(src).read(), re.M)
+    return max(os.path.getmtime(f) for f in [src] + [os.path.join(CSRC, i) for i in included])
 
 
 def _nvcc() -> str:
@@ -50,7 +57,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
     os.makedirs(OBJ, exist_ok=True)
     newest_header = max(os.path.getmtime(h) for h in headers())
     todo = [s for s in sources()
-            if force or not os.path.exists(_obj(s)) or os.path.getmtime(_obj(s)) < max(os.path.getmtime(s), newest_header)]
+            if force or not os.path.exists(_obj(s)) or os.path.getmtime(_obj(s)) < max(_changed(s), newest_header)]
 
     def compile_one(src: str):
         cmd = [nvcc] + NVCC_FLAGS + (["-Xptxas", "-v"] if verbose else []) + ["-c", "-o", _obj(src), src]

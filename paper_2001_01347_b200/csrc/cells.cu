@@ -520,7 +520,7 @@ __device__ __forceinline__ uint32_t cell_end(uint32_t start, uint32_t shift, uin
     return start + min((1u << shift) - 1u, limit - 1u - start);
 }
 
-__device__ __noinline__ bool was_asked(const uint2 *runs, int n, uint32_t c) {
+static __device__ __noinline__ bool was_asked(const uint2 *runs, int n, uint32_t c) {
     bool is = false;
 #pragma unroll 1
     for (int k = 0; k < n; ++k) is |= runs[k].x <= c && c <= runs[k].y;
@@ -1386,6 +1386,16 @@ __global__ void __launch_bounds__(FORM::THREADS, 1) k_cells(const SRC src, const
     if (G > 1) cl.barrier_wait();
 }
 
+// ------------------------------------------------------------------------------ the kernels of the forms
+// Three modules: a module is loaded whole when one of its kernels is first named, and the forms for many instances are named only for handles that make
+// such calls, the checked ones only for handles that ask for checks (all in one: the first handle of a process 28 ms, 20 before the forms).
+enum CellFormOf { FORM_CLUSTER, FORM_ALONE, FORM_THREE, FORM_FOUR, FORM_FIVE, FORM_SEVEN };
+template <class SRC> using CellKernel = void (*)(const SRC, const CellParams);
+CellKernel<MatBatch> cell_kernel_crowded(MatBatch, int form);         // RANGE; cells_crowded.cu
+CellKernel<AriBatch> cell_kernel_crowded(AriBatch, int form);
+CellKernel<MatChecked> cell_kernel_checked(int objective, int form);  // cells_checked.cu
+
+#ifndef ZL_CELLS_KERNELS_ONLY      // (cells_crowded.cu and cells_checked.cu take the search from here)
 // ------------------------------------------------------------------------------ rest
 constexpr int CELL_REST_THREADS = 512;
 
@@ -1409,7 +1419,6 @@ __global__ void __launch_bounds__(CELL_REST_THREADS) k_cell_rest(const SRC src, 
 
 // ------------------------------------------------------------------------------ host side
 // CTAs of an instance's cluster, their threads, and the cells each has room for.
-enum CellFormOf { FORM_CLUSTER, FORM_ALONE, FORM_THREE, FORM_FOUR, FORM_FIVE, FORM_SEVEN };
 struct CellShape { int cluster, threads, form, cap; size_t smem; };
 
 // What a form takes of an SM: most threads, shared memory that the kernel declares, and (`dynamic`) what lies behind the cells.
@@ -1489,19 +1498,12 @@ static CellShape cell_shape(int n, int R, int B, int objective, int num_sms) {
     return s;
 }
 
-// The kernel of a form.  (Forms with lists of the same length differ in their registers only: one of them is enough for checked rows.)
 template <int OBJ, class SRC>
-static auto cell_kernel(int form) {
-    auto kernel = form == FORM_CLUSTER ? k_cells<OBJ, SRC, CellCluster> : k_cells<OBJ, SRC, CellAlone>;
-    if constexpr (OBJ == ZL_OBJ_RANGE && std::is_same<SRC, MatChecked>::value) {
-        if (form != FORM_CLUSTER && form != FORM_ALONE) kernel = k_cells<OBJ, SRC, CellFive>;
-    } else if constexpr (OBJ == ZL_OBJ_RANGE) {
-        if (form == FORM_THREE) kernel = k_cells<OBJ, SRC, CellThree>;
-        if (form == FORM_FOUR) kernel = k_cells<OBJ, SRC, CellFour>;
-        if (form == FORM_FIVE) kernel = k_cells<OBJ, SRC, CellFive>;
-        if (form == FORM_SEVEN) kernel = k_cells<OBJ, SRC, CellSeven>;
-    }
-    return kernel;
+static CellKernel<SRC> cell_kernel(int form) {
+    if constexpr (std::is_same<SRC, MatChecked>::value) return cell_kernel_checked(OBJ, form);
+    else if (form == FORM_CLUSTER) return k_cells<OBJ, SRC, CellCluster>;
+    else if (form == FORM_ALONE) return k_cells<OBJ, SRC, CellAlone>;
+    else return cell_kernel_crowded(SRC(), form);
 }
 
 template <int OBJ, class SRC>
@@ -1558,28 +1560,40 @@ void enqueue_cells(const Pipeline &q, const FilterBufs &fb, const LaunchPlan &p,
 }
 
 template <int OBJ, class SRC>
-static cudaError_t cell_limits_t() {
+static cudaError_t cell_limits_t(bool crowded) {
     const int big = 200 * 1024;
     auto raise = [&](auto kernel) {
         const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
         return e == cudaSuccess ? cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) : e;
     };
     cudaError_t e = cudaSuccess;
-    for (int form : {FORM_CLUSTER, FORM_ALONE, FORM_THREE, FORM_FOUR, FORM_FIVE, FORM_SEVEN}) if (e == cudaSuccess) e = raise(cell_kernel<OBJ, SRC>(form));
+    if (crowded) {
+        for (int form : {FORM_THREE, FORM_FOUR, FORM_FIVE, FORM_SEVEN}) if (e == cudaSuccess) e = raise(cell_kernel<OBJ, SRC>(form));
+        return e;
+    }
+    for (int form : {FORM_CLUSTER, FORM_ALONE}) if (e == cudaSuccess) e = raise(cell_kernel<OBJ, SRC>(form));
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_cell_rest<OBJ, decltype(plain_rows(std::declval<SRC>()))>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
     return e;
 }
 
 cudaError_t cell_limits() {
-    cudaError_t e = cell_limits_t<ZL_OBJ_RANGE, MatBatch>();
-    if (e == cudaSuccess) e = cell_limits_t<ZL_OBJ_RANGE, AriBatch>();
-    if (e == cudaSuccess) e = cell_limits_t<ZL_OBJ_SUM, MatBatch>();
-    if (e == cudaSuccess) e = cell_limits_t<ZL_OBJ_SUM, AriBatch>();
+    cudaError_t e = cell_limits_t<ZL_OBJ_RANGE, MatBatch>(false);
+    if (e == cudaSuccess) e = cell_limits_t<ZL_OBJ_RANGE, AriBatch>(false);
+    if (e == cudaSuccess) e = cell_limits_t<ZL_OBJ_SUM, MatBatch>(false);
+    if (e == cudaSuccess) e = cell_limits_t<ZL_OBJ_SUM, AriBatch>(false);
     return e;
 }
-cudaError_t cell_checked_limits() {
-    const cudaError_t e = cell_limits_t<ZL_OBJ_RANGE, MatChecked>();
-    return e == cudaSuccess ? cell_limits_t<ZL_OBJ_SUM, MatChecked>() : e;
+bool cell_crowded(int objective, int B, int num_sms) { return objective == ZL_OBJ_RANGE && B > 2 * num_sms; }
+cudaError_t cell_crowded_limits() {
+    const cudaError_t e = cell_limits_t<ZL_OBJ_RANGE, MatBatch>(true);
+    return e == cudaSuccess ? cell_limits_t<ZL_OBJ_RANGE, AriBatch>(true) : e;
 }
+cudaError_t cell_checked_limits() {
+    cudaError_t e = cell_limits_t<ZL_OBJ_RANGE, MatChecked>(false);
+    if (e == cudaSuccess) e = cell_limits_t<ZL_OBJ_RANGE, MatChecked>(true);
+    return e == cudaSuccess ? cell_limits_t<ZL_OBJ_SUM, MatChecked>(false) : e;
+}
+
+#endif
 
 }  // namespace zl
