@@ -27,6 +27,10 @@
 // instructions and latencies of looking through rows (2000 cycles for 32 pieces of eight elements with 20 warps an SM, n=1024,
 // R=1024, B=64 16 of 37 us in the kernel), not what it moves (2.8 TB/s there).
 //
+// Times in this file are us a call of one seed's inputs that stay the same from call to call, unless said otherwise: they compare two ways of
+// doing something.  With inputs that change a call takes longer (n=1024, R=1024, B=64 51 instead of 44 to 46, n=128, R=256, B=1024 43 instead of 37
+// to 40), since nothing of the rows is in the L2.
+//
 // Every CTA of a cluster passes the same cluster barriers: whatever a loop or a branch around one depends on is the same
 // value in the whole cluster (never the CTA's own number of rows or cells).
 #include <cmath>
@@ -47,7 +51,7 @@ constexpr int CELL_PAIRS = 256;           // answers that a batch of cells shoul
 constexpr int CELL_CLUSTER = 16;          // most CTAs of a cluster
 // The forms of the kernel.  ONE: an instance has one CTA, and what only clusters need falls away; THREADS: most threads of an SM, and so the
 // registers of a thread; ROWS: rows that are looked through at a time, NODES: most elements in the cells that the rows are asked for at once.
-// With 96 registers (640 threads) nothing is spilled, with 72 8 bytes outside the loops, with 64 72 bytes; a cluster's kernel with 72 or 64
+// With 96 registers (640 threads) and with 72 nothing is spilled, with 80 20 bytes, with 64 48 bytes; a cluster's kernel with 72 or 64
 // spills inside the loops, and what is spilled has often left the L1 cache, past which the rows stream, by the time it is wanted back (n=1024, R=1024,
 // B=64 55 and 74 us, 44 with 96).  CTAs get registers for four warps at a time, so that 96 are good for five small CTAs an SM, 72 for seven: a thousand
 // instances are one turn instead of 1.4 (n=128, R=256, B=1024 53 us with 96, 40 with 72; n=181, R=18, B=1795 60 / 54; predicted n=131, R=41,
