@@ -58,10 +58,15 @@ constexpr int CELL_CLUSTER = 16;          // most CTAs of a cluster
 // B=1760 44 / 37).  Three CTAs of 256 threads fit with 80 (n=350, R=157, B=373 53 us with 96 and 128 threads, 44 with 80), four with 64 (n=400, R=100,
 // B=480 48 us with 96 and 128 threads, 43 with 64; n=22, R=537, B=565 54 / 49; but instances of 128 threads' work: n=30, R=60, B=580 28 / 31).
 // With lists half as long (ROWS, NODES) there is room for 1400 cells more where seven CTAs share an SM.
+// SUM, 128 threads of 96 registers / 256 of 80, three an SM (new inputs every call): n=256, R=256, B=300 282 / 194 us, n=300, R=300, B=330 167 / 127, n=128, R=128,
+// B=400 59 / 48, n=64, R=30, B=440 24.2 / 23.2; of 64, four an SM: n=200, R=200, B=500 104 / 91, n=400, R=100, B=480 136 / 122, n=256, R=100, B=512 107 / 99;
+// but instances of up to 64 timestamps a thread n=100, R=60, B=560 41.1 / 41.5, n=128, R=40, B=590 37.2 / 38.3.  (All with as many cells.)
 template <bool ONE_, int THREADS_, int ROWS_, int NODES_>
 struct CellForm { static constexpr bool ONE = ONE_; static constexpr int THREADS = THREADS_, ROWS = ROWS_, NODES = NODES_, CTAS = ONE_ ? 1 : CELL_CLUSTER; };
 typedef CellForm<false, 640, 1024, 1024> CellCluster;
-typedef CellForm<true, 640, 1024, 1024> CellAlone;        // up to two CTAs an SM, and SUM
+typedef CellForm<true, 640, 1024, 1024> CellAlone;        // up to two CTAs an SM, and SUM five and more
+typedef CellForm<true, 768, 1024, 1024> CellThreeSum;     // SUM: three an SM,
+typedef CellForm<true, 1024, 1024, 1024> CellFourSum;     // four
 typedef CellForm<true, 768, 512, 512> CellThree;          // RANGE: three an SM,
 typedef CellForm<true, 1024, 512, 512> CellFour;          // four, or eight,
 typedef CellForm<true, 640, 512, 512> CellFive;           // four of 128 threads, or five,
@@ -1391,15 +1396,17 @@ __global__ void __launch_bounds__(FORM::THREADS, 1) k_cells(const SRC src, const
 }
 
 // ------------------------------------------------------------------------------ the kernels of the forms
-// Three modules: a module is loaded whole when one of its kernels is first named, and the forms for many instances are named only for handles that make
+// Modules of their own: a module is loaded whole when one of its kernels is first named, and the forms for many instances are named only for handles that make
 // such calls, the checked ones only for handles that ask for checks (all in one: the first handle of a process 28 ms, 20 before the forms).
 enum CellFormOf { FORM_CLUSTER, FORM_ALONE, FORM_THREE, FORM_FOUR, FORM_FIVE, FORM_SEVEN };
 template <class SRC> using CellKernel = void (*)(const SRC, const CellParams);
 CellKernel<MatBatch> cell_kernel_crowded(MatBatch, int form);         // RANGE; cells_crowded.cu
 CellKernel<AriBatch> cell_kernel_crowded(AriBatch, int form);
+CellKernel<MatBatch> cell_kernel_crowded_sum(MatBatch, int form);     // SUM; cells_crowded_sum.cu
+CellKernel<AriBatch> cell_kernel_crowded_sum(AriBatch, int form);
 CellKernel<MatChecked> cell_kernel_checked(int objective, int form);  // cells_checked.cu
 
-#ifndef ZL_CELLS_KERNELS_ONLY      // (cells_crowded.cu and cells_checked.cu take the search from here)
+#ifndef ZL_CELLS_KERNELS_ONLY      // (cells_crowded.cu, cells_crowded_sum.cu and cells_checked.cu take the search from here)
 // ------------------------------------------------------------------------------ rest
 constexpr int CELL_REST_THREADS = 512;
 
@@ -1433,7 +1440,10 @@ static CellRoom cell_room_t() {
     return CellRoom{FORM::THREADS, sizeof(CellShared<OBJ, FORM>), (d + 15) & ~(size_t)15};
 }
 static CellRoom cell_room(int objective, int form) {
-    if (objective != ZL_OBJ_RANGE) return form == FORM_CLUSTER ? cell_room_t<ZL_OBJ_SUM, CellCluster>() : cell_room_t<ZL_OBJ_SUM, CellAlone>();
+    if (objective != ZL_OBJ_RANGE) {
+        return form == FORM_CLUSTER ? cell_room_t<ZL_OBJ_SUM, CellCluster>() : form == FORM_THREE ? cell_room_t<ZL_OBJ_SUM, CellThreeSum>()
+               : form == FORM_FOUR ? cell_room_t<ZL_OBJ_SUM, CellFourSum>() : cell_room_t<ZL_OBJ_SUM, CellAlone>();
+    }
     switch (form) {
         case FORM_CLUSTER: return cell_room_t<ZL_OBJ_RANGE, CellCluster>();
         case FORM_THREE: return cell_room_t<ZL_OBJ_RANGE, CellThree>();
@@ -1474,7 +1484,7 @@ static CellShape cell_shape(int n, int R, int B, int objective, int num_sms) {
     // but one turn of seven, n=128, R=256, B=1024 50 / 37).
     auto turns = [&](int per_sm) { return (ctas + per_sm * num_sms - 1) / (per_sm * num_sms); };
     const long long N = (long long)n * R;
-    s.form = s.cluster > 1 ? FORM_CLUSTER : !crowded ? FORM_ALONE : share == 3 ? FORM_THREE : share == 4 && N > 128 * 24 ? FORM_FOUR : share < 6 ? FORM_FIVE
+    s.form = s.cluster > 1 ? FORM_CLUSTER : share < 3 ? FORM_ALONE : !crowded ? (share == 3 ? FORM_THREE : share == 4 && N > 8192 ? FORM_FOUR : FORM_ALONE) : share == 3 ? FORM_THREE : share == 4 && N > 128 * 24 ? FORM_FOUR : share < 6 ? FORM_FIVE
              : turns(8) < turns(7) && n <= 384 && cells_in(FORM_FOUR, 196.0) >= least_cells ? FORM_FOUR : N >= 12288 && turns(7) > 1 ? FORM_FIVE : FORM_SEVEN;
     // threads: as many as an SM holds, whose registers CTAs get for four warps at a time
     s.threads = 128 * std::max(1, cell_room(objective, s.form).threads / 128 / share);
@@ -1507,6 +1517,7 @@ static CellKernel<SRC> cell_kernel(int form) {
     if constexpr (std::is_same<SRC, MatChecked>::value) return cell_kernel_checked(OBJ, form);
     else if (form == FORM_CLUSTER) return k_cells<OBJ, SRC, CellCluster>;
     else if (form == FORM_ALONE) return k_cells<OBJ, SRC, CellAlone>;
+    else if constexpr (OBJ == ZL_OBJ_SUM) return cell_kernel_crowded_sum(SRC(), form);
     else return cell_kernel_crowded(SRC(), form);
 }
 
@@ -1572,7 +1583,8 @@ static cudaError_t cell_limits_t(bool crowded) {
     };
     cudaError_t e = cudaSuccess;
     if (crowded) {
-        for (int form : {FORM_THREE, FORM_FOUR, FORM_FIVE, FORM_SEVEN}) if (e == cudaSuccess) e = raise(cell_kernel<OBJ, SRC>(form));
+        for (int form : {FORM_THREE, FORM_FOUR, FORM_FIVE, FORM_SEVEN})
+            if (e == cudaSuccess && (OBJ == ZL_OBJ_RANGE || form <= FORM_FOUR)) e = raise(cell_kernel<OBJ, SRC>(form));
         return e;
     }
     for (int form : {FORM_CLUSTER, FORM_ALONE}) if (e == cudaSuccess) e = raise(cell_kernel<OBJ, SRC>(form));
@@ -1587,10 +1599,11 @@ cudaError_t cell_limits() {
     if (e == cudaSuccess) e = cell_limits_t<ZL_OBJ_SUM, AriBatch>(false);
     return e;
 }
-bool cell_crowded(int objective, int B, int num_sms) { return objective == ZL_OBJ_RANGE && B > 2 * num_sms; }
-cudaError_t cell_crowded_limits() {
-    const cudaError_t e = cell_limits_t<ZL_OBJ_RANGE, MatBatch>(true);
-    return e == cudaSuccess ? cell_limits_t<ZL_OBJ_RANGE, AriBatch>(true) : e;
+bool cell_crowded(int B, int num_sms) { return B > 2 * num_sms; }
+cudaError_t cell_crowded_limits(int objective) {
+    const bool sum = objective != ZL_OBJ_RANGE;
+    const cudaError_t e = sum ? cell_limits_t<ZL_OBJ_SUM, MatBatch>(true) : cell_limits_t<ZL_OBJ_RANGE, MatBatch>(true);
+    return e != cudaSuccess ? e : sum ? cell_limits_t<ZL_OBJ_SUM, AriBatch>(true) : cell_limits_t<ZL_OBJ_RANGE, AriBatch>(true);
 }
 cudaError_t cell_checked_limits() {
     cudaError_t e = cell_limits_t<ZL_OBJ_RANGE, MatChecked>(false);

@@ -164,16 +164,17 @@ void enqueue(const Pipeline &q, const LaunchPlan &p, cudaStream_t st, cudaEvent_
 
 std::mutex g_limits_mutex;
 unsigned long long g_limits_done;                              // bit d: done for device d (devices beyond the 64th: every time)
-unsigned long long g_crowded_done;                             // the same for the cell route's forms for many instances
+unsigned long long g_crowded_done[2];                          // the same for the cell route's forms for many instances, by objective
 
 // More than the default 48 KB of dynamic shared memory for the kernels that take it: once a device, not with every handle.  `crowded`:
-// also for the cell route's forms for many instances (their module is loaded when one of them is first named).
-cudaError_t raise_shared_memory_limits(int device, bool crowded) {
+// also for the cell route's forms for many instances of the objective (their module is loaded when one of them is first named).
+cudaError_t raise_shared_memory_limits(int device, int objective, bool crowded) {
     std::lock_guard<std::mutex> lock(g_limits_mutex);
-    if (crowded && !(device < 64 && (g_crowded_done >> device) & 1ull)) {
-        const cudaError_t e = zl::cell_crowded_limits();
+    unsigned long long &done = g_crowded_done[objective == ZL_OBJ_RANGE ? 0 : 1];
+    if (crowded && !(device < 64 && (done >> device) & 1ull)) {
+        const cudaError_t e = zl::cell_crowded_limits(objective);
         if (e != cudaSuccess) return e;
-        if (device < 64) g_crowded_done |= 1ull << device;
+        if (device < 64) done |= 1ull << device;
     }
     if (device < 64 && (g_limits_done >> device) & 1ull) return cudaSuccess;
     cudaError_t e = zl::prologue_limits();
@@ -391,7 +392,7 @@ zl_status zl_create(const zl_config *cfg, zl_handle **out) {
     if (e == cudaSuccess) e = alloc((void **)&h->d_seg, seg_b);
     const size_t pred_b = (cfg->flags & ZL_FLAG_PREDICTOR) ? (size_t)cfg->max_batch * cfg->n_workers * cfg->lookahead_R * 8 : 0;
     if (e == cudaSuccess && pred_b) e = alloc((void **)&h->d_pred, pred_b);
-    if (e == cudaSuccess) e = raise_shared_memory_limits(cfg->device, zl::cell_crowded(cfg->objective, cfg->max_batch, h->num_sms));
+    if (e == cudaSuccess) e = raise_shared_memory_limits(cfg->device, cfg->objective, zl::cell_crowded(cfg->max_batch, h->num_sms));
     if (e == cudaSuccess && canaries) e = zl::cell_checked_limits();
     if (e != cudaSuccess) {
         zl_status st = cuda_fail(nullptr, e);
@@ -971,7 +972,8 @@ zl_status zl_select_batched_noalloc(int32_t n_workers, int32_t lookahead_R, int3
             void *ptr = nullptr;
             cudaError_t e = cudaGetSymbolAddress((void **)&ptr, g_noalloc_scratch);
             if (e == cudaSuccess) e = cudaDeviceGetAttribute(&g_noalloc_sms[dev], cudaDevAttrMultiProcessorCount, dev);
-            if (e == cudaSuccess) e = raise_shared_memory_limits(dev, zl::cell_crowded(ZL_OBJ_RANGE, NOALLOC_MAX_BATCH, g_noalloc_sms[dev]));
+            for (int o : {(int)ZL_OBJ_RANGE, (int)ZL_OBJ_SUM})
+                if (e == cudaSuccess) e = raise_shared_memory_limits(dev, o, zl::cell_crowded(NOALLOC_MAX_BATCH, g_noalloc_sms[dev]));
             if (e != cudaSuccess || !ptr) return ZL_ERR_CUDA;
             g_noalloc_ptr[dev] = ptr;
         }

@@ -103,8 +103,8 @@ cudaError_t bucket_route_limits();
 void enqueue_cells(const Pipeline &q, const FilterBufs &fb, const LaunchPlan &p, cudaStream_t st, cudaEvent_t *ev, const MatBatch &src);
 void enqueue_cells(const Pipeline &q, const FilterBufs &fb, const LaunchPlan &p, cudaStream_t st, cudaEvent_t *ev, const AriBatch &src);
 cudaError_t cell_limits();
-bool cell_crowded(int objective, int B, int num_sms);             // calls of so many instances may take the forms for three and more CTAs an SM ...
-cudaError_t cell_crowded_limits();                                // ... which are loaded only for handles that make such calls
+bool cell_crowded(int B, int num_sms);                            // calls of so many instances may take the forms for three and more CTAs an SM ...
+cudaError_t cell_crowded_limits(int objective);                   // ... which are loaded only for handles that make such calls
 cudaError_t cell_checked_limits();                                // ... of the kernels that check their rows
 
 // walk.cu: RANGE, small instances of up to 128 workers, a warp per instance in one launch

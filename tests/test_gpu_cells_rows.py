@@ -159,6 +159,24 @@ def test_every_form_of_ctas_that_share_an_sm(n, R, B, recipe):
         assert (sel.idx[b].cpu().numpy() == idx).all(), b
 
 
+@pytest.mark.parametrize("recipe", ["c3", "c4"])
+@pytest.mark.parametrize("n,R,B", [(90, 60, 297), (90, 100, 400), (1024, 16, 300), (1025, 16, 300), (100, 60, 444), (128, 64, 445), (129, 64, 445), (90, 120, 592), (90, 120, 593)])
+def test_every_form_of_ctas_that_share_an_sm_sum(n, R, B, recipe):
+    # three and four CTAs an SM, the first and last batch of each, few and many timestamps, one list of rows and more than one.  (A form
+    # that gave up would leave every instance to the segment sweep; that a few keep too many cells depends on their rows.)
+    d = torch.from_numpy(zi.generate(zi.CONFIGS[recipe].with_(B=B, n=n, R=R))).cuda()
+    sel, launches, left = on(("cells", "no_walk"), d, n, R, B, 1)
+    assert launches == 2 and sum(x != 0 for x in left) < B // 10
+    other, launches, _ = on(("no_cells", "no_walk"), d, n, R, B, 1)
+    assert launches != 2
+    for a, b in zip((sel.idx, sel.barrier, sel.wait, sel.status), (other.idx, other.barrier, other.wait, other.status)):
+        assert torch.equal(a, b)
+    for b in range(0, B, B // 4):
+        w, t, idx = o.sweep_window(d[b].cpu().numpy(), 1)
+        assert (int(sel.wait[b]), int(sel.barrier[b])) == (w, t), b
+        assert (sel.idx[b].cpu().numpy() == idx).all(), b
+
+
 def test_what_crowded_ctas_leave_over():
     # workers in step: more answers, or more cells, than a CTA of seven an SM has room for; the segment sweep takes the instances
     n, R, B = 1000, 20, 1000
