@@ -409,7 +409,7 @@ def main():
                "sample": f"the first {inst} of {w.B} instances of {w.name}, sweep_window (sort + one pass), {dt:.1f} s wall"}
 
     result = {"selections_per_s": world * w.B / (ms_step * 1e-3), "early_stop": route == 1,
-              "route": "cells" if h_launches == 2 else {0: "segment sweep", 1: "filter", 2: "buckets", 3: "one launch"}[route],
+              "route": "cells" if h_launches == 2 else "one launch" if h_launches == 1 else {0: "segment sweep", 1: "filter", 2: "buckets", 3: "one launch"}[route],
               "examined_fraction": examined / nts, "input_copies": copies,
               "value_counts": "all n*R*B timestamps of the batch per call (nominal: the early stop examines examined_fraction of them; "
                               "full_sweep.value counts examined timestamps only)",
